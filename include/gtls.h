@@ -82,7 +82,10 @@ typedef struct {
                                    the tensor-core window kernel waits about 1 ms on a barrier
                                    phase that nothing completes, records the timeout and stops,
                                    so that the search returns GTLS_ERR_TIMEOUT: a test of the
-                                   bounded-wait path that faults nothing */
+                                   bounded-wait path that faults nothing.  Bit 1: every window
+                                   is summed (no window is ruled out by its bound), bit 2: the
+                                   bounds are used however small the search; for tests that
+                                   compare the two, results are the same */
 } gtls_plan_params;
 
 /* Sizes of a plan (host struct filled by gtls_plan_get_info). */

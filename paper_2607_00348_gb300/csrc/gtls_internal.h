@@ -12,6 +12,26 @@
 
 namespace gtls {
 
+// Template of one duration cut into pieces for the bounds of the window
+// search (window_bounds.cuh): a few wide pieces that start at whole T0 steps
+// (first test of a window) and kBoundSegs segments (second test).
+constexpr int kBoundCuts = 13;
+constexpr int kBoundSegs = 25;
+struct BoundTab {
+    float mean_all, nu_all;       // mean of s_k, >= ||s_k - mean||
+    float root_t2;                // sqrt(sum_k s_k^2)
+    float t_max;                  // >= |s_k|
+    int32_t cuts;                 // wide pieces (0: the window sum alone is tested)
+    int32_t cut_row[kBoundCuts];  // their first T0 step
+    float cut_coef[kBoundCuts + 1];   // mean of the piece before minus mean of the piece (Abel form)
+    float cut_nu[kBoundCuts];     // >= ||s_k - mean|| over the piece
+    int32_t cut_len[kBoundCuts];  // its points
+    int32_t off[kBoundSegs + 1];  // segments [off[g], off[g + 1])
+    float mean[kBoundSegs];       // mean of s_k over the segment
+    float nu[kBoundSegs];         // >= ||s_k - mean|| over the segment
+    float inv_len[kBoundSegs];    // <= 1 / length (0 for an empty segment)
+};
+
 // Read-only plan tables on the device (passed to kernels by value).
 struct DevPlan {
     int64_t n;
@@ -49,6 +69,7 @@ struct DevPlan {
     int32_t median_half;        // half width h of the running-median window
     int32_t refine_k;           // periods re-searched with T0 step 1 (0: none)
     const int64_t* tc_off;      // offset of duration j in tc_tab (floats; kTensor durations)
+    const BoundTab* bounds;     // pieces of every duration's template
     const float* tc_tab;        // tensor-core template chunks: [chunk][hi, lo][32 x 32 core-matrix layout]
 };
 
@@ -64,12 +85,14 @@ struct DevCurve {
     int64_t* d_lat;           // rint((t - t_ref) 2^e)
     float* d_f;               // float(t - t_ref) (days): coarse cycle estimate
     PointVals* pv;            // rfx, r, w of every point
-    double* scal;             // [0] t_ref [1] chi2_0 [2] uniform weight w (0 if not uniform)
+    double* scal;             // [0] t_ref [1] chi2_0 [2] uniform weight w (0 if not uniform) [3] prefix shift
     unsigned long long* tmin_key;  // ordered key of min(t)
     unsigned int* flags;      // bit0 non-finite, bit1 dy <= 0, bit2 dy not uniform
     double* part;             // block partials of chi2_0
     unsigned int* check;      // [0] first failed device check (0 = none), [1..3] its values
 };
+
+constexpr int kListClasses = 6;   // windows are summed by groups of 1, 2, 4, ..., 32 lanes
 
 // Per-chunk scratch: `chunk` periods in flight.
 struct DevChunk {
@@ -83,6 +106,13 @@ struct DevChunk {
     float* ws;                // folded w (per-point weights only)
     float* wrs;               // folded w r (per-point weights only)
     long long* pf;            // prefix sums of rfx over the padded folded curve
+    // bounds kernel (uniform weights): the prefix sums in 32 bits, and what it
+    // leaves to sum in the wave
+    int32_t* pq;              // pf >> prefix_shift (modulo 2^32: window sums fit 31 bits)
+    int64_t list_cap;         // windows per lane-group size
+    unsigned long long* list; // windows to sum, kListClasses lists
+    int2* dense;              // (slot, tile) items for the tiled kernel
+    unsigned int* left_n;     // [0 .. kListClasses) windows listed, [kListClasses] items in `dense`
 };
 
 // Per-period outputs (np long) and the reduction scratch.
@@ -168,6 +198,7 @@ struct gtls_plan {
     // [jlo, jhi] span of a period (work items per period of that kernel),
     // its counter, and the timeout test (a wait that nothing completes)
     bool has_tensor = false;
+    bool bounds_ok = false;              // the templates admit the bounds of window_bounds.cuh
     int tc_jspan = 0;
     unsigned int* tc_counter = nullptr;
     int tc_test_wait = 0;

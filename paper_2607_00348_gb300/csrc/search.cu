@@ -11,10 +11,14 @@
 //                      folded curve, pad it with its first D_m points
 //                      (Sect. 2.3.2) and build the exact prefix sums that give
 //                      every moving average (Eq. cumsum)
+//     k_window_bounds, k_window_exact  (uniform weights) the windows that can
+//                      hold a period's minimum, and their sums
+//                      (window_bounds.cuh)
 //     k_window_tiles   every duration and T0 start (Eq. N_skip): depth
 //                      (Eqs. k, depth), chi2 - chi2_0 (Eqs. out, in),
 //                      per-period minimum; staged tiles, window_tiles.cuh
-//                      (k_window_search: one thread per window, for plans
+//                      (per-point weights, and periods the bounds leave;
+//                      k_window_search: one thread per window, for plans
 //                      whose durations do not fit a tile)
 //     k_period_finalize chi2(P), depth, T0 of each period's minimum
 //   k_sr_stats_set, k_median_sde_set        SR, SDE_raw, SDE (Sect. 2.4)
@@ -75,6 +79,8 @@ constexpr int kRankBatch = 2;         // keys a fold thread ranks before issuing
 constexpr int kScanPer = 8;           // consecutive prefix-sum positions per fold thread
 constexpr int kWeightedTilePairs = 24576;   // (w r, w) pairs staged per tile with per-point weights
 constexpr int kSearchThreads = 256;
+constexpr double kBoundsMinWpe = 5e8;  // window-point products of a search from which windows are ruled out by bounds
+constexpr int64_t kListPerSlot = 128;  // windows to sum per period and lane-group size a chunk has room for
 constexpr int kMedianThreads = 1024;
 constexpr int kMedianCap = 8192;       // values a median block sorts in shared memory
 constexpr double kRScale = 1099511627776.0;   // 2^40: fixed point of r = 1 - y
@@ -225,6 +231,18 @@ __device__ __forceinline__ bool resolve_slot(const DevSet& ds, const SlotMap& sm
     return p >= 0 && p < ds.plans[lc].np;
 }
 
+// Right shift of the exact prefix sums in their 32-bit copy, for uniform
+// weights: any sum of r over the curve is at most sum |r| <= sqrt(n sum r^2),
+// which then fits 29 bits (30 for sums that go round it twice).  64: the
+// sums may not fit the fixed point.  Computed once per curve (scal[3]).
+__device__ __forceinline__ int prefix_shift(double chi2_0, double w, int64_t n)
+{
+    const double most = sqrt((double)n * chi2_0 / w) * kRScale;
+    return most < 536870912.0 ? 0 : most < 4.0e18 ? ilogb(most) - 28 : 64;
+}
+
+__device__ __forceinline__ float prefix_unit(int shift) { return ldexpf(1.0f, shift - 40); }
+
 // Work size of the per-curve preparation kernels for n points.
 __host__ __device__ __forceinline__ int prep_blocks_for(int64_t n)
 {
@@ -235,6 +253,7 @@ __host__ __device__ __forceinline__ int prep_blocks_for(int64_t n)
 }  // namespace
 
 #include "window_tiles.cuh"
+#include "window_bounds.cuh"
 #include "window_tc.cuh"
 
 namespace {
@@ -343,6 +362,7 @@ __global__ void k_curve_reduce(const double* __restrict__ dy, const int64_t* __r
     dc.scal[0] = double_from_order_key(*dc.tmin_key);
     dc.scal[1] = s;
     dc.scal[2] = (fl & 4u) ? 0.0 : 1.0 / (dy[o] * dy[o]);
+    dc.scal[3] = (fl & 4u) ? 0.0 : (double)prefix_shift(s, dc.scal[2], n);
     flags_out[lc] = fl;
 }
 
@@ -387,6 +407,8 @@ struct FoldOut {
     float* ws;
     float* wrs;
     long long* pf;
+    int32_t* pq;              // 32-bit copy of pf, shifted right by `shift` (uniform weights)
+    int shift;
     bool uniform;
 };
 
@@ -470,6 +492,7 @@ __device__ __forceinline__ void fold_scan_run(const long long* srfx, uint32_t le
 
 // Staged path; false when a super-bucket holds more than kFoldSegKeys
 // points (only keys have been written then).
+template <bool kBounded>
 __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCurve& dc, int p,
                             unsigned long long* keys, const FoldOut& o)
 {
@@ -685,7 +708,11 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
             carry += sum;
         }
         __syncthreads();
-        for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) __stcs(o.pf + (int64_t)k0 + 1 + i, srfx[swz(i)]);
+        for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) {
+            const long long v = srfx[swz(i)];
+            __stcs(o.pf + (int64_t)k0 + 1 + i, v);
+            if (kBounded) __stcs(o.pq + (int64_t)k0 + 1 + i, (int32_t)(v >> o.shift));
+        }
         __syncthreads();   // the next super-bucket overwrites the staged keys and rfx
     }
     return true;
@@ -855,6 +882,9 @@ __device__ void fold_global(unsigned char* smem, const DevPlan& dp, const DevCur
     }
 }
 
+// kBounded: the wave's window search is the one by bounds (uniform weights),
+// which reads the 32-bit prefix sums.
+template <bool kBounded>
 __global__ void __launch_bounds__(kFoldThreads, kFoldMinBlocks)
 k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk)
 {
@@ -872,13 +902,23 @@ k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, 
     o.ws = dk.ws ? dk.ws + (int64_t)slot_id * dk.pad_stride : nullptr;
     o.wrs = dk.wrs ? dk.wrs + (int64_t)slot_id * dk.pad_stride : nullptr;
     o.pf = dk.pf + (int64_t)slot_id * dk.pad_stride;
+    o.pq = dk.pq + (int64_t)slot_id * dk.pad_stride;
     o.uniform = dc.scal[2] > 0.0;
-    if (threadIdx.x == 0) ds.outs[lc].best[p] = ~0ull;
+    o.shift = kBounded ? min((int)dc.scal[3], 63) : 0;
+    if (threadIdx.x == 0) {
+        ds.outs[lc].best[p] = ~0ull;
+        if (kBounded && slot_id == 0)
+            for (int q = 0; q <= kListClasses; ++q) dk.left_n[q] = 0u;
+    }
 
-    if (!fold_staged(smem, dp, dc, p, keys, o)) {
+    if (!fold_staged<kBounded>(smem, dp, dc, p, keys, o)) {
         __syncthreads();   // the global path reuses the shared memory
         fold_global(smem, dp, dc, p, keys, o);
+        __syncthreads();
+        if (kBounded)
+            for (int64_t k = threadIdx.x + 1; k <= dp.n; k += blockDim.x) o.pq[k] = (int32_t)(o.pf[k] >> o.shift);
     }
+    if (kBounded && threadIdx.x == 0) o.pq[0] = 0;
 
     // padding: the first D_m folded points repeat after position N-1
     const int64_t n = dp.n;
@@ -891,7 +931,11 @@ k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, 
             o.ws[n + k] = real ? o.ws[k] : 0.0f;
             o.wrs[n + k] = real ? o.wrs[k] : 0.0f;
         }
-        if (real) o.pf[n + k + 1] = tot + o.pf[k + 1];
+        if (real) {
+            const long long v = tot + o.pf[k + 1];
+            o.pf[n + k + 1] = v;
+            if (kBounded) o.pq[n + k + 1] = (int32_t)(v >> o.shift);
+        }
     }
 }
 
@@ -979,7 +1023,7 @@ k_window_search(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* s
 
 __global__ void __launch_bounds__(tiles::kThreads, tiles::kCtasPerSm)
 k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk, int buf, int weighted,
-               unsigned int* counter)
+               int listed, unsigned int* counter)
 {
     const SlotMap& sm = smq ? *smq : smv;
     using namespace tiles;
@@ -988,33 +1032,44 @@ k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
     __shared__ int s_item, s_ndur, s_total, s_task, s_lc, s_p, s_slot, s_x0, s_len, s_tau, s_tcount;
     __shared__ unsigned long long s_best[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // the items the bounds kernel left, or every (period, tile) of the wave
+    const int items = listed ? (int)dk.left_n[kListClasses] : sm.items;
     for (;;) {
         if (threadIdx.x == 0) {
             const int item = (int)atomicAdd(counter, 1u);
-            s_item = item;
-            if (item < sm.items) {
-                int g = 0;
-                while (g + 1 < sm.nseg && sm.seg[g + 1].item0 <= item) ++g;
-                const int lcg = sm.seg[g].lc;
+            s_item = item < items ? 1 : 0;
+            if (item < items) {
+                int lcg = 0, pp = -1, slot = 0, tau = 0;
+                if (listed) {
+                    const int2 it = dk.dense[item];
+                    slot = it.x;
+                    tau = it.y;
+                    if (!resolve_slot(ds, sm, slot, lcg, pp)) pp = -1;
+                } else {
+                    int g = 0;
+                    while (g + 1 < sm.nseg && sm.seg[g + 1].item0 <= item) ++g;
+                    lcg = sm.seg[g].lc;
+                    const int per = weighted ? ds.tiles[lcg].count_w : ds.tiles[lcg].count;
+                    const int rel = item - sm.seg[g].item0;
+                    const int k = rel / per;
+                    tau = rel - k * per;
+                    slot = sm.seg[g].slot0 + k;
+                    const int q = sm.seg[g].first + k;
+                    pp = sm.from_list ? ds.outs[lcg].plist[q] : q;
+                    if (!in_range(ds.curves[lcg].check, 22, pp, ds.plans[lcg].np)) pp = -1;
+                }
                 const DevTiles tl = ds.tiles[lcg];
-                const int tcount = weighted ? tl.count_w : tl.count;
-                const int rel = item - sm.seg[g].item0;
-                const int k = rel / tcount, tau = rel - k * tcount;
-                const int q = sm.seg[g].first + k;
-                int pp = sm.from_list ? ds.outs[lcg].plist[q] : q;
-                if (!in_range(ds.curves[lcg].check, 22, pp, ds.plans[lcg].np)) pp = -1;
                 s_lc = lcg;
                 s_p = pp;
-                s_slot = sm.seg[g].slot0 + k;
+                s_slot = slot;
                 s_x0 = tau * (weighted ? tl.len_w : tl.len);
                 s_len = weighted ? tl.len_w : tl.len;
                 s_tau = tau;
-                s_tcount = tcount;
+                s_tcount = weighted ? tl.count_w : tl.count;
             }
         }
         __syncthreads();
-        const int item = s_item;
-        if (item >= sm.items) break;
+        if (!s_item) break;
         const int lc = s_lc, p = s_p, slot = s_slot, x0 = s_x0, tile_len = s_len, tau = s_tau, tcount = s_tcount;
         if (p < 0) {   // block-uniform: a failed check skips the item
             __syncthreads();
@@ -1059,31 +1114,15 @@ k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
                     t.d = dp.dpts[j];
                     t.st = dp.stride[j];
                     t.m_total = (int)((n + t.st - 1) / t.st);
-                    t.m_a = (x0 + t.st - 1) / t.st;
-                    t.m_b = min(t.m_total, (x0 + tile_len + t.st - 1) / t.st);
                     t.variant = weighted ? (int)kWeighted15 : dp.cfg_variant[j];
                     t.nc = weighted ? dp.cfg_nc_w[j] : dp.cfg_nc[j];
                     t.w = variant_w(t.variant);
                     t.per_task = 32 * t.w / t.nc;
                     const int jrows = (t.d + t.st - 1) / t.st;
-                    {
-                        // whole tasks per tile where the staged buffers have room:
-                        // the duration covers windows [tau K, (tau + 1) K) of tile
-                        // tau, K a multiple of the task length with K st >= L (each
-                        // tile starts inside its buffer) and K st <= L + room /
-                        // tiles (the last tile's blocks and rows still fit), so
-                        // that only its last tile has a partly filled task
-                        const long long room =
-                            (long long)buf - 32 - (long long)(jrows + t.w) * t.st - tile_len;
-                        if (room > 0) {
-                            const long long span = tile_len + room / tcount;
-                            const long long k = span / t.st / t.per_task * t.per_task;
-                            if (k * t.st >= tile_len) {
-                                t.m_a = (int)min((long long)t.m_total, (long long)tau * k);
-                                t.m_b = (int)min((long long)t.m_total, (long long)(tau + 1) * k);
-                            }
-                        }
-                    }
+                    const TileSpan sp =
+                        tile_span(t.st, jrows, t.w, t.per_task, t.m_total, x0, tile_len, tau, tcount, buf);
+                    t.m_a = sp.m_a;
+                    t.m_b = sp.m_b;
                     const int nwin = max(0, t.m_b - t.m_a);
                     t.tasks = (!weighted && (t.variant == kWindowOnly || t.variant == kTensor))
                                   ? 0
@@ -1094,10 +1133,8 @@ k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
                     t.inv_sum_t = dp.inv_sum_t[j] * (1.0f / 1099511627776.0f);  // 2^-40 fixed point
                     t.inv_sum_t_f = dp.inv_sum_t[j];
                     t.sum_t2 = dp.sum_t2[j];
-                    // rows up to m + w + jrows - 1 and columns up to st + 31 must stay in the buffer
-                    const int m_max_start = (x0 + buf - 32) / t.st - t.w - jrows;
-                    t.hi_start = min(t.m_total - t.w, m_max_start);
-                    if (t.tasks > 0) in_range(check, 20, (int64_t)t.m_a, (int64_t)m_max_start + 1);
+                    t.hi_start = sp.hi_start;
+                    if (t.tasks > 0) in_range(check, 20, (int64_t)t.m_a, (int64_t)sp.m_max_start + 1);
                     t.first = 0;
                     dur[k] = t;
                 }
@@ -2130,6 +2167,72 @@ void pick_config_host(int d, int st, int nwin, int32_t& variant, int32_t& nc_out
         for (int nc = 2; nc <= 16; nc <<= 1) consider(tiles::kCol16R, nc);
 }
 
+// Pieces of the template s[0 .. d) with T0 step st.  Both sets are cut where
+// the sum of length x deviation, which is what the bound loses on white noise,
+// is least for the default limb darkening (0.128 D for the whole template;
+// 0.040, 0.030, 0.024, 0.017 and 0.009 D for 5, 7, 9, 13 and 25 pieces).
+BoundTab bound_table(const float* s, int d, int st)
+{
+    constexpr double kCut[kBoundSegs / 2] = {0.010, 0.024, 0.042, 0.064, 0.088, 0.116,
+                                             0.148, 0.184, 0.224, 0.270, 0.324, 0.392};
+    BoundTab b{};
+    auto piece = [&](int lo, int hi, float& mean) {
+        double m = 0.0, v = 0.0;
+        for (int k = lo; k < hi; ++k) m += s[k];
+        mean = hi > lo ? (float)(m / (hi - lo)) : 0.0f;
+        for (int k = lo; k < hi; ++k) v += ((double)s[k] - mean) * ((double)s[k] - mean);
+        return (float)(std::sqrt(v) * (1.0 + 1e-6));
+    };
+    b.off[0] = 0;
+    b.off[kBoundSegs] = d;
+    for (int g = 0; g < kBoundSegs / 2; ++g) {
+        // (short templates: at least a point each from the edges inwards)
+        const int cut = std::min(d / 2, std::max(g + 1, (int)std::lround(kCut[g] * d)));
+        b.off[1 + g] = cut;
+        b.off[kBoundSegs - 1 - g] = d - cut;
+    }
+    for (int g = 0; g < kBoundSegs; ++g) {
+        const int len = b.off[g + 1] - b.off[g];
+        b.nu[g] = piece(b.off[g], b.off[g + 1], b.mean[g]);
+        b.inv_len[g] = len > 0 ? (float)((1.0 - 1e-5) / len) : 0.0f;
+    }
+    double top = 0.0, t2 = 0.0;
+    for (int k = 0; k < d; ++k) {
+        top = std::max(top, std::fabs((double)s[k]));
+        t2 += (double)s[k] * s[k];
+    }
+    b.nu_all = piece(0, d, b.mean_all);
+    b.root_t2 = (float)std::sqrt(t2);
+    b.t_max = (float)(top * (1.0 + 1e-6));
+    if (d >= bounds::kCutPoints) {
+        // more pieces for longer windows: the bound loses in proportion to D,
+        // the best window gains with its root
+        std::vector<double> cut;
+        if (d < 200) cut = {0.078, 0.222};
+        else if (d < 1000) cut = {0.052, 0.138, 0.268};
+        else if (d < 3000) cut = {0.038, 0.098, 0.182, 0.300};
+        else cut = {0.022, 0.058, 0.104, 0.164, 0.238, 0.338};
+        std::vector<int> row = {0};
+        for (double c : cut) row.push_back((int)std::lround(c * d / st));
+        for (double c : cut) row.push_back((int)std::lround((1.0 - c) * d / st));
+        std::sort(row.begin(), row.end());
+        row.erase(std::unique(row.begin(), row.end()), row.end());
+        while ((int64_t)row.back() * st >= d) row.pop_back();
+        b.cuts = (int)row.size();
+        float before = 0.0f, mean = 0.0f;
+        for (int u = 0; u < b.cuts; ++u) {
+            const int lo = row[u] * st, hi = u + 1 < b.cuts ? row[u + 1] * st : d;
+            b.cut_row[u] = row[u];
+            b.cut_len[u] = hi - lo;
+            b.cut_nu[u] = piece(lo, hi, mean);
+            b.cut_coef[u] = before - mean;
+            before = mean;
+        }
+        b.cut_coef[b.cuts] = before;
+    }
+    return b;
+}
+
 int fold_smem_bytes(int bucket_log2)
 {
     // global path: histogram and starts, scan scratch, staged keys and folded rfx
@@ -2169,8 +2272,10 @@ gtls_status configure_kernels(int dev)
                                        optin - (int)a.sharedSizeBytes));
         return GTLS_OK;
     };
-    GTLS_TRY(allow((const void*)k_fold_sort));
+    GTLS_TRY(allow((const void*)k_fold_sort<false>));
+    GTLS_TRY(allow((const void*)k_fold_sort<true>));
     GTLS_TRY(allow((const void*)k_window_tiles));
+    GTLS_TRY(allow((const void*)bounds::k_window_bounds));
     GTLS_TRY(allow((const void*)k_median_sde));
     GTLS_TRY(allow((const void*)k_median_sde_set));
     GTLS_TRY(allow((const void*)k_topk));
@@ -2259,7 +2364,7 @@ gtls_status create_device(gtls_plan* pl)
     dk.fold_stride = (n + 31) & ~int64_t(31);
     dk.key_stride = std::max<int64_t>(dk.fold_stride, (int64_t)kFoldSegKeys * dp.fold_nsb);
     dk.pad_stride = (n + h.dmax + kPadMargin + 31) & ~int64_t(31);
-    const int64_t per_period = dk.key_stride * 8 + dk.fold_stride * 4 + dk.pad_stride * (4 + 4 + 4 + 8);
+    const int64_t per_period = dk.key_stride * 8 + dk.fold_stride * 4 + dk.pad_stride * (4 + 4 + 4 + 8 + 4);
     // 8 GiB of chunk scratch (measured on the Kepler-like search: 1024,
     // 1520 and 3040 periods per chunk took 1013, 994 and 980 ms)
     const int64_t budget = int64_t(8) << 30;
@@ -2550,6 +2655,23 @@ gtls_status create_device(gtls_plan* pl)
         GTLS_TRY(dev_alloc(pl, &pl->tc_counter, 1));
     }
 
+    // pieces of every duration's template for the bounds of the window search
+    {
+        std::vector<BoundTab> tab(dp.nd);
+        // small searches are bound by launches: two kernels more cost what
+        // they save (0.29 ms and 6e7 window-point products: 18 us slower;
+        // 1.2 ms and 2.9e9: 140 us faster)
+        const bool worth = h.wpe >= kBoundsMinWpe || (h.prm.test_flags & 4);
+        pl->bounds_ok = !pl->has_tensor && worth && !(h.prm.test_flags & 2);
+        for (int pass = 0; pass < (pl->refine_k > 0 ? 2 : 1); ++pass) {
+            for (int j = 0; j < dp.nd; ++j) {
+                tab[j] = bound_table(h.tmpl.data() + h.tmpl_off[j], h.dpts[j], pass ? 1 : h.stride[j]);
+                pl->bounds_ok = pl->bounds_ok && tab[j].mean_all > 0.0f && tab[j].root_t2 > 0.0f;
+            }
+            GTLS_TRY(upload(pl, const_cast<BoundTab**>(pass ? &pl->dp_ref.bounds : &dp.bounds), tab));
+        }
+    }
+
     // one-entry descriptor sets of this plan's own searches
     {
         DevPlan* d_plans = nullptr;
@@ -2620,6 +2742,11 @@ gtls_status ensure_chunk(gtls_plan* pl)
     GTLS_TRY(dev_alloc(pl, &dk.ws, chunk * dk.pad_stride));
     GTLS_TRY(dev_alloc(pl, &dk.wrs, chunk * dk.pad_stride));
     GTLS_TRY(dev_alloc(pl, &dk.pf, chunk * dk.pad_stride));
+    GTLS_TRY(dev_alloc(pl, &dk.pq, chunk * dk.pad_stride));
+    dk.list_cap = std::max<int64_t>(4096, chunk * kListPerSlot);
+    GTLS_TRY(dev_alloc(pl, &dk.list, kListClasses * dk.list_cap));
+    GTLS_TRY(dev_alloc(pl, &dk.dense, chunk * std::max({1, pl->tile_count, pl->tile_count_ref})));
+    GTLS_TRY(dev_alloc(pl, &dk.left_n, kListClasses + 1));
     if (pl->has_tensor) {
         unsigned char* maps = nullptr;
         GTLS_TRY(dev_alloc(pl, &maps, (size_t)tc::kMaps * sizeof(CUtensorMap)));
@@ -2636,7 +2763,8 @@ gtls_status trim_chunk(gtls_plan* pl)
 {
     if (!pl->chunk_ready) return GTLS_OK;
     GTLS_CUDA(cudaDeviceSynchronize());
-    const void* mine[] = {pl->dk.keys, pl->dk.sidx, pl->dk.rs, pl->dk.ws, pl->dk.wrs, pl->dk.pf, pl->tc_maps};
+    const void* mine[] = {pl->dk.keys, pl->dk.sidx, pl->dk.rs, pl->dk.ws, pl->dk.wrs, pl->dk.pf,
+                          pl->dk.pq, pl->dk.list, pl->dk.dense, pl->dk.left_n, pl->tc_maps};
     int kept = 0;
     for (int i = 0; i < pl->n_allocs; ++i) {
         bool chunk = false;
@@ -2653,6 +2781,10 @@ gtls_status trim_chunk(gtls_plan* pl)
     pl->dk.sidx = nullptr;
     pl->dk.rs = pl->dk.ws = pl->dk.wrs = nullptr;
     pl->dk.pf = nullptr;
+    pl->dk.dense = nullptr;
+    pl->dk.pq = nullptr;
+    pl->dk.list = nullptr;
+    pl->dk.left_n = nullptr;
     pl->dk.chunk = chunk;
     pl->tc_maps = nullptr;
     pl->chunk_ready = false;
@@ -2710,6 +2842,7 @@ struct Ctx {
     const void* tc_maps = nullptr;   // tensor-core kernel: TMA maps of dk.rs (tc::kMaps rows pitches)
     int tc_jspan = 1;        // tensor-core kernel: work items per period slot
     int tc_test = 0;         // tensor-core kernel: run the timeout test
+    bool bounds_ok = false;  // uniform weights: bounds kernel first, tiled kernel on what it leaves
     int64_t launches = 0, window_launches = 0;
     gtls_plan* prof = nullptr;   // stage marks (single search with profiling on)
     size_t ev = 0;
@@ -2730,15 +2863,24 @@ gtls_status wave_pass(Ctx& c, bool ref, const SlotMap& sm, bool tiled, bool weig
                       unsigned int* tc_counter = nullptr, const SlotMap* smq = nullptr)
 {
     const DevSet& ds = ref ? c.set_ref : c.set;
-    k_fold_sort<<<sm.slots, kFoldThreads, c.fold_smem, c.st>>>(ds, sm, smq, c.dk);
+    const bool bounded = tiled && c.bounds_ok && !weighted;
+    (bounded ? k_fold_sort<true> : k_fold_sort<false>)<<<sm.slots, kFoldThreads, c.fold_smem, c.st>>>(ds, sm, smq,
+                                                                                                     c.dk);
     GTLS_CUDA(cudaGetLastError());
     GTLS_TRY(stage_mark(c, kStageFold));
     if (tiled) {
         if (reset_counter) GTLS_CUDA(cudaMemsetAsync(counter, 0, sizeof(unsigned int), c.st));
         const int buf = weighted ? c.tile_buf_w : c.tile_buf;
         const int bytes = buf * (int)(weighted ? sizeof(float2) : sizeof(float));
-        k_window_tiles<<<c.n_sm * tiles::kCtasPerSm, tiles::kThreads, bytes, c.st>>>(ds, sm, smq, c.dk, buf,
-                                                                                   weighted ? 1 : 0, counter);
+        if (bounded) {
+            bounds::k_window_bounds<<<sm.slots, bounds::kThreads, bounds::smem_bytes(), c.st>>>(ds, sm, smq, c.dk, buf);
+            GTLS_CUDA(cudaGetLastError());
+            bounds::k_window_exact<<<c.n_sm * 8, bounds::kExactThreads, 0, c.st>>>(ds, sm, smq, c.dk);
+            GTLS_CUDA(cudaGetLastError());
+            c.launches += 2;
+        }
+        k_window_tiles<<<c.n_sm * tiles::kCtasPerSm, tiles::kThreads, bytes, c.st>>>(
+            ds, sm, smq, c.dk, buf, weighted ? 1 : 0, bounded ? 1 : 0, counter);
         if (tensor && !weighted && tc_counter) {
             // the durations marked kTensor (the tiled kernel gave them no tasks)
             GTLS_CUDA(cudaGetLastError());
@@ -2870,6 +3012,7 @@ gtls_status run_search(gtls_plan* pl, const double* t, const double* y, const do
     c.tc_jspan = pl->tc_jspan;
     c.tc_test = pl->tc_test_wait;
     c.tc_maps = pl->tc_maps;
+    c.bounds_ok = pl->bounds_ok;
     pl->profile = gtls_profile{};
     if (pl->profiling) c.prof = pl;
 
@@ -2975,6 +3118,7 @@ struct gtls_batch {
     cudaStream_t body_stream = nullptr;   // stream the loop bodies are captured on
     BatchCfg cfg;
     bool tuned = false;
+    bool bounds_ok = true;             // every plan's templates admit the bounds kernel
     // graph of everything after the curve preparation, for one set of
     // per-curve kernel classes (uniform dy and tile fit)
     std::vector<uint8_t> graph_class;
@@ -3151,6 +3295,7 @@ Ctx batch_ctx(const gtls_batch* b, cudaStream_t st)
         c.tc_test = std::max(c.tc_test, pl->tc_test_wait);
     }
     c.tc_maps = b->tc_maps;
+    c.bounds_ok = b->bounds_ok;
     return c;
 }
 
@@ -3440,6 +3585,7 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
             buf_max = std::min(buf_max, pl->tile_buf);
             any_tiled = true;
         }
+        b->bounds_ok = b->bounds_ok && pl->bounds_ok;
     }
     b->fold_smem = fold_smem_bytes(bucket_log2);
     b->topk_smem = topk;
@@ -3460,7 +3606,7 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     dk.fold_stride = fold_stride;
     dk.key_stride = key_stride;
     dk.pad_stride = pad_stride;
-    const int64_t per_slot = key_stride * 8 + fold_stride * 4 + pad_stride * (4 + 4 + 4 + 8);
+    const int64_t per_slot = key_stride * 8 + fold_stride * 4 + pad_stride * (4 + 4 + 4 + 8 + 4);
     const int64_t budget = int64_t(16) << 30;
     int64_t slots = std::min<int64_t>(4096, std::max<int64_t>(1, budget / per_slot));
     if (b->n_sm > 0 && slots >= 4 * b->n_sm) slots = slots / (4 * b->n_sm) * (4 * b->n_sm);   // whole fold waves at 1, 1/2, 1/4
@@ -3520,6 +3666,13 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     b->total_periods = total_periods;
     batch_tiles(b, b->cfg.tile_buf);
     GTLS_TRY(batch_upload_tiles(b));
+    int max_tiles = 1;
+    for (const DevTiles& t : b->tiles_host) max_tiles = std::max(max_tiles, t.count);
+    GTLS_TRY(batch_alloc(b, &b->dk.dense, slots * (int64_t)max_tiles));
+    GTLS_TRY(batch_alloc(b, &b->dk.pq, slots * pad_stride));
+    b->dk.list_cap = std::max<int64_t>(4096, slots * kListPerSlot);
+    GTLS_TRY(batch_alloc(b, &b->dk.list, kListClasses * b->dk.list_cap));
+    GTLS_TRY(batch_alloc(b, &b->dk.left_n, kListClasses + 1));
     return GTLS_OK;
 }
 

@@ -104,6 +104,47 @@ struct DurTask {
     float inv_sum_t_f;        // 1 / sum_k s_k
 };
 
+// Windows [m_a, m_b) of one duration (T0 step st, jrows rows, register blocks
+// of w windows, per_task windows per warp task, m_total windows in all) that
+// tile tau (starts x0 .. x0 + tile_len, buf staged points, tcount tiles) of a
+// period covers, and the last start hi_start a block may take.
+struct TileSpan {
+    int m_a, m_b, hi_start, m_max_start;
+};
+__device__ __forceinline__ TileSpan tile_span(int st, int jrows, int w, int per_task, int m_total, int x0, int tile_len,
+                                              int tau, int tcount, int buf)
+{
+    TileSpan t;
+    t.m_a = (x0 + st - 1) / st;
+    t.m_b = min(m_total, (x0 + tile_len + st - 1) / st);
+    // whole tasks per tile where the staged buffers have room: the duration
+    // covers windows [tau K, (tau + 1) K) of tile tau, K a multiple of the
+    // task length with K st >= L (each tile starts inside its buffer) and
+    // K st <= L + room / tiles (the last tile's blocks and rows still fit),
+    // so that only its last tile has a partly filled task
+    const long long room = (long long)buf - 32 - (long long)(jrows + w) * st - tile_len;
+    if (room > 0) {
+        const long long span = tile_len + room / tcount;
+        const long long k = span / st / per_task * per_task;
+        if (k * st >= tile_len) {
+            t.m_a = (int)min((long long)m_total, (long long)tau * k);
+            t.m_b = (int)min((long long)m_total, (long long)(tau + 1) * k);
+        }
+    }
+    // rows up to m + w + jrows - 1 and columns up to st + 31 must stay in the buffer
+    t.m_max_start = (x0 + buf - 32) / st - w - jrows;
+    t.hi_start = min(m_total - w, t.m_max_start);
+    return t;
+}
+
+// Packed (delta-chi2, duration, window) of a period's minimum.
+__device__ __forceinline__ unsigned long long window_key(float dchi, int j, long long m)
+{
+    unsigned int u = __float_as_uint(dchi);
+    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+    return ((unsigned long long)u << 32) | ((unsigned long long)j << 24) | (unsigned long long)m;
+}
+
 struct WinCtx {
     const float* tile;        // shared: folded r at x0 .. x0 + BUF
     const float2* tile2;      // shared: folded (w r, w) at x0 .. x0 + BUF (per-point weights)
@@ -134,10 +175,7 @@ __device__ __forceinline__ unsigned long long finish_window(const WinCtx& c, lon
     const long long s = m * c.st;
     const long long sfx = c.pf[s + c.d] - c.pf[s];
     const float depth = fmaxf(0.0f, fixed_to_float(sfx) * c.inv_sum_t);
-    const float dchi = c.w_uni * depth * fmaf(depth, c.sum_t2, -2.0f * c1);
-    unsigned int u = __float_as_uint(dchi);
-    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-    return ((unsigned long long)u << 32) | ((unsigned long long)c.j << 24) | (unsigned long long)m;
+    return window_key(c.w_uni * depth * fmaf(depth, c.sum_t2, -2.0f * c1), c.j, m);
 }
 
 // One recursive-halving exchange over lane bit `o`: the lane keeps the lower
@@ -233,11 +271,8 @@ __device__ __forceinline__ void reduce_pair_finish(const WinCtx& c, const float2
         const int m = mb + w;
         if (w < W && m < c.m_total) {
             const float depth = fmaxf(0.0f, e[i].y * c.inv_sum_t_f);
-            const float dchi = c.w_uni * depth * fmaf(depth, c.sum_t2, -2.0f * e[i].x);
-            unsigned int u = __float_as_uint(dchi);
-            u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
             const unsigned long long key =
-                ((unsigned long long)u << 32) | ((unsigned long long)c.j << 24) | (unsigned long long)m;
+                window_key(c.w_uni * depth * fmaf(depth, c.sum_t2, -2.0f * e[i].x), c.j, m);
             best = key < best ? key : best;
         }
     }
@@ -534,11 +569,7 @@ __device__ __forceinline__ void reduce_weighted_finish(const WinCtx& c, const fl
             const long long s0 = m * c.st;
             const long long sfx = c.pf[s0 + c.d] - c.pf[s0];
             const float depth = fmaxf(0.0f, fixed_to_float(sfx) * c.inv_sum_t);
-            const float dchi = depth * fmaf(depth, e[i].y, -2.0f * e[i].x);
-            unsigned int u = __float_as_uint(dchi);
-            u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-            const unsigned long long key =
-                ((unsigned long long)u << 32) | ((unsigned long long)c.j << 24) | (unsigned long long)m;
+            const unsigned long long key = window_key(depth * fmaf(depth, e[i].y, -2.0f * e[i].x), c.j, m);
             best = key < best ? key : best;
         }
     }
