@@ -11,13 +11,17 @@
 // pooling windows; more than a third of the curve) instead of about 320.
 //
 // Every contraction (convolution forward, data and weight gradients, head
-// forward and its two gradients) runs through one BF16 tensor-core tile GEMM
-// (mma.sync m16n8k16, FP32 accumulation) whose operand tiles are gathered
-// into shared memory by small loader functors (implicit im2col for the
-// convolutions, transposed views for the gradients).  Activations are BF16
-// [batch][length][channel]; gradients and master parameters are FP32.  The
-// whole network costs about 0.2 GFLOP per light curve for inference, so the
-// kernels favour simplicity over peak tensor throughput.
+// forward and its two gradients) runs on the BF16 tensor cores (mma.sync
+// m16n8k16, FP32 accumulation).  A convolution is an implicit GEMM: a tile of
+// 128 positions of one curve and its halo is staged once in shared memory
+// (128-byte rows, 16-byte chunks swizzled), and tap k reads the same tile
+// k dilation rows further down, so no im2col matrix exists anywhere.  The
+// gradient of a pre-activation is never stored either: the tiles of the
+// gradient kernels are made from the pooled gradient, the pooled value and
+// the pooling choice while they are staged.  Activations are BF16
+// [batch][length][channel]; gradients and master parameters are FP32.
+// The products of an output are added tap by tap, channels ascending, in
+// chains of k16 steps, in the forward pass and the data gradient.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -80,160 +84,634 @@ struct Layout {
 };
 
 // ---------------------------------------------------------------------------
-// tile GEMM: C[m][n] = sum_k A(m, k) B(n, k), 64 x 64 tiles, K steps of 32,
-// four warps of 32 x 32 (2 x 4 mma tiles of 16 x 8)
+// tensor-core building blocks
 // ---------------------------------------------------------------------------
 
-constexpr int kBM = 64, kBN = 64, kBK = 32, kLd = kBK + 8;   // +8: conflict-free fragment loads
-
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], const uint32_t (&b)[2])
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)
 {
     asm volatile(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
         "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
         : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// Operand views (value at (row, k); callers guarantee row and k in range)
-struct ConvIn {        // implicit im2col of x[B][L][C]: row = b L + l, k = tap C + c
-    const bf16* x;
-    int L, C, half, dil;   // taps at l + (tap - half) dil
-    __device__ bf16 operator()(int row, int k) const
-    {
-        const int b = row / L, l = row - b * L;
-        const int tap = k / C, c = k - tap * C;
-        const int src = l + (tap - half) * dil;
-        return (src >= 0 && src < L) ? x[((int64_t)b * L + src) * C + c] : __float2bfloat16(0.0f);
-    }
-};
-struct ConvInT {       // the same view with the roles swapped: row = tap C + c, k = b L + l
-    ConvIn in;
-    __device__ bf16 operator()(int row, int k) const { return in(k, row); }
-};
-struct RowMajor {      // m[row][k], leading dimension ld
-    const bf16* m;
-    int ld;
-    __device__ bf16 operator()(int row, int k) const { return m[(int64_t)row * ld + k]; }
-};
-struct ColMajor {      // m[k][row], leading dimension ld
-    const bf16* m;
-    int ld;
-    __device__ bf16 operator()(int row, int k) const { return m[(int64_t)k * ld + row]; }
-};
-struct FlippedW {      // data gradient: row = input channel ci, k = tap' C + co -> w[co][T-1-tap'][ci]
-    const bf16* w;
-    int taps, cin, cout;
-    __device__ bf16 operator()(int row, int k) const
-    {
-        const int tp = k / cout, co = k - tp * cout;
-        return w[((int64_t)co * taps + (taps - 1 - tp)) * cin + row];
-    }
-};
-
-enum EpiKind { kEpiPoolRelu = 0, kEpiStore = 1, kEpiAtomic = 2 };
-
-struct Epi {
-    int kind;
-    float* out;            // kEpiStore / kEpiAtomic: out[row * ld + col]
-    int ld;
-    const float* bias;     // per column, nullable
-    bf16* pooled;          // kEpiPoolRelu: pooled[(row / 2) * ld + col]
-    uint8_t* arg;          // 1 where the odd row of a pair won
-};
-
-template <class LA, class LB>
-__global__ void __launch_bounds__(128) k_gemm(int M, int N, int K, int k_chunk, LA la, LB lb, Epi ep)
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], uint32_t addr)
 {
-    __shared__ __align__(16) bf16 As[kBM][kLd];
-    __shared__ __align__(16) bf16 Bs[kBN][kLd];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int g = lane >> 2, t = lane & 3;
-    const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * kBN;
-    const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
-    const int kbeg = blockIdx.z * k_chunk;
-    const int kend = min(K, kbeg + k_chunk);
-    float acc[2][4][4];
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int u = 0; u < 4; ++u) acc[i][j][u] = 0.0f;
-    const bf16 zero = __float2bfloat16(0.0f);
-    for (int k0 = kbeg; k0 < kend; k0 += kBK) {
-        for (int e = tid; e < kBM * kBK; e += 128) {
-            const int r = e / kBK, c = e - (e / kBK) * kBK;
-            const int k = k0 + c;
-            const bool kin = k < kend;
-            As[r][c] = (kin && m0 + r < M) ? la(m0 + r, k) : zero;
-            Bs[r][c] = (kin && n0 + r < N) ? lb(n0 + r, k) : zero;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < kBK; kk += 16) {
-            uint32_t a[2][4], b[4][2];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int row = wm + i * 16 + g;
-                a[i][0] = *reinterpret_cast<const uint32_t*>(&As[row][kk + 2 * t]);
-                a[i][1] = *reinterpret_cast<const uint32_t*>(&As[row + 8][kk + 2 * t]);
-                a[i][2] = *reinterpret_cast<const uint32_t*>(&As[row][kk + 2 * t + 8]);
-                a[i][3] = *reinterpret_cast<const uint32_t*>(&As[row + 8][kk + 2 * t + 8]);
-            }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int col = wn + j * 8 + g;
-                b[j][0] = *reinterpret_cast<const uint32_t*>(&Bs[col][kk + 2 * t]);
-                b[j][1] = *reinterpret_cast<const uint32_t*>(&Bs[col][kk + 2 * t + 8]);
-            }
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) mma_bf16(acc[i][j], a[i], b[j]);
-        }
-        __syncthreads();
-    }
-    // accumulator (i, j, u): row m0 + wm + 16 i + g + 8 (u >> 1), column
-    // n0 + wn + 8 j + 2 t + (u & 1)
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+
+__device__ __forceinline__ void ldsm2t(uint32_t& r0, uint32_t& r1, uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];" : "=r"(r0), "=r"(r1) : "r"(addr));
+}
+
+// 16 bytes global -> shared, zeros when !in
+__device__ __forceinline__ void copy16(uint32_t dst, const void* src, bool in)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+}
+
+__device__ __forceinline__ void copies_done()
+{
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+}
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p)
+{
+    return (uint32_t)__cvta_generic_to_shared(p);
+}
+
+// Byte offset of 16-byte chunk c of row r in a tile of 128-byte rows: the
+// eight rows of one ldmatrix phase fall into eight different bank groups.
+__device__ __forceinline__ uint32_t at128(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
+
+constexpr int kRows = 128;                     // positions per convolution tile
+constexpr int kMaxHalo = 16;                   // rows before and after it (2 x the largest dilation)
+constexpr int kConvTaps = 5;                   // taps of convolutions 1..5
+constexpr int kWBytes = kConvTaps * kCh * 128; // their staged weights
+constexpr int kABytes = (kRows + 2 * kMaxHalo) * 128;
+
+// Where the gradient of a pre-activation comes from: the gradient of the
+// pooled output (FP32), the pooled output and which row of a pair won.
+struct PoolGrad {
+    const float* grad;
+    const bf16* pooled;
+    const uint8_t* arg;
+};
+
+// Rows [l0, l0 + rows) (l0, rows even) of the pre-activation gradient of one
+// curve of L positions, made from its pooled gradient (to the winning row of
+// each pair where the pooled value is positive, zero elsewhere), into a tile
+// of 128-byte rows; rows outside [0, L) are zero.  `first`: the curve's first
+// pooled position.
+__device__ __forceinline__ void stage_pool_grad(unsigned char* tile, const PoolGrad& pg, int64_t first, int l0, int rows,
+                                                int L)
+{
+    for (int e = threadIdx.x; e < rows / 2 * 8; e += blockDim.x) {
+        const int q = e >> 3, c = e & 7;
+        const int pos = (l0 >> 1) + q;
+        uint4 lo = make_uint4(0, 0, 0, 0), hi = lo;
+        if (pos >= 0 && pos < L / 2) {
+            const int64_t at = (first + pos) * kCh + 8 * c;
+            const float4 g0 = __ldg(reinterpret_cast<const float4*>(pg.grad + at));
+            const float4 g1 = __ldg(reinterpret_cast<const float4*>(pg.grad + at) + 1);
+            const uint4 pv = __ldg(reinterpret_cast<const uint4*>(pg.pooled + at));
+            const uint2 av = __ldg(reinterpret_cast<const uint2*>(pg.arg + at));
+            const float g[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+            const uint32_t p[4] = {pv.x, pv.y, pv.z, pv.w};
+            uint32_t a[4], b[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int row = m0 + wm + i * 16 + g + 8 * (u >> 1);
-                const int col = n0 + wn + j * 8 + 2 * t + (u & 1);
-                float v = acc[i][j][u];
-                if (ep.kind == kEpiPoolRelu) {
-                    // rows 2q and 2q+1 sit in lanes g and g ^ 1 (lane ^ 4)
-                    v = fmaxf(v + (col < N ? ep.bias[col] : 0.0f), 0.0f);
-                    const float other = __shfl_xor_sync(0xffffffffu, v, 4);
-                    if ((g & 1) == 0 && row < M && col < N) {
-                        const bool odd_wins = other > v;
-                        ep.pooled[(int64_t)(row >> 1) * ep.ld + col] = __float2bfloat16(odd_wins ? other : v);
-                        ep.arg[(int64_t)(row >> 1) * ep.ld + col] = odd_wins ? 1 : 0;
+                uint32_t even = 0, odd = 0;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t pb = h ? p[u] >> 16 : p[u] & 0xffffu;
+                    // pooled > 0: the pooled value is a ReLU's output
+                    const float v = pb != 0 && pb <= 0x7f80u ? g[2 * u + h] : 0.0f;
+                    const uint32_t bits = (uint32_t)__bfloat16_as_ushort(__float2bfloat16(v)) << (16 * h);
+                    const uint32_t won = (((u < 2 ? av.x : av.y) >> (8 * ((2 * u + h) & 3))) & 1u);
+                    if (won) odd |= bits;
+                    else even |= bits;
+                }
+                a[u] = even;
+                b[u] = odd;
+            }
+            lo = make_uint4(a[0], a[1], a[2], a[3]);
+            hi = make_uint4(b[0], b[1], b[2], b[3]);
+        }
+        *reinterpret_cast<uint4*>(tile + at128(2 * q, c)) = lo;
+        *reinterpret_cast<uint4*>(tile + at128(2 * q + 1, c)) = hi;
+    }
+}
+
+// Rows [l0, l0 + rows) of one curve's activations (L x 64, zero outside).
+__device__ __forceinline__ void stage_rows(uint32_t tile, const bf16* x, int l0, int rows, int L)
+{
+    for (int e = threadIdx.x; e < rows * 8; e += blockDim.x) {
+        const int r = e >> 3, c = e & 7, l = l0 + r;
+        const bool in = l >= 0 && l < L;
+        copy16(tile + at128(r, c), x + (int64_t)(in ? l : 0) * kCh + 8 * c, in);
+    }
+}
+
+// Bias, ReLU and max-pool of row pairs of a warp's (16 i + g, 8 j + 2 t)
+// accumulators into the staged output tile (pooled rows of 128 bytes, and 64
+// bytes of pooling choices when kArg); rows 2q and 2q + 1 sit in lanes g, g ^ 1.
+template <bool kArg>
+__device__ __forceinline__ void pool_tile(float (&acc)[2][8][4], const float* __restrict__ bias, int row0, int lane,
+                                          bf16* pool, uint8_t* arg)
+{
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const float2 bv = __ldg(reinterpret_cast<const float2*>(bias + 8 * j + 2 * t));
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float v0 = fmaxf(acc[i][j][2 * h] + bv.x, 0.0f), v1 = fmaxf(acc[i][j][2 * h + 1] + bv.y, 0.0f);
+                const float o0 = __shfl_xor_sync(0xffffffffu, v0, 4), o1 = __shfl_xor_sync(0xffffffffu, v1, 4);
+                if ((g & 1) != 0) continue;
+                const int q = (row0 + 16 * i + g + 8 * h) >> 1, col = 8 * j + 2 * t;
+                const bool w0 = o0 > v0, w1 = o1 > v1;   // the first of equal values wins
+                *reinterpret_cast<__nv_bfloat162*>(pool + q * kCh + col) =
+                    __nv_bfloat162(__float2bfloat16(w0 ? o0 : v0), __float2bfloat16(w1 ? o1 : v1));
+                if (kArg) *reinterpret_cast<uint16_t*>(arg + q * kCh + col) = (uint16_t)((w0 ? 1 : 0) | (w1 ? 256 : 0));
+            }
+        }
+    }
+}
+
+// The staged output tile to global memory (64 pooled rows, contiguous).
+template <bool kArg>
+__device__ __forceinline__ void store_pool_tile(const bf16* pool, const uint8_t* arg, bf16* out, uint8_t* arg_out)
+{
+    for (int e = threadIdx.x; e < kRows / 2 * kCh / 8; e += blockDim.x)
+        reinterpret_cast<uint4*>(out)[e] = reinterpret_cast<const uint4*>(pool)[e];
+    if (kArg)
+        for (int e = threadIdx.x; e < kRows / 2 * kCh / 16; e += blockDim.x)
+            reinterpret_cast<uint4*>(arg_out)[e] = reinterpret_cast<const uint4*>(arg)[e];
+}
+
+// ---------------------------------------------------------------------------
+// convolution 0 (one input channel, 7 taps): the taps are one zero-padded k16
+// step; the FP32 input is rounded here (and kept for the backward pass).
+// Bound by the stores of its pooled output: 256 curves 32 us (67 MB)
+// ---------------------------------------------------------------------------
+
+template <bool kTrain>
+__global__ void __launch_bounds__(128) k_conv0(const float* __restrict__ x, const bf16* __restrict__ w,
+                                               const float* __restrict__ bias, bf16* __restrict__ xb,
+                                               bf16* __restrict__ out, uint8_t* __restrict__ arg_out, int tiles)
+{
+    __shared__ bf16 xs[kRows + 16];
+    __shared__ __align__(16) bf16 pool[kRows / 2 * kCh];
+    __shared__ __align__(16) uint8_t arg[kTrain ? kRows / 2 * kCh : 16];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = lane >> 2, t = lane & 3;
+    const uint32_t last = t == 3 ? 0x0000ffffu : 0xffffffffu;   // taps 0..6 of the eight
+    uint32_t b[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const bf16* r = w + (8 * j + g) * 7 + 2 * t;
+        b[j] = (uint32_t)__bfloat16_as_ushort(r[0]) |
+               (t < 3 ? (uint32_t)__bfloat16_as_ushort(r[1]) << 16 : 0u);
+    }
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int64_t row0 = (int64_t)tile * kRows;
+        const int l0 = (int)(row0 % kBins);
+        for (int e = threadIdx.x; e < kRows + 8; e += blockDim.x) {
+            const int l = l0 + e - 3;
+            const bf16 v = __float2bfloat16(l >= 0 && l < kBins ? x[row0 + e - 3] : 0.0f);
+            xs[e] = v;
+            if (kTrain && e >= 3 && e < kRows + 3) xb[row0 + e - 3] = v;
+        }
+        __syncthreads();
+        float acc[2][8][4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            uint32_t a[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const bf16* r = xs + warp * 32 + 16 * i + 8 * h + g + 2 * t;
+                a[h] = ((uint32_t)__bfloat16_as_ushort(r[0]) | (uint32_t)__bfloat16_as_ushort(r[1]) << 16) & last;
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) acc[i][j][u] = 0.0f;
+                mma_bf16(acc[i][j], a, b[j], 0u);
+            }
+        }
+        pool_tile<kTrain>(acc, bias, warp * 32, lane, pool, arg);
+        __syncthreads();
+        store_pool_tile<kTrain>(pool, arg, out + row0 / 2 * kCh, kTrain ? arg_out + row0 / 2 * kCh : nullptr);
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// convolutions 1..5, and their data gradient (kBack: the 'same' convolution
+// of the pre-activation gradient with the flipped taps; the transposed
+// weights are read through ldmatrix.trans from the same staged weights).
+// Four warps of 32 rows x 64 columns; the weights stay staged over a CTA's
+// tiles, and three CTAs of an SM overlap their staging and their products.
+// ---------------------------------------------------------------------------
+
+struct ConvArgs {
+    const bf16* x;            // activations in (!kBack)
+    PoolGrad pg;              // pre-activation gradient in (kBack)
+    const bf16* w;            // [64][5][64]
+    const float* bias;
+    bf16* pooled;             // out (!kBack)
+    uint8_t* arg;
+    float* dx;                // out (kBack)
+    int L, dil, tiles;
+};
+
+template <bool kBack, bool kArg>
+__global__ void __launch_bounds__(128, 3) k_conv(const __grid_constant__ ConvArgs c)
+{
+    extern __shared__ __align__(128) unsigned char conv_smem[];
+    unsigned char* const ws = conv_smem;
+    unsigned char* const as = conv_smem + kWBytes;
+    const uint32_t ws_a = smem_addr(ws), as_a = smem_addr(as);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = lane >> 2, t = lane & 3, m8 = lane >> 3, r8 = lane & 7;
+    for (int e = threadIdx.x; e < kConvTaps * kCh * 8; e += blockDim.x) {
+        const int tap = e / (kCh * 8), co = (e >> 3) % kCh, ch = e & 7;
+        copy16(ws_a + tap * kCh * 128 + at128(co, ch), c.w + (co * kConvTaps + tap) * kCh + 8 * ch, true);
+    }
+    const int halo = 2 * c.dil, rows = kRows + 2 * halo;
+    const int per = c.L / kRows;
+    for (int tile = blockIdx.x; tile < c.tiles; tile += gridDim.x) {
+        const int seq = tile / per, l0 = (tile - seq * per) * kRows;
+        if (kBack) stage_pool_grad(as, c.pg, (int64_t)seq * (c.L / 2), l0 - halo, rows, c.L);
+        else stage_rows(as_a, c.x + (int64_t)seq * c.L * kCh, l0 - halo, rows, c.L);
+        copies_done();
+        __syncthreads();
+        float acc[2][8][4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) acc[i][j][u] = 0.0f;
+        for (int tap = 0; tap < kConvTaps; ++tap) {
+            const int base = warp * 32 + tap * c.dil + (lane & 15);
+            const uint32_t wt = ws_a + (kBack ? kConvTaps - 1 - tap : tap) * kCh * 128;
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+                uint32_t a[2][4];
+#pragma unroll
+                for (int i = 0; i < 2; ++i) ldsm4(a[i], as_a + at128(base + 16 * i, 2 * ks + (lane >> 4)));
+#pragma unroll
+                for (int jp = 0; jp < 4; ++jp) {
+                    uint32_t b[4];
+                    if (kBack) ldsm4t(b, wt + at128(16 * ks + 8 * (m8 & 1) + r8, 2 * jp + (m8 >> 1)));
+                    else ldsm4(b, wt + at128(16 * jp + 8 * (m8 >> 1) + r8, 2 * ks + (m8 & 1)));
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        mma_bf16(acc[i][2 * jp], a[i], b[0], b[1]);
+                        mma_bf16(acc[i][2 * jp + 1], a[i], b[2], b[3]);
                     }
-                } else if (row < M && col < N) {
-                    if (ep.bias) v += ep.bias[col];
-                    if (ep.kind == kEpiStore) ep.out[(int64_t)row * ep.ld + col] = v;
-                    else atomicAdd(&ep.out[(int64_t)row * ep.ld + col], v);
                 }
             }
         }
+        __syncthreads();   // the tile is read: its space takes the output
+        if (kBack) {
+            float* const out = c.dx + ((int64_t)seq * c.L + l0 + warp * 32) * kCh;
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        *reinterpret_cast<float2*>(out + (16 * i + g + 8 * h) * kCh + 8 * j + 2 * t) =
+                            make_float2(acc[i][j][2 * h], acc[i][j][2 * h + 1]);
+        } else {
+            bf16* const pool = reinterpret_cast<bf16*>(as);
+            uint8_t* const arg = as + kRows / 2 * 128;
+            pool_tile<kArg>(acc, c.bias, warp * 32, lane, pool, arg);
+            __syncthreads();
+            const int64_t q0 = ((int64_t)seq * c.L + l0) / 2 * kCh;
+            store_pool_tile<kArg>(pool, arg, c.pooled + q0, kArg ? c.arg + q0 : nullptr);
+            __syncthreads();
+        }
     }
 }
 
-template <class LA, class LB>
-gtls_status gemm(int M, int N, int K, int k_chunk, LA la, LB lb, Epi ep, cudaStream_t st)
+// Weight and bias gradient of convolutions 1..5: dW[co][tap][ci] = sum over
+// positions of dpre[l][co] x[l + (tap - 2) dil][ci].  Both operands are read
+// transposed from tiles of positions; a CTA keeps all 64 x 320 sums in
+// registers over its tiles (warp w: input channels 8 w .. 8 w + 7 of every
+// tap) and adds them to the gradient once.
+__global__ void __launch_bounds__(256, 1) k_conv_dw(const __grid_constant__ ConvArgs c, float* __restrict__ dw,
+                                                    float* __restrict__ db)
 {
-    if (k_chunk <= 0) k_chunk = K;
-    k_chunk = (k_chunk + kBK - 1) / kBK * kBK;
-    const dim3 grid((unsigned)((M + kBM - 1) / kBM), (unsigned)((N + kBN - 1) / kBN),
-                    (unsigned)((K + k_chunk - 1) / k_chunk));
-    k_gemm<LA, LB><<<grid, 128, 0, st>>>(M, N, K, k_chunk, la, lb, ep);
-    PROP_CUDA(cudaGetLastError());
-    return GTLS_OK;
+    extern __shared__ __align__(128) unsigned char conv_smem[];
+    unsigned char* const ds = conv_smem;               // dpre: 128 rows
+    unsigned char* const xs = conv_smem + kRows * 128; // x: 128 rows and the halo
+    const uint32_t ds_a = smem_addr(ds), xs_a = smem_addr(xs);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = lane >> 2, t = lane & 3, m8 = lane >> 3, r8 = lane & 7;
+    const int halo = 2 * c.dil, per = c.L / kRows;
+    float acc[kConvTaps][4][4];
+#pragma unroll
+    for (int tap = 0; tap < kConvTaps; ++tap)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) acc[tap][i][u] = 0.0f;
+    float colsum = 0.0f;
+    for (int tile = blockIdx.x; tile < c.tiles; tile += gridDim.x) {
+        const int seq = tile / per, l0 = (tile - seq * per) * kRows;
+        stage_rows(xs_a, c.x + (int64_t)seq * c.L * kCh, l0 - halo, kRows + 2 * halo, c.L);
+        stage_pool_grad(ds, c.pg, (int64_t)seq * (c.L / 2), l0, kRows, c.L);
+        copies_done();
+        __syncthreads();
+        for (int k0 = 0; k0 < kRows; k0 += 16) {
+            uint32_t a[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                ldsm4t(a[i], ds_a + at128(k0 + 8 * (m8 >> 1) + r8, 2 * i + (m8 & 1)));
+#pragma unroll
+            for (int tap = 0; tap < kConvTaps; ++tap) {
+                uint32_t b0, b1;
+                ldsm2t(b0, b1, xs_a + at128(k0 + tap * c.dil + 8 * (m8 & 1) + r8, warp));
+#pragma unroll
+                for (int i = 0; i < 4; ++i) mma_bf16(acc[tap][i], a[i], b0, b1);
+            }
+        }
+        {
+            const int col = threadIdx.x & 63, r0 = (threadIdx.x >> 6) * 32;
+#pragma unroll 8
+            for (int r = r0; r < r0 + 32; ++r)
+                colsum += __bfloat162float(*reinterpret_cast<const bf16*>(ds + at128(r, col >> 3) + 2 * (col & 7)));
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int tap = 0; tap < kConvTaps; ++tap)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                atomicAdd(reinterpret_cast<float2*>(dw + ((16 * i + g + 8 * h) * kConvTaps + tap) * kCh + 8 * warp + 2 * t),
+                          make_float2(acc[tap][i][2 * h], acc[tap][i][2 * h + 1]));
+    atomicAdd(db + (threadIdx.x & 63), colsum);
+}
+
+// The same for convolution 0 (one input channel, 7 taps): the warps split the
+// positions of a tile.
+__global__ void __launch_bounds__(256) k_conv0_dw(const bf16* __restrict__ x, const PoolGrad pg, float* __restrict__ dw,
+                                                  float* __restrict__ db, int tiles)
+{
+    __shared__ __align__(128) unsigned char ds[kRows * 128];
+    __shared__ bf16 xs[kRows + 16];
+    __shared__ float sum[kCh * 8];
+    const uint32_t ds_a = smem_addr(ds);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = lane >> 2, t = lane & 3, m8 = lane >> 3, r8 = lane & 7;
+    for (int e = threadIdx.x; e < kCh * 8; e += blockDim.x) sum[e] = 0.0f;
+    float acc[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[i][u] = 0.0f;
+    float colsum = 0.0f;
+    for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int64_t row0 = (int64_t)tile * kRows;
+        const int l0 = (int)(row0 % kBins);
+        stage_pool_grad(ds, pg, row0 / kBins * (kBins / 2), l0, kRows, kBins);
+        for (int e = threadIdx.x; e < kRows + 8; e += blockDim.x) {
+            const int l = l0 + e - 3;
+            xs[e] = l >= 0 && l < kBins ? x[row0 + e - 3] : __float2bfloat16(0.0f);
+        }
+        __syncthreads();
+        const int k0 = warp * 16;
+        // positions k0 + 2 t, + 1 (and + 8) and tap g (the eighth column is not used)
+        const bf16* r = xs + k0 + 2 * t + g;
+        const uint32_t b0 = (uint32_t)__bfloat16_as_ushort(r[0]) | (uint32_t)__bfloat16_as_ushort(r[1]) << 16;
+        const uint32_t b1 = (uint32_t)__bfloat16_as_ushort(r[8]) | (uint32_t)__bfloat16_as_ushort(r[9]) << 16;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            uint32_t a[4];
+            ldsm4t(a, ds_a + at128(k0 + 8 * (m8 >> 1) + r8, 2 * i + (m8 & 1)));
+            mma_bf16(acc[i], a, b0, b1);
+        }
+        const int col = threadIdx.x & 63, q0 = (threadIdx.x >> 6) * 32;
+#pragma unroll 8
+        for (int q = q0; q < q0 + 32; ++q)
+            colsum += __bfloat162float(*reinterpret_cast<const bf16*>(ds + at128(q, col >> 3) + 2 * (col & 7)));
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) atomicAdd(&sum[(16 * i + g + 8 * (u >> 1)) * 8 + 2 * t + (u & 1)], acc[i][u]);
+    __syncthreads();
+    for (int e = threadIdx.x; e < kCh * 7; e += blockDim.x) atomicAdd(dw + e, sum[e / 7 * 8 + e % 7]);
+    atomicAdd(db + (threadIdx.x & 63), colsum);
+}
+
+// ---------------------------------------------------------------------------
+// head
+// ---------------------------------------------------------------------------
+
+// z[row][reg] = bias + sum_f feat[row][f] wh[reg][f]: 16 rows x 16 regions per
+// CTA, the features split over its eight warps (a batch of 256 gives 128 CTAs,
+// one curve 8).  A lane's 16-byte loads hold the k indices of two k16 steps
+// (the same permutation of k on both sides).
+__global__ void __launch_bounds__(256) k_head(const bf16* __restrict__ feat, const bf16* __restrict__ wh,
+                                              const float* __restrict__ bias, float* __restrict__ z,
+                                              float* __restrict__ logits, float* __restrict__ scores, int B)
+{
+    __shared__ float part[8][16][17];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = lane >> 2, t = lane & 3;
+    const int row0 = blockIdx.x * 16, n0 = blockIdx.y * 16;
+    constexpr int kSpan = kFeat / 8;
+    const uint4* fa = reinterpret_cast<const uint4*>(feat + (int64_t)min(row0 + g, B - 1) * kFeat + warp * kSpan) + t;
+    const uint4* fb = reinterpret_cast<const uint4*>(feat + (int64_t)min(row0 + g + 8, B - 1) * kFeat + warp * kSpan) + t;
+    const uint4* wa = reinterpret_cast<const uint4*>(wh + (int64_t)(n0 + g) * kFeat + warp * kSpan) + t;
+    const uint4* wb = reinterpret_cast<const uint4*>(wh + (int64_t)(n0 + g + 8) * kFeat + warp * kSpan) + t;
+    float acc[2][4] = {{0.0f, 0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f, 0.0f}};
+#pragma unroll 4
+    for (int k = 0; k < kSpan / 32; ++k) {
+        const uint4 a0 = __ldg(fa + 4 * k), a1 = __ldg(fb + 4 * k), b0 = __ldg(wa + 4 * k), b1 = __ldg(wb + 4 * k);
+        const uint32_t lo[4] = {a0.x, a1.x, a0.y, a1.y}, hi[4] = {a0.z, a1.z, a0.w, a1.w};
+        mma_bf16(acc[0], lo, b0.x, b0.y);
+        mma_bf16(acc[1], lo, b1.x, b1.y);
+        mma_bf16(acc[0], hi, b0.z, b0.w);
+        mma_bf16(acc[1], hi, b1.z, b1.w);
+    }
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) part[warp][g + 8 * (u >> 1)][8 * j + 2 * t + (u & 1)] = acc[j][u];
+    __syncthreads();
+    const int r = threadIdx.x >> 4, n = threadIdx.x & 15;
+    if (row0 + r >= B) return;
+    float v = 0.0f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) v += part[w][r][n];
+    v += bias[n0 + n];
+    const int64_t o = (int64_t)(row0 + r) * kReg + n0 + n;
+    z[o] = v;
+    if (logits) logits[o] = v;
+    if (scores) scores[o] = 1.0f / (1.0f + expf(-v));
+}
+
+// The same sums in one chain of k16 steps per output (training: the gradient
+// of the logits is rounded to BF16, where the rounding of the logits would
+// show): 16 rows x 32 regions per CTA, a warp 8 regions, 256 features staged
+// ahead of the products.
+constexpr int kHeadSpan = 256;
+constexpr int kHeadBytes = (16 + 32) * kHeadSpan * 2;   // one stage
+
+__global__ void __launch_bounds__(128) k_head_chain(const bf16* __restrict__ feat, const bf16* __restrict__ wh,
+                                                    const float* __restrict__ bias, float* __restrict__ z, int B)
+{
+    __shared__ __align__(128) unsigned char hs[2 * kHeadBytes];
+    const uint32_t hs_a = smem_addr(hs);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = lane >> 2, t = lane & 3;
+    const int row0 = blockIdx.x * 16, n0 = blockIdx.y * 32;
+    // a stage: per 64 features, 16 rows of features and 32 of weights
+    auto stage = [&](int k, uint32_t to) {
+        for (int e = threadIdx.x; e < 48 * (kHeadSpan / 8); e += 128) {
+            const int c = e & 7, r = (e >> 3) % 48, sub = e / (8 * 48);
+            const int f = k * kHeadSpan + sub * 64 + 8 * c;
+            const bool in = r >= 16 || row0 + r < B;
+            const bf16* src = r < 16 ? feat + (int64_t)(in ? row0 + r : 0) * kFeat : wh + (int64_t)(n0 + r - 16) * kFeat;
+            copy16(to + sub * 48 * 128 + at128(r, c), src + f, in);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    stage(0, hs_a);
+    for (int k = 0; k < kFeat / kHeadSpan; ++k) {
+        const uint32_t at = hs_a + (k & 1) * kHeadBytes;
+        if (k + 1 < kFeat / kHeadSpan) {
+            stage(k + 1, hs_a + ((k + 1) & 1) * kHeadBytes);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+#pragma unroll
+        for (int ks = 0; ks < kHeadSpan / 16; ks += 2) {
+            const uint32_t sub = at + (ks >> 2) * 48 * 128;
+            uint32_t a0[4], a1[4], b[4];
+            ldsm4(a0, sub + at128(lane & 15, 2 * (ks & 3) + (lane >> 4)));
+            ldsm4(a1, sub + at128(lane & 15, 2 * ((ks + 1) & 3) + (lane >> 4)));
+            ldsm4(b, sub + at128(16 + 8 * warp + (lane & 7), 2 * (ks & 3) + (lane >> 3)));   // k16 steps ks, ks + 1
+            mma_bf16(acc, a0, b[0], b[1]);
+            mma_bf16(acc, a1, b[2], b[3]);
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int r = row0 + g + 8 * (u >> 1), n = n0 + 8 * warp + 2 * t + (u & 1);
+        if (r < B) z[(int64_t)r * kReg + n] = acc[u] + bias[n];
+    }
+}
+
+// dWh[reg][f] = sum_b dz[b][reg] feat[b][f] for 32 features per CTA (warp w:
+// regions 16 w ..), and the bias gradient (CTA 0).
+__global__ void __launch_bounds__(256) k_head_dw(const bf16* __restrict__ dzb, const float* __restrict__ dz,
+                                                 const bf16* __restrict__ feat, float* __restrict__ dw,
+                                                 float* __restrict__ db, int B)
+{
+    __shared__ __align__(128) unsigned char zs[64 * 256];   // 64 rows of 128 regions (two 128-byte halves)
+    __shared__ __align__(128) unsigned char fs[64 * 128];   // 64 rows of 32 features (a 128-byte row each, half used)
+    const uint32_t zs_a = smem_addr(zs), fs_a = smem_addr(fs);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = lane >> 2, t = lane & 3, m8 = lane >> 3, r8 = lane & 7;
+    const int f0 = blockIdx.x * 32;
+    float acc[4][4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[j][u] = 0.0f;
+    for (int b0 = 0; b0 < B; b0 += 64) {
+        for (int e = threadIdx.x; e < 64 * 16; e += blockDim.x) {
+            const int r = e >> 4, c = e & 15;
+            const bool in = b0 + r < B;
+            copy16(zs_a + (c >> 3) * 64 * 128 + at128(r, c & 7), dzb + (int64_t)(in ? b0 + r : 0) * kReg + 8 * c, in);
+        }
+        {
+            const int r = threadIdx.x >> 2, c = threadIdx.x & 3;
+            const bool in = b0 + r < B;
+            copy16(fs_a + at128(r, c), feat + (int64_t)(in ? b0 + r : 0) * kFeat + f0 + 8 * c, in);
+        }
+        copies_done();
+        __syncthreads();
+#pragma unroll
+        for (int k0 = 0; k0 < 64; k0 += 16) {
+            uint32_t a[4];
+            ldsm4t(a, zs_a + (warp >> 2) * 64 * 128 + at128(k0 + 8 * (m8 >> 1) + r8, 2 * (warp & 3) + (m8 & 1)));
+#pragma unroll
+            for (int jp = 0; jp < 2; ++jp) {
+                uint32_t b[4];
+                ldsm4t(b, fs_a + at128(k0 + 8 * (m8 & 1) + r8, 2 * jp + (m8 >> 1)));
+                mma_bf16(acc[2 * jp], a, b[0], b[1]);
+                mma_bf16(acc[2 * jp + 1], a, b[2], b[3]);
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            *reinterpret_cast<float2*>(dw + (int64_t)(16 * warp + g + 8 * h) * kFeat + f0 + 8 * j + 2 * t) =
+                make_float2(acc[j][2 * h], acc[j][2 * h + 1]);
+    if (blockIdx.x == 0 && threadIdx.x < kReg) {
+        float s = 0.0f;
+#pragma unroll 8
+        for (int b = 0; b < B; ++b) s += dz[(int64_t)b * kReg + threadIdx.x];
+        db[threadIdx.x] = s;
+    }
+}
+
+// dfeat[b][f] = sum_reg dz[b][reg] wh[reg][f]: 64 rows x 64 features per CTA.
+__global__ void __launch_bounds__(128) k_head_dx(const bf16* __restrict__ dzb, const bf16* __restrict__ wh,
+                                                 float* __restrict__ dfeat, int B)
+{
+    __shared__ __align__(128) unsigned char zs[64 * 256];
+    __shared__ __align__(128) unsigned char ws[kReg * 128];
+    const uint32_t zs_a = smem_addr(zs), ws_a = smem_addr(ws);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = lane >> 2, t = lane & 3, m8 = lane >> 3, r8 = lane & 7;
+    const int b0 = blockIdx.x * 64, f0 = blockIdx.y * 64;
+    for (int e = threadIdx.x; e < 64 * 16; e += blockDim.x) {
+        const int r = e >> 4, c = e & 15;
+        const bool in = b0 + r < B;
+        copy16(zs_a + (c >> 3) * 64 * 128 + at128(r, c & 7), dzb + (int64_t)(in ? b0 + r : 0) * kReg + 8 * c, in);
+    }
+    for (int e = threadIdx.x; e < kReg * 8; e += blockDim.x)
+        copy16(ws_a + at128(e >> 3, e & 7), wh + (int64_t)(e >> 3) * kFeat + f0 + 8 * (e & 7), true);
+    copies_done();
+    __syncthreads();
+    float acc[8][4];
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc[j][u] = 0.0f;
+#pragma unroll
+    for (int ks = 0; ks < kReg / 16; ++ks) {
+        uint32_t a[4];
+        ldsm4(a, zs_a + (ks >> 2) * 64 * 128 + at128(warp * 16 + (lane & 15), 2 * (ks & 3) + (lane >> 4)));
+#pragma unroll
+        for (int jp = 0; jp < 4; ++jp) {
+            uint32_t b[4];
+            ldsm4t(b, ws_a + at128(16 * ks + 8 * (m8 & 1) + r8, 2 * jp + (m8 >> 1)));
+            mma_bf16(acc[2 * jp], a, b[0], b[1]);
+            mma_bf16(acc[2 * jp + 1], a, b[2], b[3]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int r = b0 + warp * 16 + g + 8 * h;
+            if (r < B)
+                *reinterpret_cast<float2*>(dfeat + (int64_t)r * kFeat + f0 + 8 * j + 2 * t) =
+                    make_float2(acc[j][2 * h], acc[j][2 * h + 1]);
+        }
 }
 
 // ---------------------------------------------------------------------------
@@ -246,74 +724,69 @@ __global__ void k_to_bf16(const float* __restrict__ x, bf16* __restrict__ y, int
         y[i] = __float2bfloat16(x[i]);
 }
 
-// d pre-activation of a ReLU + max-pool layer: the pooled gradient goes to
-// the winning row of each pair when the pooled value is positive.
-__global__ void k_pool_back(const float* __restrict__ dpool, const bf16* __restrict__ pooled,
-                            const uint8_t* __restrict__ arg, bf16* __restrict__ dpre, int64_t n_pooled)
+// Masked logistic loss with soft targets: loss = sum mask (softplus(z) - t z)
+// / sum mask; dz = mask (sigmoid(z) - t) / sum mask (FP32 and BF16).  The FP64
+// transcendentals bound it (a warp's FP64 instruction takes an SM 16 cycles: 72
+// us at a batch of 128 on 16 SMs), so the elements are spread over all SMs; each sums the mask for itself, and
+// the last one to finish adds the blocks' parts (one per thread).
+constexpr int kLossBlocks = 128, kLossThreads = 128;
+static_assert(kLossBlocks <= kLossThreads, "the last block reads one part per thread");
+
+__device__ __forceinline__ double block_sum_fp64(double v, double* sh)
 {
-    for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < n_pooled;
-         q += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t pos = q / kCh, c = q - pos * kCh;
-        const float gsum = __bfloat162float(pooled[q]) > 0.0f ? dpool[q] : 0.0f;
-        const int a = arg[q];
-        dpre[(2 * pos + a) * kCh + c] = __float2bfloat16(gsum);
-        dpre[(2 * pos + 1 - a) * kCh + c] = __float2bfloat16(0.0f);
+    sh[threadIdx.x] = v;
+    __syncthreads();
+    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
+        if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
+        __syncthreads();
     }
+    const double r = sh[0];
+    __syncthreads();
+    return r;
 }
 
-// Column sums of a [rows][cols] matrix (bf16 or f32) into g[cols] (+=).
-template <class T>
-__global__ void k_col_sum(const T* __restrict__ m, int64_t rows, int cols, float* __restrict__ g)
-{
-    const int c = threadIdx.x % cols;
-    const int lanes = blockDim.x / cols;
-    const int r0 = threadIdx.x / cols;
-    float s = 0.0f;
-    for (int64_t r = blockIdx.x * (int64_t)lanes + r0; r < rows; r += (int64_t)gridDim.x * lanes) {
-        if constexpr (sizeof(T) == 2) s += __bfloat162float(m[r * cols + c]);
-        else s += m[r * cols + c];
-    }
-    if (r0 < lanes) atomicAdd(&g[c], s);
-}
-
-// Masked logistic loss with soft targets (one block): loss = sum mask
-// (softplus(z) - t z) / sum mask; dz = mask (sigmoid(z) - t) / sum mask.
-__global__ void __launch_bounds__(1024) k_loss(const float* __restrict__ z, const float* __restrict__ tgt,
+__global__ void __launch_bounds__(kLossThreads) k_loss(const float* __restrict__ z, const float* __restrict__ tgt,
                                                const float* __restrict__ mask, int n, float* __restrict__ dz,
-                                               double* __restrict__ loss)
+                                               bf16* __restrict__ dzb, double* __restrict__ part,
+                                               unsigned int* __restrict__ done, double* __restrict__ loss)
 {
-    __shared__ double sh[1024];
+    __shared__ double sh[kLossThreads];
+    __shared__ bool last;
+    // masks of zeros and ones are counted in integers
+    int ones = 0;
     double cnt = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) cnt += mask[i];
-    sh[threadIdx.x] = cnt;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
-    }
-    const double total = fmax(sh[0], 1.0);
-    __syncthreads();
-    double acc = 0.0;
+#pragma unroll 8
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const float m = mask[i];
+        if (m == 1.0f) ++ones;
+        else if (m != 0.0f) cnt += m;
+    }
+    const double total = fmax(block_sum_fp64(cnt + ones, sh), 1.0);
+    double acc = 0.0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const double zi = z[i], m = mask[i], ti = tgt[i];
-        const double sp = zi > 0.0 ? zi + log1p(exp(-zi)) : log1p(exp(zi));
-        acc += m * (sp - ti * zi);
-        const double sg = 1.0 / (1.0 + exp(-zi));
-        dz[i] = (float)(m * (sg - ti) / total);
+        const double e = exp(-fabs(zi)), inv = 1.0 / (1.0 + e);
+        acc += m * (fmax(zi, 0.0) + log1p(e) - ti * zi);
+        const double sg = zi >= 0.0 ? inv : e * inv;
+        const float d = (float)(m * (sg - ti) / total);
+        dz[i] = d;
+        dzb[i] = __float2bfloat16(d);
     }
-    sh[threadIdx.x] = acc;
+    acc = block_sum_fp64(acc, sh);
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = acc;
+        __threadfence();
+        last = atomicAdd(done, 1u) == gridDim.x - 1;
+    }
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
+    if (last) {   // block-uniform
+        __threadfence();
+        const double all = block_sum_fp64(threadIdx.x < gridDim.x ? __ldcg(part + threadIdx.x) : 0.0, sh);
+        if (threadIdx.x == 0) {
+            *loss = all / total;
+            *done = 0u;
+        }
     }
-    if (threadIdx.x == 0) *loss = sh[0] / total;
-}
-
-__global__ void k_sigmoid(const float* __restrict__ z, float* __restrict__ s, int n)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) s[i] = 1.0f / (1.0f + expf(-z[i]));
 }
 
 // Adam (Kingma & Ba 2015) on the FP32 master parameters, then their BF16 copy.
@@ -412,8 +885,9 @@ struct gtls_cnn {
     float* dz = nullptr;
     bf16* dz_b = nullptr;
     float* da[2] = {};        // FP32 gradient of a pooled output (ping-pong)
-    bf16* dpre = nullptr;     // BF16 gradient of a pre-activation
-    double* loss = nullptr;
+    double* loss = nullptr;   // [0] loss, [1 ..] the loss blocks' parts
+    unsigned int* loss_done = nullptr;
+    int n_sm = 0;
     int64_t* off = nullptr;   // binning offsets (max_batch + 1)
     std::vector<void*> allocs;
 };
@@ -435,72 +909,77 @@ gtls_status cnn_alloc(gtls_cnn* c, T** ptr, int64_t count)
 }
 
 int conv_len(int i) { return kBins >> i; }      // input length of conv i
-int conv_cin(int i) { return i == 0 ? 1 : kCh; }
 
-gtls_status cnn_forward(gtls_cnn* c, const float* x, int B, cudaStream_t st)
+// Logits into c->z (and the caller's arrays).  `train`: the input and the
+// pooling choices are kept for the backward pass.
+gtls_status cnn_forward(gtls_cnn* c, const float* x, int B, bool train, float* logits, float* scores, cudaStream_t st)
 {
-    const int64_t nin = (int64_t)B * kBins;
-    k_to_bf16<<<grid_for(nin), 256, 0, st>>>(x, c->act[0], nin);
+    const int tiles0 = B * (kBins / kRows), grid0 = std::min(tiles0, c->n_sm * 12);
+    const bf16* w0 = c->pb + c->lay.w[0];
+    const float* b0 = c->p + c->lay.b[0];
+    if (train) k_conv0<true><<<grid0, 128, 0, st>>>(x, w0, b0, c->act[0], c->act[1], c->arg[0], tiles0);
+    else k_conv0<false><<<grid0, 128, 0, st>>>(x, w0, b0, c->act[0], c->act[1], c->arg[0], tiles0);
     PROP_CUDA(cudaGetLastError());
-    for (int i = 0; i < kConv; ++i) {
-        const int L = conv_len(i), cin = conv_cin(i), taps = kTaps[i];
-        ConvIn a{c->act[i], L, cin, (taps - 1) / 2, kDil[i]};
-        RowMajor w{c->pb + c->lay.w[i], taps * cin};
-        Epi ep{kEpiPoolRelu, nullptr, kCh, c->p + c->lay.b[i], c->act[i + 1], c->arg[i]};
-        PROP_TRY(gemm(B * L, kCh, taps * cin, 0, a, w, ep, st));
+    for (int i = 1; i < kConv; ++i) {
+        ConvArgs a{};
+        a.x = c->act[i];
+        a.w = c->pb + c->lay.w[i];
+        a.bias = c->p + c->lay.b[i];
+        a.pooled = c->act[i + 1];
+        a.arg = c->arg[i];
+        a.L = conv_len(i);
+        a.dil = kDil[i];
+        a.tiles = B * (a.L / kRows);
+        const int grid = std::min(a.tiles, c->n_sm * 3);
+        if (train) k_conv<false, true><<<grid, 128, kWBytes + kABytes, st>>>(a);
+        else k_conv<false, false><<<grid, 128, kWBytes + kABytes, st>>>(a);
+        PROP_CUDA(cudaGetLastError());
     }
-    RowMajor f{c->act[kConv], kFeat};
-    RowMajor wh{c->pb + c->lay.wh, kFeat};
-    Epi ep{kEpiStore, c->z, kReg, c->p + c->lay.bh, nullptr, nullptr};
-    return gemm(B, kReg, kFeat, 0, f, wh, ep, st);
+    if (train)
+        k_head_chain<<<dim3((unsigned)((B + 15) / 16), kReg / 32), 128, 0, st>>>(c->act[kConv], c->pb + c->lay.wh,
+                                                                                c->p + c->lay.bh, c->z, B);
+    else
+        k_head<<<dim3((unsigned)((B + 15) / 16), kReg / 16), 256, 0, st>>>(c->act[kConv], c->pb + c->lay.wh,
+                                                                       c->p + c->lay.bh, c->z, logits, scores, B);
+    PROP_CUDA(cudaGetLastError());
+    return GTLS_OK;
 }
 
 gtls_status cnn_backward(gtls_cnn* c, const float* tgt, const float* mask, int B, cudaStream_t st)
 {
     const int nz = B * kReg;
-    k_loss<<<1, 1024, 0, st>>>(c->z, tgt, mask, nz, c->dz, c->loss);
+    k_loss<<<kLossBlocks, kLossThreads, 0, st>>>(c->z, tgt, mask, nz, c->dz, c->dz_b, c->loss + 1, c->loss_done, c->loss);
     PROP_CUDA(cudaGetLastError());
-    PROP_CUDA(cudaMemsetAsync(c->g, 0, c->lay.total * sizeof(float), st));
-    k_to_bf16<<<grid_for(nz), 256, 0, st>>>(c->dz, c->dz_b, nz);
+    // the convolutions' gradients are added up by many blocks
+    PROP_CUDA(cudaMemsetAsync(c->g, 0, c->lay.wh * sizeof(float), st));
+    k_head_dw<<<kFeat / 32, 256, 0, st>>>(c->dz_b, c->dz, c->act[kConv], c->g + c->lay.wh, c->g + c->lay.bh, B);
     PROP_CUDA(cudaGetLastError());
-    // head: dWh[r][f] = sum_b dz[b][r] feat[b][f]; dbh = sum_b dz; dfeat = dz Wh
-    {
-        ColMajor a{c->dz_b, kReg};
-        ColMajor b{c->act[kConv], kFeat};
-        Epi ep{kEpiAtomic, c->g + c->lay.wh, kFeat, nullptr, nullptr, nullptr};
-        PROP_TRY(gemm(kReg, kFeat, B, 0, a, b, ep, st));
-        k_col_sum<float><<<1, 1024, 0, st>>>(c->dz, B, kReg, c->g + c->lay.bh);
-        PROP_CUDA(cudaGetLastError());
-        RowMajor a2{c->dz_b, kReg};
-        ColMajor b2{c->pb + c->lay.wh, kFeat};
-        Epi ep2{kEpiStore, c->da[0], kFeat, nullptr, nullptr, nullptr};
-        PROP_TRY(gemm(B, kFeat, kReg, 0, a2, b2, ep2, st));
-    }
+    k_head_dx<<<dim3((unsigned)((B + 63) / 64), kFeat / 64), 128, 0, st>>>(c->dz_b, c->pb + c->lay.wh, c->da[0], B);
+    PROP_CUDA(cudaGetLastError());
     int cur = 0;
     for (int i = kConv - 1; i >= 0; --i) {
-        const int L = conv_len(i), cin = conv_cin(i), taps = kTaps[i];
-        const int64_t npool = (int64_t)B * (L / 2) * kCh;
-        k_pool_back<<<grid_for(npool), 256, 0, st>>>(c->da[cur], c->act[i + 1], c->arg[i], c->dpre, npool);
-        PROP_CUDA(cudaGetLastError());
-        const int64_t rows = (int64_t)B * L;
-        // dW[co][tap ci] = sum over positions of dpre[pos][co] x(pos, tap ci)
-        {
-            ColMajor a{c->dpre, kCh};
-            ConvInT b{ConvIn{c->act[i], L, cin, (taps - 1) / 2, kDil[i]}};
-            Epi ep{kEpiAtomic, c->g + c->lay.w[i], taps * cin, nullptr, nullptr, nullptr};
-            PROP_TRY(gemm(kCh, taps * cin, (int)rows, 8192, a, b, ep, st));
+        const PoolGrad pg{c->da[cur], c->act[i + 1], c->arg[i]};
+        const int tiles = B * (conv_len(i) / kRows);
+        if (i == 0) {
+            k_conv0_dw<<<std::min(tiles, c->n_sm * 6), 256, 0, st>>>(c->act[0], pg, c->g + c->lay.w[0],
+                                                                     c->g + c->lay.b[0], tiles);
+            PROP_CUDA(cudaGetLastError());
+            break;
         }
-        k_col_sum<bf16><<<256, 1024, 0, st>>>(c->dpre, rows, kCh, c->g + c->lay.b[i]);
+        ConvArgs a{};
+        a.x = c->act[i];
+        a.pg = pg;
+        a.w = c->pb + c->lay.w[i];
+        a.dx = c->da[cur ^ 1];
+        a.L = conv_len(i);
+        a.dil = kDil[i];
+        a.tiles = tiles;
+        k_conv_dw<<<std::min(tiles, c->n_sm), 256, kRows * 128 + kABytes, st>>>(a, c->g + c->lay.w[i],
+                                                                               c->g + c->lay.b[i]);
         PROP_CUDA(cudaGetLastError());
-        if (i > 0) {
-            // data gradient: 'same' convolution of dpre with the flipped,
-            // transposed taps -> gradient of conv i-1's pooled output
-            ConvIn a{c->dpre, L, kCh, (taps - 1) / 2, kDil[i]};
-            FlippedW b{c->pb + c->lay.w[i], taps, cin, kCh};
-            Epi ep{kEpiStore, c->da[cur ^ 1], cin, nullptr, nullptr, nullptr};
-            PROP_TRY(gemm((int)rows, cin, taps * kCh, 0, a, b, ep, st));
-            cur ^= 1;
-        }
+        k_conv<true, false><<<std::min(tiles, c->n_sm * 3), 128, kWBytes + kABytes, st>>>(a);
+        PROP_CUDA(cudaGetLastError());
+        cur ^= 1;
     }
     return GTLS_OK;
 }
@@ -560,16 +1039,22 @@ gtls_status gtls_cnn_create(int32_t max_batch, const float* params, gtls_cnn** o
     A(&c->dz_b, B * kReg);
     A(&c->da[0], B * (kBins / 2) * kCh);
     A(&c->da[1], B * (kBins / 2) * kCh);
-    A(&c->dpre, B * kBins * kCh);
-    A(&c->loss, 1);
+    A(&c->loss, 1 + kLossBlocks);
+    A(&c->loss_done, 1);
     A(&c->off, B + 1);
     if (s != GTLS_OK) return bail(s);
     std::vector<float> h(np, 0.0f);
     if (params) std::memcpy(h.data(), params, np * sizeof(float));
     if ((e = cudaMemcpy(c->p, h.data(), np * sizeof(float), cudaMemcpyHostToDevice)) != cudaSuccess ||
         (e = cudaMemset(c->m, 0, np * sizeof(float))) != cudaSuccess ||
-        (e = cudaMemset(c->v, 0, np * sizeof(float))) != cudaSuccess)
+        (e = cudaMemset(c->v, 0, np * sizeof(float))) != cudaSuccess ||
+        (e = cudaMemset(c->loss_done, 0, sizeof(unsigned int))) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&c->n_sm, cudaDevAttrMultiProcessorCount, c->device)) != cudaSuccess)
         return bail(set_error(GTLS_ERR_CUDA, cudaGetErrorString(e)));
+    for (const void* fn : {(const void*)k_conv<false, false>, (const void*)k_conv<false, true>,
+                           (const void*)k_conv<true, false>, (const void*)k_conv_dw})
+        if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kWBytes + kABytes)) != cudaSuccess)
+            return bail(set_error(GTLS_ERR_CUDA, cudaGetErrorString(e)));
     k_to_bf16<<<grid_for(np), 256>>>(c->p, c->pb, np);
     if ((e = cudaDeviceSynchronize()) != cudaSuccess) return bail(set_error(GTLS_ERR_CUDA, cudaGetErrorString(e)));
     if ((e = cudaFuncSetAttribute(k_bin, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -624,13 +1109,7 @@ gtls_status gtls_cnn_forward(gtls_cnn* c, const float* x, int32_t batch, float* 
     PROP_TRY(check_batch(c, batch));
     if (!x) return set_error(GTLS_ERR_INVALID_ARG, "null input");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    PROP_TRY(cnn_forward(c, x, batch, st));
-    const int nz = batch * kReg;
-    if (logits) PROP_CUDA(cudaMemcpyAsync(logits, c->z, nz * sizeof(float), cudaMemcpyDeviceToDevice, st));
-    if (scores) {
-        k_sigmoid<<<(nz + 255) / 256, 256, 0, st>>>(c->z, scores, nz);
-        PROP_CUDA(cudaGetLastError());
-    }
+    PROP_TRY(cnn_forward(c, x, batch, false, logits, scores, st));
     return GTLS_OK;
 }
 
@@ -640,7 +1119,7 @@ gtls_status gtls_cnn_gradient(gtls_cnn* c, const float* x, const float* target, 
     PROP_TRY(check_batch(c, batch));
     if (!x || !target || !mask) return set_error(GTLS_ERR_INVALID_ARG, "null pointer argument");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    PROP_TRY(cnn_forward(c, x, batch, st));
+    PROP_TRY(cnn_forward(c, x, batch, true, nullptr, nullptr, st));
     PROP_TRY(cnn_backward(c, target, mask, batch, st));
     if (grad) PROP_CUDA(cudaMemcpyAsync(grad, c->g, c->lay.total * sizeof(float), cudaMemcpyDeviceToHost, st));
     if (loss) PROP_CUDA(cudaMemcpyAsync(loss, c->loss, sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -655,7 +1134,7 @@ gtls_status gtls_cnn_train_step(gtls_cnn* c, const float* x, const float* target
     if (!x || !target || !mask) return set_error(GTLS_ERR_INVALID_ARG, "null pointer argument");
     if (!(lr > 0.0f)) return set_error(GTLS_ERR_INVALID_ARG, "lr must be > 0");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    PROP_TRY(cnn_forward(c, x, batch, st));
+    PROP_TRY(cnn_forward(c, x, batch, true, nullptr, nullptr, st));
     PROP_TRY(cnn_backward(c, target, mask, batch, st));
     c->step += 1;
     const float c1 = 1.0f - (float)std::pow(0.9, (double)c->step);
