@@ -1,4 +1,5 @@
-"""The proposal network at the edges of its tiles.
+"""The proposal network at the edges of its tiles, and time binning of curves
+in and out of time order.
 
 Logits and gradients do not depend on what else is in a batch: a curve's
 logits are the same bits whatever the batch (its products are added in one
@@ -56,3 +57,47 @@ def test_gradient_of_a_doubled_batch(batch):
     assert np.linalg.norm(g2 - g1) < 1e-5 * np.linalg.norm(g1)
     net.close()
 
+
+def _times(kind, n, rng):
+    t = np.sort(rng.uniform(0.0, 900.0, n))
+    if kind == "gaps":
+        t[t > 300.0] += 400.0
+    if kind == "equal":
+        t = np.repeat(t[:max(1, n // 3)], 3)[:n]
+        t = np.concatenate([t, np.full(n - t.size, t[-1])])
+    if kind == "grid":                                # points on bin edges
+        t = np.arange(n) * (900.0 / 4096)
+    if kind == "reversed":
+        t = t[::-1].copy()
+    if kind == "swapped" and n > 2:
+        t[n // 2 - 1], t[n // 2] = t[n // 2], t[n // 2 - 1]
+    if kind == "late":                                # the last point comes first
+        t = np.roll(t, 1)
+    return t
+
+
+@pytest.mark.parametrize("kind", ["sorted", "gaps", "equal", "grid", "reversed", "swapped", "late"])
+def test_binning_in_any_order(kind):
+    # FP64 sums of at most thousands of points, stored in FP32: 1e-6
+    import torch
+    rng = np.random.default_rng(7)
+    curves = []
+    for i, n in enumerate((1, 2, 3, 31, 4097, 9000, 20011)):
+        t = _times(kind, n, rng)
+        dy = np.full(n, 1e-3) if i % 2 else 1e-3 * rng.uniform(0.5, 1.5, n)
+        curves.append((t, 1.0 + rng.normal(0.0, 1e-3, n), dy))
+    offs = np.cumsum([0] + [c[0].size for c in curves])
+    net = pkg.Cnn(len(curves))
+    cat = lambda k: torch.as_tensor(np.concatenate([c[k] for c in curves]), dtype=torch.float64,  # noqa: E731
+                                    device="cuda:0")
+    for _ in range(2):      # a second call must not see the first one's flags
+        x = torch.full((len(curves), cnn.N_BINS), np.nan, dtype=torch.float32, device="cuda:0")
+        mean, wsum = torch.empty_like(x), torch.empty_like(x)
+        net.bin(cat(0), cat(1), cat(2), offs, x, mean=mean, wsum=wsum)
+        for i, (t, y, dy) in enumerate(curves):
+            swr, sw = cnn.bin_sums(t, y, dy)
+            np.testing.assert_allclose(x[i].cpu().numpy(), cnn.bin_flux(t, y, dy), rtol=1e-6, atol=1e-6)
+            np.testing.assert_allclose(wsum[i].cpu().numpy(), sw, rtol=1e-6)
+            keep = sw > 0
+            np.testing.assert_allclose(mean[i].cpu().numpy()[keep], swr[keep] / sw[keep], rtol=1e-6, atol=1e-9)
+    net.close()
