@@ -317,7 +317,7 @@ gtls_status gtls_plan_get_profile(const gtls_plan* plan, gtls_profile* out);
  * that cannot call cudaMalloc, e.g. code confined to a pre-sized memory pool
  * or to buffers handed over by another framework.)  Its scratch lives in a
  * fixed device array compiled into the library: 2^19 trial periods at most
- * (8 MiB plus a small header, held by every GPU that loads the library until
+ * (8 MiB plus a header of 20 KiB, held by every GPU that loads the library until
  * the process exits); larger inputs return GTLS_ERR_INVALID_ARG.
  *   chi2       device, n_periods doubles (input, read only)
  *   sr_out, sde_raw_out   device, n_periods doubles each, nullable (then

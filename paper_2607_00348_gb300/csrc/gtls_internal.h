@@ -115,6 +115,12 @@ struct DevChunk {
     unsigned int* left_n;     // [0 .. kListClasses) windows listed, [kListClasses] items in `dense`
 };
 
+// SR/SDE: blocks per curve of the reductions, and blocks of the running median
+// whose best SDE is kept (more: the spectrum itself is searched).
+constexpr int kSrBlocks = 128;
+constexpr int kTopBlocks = 1024;
+constexpr int kSrParts = 3 * kSrBlocks + 2 * kTopBlocks;
+
 // Per-period outputs (np long) and the reduction scratch.
 struct DevPeriod {
     unsigned long long* best; // packed (delta-chi2 key, j, window) minimum
@@ -127,6 +133,7 @@ struct DevPeriod {
     double* sde_raw;
     double* sde;
     double* stats;            // [0] chi2_min [1] mean SR [2] std SR
+    double* part;             // kSrParts: the SR/SDE blocks' minima, sums and square sums, and their best SDE
     unsigned int* check;      // same words as DevCurve::check
     int32_t* refined;         // 1 where the period was re-searched with T0 step 1
     int32_t* plist;           // the refine_k periods to re-search, in rank order

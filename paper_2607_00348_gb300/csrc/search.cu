@@ -21,7 +21,7 @@
 //                      k_window_search: one thread per window, for plans
 //                      whose durations do not fit a tile)
 //     k_period_finalize chi2(P), depth, T0 of each period's minimum
-//   k_sr_stats_set, k_median_sde_set        SR, SDE_raw, SDE (Sect. 2.4)
+//   k_sr_{min,sum,var}_set, k_median_sde_set   SR, SDE_raw, SDE (Sect. 2.4)
 //   k_topk + waves with T0 step 1           refinement of the best periods
 //                                           (Sect. 2.5), then SR/SDE again
 //   k_best                                  the candidate of largest SDE
@@ -1757,81 +1757,197 @@ __global__ void k_queue_reset(int32_t* cursors, int n)
 }
 
 // ---------------------------------------------------------------------------
-// SR, SDE_raw (one block), median detrending, argmax
+// SR, SDE_raw, median detrending, argmax
 // ---------------------------------------------------------------------------
+//
+// Three reductions (minimum of chi2, sum of SR, sum of (SR - mean)^2) over up
+// to kSrBlocks blocks; a kernel finishes the sums of the one before it, in
+// every block and in the same order.  Then the running median, whose blocks
+// also make SDE_raw.  (One block for the reductions took 1.3 ms at 199,577
+// periods.)  Doubles are compared by their order-preserving 64-bit keys: an
+// FP64 compare of a warp takes an SM 16 cycles.
 
-__device__ double block_sum_fixed(double v, double* sh)
+constexpr int kSrThreads = 256;
+
+// Blocks that share the reductions over np periods.
+__host__ __device__ __forceinline__ int sr_blocks(int np)
 {
-    // fixed-order tree over the block: deterministic for a given block size
-    sh[threadIdx.x] = v;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-        __syncthreads();
-    }
-    const double r = sh[0];
-    __syncthreads();
-    return r;
+    const int b = (np + 4 * kSrThreads - 1) / (4 * kSrThreads);
+    return b < kSrBlocks ? b : kSrBlocks;
 }
 
-__device__ void sr_stats_body(int np, const DevPeriod& dq, double* sh)
+// Sum over the block (kThreads threads, any fixed order), in thread 0: the FP64
+// pipe is so narrow that only one warp adds the warps' sums.
+template <int kThreads>
+__device__ __forceinline__ double block_sum(double v, double* sh)
 {
-    double mn = INFINITY;
-    for (int i = threadIdx.x; i < np; i += blockDim.x) mn = fmin(mn, dq.chi2[i]);
-    sh[threadIdx.x] = mn;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
     __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sh[threadIdx.x] = fmin(sh[threadIdx.x], sh[threadIdx.x + s]);
-        __syncthreads();
+    if (threadIdx.x >= 32) return 0.0;
+    v = (int)threadIdx.x < kThreads / 32 ? sh[threadIdx.x] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+template <int kThreads>
+__device__ __forceinline__ unsigned long long block_min(unsigned long long v, unsigned long long* sh)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long u = __shfl_xor_sync(0xffffffffu, v, o);
+        v = u < v ? u : v;
     }
-    const double cmin = sh[0];
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
     __syncthreads();
+    unsigned long long s = sh[0];
+#pragma unroll
+    for (int w = 1; w < kThreads / 32; ++w) s = sh[w] < s ? sh[w] : s;
+    __syncthreads();
+    return s;
+}
+
+// Sum of the first nb (<= kSrBlocks) parts, by one warp.
+__device__ __forceinline__ double sum_parts(const double* part, int nb)
+{
+    const int lane = threadIdx.x & 31;
+    double v = 0.0;
+#pragma unroll
+    for (int u = 0; u < kSrBlocks / 32; ++u) v += u * 32 + lane < nb ? part[u * 32 + lane] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Minimum of chi2 (NaN skipped).  With `check`, a value that is not finite and
+// >= 0 is recorded (code 18).
+__device__ __forceinline__ void sr_min_body(int np, int blk, const DevPeriod& dq, bool check)
+{
+    __shared__ unsigned long long sh[kSrThreads / 32];
+    const int nb = sr_blocks(np);
+    if (blk >= nb) return;
+    unsigned long long best = double_order_key(INFINITY);
+#pragma unroll 4
+    for (int i = blk * kSrThreads + threadIdx.x; i < np; i += nb * kSrThreads) {
+        const double c = dq.chi2[i];
+        const unsigned long long u = (unsigned long long)__double_as_longlong(c);
+        if (check && u > 0x7fefffffffffffffull && u != 0x8000000000000000ull) record_check(dq.check, 18, i, np);
+        const unsigned long long k = double_order_key(c);
+        if ((u & 0x7fffffffffffffffull) <= 0x7ff0000000000000ull && k < best) best = k;
+    }
+    best = block_min<kSrThreads>(best, sh);
+    if (threadIdx.x == 0) dq.part[blk] = double_from_order_key(best);
+}
+
+// SR = chi2_min / chi2 (0/0 := 1) and its sum.
+__device__ __forceinline__ void sr_sum_body(int np, int blk, const DevPeriod& dq)
+{
+    __shared__ double sh[kSrThreads / 32];
+    __shared__ unsigned long long shk[kSrThreads / 32];
+    const int nb = sr_blocks(np);
+    if (blk >= nb) return;
+    const double cmin = double_from_order_key(block_min<kSrThreads>(
+        double_order_key((int)threadIdx.x < nb ? dq.part[threadIdx.x] : INFINITY), shk));
     double acc = 0.0;
-    for (int i = threadIdx.x; i < np; i += blockDim.x) {
+    for (int i = blk * kSrThreads + threadIdx.x; i < np; i += nb * kSrThreads) {
         const double c = dq.chi2[i];
         const double sr = c > 0.0 ? cmin / c : 1.0;
         dq.sr[i] = sr;
         acc += sr;
     }
-    const double mean = block_sum_fixed(acc, sh) / (double)np;
-    acc = 0.0;
-    for (int i = threadIdx.x; i < np; i += blockDim.x) {
+    acc = block_sum<kSrThreads>(acc, sh);
+    if (threadIdx.x == 0) {
+        dq.part[kSrBlocks + blk] = acc;
+        if (blk == 0) dq.stats[0] = cmin;
+    }
+}
+
+__device__ __forceinline__ void sr_var_body(int np, int blk, const DevPeriod& dq)
+{
+    __shared__ double sh[kSrThreads / 32], s_mean;
+    const int nb = sr_blocks(np);
+    if (blk >= nb) return;
+    if (threadIdx.x < 32) {
+        const double sum = sum_parts(dq.part + kSrBlocks, nb);
+        if (threadIdx.x == 0) s_mean = sum / (double)np;
+    }
+    __syncthreads();
+    const double mean = s_mean;
+    double acc = 0.0;
+    for (int i = blk * kSrThreads + threadIdx.x; i < np; i += nb * kSrThreads) {
         const double dd = dq.sr[i] - mean;
         acc += dd * dd;
     }
-    const double var = block_sum_fixed(acc, sh) / (double)np;
-    const double sd = sqrt(var);
-    for (int i = threadIdx.x; i < np; i += blockDim.x)
-        dq.sde_raw[i] = sd > 1e-12 ? (dq.sr[i] - mean) / sd : 0.0;
-    if (threadIdx.x == 0) {
-        dq.stats[0] = cmin;
-        dq.stats[1] = mean;
-        dq.stats[2] = sd;
-    }
+    acc = block_sum<kSrThreads>(acc, sh);
+    if (threadIdx.x == 0) dq.part[2 * kSrBlocks + blk] = acc;
 }
 
-__global__ void __launch_bounds__(1024) k_sr_stats(int np, DevPeriod dq)
-{
-    __shared__ double sh[1024];
-    sr_stats_body(np, dq, sh);
-}
-
-// One block per curve lc0 + blockIdx.x.
-__global__ void __launch_bounds__(1024) k_sr_stats_set(DevSet ds, int lc0)
-{
-    __shared__ double sh[1024];
-    const int lc = lc0 + blockIdx.x;
-    const DevPeriod dq = ds.outs[lc];
-    sr_stats_body(ds.plans[lc].np, dq, sh);
-}
-
-// Lower running median of sde_raw over [i-h, i+h] (truncated), one block per
+// Lower running median of SDE_raw over [i-h, i+h] (truncated), one block per
 // `outs` consecutive outputs: the block sorts the union of its windows once
-// (bitonic, by value then position) and every thread walks the sorted list.
+// (bitonic, by value).  Wide windows: a warp takes 32 consecutive outputs,
+// finds the first one's median 32 sorted values at a time, and every lane goes
+// on from there, by the values that left the window and those that entered.
+// Narrow windows share too few values for that: bisection on the sorted
+// position.  The block also makes SDE_raw of its outputs, and its best SDE.
+constexpr int kMedianNarrow = 160;   // windows up to this many values are searched by bisection
+
+// Sorted position of the median of each lane's window [wlo, whi] (its output i
+// = first + lane while `on`), by a whole warp.
+__device__ __forceinline__ int median_walk(const uint16_t* pos, const uint16_t* inv, int np, int h, int lo, int len,
+                                           int first, int i, bool on, int wlo, int whi, int want)
+{
+    const int lane = threadIdx.x & 31;
+    // the warp's first window: sorted position r of its median (a window
+    // holds more than `want` values, so the walk ends inside the list)
+    const int flo = max(0, first - h) - lo, fhi = min(np - 1, first + h) - lo, fwant = (fhi - flo) / 2;
+    int r = 0, cnt = 0;   // values of the window before sorted position r
+    for (; r < len; r += 32) {
+        const int q = r + lane < len ? (int)pos[r + lane] : 0xffff;
+        const unsigned int in = __ballot_sync(0xffffffffu, q >= flo && q <= fhi);
+        const int c = __popc(in);
+        if (cnt + c > fwant) {
+            r += __fns(in, 0, fwant - cnt + 1);
+            cnt = fwant;
+            break;
+        }
+        cnt += c;
+    }
+    // each lane's window: what left and what entered on the way there
+    const int before = max(first, i - 1);
+    const int plo = max(0, before - h) - lo, phi = min(np - 1, before + h) - lo;
+    const unsigned int left = __ballot_sync(0xffffffffu, on && wlo > plo && (int)inv[plo] < r);
+    const unsigned int came = __ballot_sync(0xffffffffu, on && whi > phi && (int)inv[whi] < r);
+    const unsigned int upto = 0xffffffffu >> (31 - lane);
+    cnt += __popc(came & upto) - __popc(left & upto);
+    auto in = [&](int k) { return (int)pos[k] >= wlo && (int)pos[k] <= whi; };
+    while (on && r >= 0 && r < len) {
+        if (cnt > want) {
+            do --r;
+            while (r > 0 && !in(r));
+            --cnt;
+        } else if (!in(r)) {
+            ++r;
+        } else if (cnt < want) {
+            ++cnt;
+            ++r;
+        } else {
+            break;
+        }
+    }
+    return r;
+}
+
 __device__ void median_body(int np, int h, int outs, int blk, const DevPeriod& dq, unsigned char* smem)
 {
-    double* val = reinterpret_cast<double*>(smem);
-    int* pos = reinterpret_cast<int*>(val + kMedianCap);
+    __shared__ double s_mean, s_inv;
+    __shared__ unsigned long long top_key[kMedianThreads / 32];
+    __shared__ int top_idx[kMedianThreads / 32];
+    unsigned long long* key = reinterpret_cast<unsigned long long*>(smem);
+    uint16_t* pos = reinterpret_cast<uint16_t*>(key + kMedianCap);   // position - lo of sorted[k] (kNoPos: padding)
+    uint16_t* rank = pos + kMedianCap;                                // sorted position of position - lo
+    constexpr uint16_t kNoPos = 0xffff;
     const int i0 = blk * outs;
     const int lo = max(0, i0 - h);
     const int hi = min(np - 1, i0 + outs - 1 + h);
@@ -1840,57 +1956,177 @@ __device__ void median_body(int np, int h, int outs, int blk, const DevPeriod& d
         if (threadIdx.x == 0) record_check(dq.check, 16, len, kMedianCap);
         return;
     }
-    int cap = 1;
+    const int nb = sr_blocks(np);
+    if (threadIdx.x < 32) {
+        const double sum = sum_parts(dq.part + kSrBlocks, nb), var = sum_parts(dq.part + 2 * kSrBlocks, nb);
+        if (threadIdx.x == 0) {
+            const double m = sum / (double)np, sd = sqrt(var / (double)np);
+            s_mean = m;
+            s_inv = sd > 1e-12 ? 1.0 / sd : 0.0;
+            if (blk == 0) {
+                dq.stats[1] = m;
+                dq.stats[2] = sd;
+            }
+        }
+    }
+    __syncthreads();
+    const double mean = s_mean, inv = s_inv;
+    int cap = 2;
     while (cap < len) cap <<= 1;
     for (int k = threadIdx.x; k < cap; k += blockDim.x) {
         if (k < len) {
-            val[k] = dq.sde_raw[lo + k];
-            pos[k] = lo + k;
+            const double raw = inv > 0.0 ? (dq.sr[lo + k] - mean) * inv : 0.0;
+            key[k] = double_order_key(raw);
+            pos[k] = (uint16_t)k;
+            if (lo + k >= i0 && lo + k < i0 + outs) dq.sde_raw[lo + k] = raw;
         } else {
-            val[k] = INFINITY;
-            pos[k] = 0x7fffffff;
+            key[k] = ~0ull;
+            pos[k] = kNoPos;
         }
     }
     __syncthreads();
     for (int size = 2; size <= cap; size <<= 1) {
         for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int k = threadIdx.x; k < cap; k += blockDim.x) {
-                const int l = k ^ stride;
-                if (l > k) {
-                    const bool up = (k & size) == 0;
-                    const bool gt = val[k] > val[l] || (val[k] == val[l] && pos[k] > pos[l]);
-                    if (gt == up) {
-                        const double tv = val[k];
-                        val[k] = val[l];
-                        val[l] = tv;
-                        const int tp = pos[k];
-                        pos[k] = pos[l];
-                        pos[l] = tp;
-                    }
+            for (int p = threadIdx.x; p < cap >> 1; p += blockDim.x) {
+                const int k = 2 * p - (p & (stride - 1)), l = k + stride;
+                const unsigned long long a = key[k], b = key[l];
+                if ((a > b) == ((k & size) == 0) && a != b) {
+                    key[k] = b;
+                    key[l] = a;
+                    const uint16_t t = pos[k];
+                    pos[k] = pos[l];
+                    pos[l] = t;
                 }
             }
             __syncthreads();
         }
     }
-    for (int t = threadIdx.x; t < outs; t += blockDim.x) {
-        const int i = i0 + t;
-        if (i >= np) break;
-        const int wlo = max(0, i - h), whi = min(np - 1, i + h);
-        const int want = (whi - wlo) / 2;  // lower median: index (cnt-1)/2
-        int seen = 0;
-        double med = 0.0;
-        for (int k = 0; k < len; ++k) {
-            const int q = pos[k];
-            if (q >= wlo && q <= whi) {
-                if (seen == want) {
-                    med = val[k];
-                    break;
-                }
-                ++seen;
+    for (int k = threadIdx.x; k < cap; k += blockDim.x)
+        if (pos[k] != kNoPos) rank[pos[k]] = (uint16_t)k;
+    __syncthreads();
+    unsigned long long best = 0ull;
+    int best_idx = 0x7fffffff;
+    const int lane = threadIdx.x & 31;
+    const bool narrow = 2 * h + 1 <= kMedianNarrow;
+    for (int t0 = threadIdx.x & ~31; t0 < outs && i0 + t0 < np; t0 += blockDim.x) {
+        const int first = i0 + t0, i = min(first + lane, np - 1);
+        const bool on = first + lane < np;
+        const int wlo = max(0, i - h) - lo, whi = min(np - 1, i + h) - lo;
+        const int want = (whi - wlo) / 2;   // lower median: index (count - 1) / 2
+        int r;
+        if (narrow) {
+            // the smallest sorted position that more than `want` values of the
+            // window do not exceed
+            int a = 0, b = len - 1;
+            while (a < b) {
+                const int mid = (a + b) >> 1;
+                int cnt = 0;
+                for (int q = wlo; q <= whi; ++q) cnt += (int)rank[q] <= mid ? 1 : 0;
+                if (cnt > want) b = mid;
+                else a = mid + 1;
             }
+            r = a;
+            if (!on) continue;
+        } else {
+            r = median_walk(pos, rank, np, h, lo, len, first, i, on, wlo, whi, want);
+            if (!on) continue;   // (the next turn's ballots wait for these lanes)
         }
-        dq.sde[i] = dq.sde_raw[i] - med;
+        if (!in_range(dq.check, 23, r, len)) continue;
+        const double sde = dq.sde_raw[i] - double_from_order_key(key[r]);
+        dq.sde[i] = sde;
+        const unsigned long long ku = double_order_key(sde);
+        if (sde == sde && ku > best) {
+            best = ku;
+            best_idx = i;
+        }
     }
+    if (gridDim.x > (unsigned)kTopBlocks) return;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long k = __shfl_xor_sync(0xffffffffu, best, o);
+        const int b = __shfl_xor_sync(0xffffffffu, best_idx, o);
+        if (k > best || (k == best && b < best_idx)) {
+            best = k;
+            best_idx = b;
+        }
+    }
+    if ((threadIdx.x & 31) == 0) {
+        top_key[threadIdx.x >> 5] = best;
+        top_idx[threadIdx.x >> 5] = best_idx;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < kMedianThreads / 32; ++w)
+            if (top_key[w] > best || (top_key[w] == best && top_idx[w] < best_idx)) {
+                best = top_key[w];
+                best_idx = top_idx[w];
+            }
+        double* const top = dq.part + 3 * kSrBlocks + 2 * blk;
+        top[0] = __longlong_as_double((long long)best);
+        top[1] = __longlong_as_double((long long)best_idx);
+    }
+}
+
+// First index of the largest SDE (0x7fffffff: none can be ranked), in every
+// thread of a block of 1024: from the median blocks' best, or the spectrum.
+__device__ __forceinline__ int best_sde(int np, int blocks, bool kept, const DevPeriod& dq)
+{
+    __shared__ unsigned long long bk[32];
+    __shared__ int bi[32];
+    unsigned long long best = 0ull;
+    int idx = 0x7fffffff;
+    auto take = [&](unsigned long long k, int i) {
+        if (k > best || (k == best && i < idx)) {
+            best = k;
+            idx = i;
+        }
+    };
+    if (kept) {
+        for (int b = threadIdx.x; b < blocks; b += blockDim.x) {
+            const double* const top = dq.part + 3 * kSrBlocks + 2 * b;
+            const int i = (int)__double_as_longlong(top[1]);
+            if (i != 0x7fffffff) take((unsigned long long)__double_as_longlong(top[0]), i);
+        }
+    } else {
+        for (int i = threadIdx.x; i < np; i += blockDim.x) {
+            const double s = dq.sde[i];
+            if (s == s) take(double_order_key(s), i);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long k = __shfl_xor_sync(0xffffffffu, best, o);
+        const int i = __shfl_xor_sync(0xffffffffu, idx, o);
+        take(k, i);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        bk[threadIdx.x >> 5] = best;
+        bi[threadIdx.x >> 5] = idx;
+    }
+    __syncthreads();
+    for (int w = 0; w < (int)blockDim.x / 32; ++w) take(bk[w], bi[w]);
+    return idx;
+}
+
+// The reductions and the median over one spectrum (blocks of the x dimension),
+// and over every curve lc0 + blockIdx.y of a set.
+__global__ void __launch_bounds__(kSrThreads) k_sr_min(int np, DevPeriod dq) { sr_min_body(np, blockIdx.x, dq, true); }
+__global__ void __launch_bounds__(kSrThreads) k_sr_sum(int np, DevPeriod dq) { sr_sum_body(np, blockIdx.x, dq); }
+__global__ void __launch_bounds__(kSrThreads) k_sr_var(int np, DevPeriod dq) { sr_var_body(np, blockIdx.x, dq); }
+
+__global__ void __launch_bounds__(kSrThreads) k_sr_min_set(DevSet ds, int lc0)
+{
+    sr_min_body(ds.plans[lc0 + blockIdx.y].np, blockIdx.x, ds.outs[lc0 + blockIdx.y], false);
+}
+
+__global__ void __launch_bounds__(kSrThreads) k_sr_sum_set(DevSet ds, int lc0)
+{
+    sr_sum_body(ds.plans[lc0 + blockIdx.y].np, blockIdx.x, ds.outs[lc0 + blockIdx.y]);
+}
+
+__global__ void __launch_bounds__(kSrThreads) k_sr_var_set(DevSet ds, int lc0)
+{
+    sr_var_body(ds.plans[lc0 + blockIdx.y].np, blockIdx.x, ds.outs[lc0 + blockIdx.y]);
 }
 
 __global__ void __launch_bounds__(kMedianThreads) k_median_sde(int np, int h, int outs, DevPeriod dq)
@@ -1899,11 +2135,12 @@ __global__ void __launch_bounds__(kMedianThreads) k_median_sde(int np, int h, in
     median_body(np, h, outs, blockIdx.x, dq, smem);
 }
 
-// Outputs per block of the running median for half width h.
+// Outputs per block of the running median for half width h (narrow windows:
+// so many that the union of the windows fills 1024 values).
 __host__ __device__ __forceinline__ int median_outs(int h)
 {
     const int o = kMedianCap - 2 * h;
-    return (o < 1024 ? o : 1024) & ~31;
+    return (2 * h <= 512 ? 1024 - 2 * h : o < 1024 ? o : 1024) & ~31;
 }
 
 // Row blockIdx.y: curve lc0 + blockIdx.y; its blocks are the first
@@ -1998,39 +2235,16 @@ __global__ void __launch_bounds__(1024) k_topk(DevSet ds, int lc0)
 
 // Curve lc0 + blockIdx.x: the candidate of largest SDE into its result
 // (and results[lc], checks[4 lc ..] when given).
-__global__ void __launch_bounds__(1024) k_best(DevSet ds, int lc0, gtls_result* results, unsigned int* checks)
+__global__ void __launch_bounds__(1024) k_best(DevSet ds, int lc0, int median_blocks, gtls_result* results,
+                                               unsigned int* checks)
 {
-    __shared__ double bv[1024];
-    __shared__ int bi[1024];
     const int lc = lc0 + blockIdx.x;
     const DevPlan& dp = ds.plans[lc];
     const DevCurve dc = ds.curves[lc];
     const DevPeriod dq = ds.outs[lc];
-    double v = -INFINITY;
-    int idx = 0x7fffffff;
-    for (int i = threadIdx.x; i < dp.np; i += blockDim.x) {
-        const double s = dq.sde[i];
-        if (s > v) {
-            v = s;
-            idx = i;
-        }
-    }
-    bv[threadIdx.x] = v;
-    bi[threadIdx.x] = idx;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            const double ov = bv[threadIdx.x + s];
-            const int oi = bi[threadIdx.x + s];
-            if (ov > bv[threadIdx.x] || (ov == bv[threadIdx.x] && oi < bi[threadIdx.x])) {
-                bv[threadIdx.x] = ov;
-                bi[threadIdx.x] = oi;
-            }
-        }
-        __syncthreads();
-    }
+    const int outs = median_outs(dp.median_half);
+    const int b = best_sde(dp.np, (dp.np + outs - 1) / outs, median_blocks <= kTopBlocks, dq);
     if (threadIdx.x == 0) {
-        const int b = bi[0];
         gtls_result r{};
         const int j = in_range(dc.check, 17, b, dp.np) ? dq.dur[b] : -1;
         if (j < 0 || !in_range(dc.check, 18, j, dp.nd)) {
@@ -2248,12 +2462,7 @@ int fold_smem_bytes(int bucket_log2)
     return std::max(global_path, staged);
 }
 
-int topk_smem_bytes(int, int)
-{
-    return 0;   // the selection uses static shared memory only
-}
-
-constexpr int kMedianSmem = kMedianCap * (int)(sizeof(double) + sizeof(int));
+constexpr int kMedianSmem = kMedianCap * (int)(sizeof(unsigned long long) + 2 * sizeof(uint16_t));
 
 // Every kernel with dynamic shared memory may use up to the device's opt-in
 // limit (set once per device, so that plans of any size coexist).
@@ -2278,7 +2487,6 @@ gtls_status configure_kernels(int dev)
     GTLS_TRY(allow((const void*)bounds::k_window_bounds));
     GTLS_TRY(allow((const void*)k_median_sde));
     GTLS_TRY(allow((const void*)k_median_sde_set));
-    GTLS_TRY(allow((const void*)k_topk));
     GTLS_CUDA(cudaFuncSetAttribute((const void*)k_window_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    tc::kSmemRequest));
     done.push_back(dev);
@@ -2393,7 +2601,8 @@ gtls_status create_device(gtls_plan* pl)
     GTLS_TRY(dev_alloc(pl, &dq.sr, np_));
     GTLS_TRY(dev_alloc(pl, &dq.sde_raw, np_));
     GTLS_TRY(dev_alloc(pl, &dq.sde, np_));
-    GTLS_TRY(dev_alloc(pl, &dq.stats, 4));
+    GTLS_TRY(dev_alloc(pl, &dq.stats, 4 + kSrParts));
+    dq.part = dq.stats + 4;
     GTLS_TRY(dev_alloc(pl, &dq.result, 1));
     dq.check = dc.check;
 
@@ -2611,6 +2820,7 @@ gtls_status create_device(gtls_plan* pl)
         // variant (one column per lane)
         pl->refine_k = dp.refine_k;
         GTLS_TRY(dev_alloc(pl, &pl->dq.refined, dp.np));
+        GTLS_CUDA(cudaMemset(pl->dq.refined, 0, dp.np * sizeof(int32_t)));
         if (pl->refine_k > 0) {
             pl->dp_ref = dp;
             std::vector<int32_t> ones(dp.nd, 1), var1(dp.nd, tiles::kScalar15);
@@ -2663,7 +2873,7 @@ gtls_status create_device(gtls_plan* pl)
         // 1.2 ms and 2.9e9: 140 us faster)
         const bool worth = h.wpe >= kBoundsMinWpe || (h.prm.test_flags & 4);
         pl->bounds_ok = !pl->has_tensor && worth && !(h.prm.test_flags & 2);
-        for (int pass = 0; pass < (pl->refine_k > 0 ? 2 : 1); ++pass) {
+        for (int pass = 0; pass < (pl->refine_k > 0 ? 2 : 1) && pl->bounds_ok; ++pass) {
             for (int j = 0; j < dp.nd; ++j) {
                 tab[j] = bound_table(h.tmpl.data() + h.tmpl_off[j], h.dpts[j], pass ? 1 : h.stride[j]);
                 pl->bounds_ok = pl->bounds_ok && tab[j].mean_all > 0.0f && tab[j].root_t2 > 0.0f;
@@ -2742,11 +2952,13 @@ gtls_status ensure_chunk(gtls_plan* pl)
     GTLS_TRY(dev_alloc(pl, &dk.ws, chunk * dk.pad_stride));
     GTLS_TRY(dev_alloc(pl, &dk.wrs, chunk * dk.pad_stride));
     GTLS_TRY(dev_alloc(pl, &dk.pf, chunk * dk.pad_stride));
-    GTLS_TRY(dev_alloc(pl, &dk.pq, chunk * dk.pad_stride));
-    dk.list_cap = std::max<int64_t>(4096, chunk * kListPerSlot);
-    GTLS_TRY(dev_alloc(pl, &dk.list, kListClasses * dk.list_cap));
-    GTLS_TRY(dev_alloc(pl, &dk.dense, chunk * std::max({1, pl->tile_count, pl->tile_count_ref})));
-    GTLS_TRY(dev_alloc(pl, &dk.left_n, kListClasses + 1));
+    if (pl->bounds_ok) {
+        GTLS_TRY(dev_alloc(pl, &dk.pq, chunk * dk.pad_stride));
+        dk.list_cap = std::max<int64_t>(4096, chunk * kListPerSlot);
+        GTLS_TRY(dev_alloc(pl, &dk.list, kListClasses * dk.list_cap));
+        GTLS_TRY(dev_alloc(pl, &dk.dense, chunk * std::max({1, pl->tile_count, pl->tile_count_ref})));
+        GTLS_TRY(dev_alloc(pl, &dk.left_n, kListClasses + 1));
+    }
     if (pl->has_tensor) {
         unsigned char* maps = nullptr;
         GTLS_TRY(dev_alloc(pl, &maps, (size_t)tc::kMaps * sizeof(CUtensorMap)));
@@ -2837,7 +3049,7 @@ struct Ctx {
     int tile_buf_w = 0;      // (w r, w) pairs per tile with per-point weights
     int n_sm = 0;
     int median_blocks = 1;   // widest row of the running-median grid
-    int topk_smem = 0;
+    int sr_blocks = 1;       // widest row of the SR reductions' grid
     cudaStream_t st = nullptr;
     const void* tc_maps = nullptr;   // tensor-core kernel: TMA maps of dk.rs (tc::kMaps rows pitches)
     int tc_jspan = 1;        // tensor-core kernel: work items per period slot
@@ -2914,12 +3126,17 @@ gtls_status wave_pass(Ctx& c, bool ref, const SlotMap& sm, bool tiled, bool weig
 // SR, SDE_raw and the median-detrended SDE of every curve.
 gtls_status sr_sde_pass(Ctx& c)
 {
-    k_sr_stats_set<<<c.n_lc, 1024, 0, c.st>>>(c.set, 0);
+    const dim3 grid((unsigned)c.sr_blocks, (unsigned)c.n_lc);
+    k_sr_min_set<<<grid, kSrThreads, 0, c.st>>>(c.set, 0);
+    GTLS_CUDA(cudaGetLastError());
+    k_sr_sum_set<<<grid, kSrThreads, 0, c.st>>>(c.set, 0);
+    GTLS_CUDA(cudaGetLastError());
+    k_sr_var_set<<<grid, kSrThreads, 0, c.st>>>(c.set, 0);
     GTLS_CUDA(cudaGetLastError());
     k_median_sde_set<<<dim3((unsigned)c.median_blocks, (unsigned)c.n_lc), kMedianThreads, kMedianSmem, c.st>>>(
         c.set, 0);
     GTLS_CUDA(cudaGetLastError());
-    c.launches += 2;
+    c.launches += 4;
     return stage_mark(c, kStageSrSde);
 }
 
@@ -3007,7 +3224,7 @@ gtls_status run_search(gtls_plan* pl, const double* t, const double* y, const do
     c.tile_buf_w = pl->tile_buf_w;
     c.n_sm = pl->n_sm;
     c.median_blocks = (dp.np + median_outs(dp.median_half) - 1) / median_outs(dp.median_half);
-    c.topk_smem = topk_smem_bytes(dp.np, pl->refine_k);
+    c.sr_blocks = sr_blocks(dp.np);
     c.st = st;
     c.tc_jspan = pl->tc_jspan;
     c.tc_test = pl->tc_test_wait;
@@ -3036,14 +3253,14 @@ gtls_status run_search(gtls_plan* pl, const double* t, const double* y, const do
     }
     GTLS_TRY(sr_sde_pass(c));
     // two-stage T0 search (Sect. 2.5): the refine_k best periods by SDE(P)
-    // again with T0 step 1, then SR / SDE once more (k_topk also clears the
-    // refined flags when refine_k is 0)
-    k_topk<<<1, 1024, c.topk_smem, st>>>(c.set, 0);
-    GTLS_CUDA(cudaGetLastError());
-    c.launches += 1;
-    GTLS_TRY(stage_mark(c, kStageSrSde));
+    // again with T0 step 1, then SR / SDE once more (without refinement the
+    // refined flags stay as the plan cleared them)
     const int kref = pl->refine_k;
     if (kref > 0) {
+        k_topk<<<1, 1024, 0, st>>>(c.set, 0);
+        GTLS_CUDA(cudaGetLastError());
+        c.launches += 1;
+        GTLS_TRY(stage_mark(c, kStageSrSde));
         for (int r0 = 0; r0 < kref; r0 += dk.chunk) {
             const int cnt = std::min<int>(dk.chunk, kref - r0);
             GTLS_TRY(wave_pass(c, true, single_wave(r0, cnt, pl->tile_count_ref, true), tiled, false,
@@ -3051,7 +3268,7 @@ gtls_status run_search(gtls_plan* pl, const double* t, const double* y, const do
         }
         GTLS_TRY(sr_sde_pass(c));
     }
-    k_best<<<1, 1024, 0, st>>>(c.set, 0, nullptr, nullptr);
+    k_best<<<1, 1024, 0, st>>>(c.set, 0, c.median_blocks, nullptr, nullptr);
     GTLS_CUDA(cudaGetLastError());
     c.launches += 1;
     GTLS_TRY(stage_mark(c, kStageSrSde));
@@ -3097,7 +3314,7 @@ struct gtls_batch {
     std::vector<int64_t> off;          // host offsets (n_lc + 1, from 0)
     int64_t max_n = 0;
     int max_kept = 0;
-    int fold_smem = 0, topk_smem = 0, median_blocks = 1, n_sm = 0;
+    int fold_smem = 0, median_blocks = 1, sr_blocks = 1, n_sm = 0;
     int max_slots = 0;                 // chunk scratch slots allocated
     int tile_buf_max = 0;              // the smallest staged tile of the tiled plans (their own choice)
     int tile_buf_cap = 0;              // largest staged tile the device's shared memory allows
@@ -3118,6 +3335,7 @@ struct gtls_batch {
     cudaStream_t body_stream = nullptr;   // stream the loop bodies are captured on
     BatchCfg cfg;
     bool tuned = false;
+    bool refines = false;              // some plan has a refinement stage
     bool bounds_ok = true;             // every plan's templates admit the bounds kernel
     // graph of everything after the curve preparation, for one set of
     // per-curve kernel classes (uniform dy and tile fit)
@@ -3288,7 +3506,7 @@ Ctx batch_ctx(const gtls_batch* b, cudaStream_t st)
     c.tile_buf_w = b->tile_buf_w;
     c.n_sm = b->n_sm;
     c.median_blocks = b->median_blocks;
-    c.topk_smem = b->topk_smem;
+    c.sr_blocks = b->sr_blocks;
     c.st = st;
     for (const gtls_plan* pl : b->plans) {
         c.tc_jspan = std::max(c.tc_jspan, pl->tc_jspan);
@@ -3438,14 +3656,16 @@ gtls_status batch_enqueue(gtls_batch* b, Ctx& c, std::vector<LoopSpec>& coarse, 
     int qi = 0;
     for (LoopSpec& L : coarse) GTLS_TRY(capture_loop(b, c, L, qi++));
     GTLS_TRY(sr_sde_pass(c));
-    k_topk<<<c.n_lc, 1024, c.topk_smem, c.st>>>(c.set, 0);
-    GTLS_CUDA(cudaGetLastError());
-    c.launches += 1;
+    if (b->refines) {
+        k_topk<<<c.n_lc, 1024, 0, c.st>>>(c.set, 0);
+        GTLS_CUDA(cudaGetLastError());
+        c.launches += 1;
+    }
     if (!refine.empty()) {
         for (LoopSpec& L : refine) GTLS_TRY(capture_loop(b, c, L, qi++));
         GTLS_TRY(sr_sde_pass(c));
     }
-    k_best<<<c.n_lc, 1024, 0, c.st>>>(c.set, 0, b->results, b->checks);
+    k_best<<<c.n_lc, 1024, 0, c.st>>>(c.set, 0, c.median_blocks, b->results, b->checks);
     GTLS_CUDA(cudaGetLastError());
     c.launches += 1;
     return GTLS_OK;
@@ -3561,7 +3781,7 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     b->n_lc = (int)n_lc;
     b->plans.assign(plans, plans + n_lc);
     b->off.assign(1, 0);
-    int bucket_log2 = 0, max_np_blocks = 1, topk = 0, buf_max = 1 << 30;
+    int bucket_log2 = 0, max_np_blocks = 1, buf_max = 1 << 30;
     int64_t fold_stride = 32, key_stride = 32, pad_stride = 32;
     bool any_tiled = false;
     for (int i = 0; i < b->n_lc; ++i) {
@@ -3580,7 +3800,8 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
         pad_stride = std::max<int64_t>(pad_stride, pl->dk.pad_stride);
         const int mo = median_outs(pl->dp.median_half);
         max_np_blocks = std::max(max_np_blocks, (pl->dp.np + mo - 1) / mo);
-        topk = std::max(topk, topk_smem_bytes(pl->dp.np, pl->refine_k));
+        b->sr_blocks = std::max(b->sr_blocks, sr_blocks(pl->dp.np));
+        b->refines = b->refines || pl->refine_k > 0;
         if (pl->tile_ok) {
             buf_max = std::min(buf_max, pl->tile_buf);
             any_tiled = true;
@@ -3588,7 +3809,6 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
         b->bounds_ok = b->bounds_ok && pl->bounds_ok;
     }
     b->fold_smem = fold_smem_bytes(bucket_log2);
-    b->topk_smem = topk;
     b->median_blocks = max_np_blocks;
     b->n_sm = plans[0]->n_sm;
     b->tile_buf_max = any_tiled ? buf_max : 0;
@@ -3666,13 +3886,15 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     b->total_periods = total_periods;
     batch_tiles(b, b->cfg.tile_buf);
     GTLS_TRY(batch_upload_tiles(b));
-    int max_tiles = 1;
-    for (const DevTiles& t : b->tiles_host) max_tiles = std::max(max_tiles, t.count);
-    GTLS_TRY(batch_alloc(b, &b->dk.dense, slots * (int64_t)max_tiles));
-    GTLS_TRY(batch_alloc(b, &b->dk.pq, slots * pad_stride));
-    b->dk.list_cap = std::max<int64_t>(4096, slots * kListPerSlot);
-    GTLS_TRY(batch_alloc(b, &b->dk.list, kListClasses * b->dk.list_cap));
-    GTLS_TRY(batch_alloc(b, &b->dk.left_n, kListClasses + 1));
+    if (b->bounds_ok) {
+        int max_tiles = 1;
+        for (const DevTiles& t : b->tiles_host) max_tiles = std::max(max_tiles, t.count);
+        GTLS_TRY(batch_alloc(b, &b->dk.dense, slots * (int64_t)max_tiles));
+        GTLS_TRY(batch_alloc(b, &b->dk.pq, slots * pad_stride));
+        b->dk.list_cap = std::max<int64_t>(4096, slots * kListPerSlot);
+        GTLS_TRY(batch_alloc(b, &b->dk.list, kListClasses * b->dk.list_cap));
+        GTLS_TRY(batch_alloc(b, &b->dk.left_n, kListClasses + 1));
+    }
     return GTLS_OK;
 }
 
@@ -4087,53 +4309,24 @@ const char* gtls_status_string(gtls_status s)
 namespace {
 
 constexpr int64_t kNoAllocMaxPeriods = int64_t(1) << 19;  // 524,288 trial periods
-constexpr int64_t kNoAllocHead = 32;                        // doubles before the SR / SDE_raw areas
+constexpr int64_t kNoAllocHead = 32 + kSrParts;             // doubles before the SR / SDE_raw areas
 // [0..4) stats  [4..8) check words  [8] best SDE  [9] best index (bits)
-// [32 .. 32+max) SR   [32+max .. 32+2 max) SDE_raw
+// [32 .. head) parts of the reductions, then SR and SDE_raw
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocHead + 2 * kNoAllocMaxPeriods];
 
 std::mutex g_noalloc_mutex;
 double* g_noalloc_ptr[64] = {};   // device address of g_noalloc_scratch per device
 
-// Argmax of SDE (ties: lower index) and a check of the caller's chi2(P): every
-// value must be finite and >= 0 (check 18); an argmax that finds no index
-// (every SDE NaN) records check 17.
-__global__ void __launch_bounds__(1024) k_argmax_noalloc(int np, const double* __restrict__ chi2,
-                                                         const double* __restrict__ sde, double* head)
+// Argmax of SDE (ties: lower index); one that finds no index (every SDE NaN)
+// records check 17.
+__global__ void __launch_bounds__(1024) k_argmax_noalloc(int np, int blocks, DevPeriod dq, double* head)
 {
-    __shared__ double bv[1024];
-    __shared__ int bi[1024];
-    unsigned int* check = reinterpret_cast<unsigned int*>(head + 4);
-    double v = -INFINITY;
-    int idx = 0x7fffffff;
-    for (int i = threadIdx.x; i < np; i += blockDim.x) {
-        const double c = chi2[i];
-        if (!(c >= 0.0 && c <= DBL_MAX)) record_check(check, 18, i, np);
-        const double x = sde[i];
-        if (x > v || (x == v && i < idx)) {
-            v = x;
-            idx = i;
-        }
-    }
-    bv[threadIdx.x] = v;
-    bi[threadIdx.x] = idx;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) {
-            const double ov = bv[threadIdx.x + s];
-            const int oi = bi[threadIdx.x + s];
-            if (ov > bv[threadIdx.x] || (ov == bv[threadIdx.x] && oi < bi[threadIdx.x])) {
-                bv[threadIdx.x] = ov;
-                bi[threadIdx.x] = oi;
-            }
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        if (bi[0] < 0 || bi[0] >= np) record_check(check, 17, bi[0], np);
-        head[8] = bv[0];
-        head[9] = __longlong_as_double((long long)bi[0]);
-    }
+    const int b = best_sde(np, blocks, blocks <= kTopBlocks, dq);
+    if (threadIdx.x != 0) return;
+    const bool ok = b >= 0 && b < np;
+    if (!ok) record_check(dq.check, 17, b, np);
+    head[8] = ok ? dq.sde[b] : -INFINITY;
+    head[9] = __longlong_as_double((long long)b);
 }
 
 // Where `p` lives: device memory of the current device (or managed memory)
@@ -4189,7 +4382,7 @@ extern "C" gtls_status gtls_sr_sde_noalloc(const double* chi2, int64_t n_periods
     const int np = (int)n_periods;
     const int win = median_window > 0 ? median_window : std::max(3, 2 * (np / 200) + 1);
     const int hwin = win / 2;
-    const int outs = std::min(1024, kMedianCap - 2 * hwin) & ~31;
+    const int outs = median_outs(hwin);
     if (outs < 32) return fail(GTLS_ERR_INVALID_ARG, "median window too large for the device median");
     int dev = -1;
     GTLS_CUDA(cudaGetDevice(&dev));
@@ -4207,15 +4400,20 @@ extern "C" gtls_status gtls_sr_sde_noalloc(const double* chi2, int64_t n_periods
     dq.sde_raw = sde_raw_out ? sde_raw_out : head + kNoAllocHead + kNoAllocMaxPeriods;
     dq.sde = sde_out;
     dq.stats = head;
+    dq.part = head + 32;
     dq.check = reinterpret_cast<unsigned int*>(head + 4);
     // the array keeps the previous call's contents: clear the check words
     GTLS_CUDA(cudaMemsetAsync(head + 4, 0, 4 * sizeof(double), st));
-    k_sr_stats<<<1, 1024, 0, st>>>(np, dq);
+    const int blocks = (np + outs - 1) / outs;
+    k_sr_min<<<sr_blocks(np), kSrThreads, 0, st>>>(np, dq);
     GTLS_CUDA(cudaGetLastError());
-    k_median_sde<<<(np + outs - 1) / outs, kMedianThreads, kMedianCap * (int)(sizeof(double) + sizeof(int)), st>>>(
-        np, hwin, outs, dq);
+    k_sr_sum<<<sr_blocks(np), kSrThreads, 0, st>>>(np, dq);
     GTLS_CUDA(cudaGetLastError());
-    k_argmax_noalloc<<<1, 1024, 0, st>>>(np, chi2, sde_out, head);
+    k_sr_var<<<sr_blocks(np), kSrThreads, 0, st>>>(np, dq);
+    GTLS_CUDA(cudaGetLastError());
+    k_median_sde<<<blocks, kMedianThreads, kMedianSmem, st>>>(np, hwin, outs, dq);
+    GTLS_CUDA(cudaGetLastError());
+    k_argmax_noalloc<<<1, 1024, 0, st>>>(np, blocks, dq, head);
     GTLS_CUDA(cudaGetLastError());
     double res[2] = {0.0, 0.0};
     unsigned int chk[4] = {0, 0, 0, 0};
