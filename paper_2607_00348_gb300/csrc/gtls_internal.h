@@ -13,23 +13,36 @@
 namespace gtls {
 
 // Template of one duration cut into pieces for the bounds of the window
-// search (window_bounds.cuh): a few wide pieces that start at whole T0 steps
-// (first test of a window) and kBoundSegs segments (second test).
-constexpr int kBoundCuts = 13;
+// search (window_bounds.cuh): a few wide pieces (first test of a window) and
+// kBoundSegs segments (second test).
+constexpr int kBoundCuts = 17;
+constexpr int kBoundCutSlots = kBoundCuts - 1;   // the first one starts at 0 and is kept apart
 constexpr int kBoundSegs = 25;
-struct BoundTab {
-    float mean_all, nu_all;       // mean of s_k, >= ||s_k - mean||
+struct alignas(16) BoundTab {
+    float4 seg[kBoundSegs];       // end (point, integer bits), mean of s_k, >= ||s_k - mean||, <= 1 / length
+    float mean_all, nu_all;       // mean of s_k over the template, >= ||s_k - mean||
     float root_t2;                // sqrt(sum_k s_k^2)
     float t_max;                  // >= |s_k|
     int32_t cuts;                 // wide pieces (0: the window sum alone is tested)
-    int32_t cut_row[kBoundCuts];  // their first T0 step
-    float cut_coef[kBoundCuts + 1];   // mean of the piece before minus mean of the piece (Abel form)
+    float cut_jumps, seg_jumps;   // sums of |mean - mean before| over the wide pieces, the segments
     float cut_nu[kBoundCuts];     // >= ||s_k - mean|| over the piece
     int32_t cut_len[kBoundCuts];  // its points
-    int32_t off[kBoundSegs + 1];  // segments [off[g], off[g + 1])
-    float mean[kBoundSegs];       // mean of s_k over the segment
-    float nu[kBoundSegs];         // >= ||s_k - mean|| over the segment
-    float inv_len[kBoundSegs];    // <= 1 / length (0 for an empty segment)
+};
+
+// What the bounds need of one duration for every period (staged in shared
+// memory by the words).
+struct alignas(16) BoundDur {
+    int32_t j, d, st, m_total;    // grid index, points, T0 step, windows
+    int32_t subs, wsub;           // chunks (of the curve or a stretch; 0: not searched here), windows per chunk
+    int32_t lg_nc, mode, test;    // lanes per window, summation order and first test (window_bounds.cuh)
+    int32_t row_max;              // first T0 step of the last wide piece
+    int32_t cuts4;                // wide pieces after the first, rounded up to a multiple of 4
+    float lam;                    // first-test value times lam estimates C1 / sqrt(sum s_k^2)
+    float cut_last;               // mean of the last wide piece
+    float coef0;                  // minus the mean of the first
+    int32_t pad[2];
+    float coef[kBoundCutSlots];   // of the others: mean of the piece before minus its mean (Abel form; 0 past the last)
+    int32_t row[kBoundCutSlots];  // their first T0 steps, or points
 };
 
 // Read-only plan tables on the device (passed to kernels by value).
@@ -70,6 +83,8 @@ struct DevPlan {
     int32_t refine_k;           // periods re-searched with T0 step 1 (0: none)
     const int64_t* tc_off;      // offset of duration j in tc_tab (floats; kTensor durations)
     const BoundTab* bounds;     // pieces of every duration's template
+    const BoundDur* bound_durs;
+    int32_t bound_lg;           // chunks of the window search are 2^bound_lg times the usual size
     const float* tc_tab;        // tensor-core template chunks: [chunk][hi, lo][32 x 32 core-matrix layout]
 };
 
@@ -210,7 +225,8 @@ struct gtls_plan {
     unsigned int* tc_counter = nullptr;
     int tc_test_wait = 0;
     const void* tc_maps = nullptr;      // TMA maps of dk.rs (made with the chunk scratch)
-    std::vector<int32_t> variant_host;   // window-kernel variant per duration (host copy)
+    std::vector<int32_t> variant_host;   // window-kernel variant per duration (host copies)
+    std::vector<int32_t> variant_ref_host, nc_host;
     int n_sm = 0;
     unsigned int* tile_counter = nullptr;
     // refinement stage (T0 step 1 on the best periods): plan tables with

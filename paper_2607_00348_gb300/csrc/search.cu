@@ -31,6 +31,7 @@
 
 #include <algorithm>
 #include <cfloat>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -401,6 +402,28 @@ __device__ __forceinline__ uint32_t fold_fine(long long rho, int sh, uint32_t mu
     return (uint32_t)((((unsigned long long)rho >> sh) * (unsigned long long)mulf) >> 32);
 }
 
+// Shapes for CTAs of T threads: 8 T staged keys, two fine buckets per thread.
+// Curves of up to 8 T points take the smallest T (256, 512, 1024) and a single
+// super-bucket, whose keys never leave the CTA; several such CTAs share an SM
+// (1440 points: 0.27 ms at 1024 threads, 0.17 at 512).  At more than one
+// super-bucket two CTAs of 512 threads were slower than one of 1024 (Kepler-like
+// fold 308 against 250 ms): twice as many barrier-separated rounds.
+template <int T>
+struct FoldCfg {
+    static constexpr bool kSingle = T < kFoldThreads;
+    static constexpr int kSegKeys = 8 * T;
+    static constexpr int kFineLog2 = T == 1024 ? kFoldFineLog2 : T == 512 ? 10 : 9;
+    static constexpr int kMaxSb = kSingle ? 2 : 1 << kFoldMaxSbLog2;
+    static constexpr int kStagedBytes = 33 * 8 + 2 * kSegKeys * 8 + (2 << kFineLog2) * 4 + 2 * kMaxSb * 4 +
+                                        2 * kSegKeys * 2 + 16;
+};
+
+// Threads of the fold's CTAs for curves of at most n points.
+__host__ __device__ __forceinline__ int fold_threads(int64_t n)
+{
+    return n <= FoldCfg<256>::kSegKeys ? 256 : n <= FoldCfg<512>::kSegKeys ? 512 : 1024;
+}
+
 struct FoldOut {
     int32_t* sidx;
     float* rs;
@@ -492,7 +515,7 @@ __device__ __forceinline__ void fold_scan_run(const long long* srfx, uint32_t le
 
 // Staged path; false when a super-bucket holds more than kFoldSegKeys
 // points (only keys have been written then).
-template <bool kBounded>
+template <bool kBounded, int T>
 __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCurve& dc, int p,
                             unsigned long long* keys, const FoldOut& o)
 {
@@ -502,12 +525,14 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
     const int sh = dp.bucket_shift[p];
     const int ib = dp.idx_bits;
     const unsigned long long idx_mask = (1ull << ib) - 1ull;
-    const int nsb = dp.fold_nsb;
+    using L = FoldCfg<T>;
+    constexpr int kFoldThreads = T, kFoldSegKeys = L::kSegKeys, kFoldFineLog2 = L::kFineLog2;
+    const int nsb = L::kSingle ? 1 : dp.fold_nsb;
     const uint32_t mulf = (uint32_t)(((unsigned long long)nsb << (kFoldFineLog2 + 32)) /
                                      (((unsigned long long)P >> sh) + 1ull));
     constexpr uint32_t kFineMask = (1u << kFoldFineLog2) - 1u;
     static_assert((1 << kFoldFineLog2) % kFoldThreads == 0, "fine buckets split evenly over the threads");
-    static_assert((1 << kFoldMaxSbLog2) <= kFoldThreads, "one super-bucket count per thread");
+    static_assert(L::kSingle || (1 << kFoldMaxSbLog2) <= kFoldThreads, "one super-bucket count per thread");
     static_assert(kFoldFineLog2 <= 16, "fine bucket indices are kept as 16-bit values");
 
     long long* warp_sums = reinterpret_cast<long long*>(smem);
@@ -517,52 +542,57 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
     uint32_t* fcnt = reinterpret_cast<uint32_t*>(sorted + kFoldSegKeys);
     uint32_t* fcur = fcnt + (1 << kFoldFineLog2);
     uint32_t* sb_cnt = fcur + (1 << kFoldFineLog2);
-    uint32_t* sb_start = sb_cnt + (1 << kFoldMaxSbLog2);
-    uint16_t* inv = reinterpret_cast<uint16_t*>(sb_start + (1 << kFoldMaxSbLog2));       // final position -> sorted position
+    uint32_t* sb_start = sb_cnt + L::kMaxSb;
+    uint16_t* inv = reinterpret_cast<uint16_t*>(sb_start + L::kMaxSb);       // final position -> sorted position
     uint16_t* sorted_f = inv + kFoldSegKeys;                                              // fine bucket of sorted[q]
     int* overflow = reinterpret_cast<int*>(sorted_f + kFoldSegKeys);
 
-    for (int q = threadIdx.x; q < nsb; q += blockDim.x) sb_cnt[q] = 0;
-    if (threadIdx.x == 0) *overflow = 0;
-    __syncthreads();
+    // A single super-bucket (n <= kFoldSegKeys): its keys go straight to the
+    // registers of step B.
+    const bool single = nsb == 1;
+    if (!single) {
+        for (int q = threadIdx.x; q < nsb; q += blockDim.x) sb_cnt[q] = 0;
+        if (threadIdx.x == 0) *overflow = 0;
+        __syncthreads();
 
-    // A. super-bucket of every point; its key goes to the next slot of the
-    // super-bucket's region (a shared-memory atomic per point: aggregating
-    // the lanes of a warp with equal super-buckets first measured slower)
-    const int64_t bs = blockDim.x;
-    for (int64_t g0 = 0; g0 < n; g0 += kFoldUnroll * bs) {
-        long long dl[kFoldUnroll];
-        float df[kFoldUnroll];
+        // A. super-bucket of every point; its key goes to the next slot of the
+        // super-bucket's region (a shared-memory atomic per point: aggregating
+        // the lanes of a warp with equal super-buckets first measured slower)
+        const int64_t bs = blockDim.x;
+        for (int64_t g0 = 0; g0 < n; g0 += kFoldUnroll * bs) {
+            long long dl[kFoldUnroll];
+            float df[kFoldUnroll];
 #pragma unroll
-        for (int u = 0; u < kFoldUnroll; ++u) {
-            const int64_t i = g0 + u * bs + threadIdx.x;
-            dl[u] = i < n ? dc.d_lat[i] : 0;
-            df[u] = i < n ? dc.d_f[i] : 0.0f;
-        }
+            for (int u = 0; u < kFoldUnroll; ++u) {
+                const int64_t i = g0 + u * bs + threadIdx.x;
+                dl[u] = i < n ? dc.d_lat[i] : 0;
+                df[u] = i < n ? dc.d_f[i] : 0.0f;
+            }
 #pragma unroll
-        for (int u = 0; u < kFoldUnroll; ++u) {
-            const int64_t i = g0 + u * bs + threadIdx.x;
-            const long long rho = lattice_rho(dl[u], df[u], P, inv_p);
-            const uint32_t sb = fold_fine(rho, sh, mulf) >> kFoldFineLog2;
-            const bool ok = i < n && in_range(dc.check, 2, rho, P) && in_range32(dc.check, 1, sb, nsb);
-            if (ok) {
-                const uint32_t slot = atomicAdd(&sb_cnt[sb], 1u);
-                if (slot < (uint32_t)kFoldSegKeys)
-                    keys[(int64_t)sb * kFoldSegKeys + slot] = ((unsigned long long)rho << ib) | (unsigned long long)i;
-                else
-                    *overflow = 1;
+            for (int u = 0; u < kFoldUnroll; ++u) {
+                const int64_t i = g0 + u * bs + threadIdx.x;
+                const long long rho = lattice_rho(dl[u], df[u], P, inv_p);
+                const uint32_t sb = fold_fine(rho, sh, mulf) >> kFoldFineLog2;
+                const bool ok = i < n && in_range(dc.check, 2, rho, P) && in_range32(dc.check, 1, sb, nsb);
+                if (ok) {
+                    const uint32_t slot = atomicAdd(&sb_cnt[sb], 1u);
+                    if (slot < (uint32_t)kFoldSegKeys)
+                        keys[(int64_t)sb * kFoldSegKeys + slot] = ((unsigned long long)rho << ib) | (unsigned long long)i;
+                    else
+                        *overflow = 1;
+                }
             }
         }
+        __syncthreads();
+        if (*overflow) return false;
+        {
+            // positions of the super-buckets in the folded order
+            const uint32_t c = threadIdx.x < nsb ? sb_cnt[threadIdx.x] : 0u;
+            const long long st = block_exclusive_scan(c, warp_sums, total);
+            if (threadIdx.x < nsb) sb_start[threadIdx.x] = (uint32_t)st;
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    if (*overflow) return false;
-    {
-        // positions of the super-buckets in the folded order
-        const uint32_t c = threadIdx.x < nsb ? sb_cnt[threadIdx.x] : 0u;
-        const long long st = block_exclusive_scan(c, warp_sums, total);
-        if (threadIdx.x < nsb) sb_start[threadIdx.x] = (uint32_t)st;
-    }
-    __syncthreads();
 
     // B. each super-bucket in shared memory: the keys staged with their fine
     // bucket, counting-sorted by fine bucket and ranked inside it, which
@@ -579,7 +609,7 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
     long long carry = 0;
     if (threadIdx.x == 0) o.pf[0] = 0;
     for (int sb = 0; sb < nsb; ++sb) {
-        const uint32_t k0 = sb_start[sb], len = sb_cnt[sb];
+        const uint32_t k0 = single ? 0u : sb_start[sb], len = single ? (uint32_t)n : sb_cnt[sb];
         if (len == 0) continue;
         const unsigned long long* region = keys + (int64_t)sb * kFoldSegKeys;
         for (int f = threadIdx.x; f < (1 << kFoldFineLog2); f += blockDim.x) fcnt[f] = 0;
@@ -588,10 +618,31 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
         // registers from the count to the scatter
         unsigned long long kv[kPerThread];
         uint32_t kf[kPerThread / 2];   // two 16-bit fine buckets per register
+        if (single) {
 #pragma unroll
-        for (int u = 0; u < kPerThread; ++u) {
-            const uint32_t q = threadIdx.x + u * kFoldThreads;
-            kv[u] = q < len ? __ldcs(region + q) : 0ull;   // last use of the staged key
+            for (int h = 0; h < kPerThread; h += kFoldUnroll) {
+                long long dl[kFoldUnroll];
+                float df[kFoldUnroll];
+#pragma unroll
+                for (int u = 0; u < kFoldUnroll; ++u) {
+                    const uint32_t q = threadIdx.x + (h + u) * kFoldThreads;
+                    dl[u] = q < len ? dc.d_lat[q] : 0;
+                    df[u] = q < len ? dc.d_f[q] : 0.0f;
+                }
+#pragma unroll
+                for (int u = 0; u < kFoldUnroll; ++u) {
+                    const uint32_t q = threadIdx.x + (h + u) * kFoldThreads;
+                    const long long rho = lattice_rho(dl[u], df[u], P, inv_p);
+                    const bool ok = q < len && in_range(dc.check, 2, rho, P);
+                    kv[h + u] = ok ? ((unsigned long long)rho << ib) | (unsigned long long)q : 0ull;
+                }
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < kPerThread; ++u) {
+                const uint32_t q = threadIdx.x + u * kFoldThreads;
+                kv[u] = q < len ? __ldcs(region + q) : 0ull;   // last use of the staged key
+            }
         }
 #pragma unroll
         for (int u = 0; u < kPerThread; ++u) {
@@ -606,7 +657,7 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
         // region's lines from L2 without writing them back (the next period
         // writes the region again before reading it), so that the keys
         // cost no DRAM traffic when they stayed in L2
-        {
+        if (!single) {
             const uint32_t lines = (len * (uint32_t)sizeof(unsigned long long) + 127u) / 128u;
             for (uint32_t l = threadIdx.x; l < lines; l += blockDim.x)
                 asm volatile("discard.global.L2 [%0], 128;" ::"l"(region + 16 * l) : "memory");
@@ -676,11 +727,13 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
                 const uint32_t i = threadIdx.x + (h + j) * kFoldThreads;
                 if (!ok[j]) continue;
                 const int64_t g = (int64_t)k0 + i;
-                // streaming stores: the window kernels read the folded curve
-                // after the whole chunk is folded, from DRAM, so these lines
-                // go first when L2 needs room (the super-bucket regions stay)
+                // streaming stores: what the window kernels read after the
+                // whole chunk is folded comes from DRAM, so these lines go
+                // first when L2 needs room (the super-bucket regions stay, and
+                // what window_bounds reads right here)
                 __stcs(o.sidx + g, id[j]);
-                __stcs(o.rs + g, pv[j].r);
+                if (kBounded) o.rs[g] = pv[j].r;
+                else __stcs(o.rs + g, pv[j].r);
                 srfx[swz(i)] = pv[j].rfx;
                 if (!o.uniform) {
                     __stcs(o.ws + g, pv[j].w);
@@ -711,7 +764,7 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
         for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) {
             const long long v = srfx[swz(i)];
             __stcs(o.pf + (int64_t)k0 + 1 + i, v);
-            if (kBounded) __stcs(o.pq + (int64_t)k0 + 1 + i, (int32_t)(v >> o.shift));
+            if (kBounded) o.pq[(int64_t)k0 + 1 + i] = (int32_t)(v >> o.shift);
         }
         __syncthreads();   // the next super-bucket overwrites the staged keys and rfx
     }
@@ -882,11 +935,11 @@ __device__ void fold_global(unsigned char* smem, const DevPlan& dp, const DevCur
     }
 }
 
-// kBounded: the wave's window search is the one by bounds (uniform weights),
-// which reads the 32-bit prefix sums.
-template <bool kBounded>
-__global__ void __launch_bounds__(kFoldThreads, kFoldMinBlocks)
-k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk)
+// kBounded: the window search is the one by bounds (uniform weights), whose
+// first steps follow here.
+template <bool kBounded, int T>
+__global__ void __launch_bounds__(T, kFoldThreads * kFoldMinBlocks / T)
+k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk, int tile_buf)
 {
     const SlotMap& sm = smq ? *smq : smv;
     extern __shared__ unsigned char smem[];
@@ -911,7 +964,8 @@ k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, 
             for (int q = 0; q <= kListClasses; ++q) dk.left_n[q] = 0u;
     }
 
-    if (!fold_staged<kBounded>(smem, dp, dc, p, keys, o)) {
+    bool staged = fold_staged<kBounded, T>(smem, dp, dc, p, keys, o);
+    if constexpr (!FoldCfg<T>::kSingle) if (!staged) {
         __syncthreads();   // the global path reuses the shared memory
         fold_global(smem, dp, dc, p, keys, o);
         __syncthreads();
@@ -936,6 +990,10 @@ k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, 
             o.pf[n + k + 1] = v;
             if (kBounded) o.pq[n + k + 1] = (int32_t)(v >> o.shift);
         }
+    }
+    if (kBounded) {
+        __syncthreads();
+        bounds::window_bounds<T>(smem, ds, dk, slot_id, lc, p, tile_buf);
     }
 }
 
@@ -2381,15 +2439,18 @@ void pick_config_host(int d, int st, int nwin, int32_t& variant, int32_t& nc_out
         for (int nc = 2; nc <= 16; nc <<= 1) consider(tiles::kCol16R, nc);
 }
 
-// Pieces of the template s[0 .. d) with T0 step st.  Both sets are cut where
-// the sum of length x deviation, which is what the bound loses on white noise,
-// is least for the default limb darkening (0.128 D for the whole template;
-// 0.040, 0.030, 0.024, 0.017 and 0.009 D for 5, 7, 9, 13 and 25 pieces).
-BoundTab bound_table(const float* s, int d, int st)
+// Pieces of the template s[0 .. d) with T0 step st, and what the bounds need of
+// the duration (window_bounds.cuh).  Both sets of pieces are cut where the sum
+// of length x deviation, which is what the bound loses on white noise, is least
+// for the default limb darkening (0.128 D for the whole template; 0.040, 0.024,
+// 0.017, 0.013 and 0.009 D for 5, 9, 13, 17 and 25 pieces).
+void bound_tables(const float* s, int j, int d, int st, int64_t n, int clg, int variant, int nc, BoundTab& b,
+                  BoundDur& bd)
 {
     constexpr double kCut[kBoundSegs / 2] = {0.010, 0.024, 0.042, 0.064, 0.088, 0.116,
                                              0.148, 0.184, 0.224, 0.270, 0.324, 0.392};
-    BoundTab b{};
+    b = BoundTab{};
+    bd = BoundDur{};
     auto piece = [&](int lo, int hi, float& mean) {
         double m = 0.0, v = 0.0;
         for (int k = lo; k < hi; ++k) m += s[k];
@@ -2397,19 +2458,29 @@ BoundTab bound_table(const float* s, int d, int st)
         for (int k = lo; k < hi; ++k) v += ((double)s[k] - mean) * ((double)s[k] - mean);
         return (float)(std::sqrt(v) * (1.0 + 1e-6));
     };
-    b.off[0] = 0;
-    b.off[kBoundSegs] = d;
+    int off[kBoundSegs + 1];
+    off[0] = 0;
+    off[kBoundSegs] = d;
     for (int g = 0; g < kBoundSegs / 2; ++g) {
         // (short templates: at least a point each from the edges inwards)
         const int cut = std::min(d / 2, std::max(g + 1, (int)std::lround(kCut[g] * d)));
-        b.off[1 + g] = cut;
-        b.off[kBoundSegs - 1 - g] = d - cut;
+        off[1 + g] = cut;
+        off[kBoundSegs - 1 - g] = d - cut;
     }
     for (int g = 0; g < kBoundSegs; ++g) {
-        const int len = b.off[g + 1] - b.off[g];
-        b.nu[g] = piece(b.off[g], b.off[g + 1], b.mean[g]);
-        b.inv_len[g] = len > 0 ? (float)((1.0 - 1e-5) / len) : 0.0f;
+        const int len = off[g + 1] - off[g];
+        float mean = 0.0f;
+        const float nu = piece(off[g], off[g + 1], mean);
+        float end;
+        std::memcpy(&end, &off[g + 1], sizeof end);
+        b.seg[g] = make_float4(end, mean, nu, len > 0 ? (float)((1.0 - 1e-5) / len) : 0.0f);
     }
+    double seg_jumps = 0.0, seg_before = 0.0;
+    for (int g = 0; g < kBoundSegs; ++g) {
+        seg_jumps += std::fabs(b.seg[g].y - seg_before);
+        seg_before = b.seg[g].y;
+    }
+    b.seg_jumps = (float)((seg_jumps + std::fabs(seg_before)) * (1.0 + 1e-6));
     double top = 0.0, t2 = 0.0;
     for (int k = 0; k < d; ++k) {
         top = std::max(top, std::fabs((double)s[k]));
@@ -2418,33 +2489,78 @@ BoundTab bound_table(const float* s, int d, int st)
     b.nu_all = piece(0, d, b.mean_all);
     b.root_t2 = (float)std::sqrt(t2);
     b.t_max = (float)(top * (1.0 + 1e-6));
+
+    bd.j = j;
+    bd.d = d;
+    bd.st = st;
+    bd.m_total = (int32_t)((n + st - 1) / st);
+    while ((1 << bd.lg_nc) < nc) ++bd.lg_nc;
+    bd.mode = variant == tiles::kScalar15 ? bounds::kModePairS
+              : variant == tiles::kCol16R ? bounds::kModeRot
+              : tiles::variant_colpair(variant) ? bounds::kModeCols : bounds::kModeWin;
+    bd.test = bounds::kTestSum;
     if (d >= bounds::kCutPoints) {
         // more pieces for longer windows: the bound loses in proportion to D,
         // the best window gains with its root
         std::vector<double> cut;
         if (d < 200) cut = {0.078, 0.222};
-        else if (d < 1000) cut = {0.052, 0.138, 0.268};
-        else if (d < 3000) cut = {0.038, 0.098, 0.182, 0.300};
-        else cut = {0.022, 0.058, 0.104, 0.164, 0.238, 0.338};
-        std::vector<int> row = {0};
-        for (double c : cut) row.push_back((int)std::lround(c * d / st));
-        for (double c : cut) row.push_back((int)std::lround((1.0 - c) * d / st));
-        std::sort(row.begin(), row.end());
-        row.erase(std::unique(row.begin(), row.end()), row.end());
-        while ((int64_t)row.back() * st >= d) row.pop_back();
-        b.cuts = (int)row.size();
+        else if (d < 1000) cut = {0.038, 0.098, 0.182, 0.300};
+        else if (d < 4000) cut = {0.022, 0.058, 0.104, 0.164, 0.238, 0.338};
+        else cut = {0.016, 0.040, 0.072, 0.110, 0.156, 0.210, 0.276, 0.362};
+        const bool coarse = d >= bounds::kCoarseSteps << clg;
+        const int unit = coarse ? 1 : st;   // cuts at whole T0 steps
+        std::vector<int> at = {0};
+        for (double c : cut) at.push_back((int)std::lround(c * d / unit) * unit);
+        for (double c : cut) at.push_back((int)std::lround((1.0 - c) * d / unit) * unit);
+        std::sort(at.begin(), at.end());
+        at.erase(std::unique(at.begin(), at.end()), at.end());
+        while (at.back() >= d) at.pop_back();
+        b.cuts = (int)at.size();
+        bd.row_max = at.back() / st;
+        bd.test = coarse ? bounds::kTestCoarse
+                  : bounds::kGroup + bd.row_max <= bounds::kRowBuf ? bounds::kTestCuts : bounds::kTestCutsDirect;
         float before = 0.0f, mean = 0.0f;
+        double jumps = 0.0;
         for (int u = 0; u < b.cuts; ++u) {
-            const int lo = row[u] * st, hi = u + 1 < b.cuts ? row[u + 1] * st : d;
-            b.cut_row[u] = row[u];
-            b.cut_len[u] = hi - lo;
-            b.cut_nu[u] = piece(lo, hi, mean);
-            b.cut_coef[u] = before - mean;
+            const int hi = u + 1 < b.cuts ? at[u + 1] : d;
+            b.cut_len[u] = hi - at[u];
+            b.cut_nu[u] = piece(at[u], hi, mean);
+            if (u == 0) bd.coef0 = -mean;
+            else bd.coef[u - 1] = before - mean;
+            if (u > 0) bd.row[u - 1] = bd.test == bounds::kTestCuts ? at[u] / st : at[u];
+            jumps += std::fabs((double)before - mean);
             before = mean;
         }
-        b.cut_coef[b.cuts] = before;
+        bd.cut_last = before;
+        b.cut_jumps = (float)((jumps + std::fabs((double)before)) * (1.0 + 1e-6));
+        bd.cuts4 = (b.cuts + 2) / 4 * 4;
     }
-    return b;
+    bd.lam = (b.cuts == 0 ? b.mean_all : 1.0f) / b.root_t2;
+}
+
+// Chunk sizes of the durations (variants kWindowOnly excepted) for CTAs with
+// room for `most` chunks: the smallest lg with which every period's fit.
+int bound_chunks(std::vector<BoundDur>& bd, const std::vector<int32_t>& variant, const PlanHost& h, int most)
+{
+    for (int lg = 0;; ++lg) {
+        const int64_t tile = (int64_t)bounds::kTileStarts << lg;
+        std::vector<int64_t> sum(bd.size() + 1, 0);
+        for (size_t j = 0; j < bd.size(); ++j) {
+            BoundDur& b = bd[j];
+            b.subs = b.wsub = 0;
+            if (variant[j] != tiles::kWindowOnly) {
+                const bool nearby = b.st <= bounds::kNearStep;
+                const int64_t group = (int64_t)(nearby ? bounds::kChunkGroups : 1) * bounds::kGroup << lg;
+                const int64_t wins = nearby ? std::min<int64_t>(b.m_total, tile / b.st + 1) : b.m_total;
+                b.subs = (int32_t)((wins + group - 1) / group);
+                b.wsub = (int32_t)(((wins + b.subs - 1) / b.subs + 31) & ~int64_t(31));   // equal chunks, whole warps
+            }
+            sum[j + 1] = sum[j] + b.subs * (b.st <= bounds::kNearStep ? (h.n + tile - 1) / tile : 1);
+        }
+        int64_t worst = 0;
+        for (size_t p = 0; p < h.jlo.size(); ++p) worst = std::max(worst, sum[h.jhi[p] + 1] - sum[h.jlo[p]]);
+        if (worst <= most) return lg;
+    }
 }
 
 int fold_smem_bytes(int bucket_log2)
@@ -2455,11 +2571,7 @@ int fold_smem_bytes(int bucket_log2)
     // staged path: scan scratch, rfx in final order, keys in fine-bucket
     // order, fine-bucket counts and ends, super-bucket counts and starts,
     // inverse permutation, fine buckets of the sorted keys, overflow flag
-    const int staged = 33 * (int)sizeof(long long) + 2 * kFoldSegKeys * (int)sizeof(unsigned long long) +
-                       (2 << kFoldFineLog2) * (int)sizeof(uint32_t) +
-                       2 * (1 << kFoldMaxSbLog2) * (int)sizeof(uint32_t) +
-                       2 * kFoldSegKeys * (int)sizeof(uint16_t) + (int)sizeof(int);
-    return std::max(global_path, staged);
+    return std::max(global_path, FoldCfg<kFoldThreads>::kStagedBytes);
 }
 
 constexpr int kMedianSmem = kMedianCap * (int)(sizeof(unsigned long long) + 2 * sizeof(uint16_t));
@@ -2481,10 +2593,12 @@ gtls_status configure_kernels(int dev)
                                        optin - (int)a.sharedSizeBytes));
         return GTLS_OK;
     };
-    GTLS_TRY(allow((const void*)k_fold_sort<false>));
-    GTLS_TRY(allow((const void*)k_fold_sort<true>));
+    for (const void* fn : {(const void*)k_fold_sort<false, 256>, (const void*)k_fold_sort<false, 512>,
+                           (const void*)k_fold_sort<false, 1024>, (const void*)k_fold_sort<true, 256>,
+                           (const void*)k_fold_sort<true, 512>, (const void*)k_fold_sort<true, 1024>})
+        GTLS_TRY(allow(fn));
     GTLS_TRY(allow((const void*)k_window_tiles));
-    GTLS_TRY(allow((const void*)bounds::k_window_bounds));
+    GTLS_TRY(allow((const void*)bounds::k_window_exact));
     GTLS_TRY(allow((const void*)k_median_sde));
     GTLS_TRY(allow((const void*)k_median_sde_set));
     GTLS_CUDA(cudaFuncSetAttribute((const void*)k_window_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2508,7 +2622,7 @@ gtls_status create_device(gtls_plan* pl)
         // super-buckets of the staged fold: about kFoldFillKeys points each
         // on average (regions of kFoldSegKeys slots)
         const int64_t nsb = (h.n + kFoldFillKeys - 1) / kFoldFillKeys;
-        dp.fold_nsb = (int32_t)std::max<int64_t>(1, std::min<int64_t>(nsb, 1 << kFoldMaxSbLog2));
+        dp.fold_nsb = h.n <= kFoldSegKeys ? 1 : (int32_t)std::min<int64_t>(nsb, 1 << kFoldMaxSbLog2);
     }
     dp.max_kept = h.max_kept;
     dp.median_half = h.median_window / 2;
@@ -2755,6 +2869,7 @@ gtls_status create_device(gtls_plan* pl)
         GTLS_TRY(upload(pl, const_cast<float**>(&dp.tc_tab), tc_tab));
         GTLS_TRY(upload(pl, const_cast<int32_t**>(&dp.cfg_variant), var));
         pl->variant_host = var;
+        pl->nc_host = ncs;
         GTLS_TRY(upload(pl, const_cast<int32_t**>(&dp.cfg_nc), ncs));
         GTLS_TRY(upload(pl, const_cast<int64_t**>(&dp.tmpl2_off), off2));
         if (t2.empty()) t2.assign(1, make_float2(0.0f, 0.0f));
@@ -2860,25 +2975,34 @@ gtls_status create_device(gtls_plan* pl)
                 pl->tile_count_ref = (int)((n + len1 - 1) / len1);
             }
             GTLS_TRY(upload(pl, const_cast<int32_t**>(&pl->dp_ref.cfg_variant), var1));
+            pl->variant_ref_host = var1;
         }
         GTLS_TRY(dev_alloc(pl, &pl->tile_counter, 1));
         GTLS_TRY(dev_alloc(pl, &pl->tc_counter, 1));
     }
 
-    // pieces of every duration's template for the bounds of the window search
+    // tables of the window search by bounds
     {
-        std::vector<BoundTab> tab(dp.nd);
         // small searches are bound by launches: two kernels more cost what
         // they save (0.29 ms and 6e7 window-point products: 18 us slower;
         // 1.2 ms and 2.9e9: 140 us faster)
         const bool worth = h.wpe >= kBoundsMinWpe || (h.prm.test_flags & 4);
         pl->bounds_ok = !pl->has_tensor && worth && !(h.prm.test_flags & 2);
+        std::vector<BoundTab> tab(dp.nd);
+        std::vector<BoundDur> bd(dp.nd);
+        const int threads = fold_threads(h.n), most = bounds::max_chunks(threads);
+        const int clg = bounds::coarse_log2(threads, h.n, h.dmax);
         for (int pass = 0; pass < (pl->refine_k > 0 ? 2 : 1) && pl->bounds_ok; ++pass) {
+            const std::vector<int32_t>& var = pass ? pl->variant_ref_host : pl->variant_host;
             for (int j = 0; j < dp.nd; ++j) {
-                tab[j] = bound_table(h.tmpl.data() + h.tmpl_off[j], h.dpts[j], pass ? 1 : h.stride[j]);
+                bound_tables(h.tmpl.data() + h.tmpl_off[j], j, h.dpts[j], pass ? 1 : h.stride[j], h.n, clg, var[j],
+                             pass ? 1 : pl->nc_host[j], tab[j], bd[j]);
                 pl->bounds_ok = pl->bounds_ok && tab[j].mean_all > 0.0f && tab[j].root_t2 > 0.0f;
             }
-            GTLS_TRY(upload(pl, const_cast<BoundTab**>(pass ? &pl->dp_ref.bounds : &dp.bounds), tab));
+            DevPlan& q = pass ? pl->dp_ref : dp;
+            q.bound_lg = bound_chunks(bd, var, h, most);
+            GTLS_TRY(upload(pl, const_cast<BoundTab**>(&q.bounds), tab));
+            GTLS_TRY(upload(pl, const_cast<BoundDur**>(&q.bound_durs), bd));
         }
     }
 
@@ -3050,6 +3174,7 @@ struct Ctx {
     int n_sm = 0;
     int median_blocks = 1;   // widest row of the running-median grid
     int sr_blocks = 1;       // widest row of the SR reductions' grid
+    int64_t max_d = 0;       // longest duration of any curve
     cudaStream_t st = nullptr;
     const void* tc_maps = nullptr;   // tensor-core kernel: TMA maps of dk.rs (tc::kMaps rows pitches)
     int tc_jspan = 1;        // tensor-core kernel: work items per period slot
@@ -3065,6 +3190,30 @@ gtls_status stage_mark(Ctx& c, int stage)
     return c.prof ? mark(c.prof, c.st, stage, c.ev) : GTLS_OK;
 }
 
+template <bool kBounded, int T>
+void launch_fold_as(Ctx& c, const DevSet& ds, const SlotMap& sm, const SlotMap* smq)
+{
+    int smem = T == kFoldThreads ? c.fold_smem : FoldCfg<T>::kStagedBytes;
+    if (kBounded) smem = std::max(smem, (int)bounds::smem_bytes(T));
+    k_fold_sort<kBounded, T><<<sm.slots, T, smem, c.st>>>(ds, sm, smq, c.dk, c.tile_buf);
+}
+
+// The fold of one wave (with the first steps of the window search when
+// bounded) in CTAs of `threads` threads.
+gtls_status launch_fold(Ctx& c, const DevSet& ds, const SlotMap& sm, const SlotMap* smq, bool bounded, int threads)
+{
+    if (bounded) {
+        if (threads == 256) launch_fold_as<true, 256>(c, ds, sm, smq);
+        else if (threads == 512) launch_fold_as<true, 512>(c, ds, sm, smq);
+        else launch_fold_as<true, 1024>(c, ds, sm, smq);
+    } else {
+        if (threads == 256) launch_fold_as<false, 256>(c, ds, sm, smq);
+        else if (threads == 512) launch_fold_as<false, 512>(c, ds, sm, smq);
+        else launch_fold_as<false, 1024>(c, ds, sm, smq);
+    }
+    return GTLS_OK;
+}
+
 // One wave: fold + sort, every window, per-period results.  `counter` must
 // be zero when the window kernel starts (reset here when reset_counter).
 // With smq (a wave cut on the device, see k_wave_next) the kernels read the
@@ -3076,8 +3225,7 @@ gtls_status wave_pass(Ctx& c, bool ref, const SlotMap& sm, bool tiled, bool weig
 {
     const DevSet& ds = ref ? c.set_ref : c.set;
     const bool bounded = tiled && c.bounds_ok && !weighted;
-    (bounded ? k_fold_sort<true> : k_fold_sort<false>)<<<sm.slots, kFoldThreads, c.fold_smem, c.st>>>(ds, sm, smq,
-                                                                                                     c.dk);
+    GTLS_TRY(launch_fold(c, ds, sm, smq, bounded, fold_threads(max_n)));
     GTLS_CUDA(cudaGetLastError());
     GTLS_TRY(stage_mark(c, kStageFold));
     if (tiled) {
@@ -3085,11 +3233,12 @@ gtls_status wave_pass(Ctx& c, bool ref, const SlotMap& sm, bool tiled, bool weig
         const int buf = weighted ? c.tile_buf_w : c.tile_buf;
         const int bytes = buf * (int)(weighted ? sizeof(float2) : sizeof(float));
         if (bounded) {
-            bounds::k_window_bounds<<<sm.slots, bounds::kThreads, bounds::smem_bytes(), c.st>>>(ds, sm, smq, c.dk, buf);
+            // as many windows at a time as their points and templates leave room for
+            const int room = (int)std::min<int64_t>((c.max_d + 3) & ~3, bounds::kExactRoom);
+            const int ctas = std::max(1, std::min(16, (int)(200000 / (room * 8 + 1024))));
+            bounds::k_window_exact<<<c.n_sm * ctas, 32, room * 2 * sizeof(float), c.st>>>(ds, sm, smq, c.dk, room);
             GTLS_CUDA(cudaGetLastError());
-            bounds::k_window_exact<<<c.n_sm * 8, bounds::kExactThreads, 0, c.st>>>(ds, sm, smq, c.dk);
-            GTLS_CUDA(cudaGetLastError());
-            c.launches += 2;
+            c.launches += 1;
         }
         k_window_tiles<<<c.n_sm * tiles::kCtasPerSm, tiles::kThreads, bytes, c.st>>>(
             ds, sm, smq, c.dk, buf, weighted ? 1 : 0, bounded ? 1 : 0, counter);
@@ -3225,6 +3374,7 @@ gtls_status run_search(gtls_plan* pl, const double* t, const double* y, const do
     c.n_sm = pl->n_sm;
     c.median_blocks = (dp.np + median_outs(dp.median_half) - 1) / median_outs(dp.median_half);
     c.sr_blocks = sr_blocks(dp.np);
+    c.max_d = h.dmax;
     c.st = st;
     c.tc_jspan = pl->tc_jspan;
     c.tc_test = pl->tc_test_wait;
@@ -3511,6 +3661,7 @@ Ctx batch_ctx(const gtls_batch* b, cudaStream_t st)
     for (const gtls_plan* pl : b->plans) {
         c.tc_jspan = std::max(c.tc_jspan, pl->tc_jspan);
         c.tc_test = std::max(c.tc_test, pl->tc_test_wait);
+        c.max_d = std::max(c.max_d, pl->host.dmax);
     }
     c.tc_maps = b->tc_maps;
     c.bounds_ok = b->bounds_ok;

@@ -10,96 +10,140 @@
 // (Cauchy-Schwarz), where S_g is the exact sum of r over the segment and E_g
 // an upper bound of its sum of r^2.  A window whose bound stays below what
 // some window of the period is known to reach cannot be the minimum, and its
-// D products need not be summed.  On white noise (the hardest case: the best
-// window stands out least) this leaves 0.01-3 % of the windows.
+// D products need not be summed.
 //
-// k_window_bounds, one CTA per period:
-//   1. sums of r^2 over blocks of 2^lb folded points and their prefix
-//      (shared memory), and from it the largest energy of any stretch of a
-//      length;
-//   2. one pass over all windows, chunk by chunk: the window sum (short
-//      windows) or the bound's main term over a few wide pieces; the largest
-//      value of every chunk and the four most promising windows are kept;
-//   3. those four are summed: the lowest delta-chi2 T is the threshold;
+// window_bounds, by the CTA that has just folded the period (so that its
+// prefix sums are still in L2):
+//   1. one pass over the prefix sums: a coarse copy of them (every 2^clg-th,
+//      in shared memory), the energies of blocks of 2^lb points and their
+//      prefix, and from it the largest energy of any stretch of a length;
+//   2. first test, one pass over all windows, chunk by chunk: the window sum
+//      (short windows) or the bound's main term over a few wide pieces; the
+//      largest value of every chunk and the most promising windows are kept;
+//   3. those are summed: the lowest delta-chi2 T is the threshold;
 //   4. chunks whose largest value can beat T are walked again; windows that
-//      also pass the kBoundSegs-segment bound are listed for step 5.
+//      also pass the kBoundSegs-segment bound are summed, a warp each, and
+//      those within the rounding of the lowest sum are listed.
 // k_window_exact:
-//   5. the listed windows of all periods of the wave are summed, adding the
-//      products of a window in the order of the tiled kernel
-//      (window_tiles.cuh): the same columns per lane, the same rows, the same
-//      tree over the lanes, for the rotated variant also the same first round
-//      of every block that covers the window there; so the minimum, its
-//      duration, its start and every bit of its delta-chi2 are those of the
-//      tiled kernel.
+//   5. the listed windows of all periods of the wave (one or two per period)
+//      are summed again, adding the products of a window in the order of the
+//      tiled kernel (window_tiles.cuh): the same columns per lane, the same
+//      rows, the same tree over the lanes, for the rotated variant also the
+//      same first round of every block that covers the window there; so the
+//      minimum, its duration, its start and every bit of its delta-chi2 are
+//      those of the tiled kernel.
 //
 // Periods for which nothing is gained (no window has a negative delta-chi2,
 // so that signed zeros decide; too many windows left; a value is not finite)
 // are listed for the tiled kernel, which then runs on that list.
 //
-// The window sums of steps 2 and 4 come from 32-bit prefix sums: the exact
-// ones shifted right so far that any window sum fits 31 bits; differences
-// modulo 2^32 are then off by at most one unit.
+// The window sums of steps 1 to 4 come from 32-bit prefix sums: the exact ones
+// shifted right so far that any sum fits 31 bits; differences are then off by
+// at most one unit.
 //
-// What bounds it: the prefix reads of step 2 (a lane whose start lies in a
-// cache line of its own costs the L1 a cycle) and about 40 instructions per
-// window.  Windows of small T0 steps are walked position-major -- all
-// durations of a stretch of kTileStarts starts before the next -- to keep the
-// prefix sums in L1.  Measured on the Kepler-like search (62,363 points,
-// 199,577 periods, 3.1e10 windows): 193 ms for the window stage, against
-// 698 ms for the tiled kernel alone; 46 windows of a period are left to sum
-// on average, out of 154,000.
+// What bounds it: shared-memory reads of the coarse prefix and about 50
+// instructions per window.  A lane that reads global memory at a cache line
+// of its own costs the L1 a cycle, which made the same tests on the prefix
+// sums themselves slower by half; only short windows (T0 steps of a few points, so
+// that neighbours share lines) read those,
+// position-major -- all durations of a stretch of kTileStarts starts before
+// the next -- to stay in L1.
 #pragma once
 
 namespace gtls {
 namespace bounds {
 
-constexpr int kThreads = 512;
-constexpr int kWarps = kThreads / 32;
-constexpr int kMinBlocks = 2;       // resident CTAs per SM
-constexpr int kMaxBlocks = 8192;    // energy blocks of a period
-constexpr int kEnergyLens = 48;     // lengths 8, 11, 16, 22, ... whose largest energy is kept
-constexpr int kMaxChunks = 4096;    // window chunks of a period
+constexpr int kShortSpans = 16;     // spans of blocks whose largest energy is kept: 0 .. 15,
+constexpr int kEnergySpans = kShortSpans + 32;   // then 16, 22, 32, 45, ... (up to every block there is)
 constexpr int kTileStarts = 8192;   // window starts walked before the next stretch
 constexpr int kGroup = 128;         // windows a warp tests at a time (4 per lane)
 constexpr int kChunkGroups = 4;     // groups per chunk (at most)
 constexpr int kNearStep = kTileStarts / kGroup;   // T0 steps up to this fill a group in one stretch
-constexpr int kSieve = kWarps * kGroup;   // windows waiting for the segment bound: one group per warp always fits
-constexpr int kListed = 2048;       // windows listed of a period before the tiled kernel is cheaper
-constexpr int kCand = 4;            // windows summed for the threshold
-constexpr int kRowBuf = 336;        // prefix sums at whole T0 steps a warp stages for one group
-constexpr int kCutSlots = (kBoundCuts + 3) / 4 * 4;
+constexpr int kListed = 256;        // windows listed of a period before the tiled kernel is cheaper
+constexpr int kCand = 2;            // windows summed for the threshold
+constexpr int kRowBuf = 168;        // prefix sums at whole T0 steps a warp stages for one group
 constexpr int kCutPoints = 60;      // windows of at least this many points are first tested by wide pieces
-constexpr int kExactThreads = 256;
+constexpr int kCoarseSteps = 64;    // ... and from this many coarse steps on from the coarse prefix
+constexpr int kExactRoom = 24576;   // points of a window (and its template) staged by k_window_exact, at most
 constexpr unsigned int kNone = 0xffffffffu;
 
 enum Mode : int { kModePairS = 0, kModeCols = 1, kModeRot = 2, kModeWin = 3 };
-enum Test : int { kTestSum = 0, kTestCuts = 1, kTestCutsDirect = 2 };
+enum Test : int { kTestSum = 0, kTestCuts = 1, kTestCutsDirect = 2, kTestCoarse = 3 };
 
+// One duration of a period: the plan's part (BoundDur) and the period's.
 struct Dur {
-    int j, d, st, m_total;
-    int first, wsub;            // first chunk (of a stretch for T0 steps up to kNearStep), windows per chunk
-    int lg_nc, mode, test;
-    float lam;                  // first-test value times lam estimates C1 / sqrt(sum s_k^2)
+    BoundDur b;
+    int first;                  // first chunk (near durations: of a stretch)
     float emax;                 // upper bound of sum r^2 over any window of the duration
     float first_min, cmin;      // thresholds of the first test (32-bit prefix units) and of the segment bound
     float smin;                 // lowest window sum that can have a depth (32-bit prefix units)
-    int row_max;                // first T0 step of the last piece
-    int cuts4;                  // wide pieces, rounded up to a multiple of 4
-    float cut_last;             // mean of the last piece
-    alignas(16) float coef[kCutSlots];   // the pieces' coefficients (0 past the last)
-    alignas(16) int row[kCutSlots];      // and first T0 steps
+    float blur;                 // what FP32 sums of C1 can be off by
+    float cmin_coarse;          // cmin for sums from the coarse prefix
+    int pad[1];
 };
 
-__host__ __device__ inline size_t smem_bytes()
+// Chunks of windows: durations of T0 steps above kNearStep (far ones) are cut
+// into groups over the whole curve; the others (near ones) into chunks of at
+// most kChunkGroups 2^lg groups inside every stretch of kTileStarts 2^lg
+// starts.  Far chunks come first.
+struct Chunks {
+    int ndur, near_durs;        // durations (ascending); the first near_durs are near
+    int far, per_tile;          // far chunks, near chunks per stretch
+    int total;
+};
+
+// Shared memory for CTAs of T threads (curves of up to 8 T points when
+// T < 1024).  At 1024 it stays below 195 KB: the next size the SM offers leaves
+// 28 instead of 60 KB of L1, which the fold's gathers feel.
+template <int T>
+struct Smem {
+    static constexpr int kWarps = T / 32;
+    static constexpr int kSieve = kWarps * kGroup;   // one group per warp always fits
+    static constexpr int kMaxBlocks = T == 1024 ? 9 * T : 2 * T;
+    static constexpr int kMaxCoarse = T == 1024 ? 18 * T : 3 * T;
+    static constexpr int kMaxChunks = 2 * T;
+    static constexpr int kFinal = T;                 // windows past the segment bound
+    Dur dur[tiles::kMaxDur];
+    unsigned int sieve[kSieve];                      // (duration, window) past the first test
+    float pre[kMaxBlocks + 8];                       // energy prefix
+    float cmax[kMaxChunks];                          // largest first-test value per chunk
+    float row_buf[kWarps * kRowBuf];
+    float coarse[kMaxCoarse + kMaxCoarse / 32 + 1];  // see at_coarse
+    unsigned int fin[kFinal];
+    float fin_v[kFinal];
+    Chunks ck;
+    int next, sieved, n_fin, n_listed, dev, big;
+    float wsum[kWarps], energy[kEnergySpans];
+    float top[kWarps], c1[kWarps], s[kWarps], thr;
+    int top_at[kWarps], cand[kCand];
+};
+
+__host__ inline size_t smem_bytes(int threads)
 {
-    return (size_t)kSieve * sizeof(unsigned int) +
-           (size_t)(kMaxBlocks + 8 + kMaxChunks + kWarps * kRowBuf) * sizeof(float);
+    return threads == 256 ? sizeof(Smem<256>) : threads == 512 ? sizeof(Smem<512>) : sizeof(Smem<1024>);
 }
+
+// log2 of the coarse step for curves of n points and durations of up to d.
+__host__ inline int coarse_log2(int threads, int64_t n, int64_t d)
+{
+    const int64_t room = threads == 1024 ? Smem<1024>::kMaxCoarse : threads == 512 ? Smem<512>::kMaxCoarse
+                                                                                   : Smem<256>::kMaxCoarse;
+    int lg = 2;
+    while (((n + d) >> lg) + 2 > room) ++lg;
+    return lg;
+}
+
+// Chunks a CTA of T threads has room for.
+__host__ inline int max_chunks(int threads) { return 2 * threads; }
 
 // Relative error allowed for a sum of n products in FP32 (twice the bound).
 __device__ __forceinline__ float sum_slack(int n) { return 1.2e-7f * (float)(n + 8); }
 
 __device__ __forceinline__ float root(float x) { return x > 0.0f ? x * rsqrtf(x) : (x == 0.0f ? 0.0f : x); }
+
+// Place of coarse entry e: one word further every 32, so that lanes whose
+// entries are a power of two apart read different banks.
+__device__ __forceinline__ int at_coarse(int e) { return e + (e >> 5); }
 
 // Sum of one window by the nc lanes of a group, in the order of the tiled
 // kernel; every lane of the group returns the totals (y: window sum of the
@@ -116,14 +160,14 @@ __device__ __forceinline__ float2 window_sum(const float* __restrict__ r, const 
 #pragma unroll 8
                 for (int k = rho; k < d; k += st) {
                     const float v = r[k];
-                    x = fmaf(v, __ldg(t + k), x);
+                    x = fmaf(v, t[k], x);
                     y = v + y;
                 }
             }
         } else if (mode == kModeWin) {
             for (int rho = c; rho < st; rho += nc) {
 #pragma unroll 8
-                for (int k = rho; k < d; k += st) x = fmaf(r[k], __ldg(t + k), x);
+                for (int k = rho; k < d; k += st) x = fmaf(r[k], t[k], x);
             }
         } else {
             const int rounds = (st + 2 * nc - 1) >> (lg_nc + 1);
@@ -136,10 +180,10 @@ __device__ __forceinline__ float2 window_sum(const float* __restrict__ r, const 
                 int k = rho;
 #pragma unroll 8
                 for (; k < both; k += st) {
-                    x = fmaf(r[k], __ldg(t + k), x);
-                    y = fmaf(r[k + nc], __ldg(t + k + nc), y);
+                    x = fmaf(r[k], t[k], x);
+                    y = fmaf(r[k + nc], t[k + nc], y);
                 }
-                for (; k < end; k += st) x = fmaf(r[k], __ldg(t + k), x);
+                for (; k < end; k += st) x = fmaf(r[k], t[k], x);
             }
         }
     }
@@ -154,100 +198,53 @@ __device__ __forceinline__ float2 window_sum(const float* __restrict__ r, const 
     return make_float2(x, y);
 }
 
-// Chunks of windows: durations of T0 steps above kNearStep (far ones) are cut
-// into groups over the whole curve; the others (near ones) into chunks of at
-// most kChunkGroups 2^lg groups inside every stretch of kTileStarts 2^lg
-// starts.  Far chunks come first.
-struct Chunks {
-    int ndur, near_durs;        // durations (ascending); the first near_durs are near
-    int far, per_tile, lg;      // far chunks, near chunks per stretch
-    int total;
-};
-
-// Durations of period p the kernel searches (kept, not marked kWindowOnly)
-// into dur[] and their chunks into ck (by one warp).
-__device__ __forceinline__ void list_durations(const DevPlan& dp, unsigned int* check, int p, int n, Dur* dur, Chunks* ck,
+// Durations of period p the kernel searches (kept, not marked kWindowOnly):
+// their grid indices into list[] and the chunks of dur[] (by one warp; the
+// plan's part of dur[] is copied by the caller).
+__device__ __forceinline__ void list_durations(const DevPlan& dp, unsigned int* check, int p, int n, Dur* dur, Chunks& ck,
                                                int lane)
 {
     const int lo = dp.jlo[p], hi = dp.jhi[p];
-    int count = 0;
+    int count = 0, run_near = 0, run_far = 0, near_durs = 0;
     for (int base = 0; base <= hi - lo; base += 32) {
         const int j = lo + base + lane;
+        const int subs = j <= hi ? dp.bound_durs[j].subs : 0;
+        const bool nearby = j <= hi && dp.bound_durs[j].st <= kNearStep;
         const int d = j <= hi ? dp.dpts[j] : 0, before = j <= hi && j > lo ? dp.dpts[j - 1] : -1;
-        const int v = j <= hi ? dp.cfg_variant[j] : (int)tiles::kWindowOnly;
-        const bool kept = j <= hi && d != before && v != tiles::kWindowOnly;
+        bool kept = j <= hi && d != before && subs > 0;
         const unsigned int mask = __ballot_sync(0xffffffffu, kept);
         const int k = count + __popc(mask & ((1u << lane) - 1u));
-        if (kept && in_range(check, 19, k, tiles::kMaxDur)) {
-            const BoundTab& bt = dp.bounds[j];
-            Dur t;
-            t.j = j;
-            t.d = d;
-            t.st = dp.stride[j];
-            t.m_total = (n + t.st - 1) / t.st;
-            t.lg_nc = __ffs(dp.cfg_nc[j]) - 1;
-            t.mode = v == tiles::kScalar15 ? kModePairS
-                     : v == tiles::kCol16R ? kModeRot
-                     : tiles::variant_colpair(v) ? kModeCols : kModeWin;
-            t.lam = (bt.cuts == 0 ? bt.mean_all : 1.0f) / bt.root_t2;
-            t.test = bt.cuts == 0 ? kTestSum
-                     : kGroup + bt.cut_row[bt.cuts - 1] <= kRowBuf ? kTestCuts : kTestCutsDirect;
-            t.emax = 0.0f;
-            t.cuts4 = (bt.cuts + 3) / 4 * 4;
-            t.row_max = bt.cuts ? bt.cut_row[bt.cuts - 1] : 0;
-            t.cut_last = bt.cut_coef[bt.cuts];
+        kept = kept && in_range(check, 19, k, tiles::kMaxDur);
+        int a = kept && nearby ? subs : 0, b = kept && !nearby ? subs : 0;
+        const int a0 = a, b0 = b;
 #pragma unroll
-            for (int u = 0; u < kCutSlots; ++u) {
-                const bool in = u < bt.cuts;
-                t.coef[u] = in ? bt.cut_coef[min(u, kBoundCuts)] : 0.0f;
-                t.row[u] = in ? bt.cut_row[min(u, kBoundCuts - 1)] : 0;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int ya = __shfl_up_sync(0xffffffffu, a, o), yb = __shfl_up_sync(0xffffffffu, b, o);
+            if (lane >= o) {
+                a += ya;
+                b += yb;
             }
-            dur[k] = t;
         }
+        if (kept) {
+            dur[k].b.j = j;
+            dur[k].first = nearby ? run_near + a - a0 : run_far + b - b0;
+            dur[k].emax = 0.0f;
+        }
+        run_near += __shfl_sync(0xffffffffu, a, 31);
+        run_far += __shfl_sync(0xffffffffu, b, 31);
+        near_durs += __popc(__ballot_sync(0xffffffffu, kept && nearby));
         count += __popc(mask);
     }
-    count = min(count, tiles::kMaxDur);
-    __syncwarp();
-    for (int lg = 0;; ++lg) {   // larger chunks until kMaxChunks hold any curve length
-        int run_near = 0, run_far = 0, near_durs = 0;
-        for (int base = 0; base < count; base += 32) {
-            const int k = base + lane;
-            const bool on = k < count;
-            const int st = on ? dur[k].st : 1, m_total = on ? dur[k].m_total : 0;
-            const bool nearby = st <= kNearStep;
-            const int group = (nearby ? kChunkGroups : 1) * kGroup << lg;
-            const int wins = nearby ? min(m_total, (kTileStarts << lg) / st + 1) : m_total;
-            const int subs = on ? (wins + group - 1) / group : 0;
-            int a = nearby ? subs : 0, b = nearby ? 0 : subs;
-            const int a0 = a, b0 = b;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int ya = __shfl_up_sync(0xffffffffu, a, o), yb = __shfl_up_sync(0xffffffffu, b, o);
-                if (lane >= o) {
-                    a += ya;
-                    b += yb;
-                }
-            }
-            if (on) {
-                dur[k].first = nearby ? run_near + a - a0 : run_far + b - b0;
-                // equal chunks, whole groups of 32 windows
-                dur[k].wsub = ((wins + subs - 1) / subs + 31) & ~31;
-            }
-            run_near += __shfl_sync(0xffffffffu, a, 31);
-            run_far += __shfl_sync(0xffffffffu, b, 31);
-            near_durs += __popc(__ballot_sync(0xffffffffu, on && nearby));
-        }
-        const int tile = kTileStarts << lg;
-        const long long total = run_far + (long long)((n + tile - 1) / tile) * run_near;
-        if (total > kMaxChunks) continue;
-        if (lane == 0) *ck = Chunks{count, near_durs, run_far, run_near, lg, (int)total};
-        break;
-    }
+    const int tile = kTileStarts << dp.bound_lg;
+    if (lane == 0)
+        ck = Chunks{min(count, tiles::kMaxDur), near_durs, run_far, run_near,
+                    run_far + (n + tile - 1) / tile * run_near};
     __syncwarp();
 }
 
 // Duration k and windows [lo, hi) of chunk c (warp-uniform).
-__device__ __forceinline__ void chunk_range(const Chunks& ck, const Dur* dur, int c, int lane, int& k, int& lo, int& hi)
+__device__ __forceinline__ void chunk_range(const Chunks& ck, const Dur* dur, int lg, int c, int lane, int& k, int& lo,
+                                            int& hi)
 {
     const bool far = c < ck.far;
     int rel = c, x = 0;
@@ -262,11 +259,11 @@ __device__ __forceinline__ void chunk_range(const Chunks& ck, const Dur* dur, in
         a = __ballot_sync(0xffffffffu, k0 + 32 + lane < k1 && dur[min(k0 + 32 + lane, k1 - 1)].first <= rel);
         k += __popc(a);
     }
-    const int wsub = dur[k].wsub;
+    const int wsub = dur[k].b.wsub;
     lo = (rel - dur[k].first) * wsub;
-    int end = dur[k].m_total;
+    int end = dur[k].b.m_total;
     if (!far) {
-        const int st = dur[k].st, tile = kTileStarts << ck.lg;
+        const int st = dur[k].b.st, tile = kTileStarts << lg;
         lo += (x * tile + st - 1) / st;
         end = min(end, (int)(((long long)(x + 1) * tile + st - 1) / st));
     }
@@ -276,12 +273,38 @@ __device__ __forceinline__ void chunk_range(const Chunks& ck, const Dur* dur, in
 // First test of windows at .. at + cnt - 1 (cnt <= kGroup) of one duration:
 // acc[q] of lane l belongs to window at + 32 q + l.  kTestSum: the window sum;
 // else sum_u mean_u S_u over the wide pieces u, from prefix sums relative to
-// the first window's start (in the warp's rb when they fit there); both in
-// units of the 32-bit prefix.
-__device__ __forceinline__ void first_test(const Dur& t, const int* __restrict__ pq, int at, int cnt, float* rb, int lane,
-                                           float (&acc)[4])
+// the first window's start (kTestCuts: staged in the warp's rb) or from the
+// coarse prefix (kTestCoarse: every position taken to the nearest multiple of
+// 2^clg); in units of the 32-bit prefix.
+__device__ __forceinline__ void first_test(const BoundDur& t, const int* __restrict__ pq, const float* coarse, int clg,
+                                           int at, int cnt, float* rb, int lane, float (&acc)[4])
 {
     const int st = t.st, d = t.d, test = t.test;
+    const int cuts4 = t.cuts4;
+    const float last = t.cut_last;
+    if (test == kTestCoarse) {
+        int s[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s[q] = (at + min(q * 32 + lane, cnt - 1)) * st + (1 << clg >> 1);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            acc[q] = last * coarse[at_coarse((s[q] + d) >> clg)];
+            acc[q] = fmaf(t.coef0, coarse[at_coarse(s[q] >> clg)], acc[q]);
+        }
+        for (int u = 0; u < cuts4; u += 4) {
+            const float4 w = *reinterpret_cast<const float4*>(t.coef + u);
+            const int4 r = *reinterpret_cast<const int4*>(t.row + u);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (q * 32 >= cnt) break;
+                acc[q] = fmaf(w.x, coarse[at_coarse((s[q] + r.x) >> clg)], acc[q]);
+                acc[q] = fmaf(w.y, coarse[at_coarse((s[q] + r.y) >> clg)], acc[q]);
+                acc[q] = fmaf(w.z, coarse[at_coarse((s[q] + r.z) >> clg)], acc[q]);
+                acc[q] = fmaf(w.w, coarse[at_coarse((s[q] + r.w) >> clg)], acc[q]);
+            }
+        }
+        return;
+    }
     const int* const a = pq + at * st;
     int i[4], v[4];
 #pragma unroll
@@ -293,9 +316,7 @@ __device__ __forceinline__ void first_test(const Dur& t, const int* __restrict__
         for (int q = 0; q < 4; ++q) acc[q] = q * 32 < cnt ? (float)(v[q] - a[i[q]]) : 0.0f;
         return;
     }
-    const int cuts4 = t.cuts4;
     const int base = a[0];
-    const float last = t.cut_last;
     if (test == kTestCuts) {
         const int nr = cnt + t.row_max;
         __syncwarp();   // the previous group's reads are done
@@ -311,11 +332,13 @@ __device__ __forceinline__ void first_test(const Dur& t, const int* __restrict__
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[q] = last * (float)(v[q] - base);
         const float* const b = rb + lane;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] = fmaf(t.coef0, b[q * 32], acc[q]);   // (past cnt: not used)
         for (int u = 0; u < cuts4; u += 4) {
             const float4 w = *reinterpret_cast<const float4*>(t.coef + u);
             const int4 r = *reinterpret_cast<const int4*>(t.row + u);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {   // (past cnt: not used)
+            for (int q = 0; q < 4; ++q) {
                 acc[q] = fmaf(w.x, b[r.x + q * 32], acc[q]);
                 acc[q] = fmaf(w.y, b[r.y + q * 32], acc[q]);
                 acc[q] = fmaf(w.z, b[r.z + q * 32], acc[q]);
@@ -324,83 +347,164 @@ __device__ __forceinline__ void first_test(const Dur& t, const int* __restrict__
         }
     } else {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[q] = last * (float)(v[q] - base);
+        for (int q = 0; q < 4; ++q) {
+            acc[q] = last * (float)(v[q] - base);
+            acc[q] = fmaf(t.coef0, (float)(a[i[q]] - base), acc[q]);
+        }
         for (int u = 0; u < cuts4; ++u) {
             const float w = t.coef[u];
-            const int* const b = a + t.row[u] * st;
+            const int* const b = a + t.row[u];
 #pragma unroll
             for (int q = 0; q < 4; ++q) acc[q] = fmaf(w, (float)(b[i[q]] - base), acc[q]);
         }
     }
 }
 
-static __global__ void __launch_bounds__(kThreads, kMinBlocks)
-k_window_bounds(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk, int buf)
+// One pass over the 32-bit prefix sums P[0 .. total]: block energies into
+// pre[] (from the differences of P, each off by at most a unit), the coarse
+// prefix, the largest |entry| of it, and the furthest any P is from the entry
+// its position is taken to.  A thread takes runs of 2^max(lb, clg) positions.
+template <int T>
+__device__ __forceinline__ void scan_prefix(Smem<T>& S, const int* __restrict__ pq, int total, int lb, int clg,
+                                            float unit)
 {
-    const SlotMap& sm = smq ? *smq : smv;
-    extern __shared__ unsigned int bound_smem[];
-    unsigned int* const sieve = bound_smem;                 // (duration, window) past the first test
-    float* const pre = reinterpret_cast<float*>(sieve + kSieve);   // energy prefix
-    float* const cmax = pre + kMaxBlocks + 8;               // largest first-test value per chunk
-    float* const row_buf = cmax + kMaxChunks;
-    __shared__ Dur dur[tiles::kMaxDur];
-    __shared__ Chunks s_ck;
-    __shared__ int s_next, s_sieved, s_listed;
-    __shared__ float s_wsum[kWarps], s_energy[kEnergyLens];
-    __shared__ float s_top[kWarps], s_c1[kWarps], s_s[kWarps], s_thr;
-    __shared__ int s_top_at[kWarps], s_cand[kCand];
+    const int lrun = max(lb, clg), run = 1 << lrun, bmask = (1 << lb) - 1, cstep = 1 << clg, half = cstep >> 1;
+    int dev = 0, big = 0;
+    if (lb == 3 && clg == 2) {
+        // the usual sizes: eight positions and the next one, which the next lane holds
+        const int lane = threadIdx.x & 31;
+#pragma unroll 3
+        for (int r0 = threadIdx.x * 8; r0 - lane * 8 + 256 <= total; r0 += T * 8) {   // whole warps
+            const int4 a = *reinterpret_cast<const int4*>(pq + r0), b = *reinterpret_cast<const int4*>(pq + r0 + 4);
+            int next = __shfl_down_sync(0xffffffffu, a.x, 1);
+            if (lane == 31) next = pq[r0 + 8];
+            const int v[9] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, next};
+            float e = 0.0f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const float x = (float)(abs(v[u + 1] - v[u]) + 1);
+                e = fmaf(x, x, e);
+            }
+            S.pre[r0 >> 3] = e * unit * unit;
+            S.coarse[at_coarse(r0 >> 2)] = (float)v[0];
+            S.coarse[at_coarse((r0 >> 2) + 1)] = (float)v[4];
+            big = max(big, max(abs(v[0]), abs(v[4])));
+            dev = max(dev, max(max(abs(v[1] - v[0]), abs(v[2] - v[4])), max(abs(v[3] - v[4]), abs(v[5] - v[4]))));
+            dev = max(dev, max(abs(v[6] - v[8]), abs(v[7] - v[8])));
+        }
+    }
+    // (the rest: what is not a whole warp's span above, or every position)
+    const int done = lb == 3 && clg == 2 ? total / 256 * 256 : 0;
+    for (int r0 = done + (threadIdx.x << lrun); r0 <= total; r0 += T << lrun) {
+        int cur = 0, lo = 0, hi = 0, prev = 0;
+        float e = 0.0f;
+        const int end = min(run, total - r0);   // last position of the run's span (inclusive)
+        for (int g0 = 0; g0 <= end; g0 += 4) {
+            // (the vector stays inside the padded array; values past `end` are not used)
+            const int4 v4 = *reinterpret_cast<const int4*>(pq + r0 + g0);
+            const int v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int g = g0 + u;
+                if (g > end) break;
+                if (g > 0) {
+                    const float x = (float)(abs(v[u] - prev) + 1);
+                    e = fmaf(x, x, e);
+                    if ((g & bmask) == 0) {   // the block before g ends here
+                        S.pre[(r0 + g - 1) >> lb] = e * unit * unit;
+                        e = 0.0f;
+                    }
+                }
+                prev = v[u];
+                const int in = g & (cstep - 1);
+                if (in == 0) {
+                    if (g > 0) dev = max(dev, max(abs(hi - v[u]), abs(lo - v[u])));
+                    cur = lo = hi = v[u];
+                    if (g < run) {
+                        S.coarse[at_coarse((r0 + g) >> clg)] = (float)v[u];
+                        big = max(big, abs(v[u]));
+                    }
+                } else if (in < half) {
+                    dev = max(dev, abs(v[u] - cur));
+                } else {
+                    // taken to the next entry: kept until that is known
+                    lo = in == half ? v[u] : min(lo, v[u]);
+                    hi = in == half ? v[u] : max(hi, v[u]);
+                }
+            }
+        }
+        if (end < run) {   // the curve ends inside this run
+            if ((end & bmask) != 0) S.pre[(r0 + end) >> lb] = e * unit * unit;
+            if ((end & (cstep - 1)) >= half) {   // and in the upper half of a step: its end is the entry
+                S.coarse[at_coarse(((r0 + end) >> clg) + 1)] = (float)prev;
+                big = max(big, abs(prev));
+                dev = max(dev, max(abs(hi - prev), abs(lo - prev)));
+            }
+        }
+    }
+    dev = __reduce_max_sync(0xffffffffu, dev);
+    big = __reduce_max_sync(0xffffffffu, big);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&S.dev, dev);
+        atomicMax(&S.big, big);
+    }
+}
+
+// Steps 1 to 4 for one period, by a CTA of T threads.
+template <int T>
+__device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet& ds, const DevChunk& dk, int slot, int lc,
+                                              int p, int buf)
+{
+    using M = Smem<T>;
+    constexpr int kWarps = T / 32;
+    M& S = *reinterpret_cast<M*>(smem);
+    Dur* const dur = S.dur;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int slot = blockIdx.x;
-    int lc, p;
-    if (!resolve_slot(ds, sm, slot, lc, p)) return;
     const DevPlan& dp = ds.plans[lc];
-    unsigned int* const check = ds.curves[lc].check;
     const float w_uni = (float)ds.curves[lc].scal[2];
     const int n = (int)dp.n;
     const int total = n + dp.dmax_p[p];
-    float* const rb = row_buf + warp * kRowBuf;
+    float* const rb = S.row_buf + warp * kRowBuf;
     const float* const rs = dk.rs + (int64_t)slot * dk.pad_stride;
     const int* const pq = dk.pq + (int64_t)slot * dk.pad_stride;
     const int shift = (int)ds.curves[lc].scal[3];
     const float unit = prefix_unit(shift);   // of the 32-bit prefix
+    const int lg = dp.bound_lg;
 
     if (warp == 0) {
-        list_durations(dp, check, p, n, dur, &s_ck, lane);
-        if (lane == 0) {
-            s_next = 0;
-            s_sieved = 0;
-            s_listed = 0;
-        }
+        list_durations(dp, ds.curves[lc].check, p, n, dur, S.ck, lane);
+        for (int k = lane; k < kEnergySpans; k += 32) S.energy[k] = 0.0f;
+        if (lane == 0) S.next = S.sieved = S.n_fin = S.n_listed = S.dev = S.big = 0;
     }
-    for (int i = threadIdx.x; i < kSieve; i += kThreads) sieve[i] = kNone;
-    // 1. energies: blocks of 2^lb points, their exclusive prefix
-    int lb = 3;
-    while (((total + (1 << lb) - 1) >> lb) > kMaxBlocks) ++lb;
-    const int bsize = 1 << lb, nb = (total + bsize - 1) >> lb;
-    for (int b = threadIdx.x; b < nb; b += kThreads) {
-        const float4* q = reinterpret_cast<const float4*>(rs + ((int64_t)b << lb));   // zeros follow the padded curve
-        float e0 = 0.0f, e1 = 0.0f, e2 = 0.0f, e3 = 0.0f;
-#pragma unroll 4
-        for (int k = 0; k < bsize / 4; ++k) {
-            const float4 v = q[k];
-            e0 = fmaf(v.x, v.x, e0);
-            e1 = fmaf(v.y, v.y, e1);
-            e2 = fmaf(v.z, v.z, e2);
-            e3 = fmaf(v.w, v.w, e3);
-        }
-        pre[b] = (e0 + e1) + (e2 + e3);
-    }
+    for (int i = threadIdx.x; i < M::kSieve; i += T) S.sieve[i] = kNone;
     __syncthreads();
-    const Chunks ck = s_ck;
+    const Chunks ck = S.ck;
     const int ndur = ck.ndur;
     {
-        constexpr int kPer = kMaxBlocks / kThreads;
+        // the plan's part of the durations
+        constexpr int kWords = sizeof(BoundDur) / 4;
+        for (int e = threadIdx.x; e < ndur * kWords; e += T) {
+            const int k = e / kWords, u = e - k * kWords;
+            if (u > 0)   // (word 0: j, set already)
+                reinterpret_cast<int*>(&dur[k].b)[u] =
+                    __ldg(reinterpret_cast<const int*>(dp.bound_durs + dur[k].b.j) + u);
+        }
+    }
+    // 1. energies: blocks of 2^lb points, their exclusive prefix
+    int lb = 3, clg = 2;
+    while (((total + (1 << lb) - 1) >> lb) > M::kMaxBlocks) ++lb;
+    while ((total >> clg) + 2 > M::kMaxCoarse) ++clg;
+    const int bsize = 1 << lb, nb = (total + bsize - 1) >> lb;
+    scan_prefix<T>(S, pq, total, lb, clg, unit);
+    __syncthreads();
+    {
+        constexpr int kPer = M::kMaxBlocks / T;
         const int b0 = threadIdx.x * kPer;
         float v[kPer], run = 0.0f;
 #pragma unroll
         for (int u = 0; u < kPer; ++u) {
             v[u] = run;
-            run += b0 + u < nb ? pre[b0 + u] : 0.0f;
+            run += b0 + u < nb ? S.pre[b0 + u] : 0.0f;
         }
         float x = run;
 #pragma unroll
@@ -408,70 +512,97 @@ k_window_bounds(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* s
             const float y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
-        if (lane == 31) s_wsum[warp] = x;
+        if (lane == 31) S.wsum[warp] = x;
         __syncthreads();
-        float base = 0.0f;
-        for (int w = 0; w < warp; ++w) base += s_wsum[w];
+        float base = lane < warp ? S.wsum[lane] : 0.0f;   // sums of the lower warps
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) base += __shfl_xor_sync(0xffffffffu, base, o);
         const float excl = __shfl_up_sync(0xffffffffu, x, 1);   // sums of the lower lanes
         base += lane > 0 ? excl : 0.0f;
 #pragma unroll
         for (int u = 0; u < kPer; ++u)
-            if (b0 + u <= nb) pre[b0 + u] = base + v[u];
-        if (b0 + kPer == nb && nb == kMaxBlocks) pre[nb] = base + run;
+            if (b0 + u <= nb) S.pre[b0 + u] = base + v[u];
+        if (b0 + kPer == nb && nb == M::kMaxBlocks) S.pre[nb] = base + run;
     }
     __syncthreads();
-    const float e_all = pre[nb];
+    const float e_all = S.pre[nb];
     // rounding of block sums and prefix: an energy E read from the prefix is
     // at most E (1 + e_rel) + e_abs
     const float e_rel = sum_slack(bsize), e_abs = sum_slack(bsize + 64) * e_all;
 
-    // largest energy of any stretch of a length (a warp per length; starts in
-    // blocks [i, i + step) reach `span` blocks further): a row of lengths
-    // sqrt(2) apart, and D of the durations that are tested by their sum
-    auto max_energy = [&](int len) {
-        const int span = (len + bsize - 2) >> lb;
-        const int step = max(1, (len >> lb) >> 3);
-        float best = 0.0f;
-        for (int i = lane * step; i < nb; i += 32 * step)
-            best = fmaxf(best, pre[min(nb, i + step + span)] - pre[i]);
+    // largest energy of any stretch that reaches `span` blocks past its first:
+    // spans 0 .. kShortSpans - 1, and from there a row of spans sqrt(2) apart
+    // (starts in blocks [i, i + step) taken together)
+    {
+        float best[kShortSpans];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-        return fmaf(best, 1.0f + e_rel, e_abs);
-    };
-    for (int k = warp; k < kEnergyLens + ndur; k += kWarps) {
-        if (k < kEnergyLens) {
-            const int len = (k & 1 ? 11 : 8) << (k >> 1);
-            const float e = len < 2 * total ? max_energy(len) : fmaf(e_all, 1.0f + e_rel, e_abs);
-            if (lane == 0) s_energy[k] = e;
-        } else if (dur[k - kEnergyLens].test == kTestSum) {
-            const float e = max_energy(dur[k - kEnergyLens].d);
-            if (lane == 0) dur[k - kEnergyLens].emax = e;
+        for (int q = 0; q < kShortSpans; ++q) best[q] = 0.0f;
+        for (int i = threadIdx.x; i < nb; i += T) {
+            const float from = S.pre[i];
+#pragma unroll
+            for (int q = 0; q < kShortSpans; ++q) best[q] = fmaxf(best[q], S.pre[min(nb, i + 1 + q)] - from);
+        }
+#pragma unroll
+        for (int q = 0; q < kShortSpans; ++q) {
+            // (not negative: as integers they are ordered the same)
+            const int top = __reduce_max_sync(0xffffffffu, __float_as_int(best[q]));
+            if (lane == 0) atomicMax(reinterpret_cast<int*>(S.energy + q), top);
+        }
+        for (int q = warp; q < kEnergySpans - kShortSpans; q += kWarps) {
+            const int span = (q & 1 ? (kShortSpans * 181) >> 7 : kShortSpans) << (q >> 1), step = max(1, span >> 3);
+            float top = span < nb ? 0.0f : e_all;
+            if (span < nb) {
+#pragma unroll 4
+                for (int i = lane * step; i < nb; i += 32 * step)
+                    top = fmaxf(top, S.pre[min(nb, i + step + span)] - S.pre[i]);
+            }
+            const int t = __reduce_max_sync(0xffffffffu, __float_as_int(top));
+            if (lane == 0) S.energy[kShortSpans + q] = __int_as_float(t);
         }
     }
-    // first of those lengths that is at least len
+    // upper bound of sum r^2 over any len points
     auto energy_of = [&](int len) {
-        const int o = 31 - __clz(max(len - 1, 1) >> 3);     // len - 1 in [8 << o, 16 << o) (o = -1: below 8)
-        if (len <= 8) return s_energy[0];
-        return s_energy[len <= (11 << o) ? 2 * o + 1 : 2 * o + 2];
+        const int span = (len + bsize - 2) >> lb;
+        int q = span;
+        if (span >= kShortSpans) {   // first of the long spans that is at least this one
+            const int o = 31 - __clz(max(span - 1, kShortSpans) / kShortSpans);   // kShortSpans << o <= max(span - 1, ..)
+            q = kShortSpans + 2 * o;
+            while (((q - kShortSpans) & 1 ? (kShortSpans * 181) >> 7 : kShortSpans) << ((q - kShortSpans) >> 1) < span) ++q;
+        }
+        return fmaf(S.energy[min(q, kEnergySpans - 1)], 1.0f + e_rel, e_abs);
     };
 
-    // 2. largest window sum of every chunk; each warp's most promising chunk
+    // 2. largest first-test value of every chunk; each warp's best group
     float top = -INFINITY;   // this lane's best estimate of C1 / sqrt(sum s_k^2)
     int top_at = 0;          // its duration and group of windows
     int top_cnt = 0;
     for (;;) {
         int c = 0;
-        if (lane == 0) c = atomicAdd(&s_next, 1);
+        if (lane == 0) c = atomicAdd(&S.next, 1);
         c = __shfl_sync(0xffffffffu, c, 0);
         if (c >= ck.total) break;
         int k, lo, hi;
-        chunk_range(ck, dur, c, lane, k, lo, hi);
-        const float lam = dur[k].lam;
+        chunk_range(ck, dur, lg, c, lane, k, lo, hi);
+        const float lam = dur[k].b.lam;
         float f = -INFINITY;
-        for (int at = lo; at < hi; at += kGroup) {
+        if (dur[k].b.test == kTestSum) {
+            // the largest sum of the chunk, in integers
+            const int st = dur[k].b.st, d = dur[k].b.d;
+            const int* a = pq + (lo + lane) * st;
+            int best = INT_MIN;
+#pragma unroll 4
+            for (int i = lo + lane; i < hi; i += 32, a += 32 * st) best = max(best, a[d] - a[0]);
+            if (best > INT_MIN) f = (float)best;
+            if (f * lam > top) {
+                top = f * lam;
+                top_at = (k << 24) | lo;
+                top_cnt = hi - lo;
+            }
+        }
+        for (int at = dur[k].b.test == kTestSum ? hi : lo; at < hi; at += kGroup) {
             float acc[4];
             const int cnt = min(kGroup, hi - at);
-            first_test(dur[k], pq, at, cnt, rb, lane, acc);
+            first_test(dur[k].b, pq, S.coarse, clg, at, cnt, rb, lane, acc);
             float g = -INFINITY;
 #pragma unroll
             for (int q = 0; q < 4; ++q) g = fmaxf(g, q * 32 + lane < cnt ? acc[q] : -INFINITY);
@@ -483,7 +614,7 @@ k_window_bounds(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* s
             }
         }
         f = float_from_order_key(__reduce_max_sync(0xffffffffu, float_order_key(f)));
-        if (lane == 0) cmax[c] = f;
+        if (lane == 0) S.cmax[c] = f;
     }
 
     // 3. threshold: the most promising windows of the warps, kWarps / kCand
@@ -494,37 +625,42 @@ k_window_bounds(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* s
         const float most = __shfl_sync(0xffffffffu, top, who);
         const int group = __shfl_sync(0xffffffffu, top_at, who), cnt = __shfl_sync(0xffffffffu, top_cnt, who);
         if (most > -INFINITY) {   // the group again: which of the lane's windows it was
-            float acc[4];
-            const Dur& t = dur[group >> 24];
-            first_test(t, pq, group & 0xffffff, cnt, rb, lane, acc);
-            int q = 0;
-            while (q < 3 && (q * 32 + lane >= cnt || acc[q] * t.lam != top)) ++q;
-            top_at = min(group + q * 32 + lane, group + cnt - 1);
+            const BoundDur& t = dur[group >> 24].b;
+            const int g0 = group & 0xffffff;
+            int found = -1;
+            for (int at = g0; at < g0 + cnt; at += kGroup) {   // (one group, or the chunk of a sum test)
+                float acc[4];
+                first_test(t, pq, S.coarse, clg, at, min(kGroup, g0 + cnt - at), rb, lane, acc);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (at + q * 32 + lane < g0 + cnt && acc[q] * t.lam == top) found = at + q * 32 + lane;
+            }
+            top_at = (group & ~0xffffff) | (found < 0 ? g0 : found);
         }
         if (lane == who) {
-            s_top[warp] = top;
-            s_top_at[warp] = top_at;
+            S.top[warp] = top;
+            S.top_at[warp] = top_at;
         }
-        if (threadIdx.x < kCand) s_cand[threadIdx.x] = -1;
+        if (threadIdx.x < kCand) S.cand[threadIdx.x] = -1;
     }
     __syncthreads();
     if (threadIdx.x < kWarps) {
-        const float v = s_top[threadIdx.x];
+        const float v = S.top[threadIdx.x];
         int rank = 0;
         for (int w = 0; w < kWarps; ++w)
-            rank += s_top[w] > v || (s_top[w] == v && w < (int)threadIdx.x) ? 1 : 0;
-        if (rank < kCand && v > -INFINITY) s_cand[rank] = s_top_at[threadIdx.x];
+            rank += S.top[w] > v || (S.top[w] == v && w < (int)threadIdx.x) ? 1 : 0;
+        if (rank < kCand && v > -INFINITY) S.cand[rank] = S.top_at[threadIdx.x];
     }
     __syncthreads();
     constexpr int kTeam = kWarps / kCand, kTeamThreads = kTeam * 32;
     {
-        const int cand = s_cand[warp / kTeam];
+        const int cand = S.cand[warp / kTeam];
         float c1 = 0.0f, sum = 0.0f;
         if (cand >= 0) {
-            const Dur& t = dur[cand >> 24];
+            const BoundDur& t = dur[cand >> 24].b;
             const float* const r = rs + (cand & 0xffffff) * t.st;
             const float* const s = dp.tmpl + dp.tmpl_off[t.j];
-#pragma unroll 4
+#pragma unroll 8
             for (int i = threadIdx.x % kTeamThreads; i < t.d; i += kTeamThreads) {
                 const float v = r[i];
                 c1 = fmaf(v, __ldg(s + i), c1);
@@ -537,30 +673,30 @@ k_window_bounds(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* s
             sum += __shfl_xor_sync(0xffffffffu, sum, o);
         }
         if (lane == 0) {
-            s_c1[warp] = c1;
-            s_s[warp] = sum;
+            S.c1[warp] = c1;
+            S.s[warp] = sum;
         }
     }
     __syncthreads();
     if (threadIdx.x == 0) {
         float thr = INFINITY;
         for (int q = 0; q < kCand; ++q) {
-            if (s_cand[q] < 0) continue;
-            const int j = dur[s_cand[q] >> 24].j;
+            if (S.cand[q] < 0) continue;
+            const int j = dur[S.cand[q] >> 24].b.j;
             float c1 = 0.0f, sum = 0.0f;
             for (int w = q * kTeam; w < (q + 1) * kTeam; ++w) {
-                c1 += s_c1[w];
-                sum += s_s[w];
+                c1 += S.c1[w];
+                sum += S.s[w];
             }
             const float depth = fmaxf(0.0f, sum * dp.inv_sum_t[j]);
             const float v = w_uni * depth * fmaf(depth, dp.sum_t2[j], -2.0f * c1);
             thr = v < thr || isnan(v) ? v : thr;
         }
-        s_thr = thr;
-        s_next = 0;
+        S.thr = thr;
+        S.next = 0;
     }
     __syncthreads();
-    const float thr = s_thr;
+    const float thr = S.thr;
     // no negative delta-chi2, or values out of range: the tiled kernel decides
     const bool sane = thr < 0.0f && thr > -INFINITY && e_all < INFINITY && w_uni < INFINITY && shift < 64;
     if (sane) {
@@ -571,26 +707,36 @@ k_window_bounds(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* s
         // row) ||r|| ||s||, 2^-41 of fixed point per point, and the prefix
         // units of the sums)
         const float reach = sqrtf(-thr / w_uni) * (1.0f - 1e-4f);
-        for (int k = threadIdx.x; k < ndur; k += kThreads) {
+        for (int k = threadIdx.x; k < ndur; k += T) {
             Dur& t = dur[k];
-            const BoundTab& bt = dp.bounds[t.j];
-            const int nc = 1 << t.lg_nc;
-            const int chain = ((t.st + nc - 1) >> t.lg_nc) * ((t.d + t.st - 1) / t.st) + 6;
-            if (t.test != kTestSum) t.emax = energy_of(t.d);
-            const float norm = sqrtf((float)t.d * t.emax);
-            const float lost = (sum_slack(chain) + 8e-6f) * norm + (float)t.d * 1e-12f;
+            const BoundTab& bt = dp.bounds[t.b.j];
+            const int nc = 1 << t.b.lg_nc, d = t.b.d, st = t.b.st;
+            const int chain = ((st + nc - 1) >> t.b.lg_nc) * ((d + st - 1) / st) + 6;
+            t.emax = energy_of(d);
+            const float norm = sqrtf((float)d * t.emax);
+            const float lost = (sum_slack(chain) + 8e-6f) * norm + (float)d * 1e-12f;
             t.cmin = reach * bt.root_t2 - (lost + (float)(kBoundSegs + 1) * unit) * bt.t_max;
+            t.blur = ((sum_slack(chain) + sum_slack(d / 32 + 8)) * norm + (float)d * 1e-12f) * fmaxf(bt.t_max, 1.0f);
             // depth is zero without a positive sum (exact, or FP32 for the pairs)
-            const float low = (t.mode == kModePairS ? -lost : 0.0f) - 2.0f * unit;
+            const float low = (t.b.mode == kModePairS ? -lost : 0.0f) - 2.0f * unit;
             float c0;
-            if (t.test == kTestSum) {
+            if (t.b.test == kTestSum) {
                 c0 = fmaxf((t.cmin - bt.nu_all * sqrtf(t.emax)) / bt.mean_all, low);
             } else {
                 float lose = 0.0f;
                 for (int u = 0; u < bt.cuts; ++u) lose = fmaf(bt.cut_nu[u], sqrtf(energy_of(bt.cut_len[u])), lose);
-                // rounding of the prefix sums, which reach over the whole group
-                const float over = (float)(kGroup * t.st) / (float)t.d + 2.0f;
-                c0 = t.cmin - lose - 1.2e-7f * (float)(bt.cuts + 4) * 2.0f * over * norm * bt.t_max;
+                if (t.b.test == kTestCoarse) {
+                    // every position is off by at most S.dev in its prefix
+                    // sum; the coarse entries are rounded to FP32
+                    lose = fmaf(bt.cut_jumps * unit, (float)S.dev + 1.2e-7f * (float)(bt.cuts + 4) * (float)S.big, lose);
+                    t.cmin_coarse = t.cmin - bt.seg_jumps * unit *
+                                                 ((float)S.dev + 1.2e-7f * (float)(2 * kBoundSegs + 4) * (float)S.big);
+                } else {
+                    // rounding of the prefix sums, which reach over the whole group
+                    const float over = (float)(kGroup * st) / (float)d + 2.0f;
+                    lose += 1.2e-7f * (float)(bt.cuts + 4) * 2.0f * over * norm * bt.t_max;
+                }
+                c0 = t.cmin - lose;
             }
             t.first_min = (c0 - 1e-5f * fabsf(c0)) / unit;
             t.smin = low / unit;
@@ -598,21 +744,21 @@ k_window_bounds(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* s
     }
     __syncthreads();
 
-    // 4. windows that may hold the minimum: chunks whose largest sum passes,
-    // their windows by sum or rows into the sieve, those by segments into the
-    // queues; a full sieve is emptied before the walk goes on
+    // 4. windows that may hold the minimum: chunks whose largest value passes,
+    // their windows by the first test into the sieve, those by segments into
+    // the final list; a full sieve is emptied before the walk goes on
     int c = -1, k = 0, at = 0, hi = 0;
     while (sane) {
         for (;;) {
             if (c < 0) {
-                if (lane == 0) c = atomicAdd(&s_next, 1);
+                if (lane == 0) c = atomicAdd(&S.next, 1);
                 c = __shfl_sync(0xffffffffu, c, 0);
                 if (c >= ck.total) {
                     c = -1;
                     break;
                 }
-                chunk_range(ck, dur, c, lane, k, at, hi);
-                if (cmax[c] < dur[k].first_min) {
+                chunk_range(ck, dur, lg, c, lane, k, at, hi);
+                if (S.cmax[c] < dur[k].first_min) {
                     c = -1;
                     continue;
                 }
@@ -622,30 +768,26 @@ k_window_bounds(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* s
             for (; at < hi; at += kGroup) {
                 const int cnt = min(kGroup, hi - at);
                 float acc[4];
-                first_test(dur[k], pq, at, cnt, rb, lane, acc);
-                unsigned int pass = 0;
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (q * 32 + lane < cnt && !(acc[q] < first_min)) pass |= 1u << q;
+                first_test(dur[k].b, pq, S.coarse, clg, at, cnt, rb, lane, acc);
                 unsigned int vote[4];
                 int sum = 0;
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    vote[q] = __ballot_sync(0xffffffffu, (pass >> q) & 1u);
+                    vote[q] = __ballot_sync(0xffffffffu, q * 32 + lane < cnt && !(acc[q] < first_min));
                     sum += __popc(vote[q]);
                 }
                 if (sum == 0) continue;
                 int pos = 0;
-                if (lane == 0) pos = atomicAdd(&s_sieved, sum);
+                if (lane == 0) pos = atomicAdd(&S.sieved, sum);
                 pos = __shfl_sync(0xffffffffu, pos, 0);
-                if (pos + sum > kSieve) {   // the group is tested again after the sieve is emptied
+                if (pos + sum > M::kSieve) {   // the group is tested again after the sieve is emptied
                     full = true;
                     break;
                 }
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    if ((pass >> q) & 1u)
-                        sieve[pos + __popc(vote[q] & ((1u << lane) - 1u))] =
+                    if ((vote[q] >> lane) & 1u)
+                        S.sieve[pos + __popc(vote[q] & ((1u << lane) - 1u))] =
                             ((unsigned int)k << 24) | (unsigned int)(at + q * 32 + lane);
                     pos += __popc(vote[q]);
                 }
@@ -654,55 +796,118 @@ k_window_bounds(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* s
             c = -1;
         }
         __syncthreads();
-        const int sieved = min(s_sieved, kSieve);
-        for (int i = threadIdx.x; i < sieved; i += kThreads) {
-            const unsigned int e = sieve[i];
-            sieve[i] = kNone;
+        const int sieved = min(S.sieved, M::kSieve);
+        for (int i = threadIdx.x; i < sieved; i += T) {
+            const unsigned int e = S.sieve[i];
+            S.sieve[i] = kNone;
             if (e == kNone) continue;
             const int kk = e >> 24, m = e & 0xffffffu;
             const Dur& t = dur[kk];
-            const int s = m * t.st;
-            const int p0 = pq[s];
-            if ((float)(pq[s + t.d] - p0) < t.smin) continue;
-            {
-                const BoundTab& bt = dp.bounds[t.j];
-                float c1 = 0.0f;
-                int last = p0, e0 = s;
+            const int s = m * t.b.st;
+            const float4* const seg = dp.bounds[t.b.j].seg;
+            if (t.b.test == kTestCoarse) {
+                // the same bound from the coarse prefix first: no global reads
+                const int s1 = s + (1 << clg >> 1);
+                float c1 = 0.0f, from = S.coarse[at_coarse(s1 >> clg)];
+                int e0 = s;
 #pragma unroll 5
                 for (int g = 0; g < kBoundSegs; ++g) {
-                    const int e1 = s + __ldg(bt.off + g + 1);
-                    const int nx = pq[e1];
-                    const float sg = (float)(nx - last) * unit;
-                    const float en = fmaf(pre[(e1 + bsize - 1) >> lb] - pre[e0 >> lb], 1.0f + e_rel, e_abs);
-                    const float len = __ldg(bt.inv_len + g) * fmaxf(fabsf(sg) - unit, 0.0f) * fmaxf(fabsf(sg) - unit, 0.0f);
-                    c1 += fmaf(__ldg(bt.mean + g), sg, __ldg(bt.nu + g) * root(en - len));
-                    last = nx;
-                    e0 = e1;
+                    const float4 q = __ldg(seg + g);
+                    const int off = __float_as_int(q.x);
+                    const float to = S.coarse[at_coarse((s1 + off) >> clg)];
+                    const float en = fmaf(S.pre[(s + off + bsize - 1) >> lb] - S.pre[e0 >> lb], 1.0f + e_rel, e_abs);
+                    c1 = fmaf(q.y, (to - from) * unit, fmaf(q.z, root(en), c1));
+                    from = to;
+                    e0 = s + off;
                 }
-                if (c1 < t.cmin) continue;
+                if (c1 < t.cmin_coarse) continue;
             }
+            int last = pq[s], e0 = s;
+            if ((float)(pq[s + t.b.d] - last) < t.smin) continue;
+            float c1 = 0.0f;
+#pragma unroll 5
+            for (int g = 0; g < kBoundSegs; ++g) {
+                const float4 q = __ldg(seg + g);   // end, mean, nu, 1 / length
+                const int e1 = s + __float_as_int(q.x);
+                const int nx = pq[e1];
+                const float sg = (float)(nx - last) * unit;
+                const float en = fmaf(S.pre[(e1 + bsize - 1) >> lb] - S.pre[e0 >> lb], 1.0f + e_rel, e_abs);
+                const float sm = fmaxf(fabsf(sg) - unit, 0.0f);
+                c1 += fmaf(q.y, sg, q.z * root(en - q.w * sm * sm));
+                last = nx;
+                e0 = e1;
+            }
+            if (c1 < t.cmin) continue;
+            const int to = atomicAdd(&S.n_fin, 1);
+            if (to < M::kFinal) S.fin[to] = e;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) S.sieved = 0;
+        if (!__syncthreads_or(c >= 0)) break;
+    }
+    // their sums (a warp each, any order): v - err <= delta-chi2 <= v + err,
+    // whatever the order of the products
+    const int nfin = sane ? S.n_fin : 0;   // (final after the last barrier)
+    bool fits = sane && nfin <= M::kFinal;
+    if (fits) {
+        float best = INFINITY;   // lowest upper end
+        bool odd = false;        // a sum that is not finite
+        for (int i = warp; i < nfin; i += kWarps) {
+            const unsigned int e = S.fin[i];
+            const Dur& t = dur[e >> 24];
+            const int s = (int)(e & 0xffffffu) * t.b.st, d = t.b.d;
+            const float* const r = rs + s;
+            const float* const tm = dp.tmpl + dp.tmpl_off[t.b.j];
+            const long long* const pf = dk.pf + (int64_t)slot * dk.pad_stride + s;
+            const long long sfx = pf[d] - pf[0];
+            float c1 = 0.0f;
+#pragma unroll 16
+            for (int q = lane; q < d; q += 32) c1 = fmaf(r[q], __ldg(tm + q), c1);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) c1 += __shfl_xor_sync(0xffffffffu, c1, o);
+            const float inv = dp.inv_sum_t[t.b.j], t2 = dp.sum_t2[t.b.j];
+            const float depth = fmaxf(0.0f, tiles::fixed_to_float(sfx) * (inv * (1.0f / 1099511627776.0f)));
+            const float v = w_uni * depth * fmaf(depth, t2, -2.0f * c1);
+            // C1 is off by at most blur, the depth of the pairs by blur / sum s_k
+            const float off = t.blur, dd = t.b.mode == kModePairS ? off * inv : 0.0f;
+            const float err = w_uni * (2.0f * (depth + dd) * off + 2.0f * dd * fabsf(fmaf(depth, t2, -c1)) + dd * dd * t2) +
+                              1e-6f * fabsf(v) + 2e-6f * w_uni * depth * fabsf(c1);
+            if (lane == 0) S.fin_v[i] = v - err;
+            odd = odd || !(v - err > -INFINITY && v + err < INFINITY);
+            best = fminf(best, v + err);
+        }
+        if (lane == 0) S.top[warp] = best;
+        fits = !__syncthreads_or(odd);
+        best = lane < kWarps ? S.top[lane] : INFINITY;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+        for (int i = threadIdx.x; i < nfin && fits; i += T) {
+            if (S.fin_v[i] > best) continue;
+            const unsigned int e = S.fin[i];
+            const Dur& t = dur[e >> 24];
+            const int m = (int)(e & 0xffffffu);
             auto push = [&](int rot) {
                 const unsigned int to =
-                    atomicAdd(&s_listed, 1) < kListed ? atomicAdd(dk.left_n + t.lg_nc, 1u) : 0xffffffffu;
+                    atomicAdd(&S.n_listed, 1) < kListed ? atomicAdd(dk.left_n + t.b.lg_nc, 1u) : 0xffffffffu;
                 if (to < dk.list_cap)
-                    dk.list[t.lg_nc * dk.list_cap + to] = ((unsigned long long)slot << 40) |
-                                                          ((unsigned long long)t.j << 32) |
-                                                          ((unsigned long long)rot << 24) | (unsigned long long)m;
+                    dk.list[t.b.lg_nc * dk.list_cap + to] = ((unsigned long long)slot << 40) |
+                                                            ((unsigned long long)t.b.j << 32) |
+                                                            ((unsigned long long)rot << 24) | (unsigned long long)m;
                 else
-                    s_listed = 2 * kListed;   // (more may be added: it stays above kListed)
+                    S.n_listed = 2 * kListed;   // (more may be added: it stays above kListed)
             };
-            if (t.mode != kModeRot) {
+            if (t.b.mode != kModeRot) {
                 push(0);
                 continue;
             }
             // every block of the tiled kernel that covers window m, with its first round
-            const int nc = 1 << t.lg_nc, rounds = (t.st + 2 * nc - 1) >> (t.lg_nc + 1), blocks = 32 >> t.lg_nc;
+            const int nc = 1 << t.b.lg_nc, st = t.b.st, rounds = (st + 2 * nc - 1) >> (t.b.lg_nc + 1);
+            const int blocks = 32 >> t.b.lg_nc;
             auto push_block = [&](int b) { push(b % blocks % rounds); };
             const DevTiles tl = ds.tiles[lc];
             for (int tau = 0; tau < tl.count; ++tau) {
-                const tiles::TileSpan sp =
-                    tiles::tile_span(t.st, (t.d + t.st - 1) / t.st, 16, 16 * blocks, t.m_total, tau * tl.len, tl.len,
-                                     tau, tl.count, buf);
+                const tiles::TileSpan sp = tiles::tile_span(st, (t.b.d + st - 1) / st, 16, 16 * blocks, t.b.m_total,
+                                                            tau * tl.len, tl.len, tau, tl.count, buf);
                 const int nblk = (sp.m_b - sp.m_a + 15) / 16;
                 if (nblk <= 0) continue;
                 const int clamped = sp.hi_start < sp.m_a ? 0 : (sp.hi_start - sp.m_a) / 16 + 1;
@@ -714,56 +919,64 @@ k_window_bounds(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* s
             }
         }
         __syncthreads();
-        if (threadIdx.x == 0) s_sieved = 0;
-        if (!__syncthreads_or(c >= 0)) break;
+        fits = fits && S.n_listed <= kListed;
     }
-    __syncthreads();
-    if (!sane || s_listed > kListed) {   // block-uniform
-        if (threadIdx.x == 0) {
-            const int tc = ds.tiles[lc].count;
-            const unsigned int to = atomicAdd(dk.left_n + kListClasses, (unsigned int)tc);
-            for (int tau = 0; tau < tc; ++tau) dk.dense[to + tau] = make_int2(slot, tau);
-        }
+    if (!fits && threadIdx.x == 0) {
+        const int tc = ds.tiles[lc].count;
+        const unsigned int to = atomicAdd(dk.left_n + kListClasses, (unsigned int)tc);
+        for (int tau = 0; tau < tc; ++tau) dk.dense[to + tau] = make_int2(slot, tau);
     }
 }
 
-// 5. exact sums of the listed windows: groups of nc lanes, the lists of the
-// six group sizes one after the other.
-static __global__ void __launch_bounds__(kExactThreads)
-k_window_exact(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk)
+// 5. exact sums of the listed windows: one window per CTA of a warp at a time,
+// its points and its template staged in shared memory first (`room` floats
+// each; longer ones are read in place), because the chain of products would
+// wait for every row's loads (170 us per wave instead of 30).
+static __global__ void __launch_bounds__(32)
+k_window_exact(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk, int room)
 {
     const SlotMap& sm = smq ? *smq : smv;
-    const int lane = threadIdx.x & 31;
-    const int warps = gridDim.x * (kExactThreads / 32);
-    int item = blockIdx.x * (kExactThreads / 32) + (threadIdx.x >> 5);
+    extern __shared__ float exact_smem[];
+    const int lane = threadIdx.x;
+    int item = blockIdx.x;
     for (int q = 0; q < kListClasses; ++q) {
-        const unsigned int cnt = (unsigned int)min((int64_t)dk.left_n[q], dk.list_cap);
-        const int groups = 32 >> q, items = (int)((cnt + groups - 1) / groups);
-        for (; item < items; item += warps) {
-            const unsigned int e = (unsigned int)item * groups + (lane >> q);
-            const unsigned long long en = dk.list[q * dk.list_cap + min(e, cnt - 1)];
+        const int cnt = (int)min((int64_t)dk.left_n[q], dk.list_cap);
+        for (; item < cnt; item += gridDim.x) {
+            const unsigned long long en = dk.list[q * dk.list_cap + item];
             const int slot = (int)(en >> 40), j = (int)(en >> 32) & 0xff, rot = (int)(en >> 24) & 0xff;
             const int m = (int)(en & 0xffffffull);
             int lc, p;
-            const bool on = resolve_slot(ds, sm, slot, lc, p) && e < cnt;
-            if (!on) lc = p = 0;
+            if (!resolve_slot(ds, sm, slot, lc, p)) continue;   // warp-uniform
             const DevPlan& dp = ds.plans[lc];
             const int d = dp.dpts[j], st = dp.stride[j], v = dp.cfg_variant[j];
             const int mode = v == tiles::kScalar15 ? kModePairS
                              : v == tiles::kCol16R || tiles::variant_colpair(v) ? kModeCols : kModeWin;
             const int64_t base = (int64_t)slot * dk.pad_stride + (int64_t)m * st;
-            const float2 sum = window_sum(dk.rs + base, dp.tmpl + dp.tmpl_off[j], d, st, q, mode, rot, on, lane);
-            if (!on || (lane & ((1 << q) - 1)) != 0) continue;
+            const float* r = dk.rs + base;
+            const float* t = dp.tmpl + dp.tmpl_off[j];
+            const long long sfx = dk.pf[base + d] - dk.pf[base];
+            if (d <= room) {
+                __syncwarp();
+                for (int k = lane; k < d; k += 32) {
+                    const uint32_t to = (uint32_t)__cvta_generic_to_shared(exact_smem + k);
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to), "l"(r + k) : "memory");
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to + room * 4), "l"(t + k) : "memory");
+                }
+                asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+                __syncwarp();
+            }
+            const float2 sum = d <= room ? window_sum(exact_smem, exact_smem + room, d, st, q, mode, rot, lane < (1 << q), lane)
+                                         : window_sum(r, t, d, st, q, mode, rot, lane < (1 << q), lane);
+            if (lane != 0) continue;
             const float inv = dp.inv_sum_t[j];
-            const float depth =
-                fmaxf(0.0f, mode == kModePairS
-                                ? sum.y * inv
-                                : tiles::fixed_to_float(dk.pf[base + d] - dk.pf[base]) * (inv * (1.0f / 1099511627776.0f)));
+            const float depth = fmaxf(0.0f, mode == kModePairS
+                                                ? sum.y * inv
+                                                : tiles::fixed_to_float(sfx) * (inv * (1.0f / 1099511627776.0f)));
             const float w_uni = (float)ds.curves[lc].scal[2];
             atomicMin(&ds.outs[lc].best[p],
                       tiles::window_key(w_uni * depth * fmaf(depth, dp.sum_t2[j], -2.0f * sum.x), j, m));
         }
-        item -= items;
+        item -= cnt;
     }
 }
 
