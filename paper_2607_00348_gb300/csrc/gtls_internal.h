@@ -18,6 +18,7 @@ namespace gtls {
 constexpr int kBoundCuts = 17;
 constexpr int kBoundCutSlots = kBoundCuts - 1;   // the first one starts at 0 and is kept apart
 constexpr int kBoundSegs = 25;
+constexpr int kBoundLevels = 6;
 struct alignas(16) BoundTab {
     float4 seg[kBoundSegs];       // end (point, integer bits), mean of s_k, >= ||s_k - mean||, <= 1 / length
     float mean_all, nu_all;       // mean of s_k over the template, >= ||s_k - mean||
@@ -27,6 +28,11 @@ struct alignas(16) BoundTab {
     float cut_jumps, seg_jumps;   // sums of |mean - mean before| over the wide pieces, the segments
     float cut_nu[kBoundCuts];     // >= ||s_k - mean|| over the piece
     int32_t cut_len[kBoundCuts];  // its points
+    // per-point weights: sum w s_k^2 >= sum_l lev_up (smallest sum of w over
+    // lev_len points), and the smallest s_k^2 of every segment
+    int32_t lev_len[kBoundLevels];
+    float lev_up[kBoundLevels];
+    float seg_low[kBoundSegs];
 };
 
 // What the bounds need of one duration for every period (staged in shared
@@ -100,7 +106,8 @@ struct DevCurve {
     int64_t* d_lat;           // rint((t - t_ref) 2^e)
     float* d_f;               // float(t - t_ref) (days): coarse cycle estimate
     PointVals* pv;            // rfx, r, w of every point
-    double* scal;             // [0] t_ref [1] chi2_0 [2] uniform weight w (0 if not uniform) [3] prefix shift
+    double* scal;             // [0] t_ref [1] chi2_0 [2] uniform weight w (0 if not uniform) [3] prefix shift (per-point
+                              // weights: [3], [4] exponents of the units of the w r and w prefix sums)
     unsigned long long* tmin_key;  // ordered key of min(t)
     unsigned int* flags;      // bit0 non-finite, bit1 dy <= 0, bit2 dy not uniform
     double* part;             // block partials of chi2_0
@@ -221,6 +228,7 @@ struct gtls_plan {
     // its counter, and the timeout test (a wait that nothing completes)
     bool has_tensor = false;
     bool bounds_ok = false;              // the templates admit the bounds of window_bounds.cuh
+    bool bounds_w_ok = false;            // ... with per-point weights
     int tc_jspan = 0;
     unsigned int* tc_counter = nullptr;
     int tc_test_wait = 0;

@@ -80,6 +80,7 @@ constexpr int kRankBatch = 2;         // keys a fold thread ranks before issuing
 constexpr int kScanPer = 8;           // consecutive prefix-sum positions per fold thread
 constexpr int kWeightedTilePairs = 24576;   // (w r, w) pairs staged per tile with per-point weights
 constexpr int kSearchThreads = 256;
+constexpr int kPrepBlocks = 1024;     // blocks per curve of its preparation, at most
 constexpr double kBoundsMinWpe = 5e8;  // window-point products of a search from which windows are ruled out by bounds
 constexpr int64_t kListPerSlot = 128;  // windows to sum per period and lane-group size a chunk has room for
 constexpr int kMedianThreads = 1024;
@@ -244,11 +245,19 @@ __device__ __forceinline__ int prefix_shift(double chi2_0, double w, int64_t n)
 
 __device__ __forceinline__ float prefix_unit(int shift) { return ldexpf(1.0f, shift - 40); }
 
+// Per-point weights: exponent of the unit of 32-bit prefix sums that stay
+// below 2^29 units over the curve (`most` bounds its sum of absolute values);
+// kNoUnit where that leaves FP32.
+__device__ __forceinline__ int prefix_exponent(double most)
+{
+    return most > 1e-25 && most < 1e25 ? ilogb(most) - 28 : 1000;
+}
+
 // Work size of the per-curve preparation kernels for n points.
 __host__ __device__ __forceinline__ int prep_blocks_for(int64_t n)
 {
     const int64_t b = (n + 255) / 256;
-    return (int)(b < 1024 ? b : 1024);
+    return (int)(b < kPrepBlocks ? b : kPrepBlocks);
 }
 
 }  // namespace
@@ -313,7 +322,7 @@ __global__ void k_curve_prep(const double* __restrict__ t, const double* __restr
                              const double* __restrict__ dy, const int64_t* __restrict__ off,
                              DevSet ds, int lc0)
 {
-    __shared__ double red[32];
+    __shared__ double red[32], red_w[32];
     const int lc = lc0 + blockIdx.y;
     const int64_t o = off[lc], n = off[lc + 1] - o;
     const int nb = prep_blocks_for(n);
@@ -325,7 +334,7 @@ __global__ void k_curve_prep(const double* __restrict__ t, const double* __restr
     const int e = ds.plans[lc].time_exponent;
     const double t_ref = double_from_order_key(*dc.tmin_key);
     const double scale = ldexp(1.0, e);
-    double acc = 0.0;
+    double acc = 0.0, wacc = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)nb * blockDim.x) {
         const double dt = t[i] - t_ref;
         const double r = 1.0 - y[i];
@@ -334,15 +343,23 @@ __global__ void k_curve_prep(const double* __restrict__ t, const double* __restr
         dc.d_f[i] = (float)dt;
         dc.pv[i] = PointVals{__double2ll_rn(r * kRScale), (float)r, (float)w};
         acc += w * r * r;
+        wacc += w;
     }
 #pragma unroll
-    for (int o2 = 16; o2 > 0; o2 >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o2);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    for (int o2 = 16; o2 > 0; o2 >>= 1) {
+        acc += __shfl_xor_sync(0xffffffffu, acc, o2);
+        wacc += __shfl_xor_sync(0xffffffffu, wacc, o2);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        red[threadIdx.x >> 5] = acc;
+        red_w[threadIdx.x >> 5] = wacc;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 64 && (threadIdx.x & 31) == 0) {
+        const double* const from = threadIdx.x == 0 ? red : red_w;
         double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        dc.part[blockIdx.x] = s;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += from[w];
+        dc.part[blockIdx.x + (threadIdx.x == 0 ? 0 : kPrepBlocks)] = s;
     }
 }
 
@@ -357,13 +374,18 @@ __global__ void k_curve_reduce(const double* __restrict__ dy, const int64_t* __r
     const int64_t o = off[lc], n = off[lc + 1] - o;
     const DevCurve dc = ds.curves[lc];
     const int nparts = prep_blocks_for(n);
-    double s = 0.0;
-    for (int i = 0; i < nparts; ++i) s += dc.part[i];
+    double s = 0.0, sum_w = 0.0;
+    for (int i = 0; i < nparts; ++i) {
+        s += dc.part[i];
+        sum_w += dc.part[kPrepBlocks + i];
+    }
     const unsigned int fl = *dc.flags;
     dc.scal[0] = double_from_order_key(*dc.tmin_key);
     dc.scal[1] = s;
     dc.scal[2] = (fl & 4u) ? 0.0 : 1.0 / (dy[o] * dy[o]);
-    dc.scal[3] = (fl & 4u) ? 0.0 : (double)prefix_shift(s, dc.scal[2], n);
+    // (sum |w r| <= sqrt(sum w sum w r^2))
+    dc.scal[3] = (fl & 4u) ? (double)prefix_exponent(sqrt(sum_w * s)) : (double)prefix_shift(s, dc.scal[2], n);
+    dc.scal[4] = (double)prefix_exponent(sum_w);
     flags_out[lc] = fl;
 }
 
@@ -423,6 +445,10 @@ __host__ __device__ __forceinline__ int fold_threads(int64_t n)
 {
     return n <= FoldCfg<256>::kSegKeys ? 256 : n <= FoldCfg<512>::kSegKeys ? 512 : 1024;
 }
+
+// What follows the fold in its kernel: nothing, or the window search by bounds
+// for uniform or per-point weights.
+enum class Fold { kPlain, kBounds, kBoundsW };
 
 struct FoldOut {
     int32_t* sidx;
@@ -515,10 +541,11 @@ __device__ __forceinline__ void fold_scan_run(const long long* srfx, uint32_t le
 
 // Staged path; false when a super-bucket holds more than kFoldSegKeys
 // points (only keys have been written then).
-template <bool kBounded, int T>
+template <Fold kFold, int T>
 __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCurve& dc, int p,
                             unsigned long long* keys, const FoldOut& o)
 {
+    constexpr bool kBounded = kFold == Fold::kBounds, kBoundedW = kFold == Fold::kBoundsW;
     const int64_t n = dp.n;
     const long long P = dp.p_lat[p];
     const float inv_p = dp.inv_p[p];
@@ -733,9 +760,12 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
                 // what window_bounds reads right here)
                 __stcs(o.sidx + g, id[j]);
                 if (kBounded) o.rs[g] = pv[j].r;
-                else __stcs(o.rs + g, pv[j].r);
+                else if (!kBoundedW) __stcs(o.rs + g, pv[j].r);
                 srfx[swz(i)] = pv[j].rfx;
-                if (!o.uniform) {
+                if (kBoundedW) {
+                    o.ws[g] = pv[j].w;
+                    o.wrs[g] = pv[j].w * pv[j].r;
+                } else if (!kBounded && !o.uniform) {
                     __stcs(o.ws + g, pv[j].w);
                     __stcs(o.wrs + g, pv[j].w * pv[j].r);
                 }
@@ -935,12 +965,11 @@ __device__ void fold_global(unsigned char* smem, const DevPlan& dp, const DevCur
     }
 }
 
-// kBounded: the window search is the one by bounds (uniform weights), whose
-// first steps follow here.
-template <bool kBounded, int T>
+template <Fold kFold, int T>
 __global__ void __launch_bounds__(T, kFoldThreads * kFoldMinBlocks / T)
 k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk, int tile_buf)
 {
+    constexpr bool kBounded = kFold == Fold::kBounds, kBoundedW = kFold == Fold::kBoundsW;
     const SlotMap& sm = smq ? *smq : smv;
     extern __shared__ unsigned char smem[];
     const int slot_id = blockIdx.x;
@@ -960,11 +989,11 @@ k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, 
     o.shift = kBounded ? min((int)dc.scal[3], 63) : 0;
     if (threadIdx.x == 0) {
         ds.outs[lc].best[p] = ~0ull;
-        if (kBounded && slot_id == 0)
+        if (kFold != Fold::kPlain && slot_id == 0)
             for (int q = 0; q <= kListClasses; ++q) dk.left_n[q] = 0u;
     }
 
-    bool staged = fold_staged<kBounded, T>(smem, dp, dc, p, keys, o);
+    bool staged = fold_staged<kFold, T>(smem, dp, dc, p, keys, o);
     if constexpr (!FoldCfg<T>::kSingle) if (!staged) {
         __syncthreads();   // the global path reuses the shared memory
         fold_global(smem, dp, dc, p, keys, o);
@@ -980,7 +1009,7 @@ k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, 
     const long long tot = o.pf[n];
     for (int64_t k = threadIdx.x; k < dm + kPadMargin; k += blockDim.x) {
         const bool real = k < dm;
-        o.rs[n + k] = real ? o.rs[k] : 0.0f;
+        if (!kBoundedW) o.rs[n + k] = real ? o.rs[k] : 0.0f;
         if (!o.uniform) {
             o.ws[n + k] = real ? o.ws[k] : 0.0f;
             o.wrs[n + k] = real ? o.wrs[k] : 0.0f;
@@ -991,9 +1020,9 @@ k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, 
             if (kBounded) o.pq[n + k + 1] = (int32_t)(v >> o.shift);
         }
     }
-    if (kBounded) {
+    if (kFold != Fold::kPlain) {
         __syncthreads();
-        bounds::window_bounds<T>(smem, ds, dk, slot_id, lc, p, tile_buf);
+        bounds::window_bounds<T, kBoundedW>(smem, ds, dk, slot_id, lc, p, tile_buf);
     }
 }
 
@@ -2486,6 +2515,23 @@ void bound_tables(const float* s, int j, int d, int st, int64_t n, int clg, int 
         top = std::max(top, std::fabs((double)s[k]));
         t2 += (double)s[k] * s[k];
     }
+    // per-point weights: nested parts of the template and what s_k^2 is at
+    // least there, and on the segments
+    auto least = [&](int lo, int hi) {
+        double m = hi > lo ? 1e300 : 0.0;
+        for (int k = lo; k < hi; ++k) m = std::min(m, (double)s[k] * s[k]);
+        return m * (1.0 - 1e-6);
+    };
+    constexpr double kLevel[kBoundLevels] = {0.0, 0.01, 0.03, 0.07, 0.15, 0.28};
+    double level = 0.0;
+    for (int l = 0; l < kBoundLevels; ++l) {
+        const int at = (int)(kLevel[l] * d);
+        const double c = std::max(level, least(at, d - at));
+        b.lev_len[l] = d - 2 * at;
+        b.lev_up[l] = (float)((c - level) * (1.0 - 1e-6));
+        level = c;
+    }
+    for (int g = 0; g < kBoundSegs; ++g) b.seg_low[g] = (float)least(off[g], off[g + 1]);
     b.nu_all = piece(0, d, b.mean_all);
     b.root_t2 = (float)std::sqrt(t2);
     b.t_max = (float)(top * (1.0 + 1e-6));
@@ -2593,12 +2639,16 @@ gtls_status configure_kernels(int dev)
                                        optin - (int)a.sharedSizeBytes));
         return GTLS_OK;
     };
-    for (const void* fn : {(const void*)k_fold_sort<false, 256>, (const void*)k_fold_sort<false, 512>,
-                           (const void*)k_fold_sort<false, 1024>, (const void*)k_fold_sort<true, 256>,
-                           (const void*)k_fold_sort<true, 512>, (const void*)k_fold_sort<true, 1024>})
+    for (const void* fn :
+         {(const void*)k_fold_sort<Fold::kPlain, 256>, (const void*)k_fold_sort<Fold::kPlain, 512>,
+          (const void*)k_fold_sort<Fold::kPlain, 1024>, (const void*)k_fold_sort<Fold::kBounds, 256>,
+          (const void*)k_fold_sort<Fold::kBounds, 512>, (const void*)k_fold_sort<Fold::kBounds, 1024>,
+          (const void*)k_fold_sort<Fold::kBoundsW, 256>, (const void*)k_fold_sort<Fold::kBoundsW, 512>,
+          (const void*)k_fold_sort<Fold::kBoundsW, 1024>})
         GTLS_TRY(allow(fn));
     GTLS_TRY(allow((const void*)k_window_tiles));
     GTLS_TRY(allow((const void*)bounds::k_window_exact));
+    GTLS_TRY(allow((const void*)bounds::k_window_exact_w));
     GTLS_TRY(allow((const void*)k_median_sde));
     GTLS_TRY(allow((const void*)k_median_sde_set));
     GTLS_CUDA(cudaFuncSetAttribute((const void*)k_window_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2679,7 +2729,7 @@ gtls_status create_device(gtls_plan* pl)
     GTLS_TRY(dev_alloc(pl, &dc.scal, 8));
     GTLS_TRY(dev_alloc(pl, &dc.tmin_key, 1));
     GTLS_TRY(dev_alloc(pl, &dc.flags, 1));
-    GTLS_TRY(dev_alloc(pl, &dc.part, 1024));
+    GTLS_TRY(dev_alloc(pl, &dc.part, 2 * kPrepBlocks));
     GTLS_TRY(dev_alloc(pl, &dc.check, 4));
 
     DevChunk& dk = pl->dk;
@@ -3004,6 +3054,9 @@ gtls_status create_device(gtls_plan* pl)
             GTLS_TRY(upload(pl, const_cast<BoundTab**>(&q.bounds), tab));
             GTLS_TRY(upload(pl, const_cast<BoundDur**>(&q.bound_durs), bd));
         }
+        // (the 32-bit prefix sums of w take the fold's keys' place)
+        pl->bounds_w_ok = pl->bounds_ok && pl->tile_w_ok && !pl->has_window_only &&
+                          4 * (n + h.dmax + 16) <= 8 * pl->dk.key_stride;
     }
 
     // one-entry descriptor sets of this plan's own searches
@@ -3080,7 +3133,7 @@ gtls_status ensure_chunk(gtls_plan* pl)
         GTLS_TRY(dev_alloc(pl, &dk.pq, chunk * dk.pad_stride));
         dk.list_cap = std::max<int64_t>(4096, chunk * kListPerSlot);
         GTLS_TRY(dev_alloc(pl, &dk.list, kListClasses * dk.list_cap));
-        GTLS_TRY(dev_alloc(pl, &dk.dense, chunk * std::max({1, pl->tile_count, pl->tile_count_ref})));
+        GTLS_TRY(dev_alloc(pl, &dk.dense, chunk * std::max({1, pl->tile_count, pl->tile_count_ref, pl->tile_count_w})));
         GTLS_TRY(dev_alloc(pl, &dk.left_n, kListClasses + 1));
     }
     if (pl->has_tensor) {
@@ -3179,7 +3232,8 @@ struct Ctx {
     const void* tc_maps = nullptr;   // tensor-core kernel: TMA maps of dk.rs (tc::kMaps rows pitches)
     int tc_jspan = 1;        // tensor-core kernel: work items per period slot
     int tc_test = 0;         // tensor-core kernel: run the timeout test
-    bool bounds_ok = false;  // uniform weights: bounds kernel first, tiled kernel on what it leaves
+    bool bounds_ok = false;  // window search by bounds first, tiled kernel on what it leaves
+    bool bounds_w_ok = false;   // ... with per-point weights
     int64_t launches = 0, window_launches = 0;
     gtls_plan* prof = nullptr;   // stage marks (single search with profiling on)
     size_t ev = 0;
@@ -3190,28 +3244,22 @@ gtls_status stage_mark(Ctx& c, int stage)
     return c.prof ? mark(c.prof, c.st, stage, c.ev) : GTLS_OK;
 }
 
-template <bool kBounded, int T>
+template <Fold kFold, int T>
 void launch_fold_as(Ctx& c, const DevSet& ds, const SlotMap& sm, const SlotMap* smq)
 {
     int smem = T == kFoldThreads ? c.fold_smem : FoldCfg<T>::kStagedBytes;
-    if (kBounded) smem = std::max(smem, (int)bounds::smem_bytes(T));
-    k_fold_sort<kBounded, T><<<sm.slots, T, smem, c.st>>>(ds, sm, smq, c.dk, c.tile_buf);
+    if (kFold != Fold::kPlain) smem = std::max(smem, (int)bounds::smem_bytes(T));
+    k_fold_sort<kFold, T><<<sm.slots, T, smem, c.st>>>(ds, sm, smq, c.dk, c.tile_buf);
 }
 
 // The fold of one wave (with the first steps of the window search when
-// bounded) in CTAs of `threads` threads.
-gtls_status launch_fold(Ctx& c, const DevSet& ds, const SlotMap& sm, const SlotMap* smq, bool bounded, int threads)
+// by bounds) in CTAs of `threads` threads.
+template <Fold kFold>
+void launch_fold(Ctx& c, const DevSet& ds, const SlotMap& sm, const SlotMap* smq, int threads)
 {
-    if (bounded) {
-        if (threads == 256) launch_fold_as<true, 256>(c, ds, sm, smq);
-        else if (threads == 512) launch_fold_as<true, 512>(c, ds, sm, smq);
-        else launch_fold_as<true, 1024>(c, ds, sm, smq);
-    } else {
-        if (threads == 256) launch_fold_as<false, 256>(c, ds, sm, smq);
-        else if (threads == 512) launch_fold_as<false, 512>(c, ds, sm, smq);
-        else launch_fold_as<false, 1024>(c, ds, sm, smq);
-    }
-    return GTLS_OK;
+    if (threads == 256) launch_fold_as<kFold, 256>(c, ds, sm, smq);
+    else if (threads == 512) launch_fold_as<kFold, 512>(c, ds, sm, smq);
+    else launch_fold_as<kFold, 1024>(c, ds, sm, smq);
 }
 
 // One wave: fold + sort, every window, per-period results.  `counter` must
@@ -3224,8 +3272,11 @@ gtls_status wave_pass(Ctx& c, bool ref, const SlotMap& sm, bool tiled, bool weig
                       unsigned int* tc_counter = nullptr, const SlotMap* smq = nullptr)
 {
     const DevSet& ds = ref ? c.set_ref : c.set;
-    const bool bounded = tiled && c.bounds_ok && !weighted;
-    GTLS_TRY(launch_fold(c, ds, sm, smq, bounded, fold_threads(max_n)));
+    const bool bounded = tiled && (weighted ? c.bounds_w_ok : c.bounds_ok);
+    const int threads = fold_threads(max_n);
+    if (!bounded) launch_fold<Fold::kPlain>(c, ds, sm, smq, threads);
+    else if (weighted) launch_fold<Fold::kBoundsW>(c, ds, sm, smq, threads);
+    else launch_fold<Fold::kBounds>(c, ds, sm, smq, threads);
     GTLS_CUDA(cudaGetLastError());
     GTLS_TRY(stage_mark(c, kStageFold));
     if (tiled) {
@@ -3234,9 +3285,11 @@ gtls_status wave_pass(Ctx& c, bool ref, const SlotMap& sm, bool tiled, bool weig
         const int bytes = buf * (int)(weighted ? sizeof(float2) : sizeof(float));
         if (bounded) {
             // as many windows at a time as their points and templates leave room for
-            const int room = (int)std::min<int64_t>((c.max_d + 3) & ~3, bounds::kExactRoom);
-            const int ctas = std::max(1, std::min(16, (int)(200000 / (room * 8 + 1024))));
-            bounds::k_window_exact<<<c.n_sm * ctas, 32, room * 2 * sizeof(float), c.st>>>(ds, sm, smq, c.dk, room);
+            const int per = 2 * (int)(weighted ? sizeof(float2) : sizeof(float));
+            const int room = (int)std::min<int64_t>((c.max_d + 3) & ~3, bounds::kExactRoom * 8 / per);
+            const int ctas = std::max(1, std::min(16, 200000 / (room * per + 1024)));
+            auto* const exact = weighted ? bounds::k_window_exact_w : bounds::k_window_exact;
+            exact<<<c.n_sm * ctas, 32, room * per, c.st>>>(ds, sm, smq, c.dk, room);
             GTLS_CUDA(cudaGetLastError());
             c.launches += 1;
         }
@@ -3380,6 +3433,7 @@ gtls_status run_search(gtls_plan* pl, const double* t, const double* y, const do
     c.tc_test = pl->tc_test_wait;
     c.tc_maps = pl->tc_maps;
     c.bounds_ok = pl->bounds_ok;
+    c.bounds_w_ok = pl->bounds_w_ok;
     pl->profile = gtls_profile{};
     if (pl->profiling) c.prof = pl;
 
@@ -3486,7 +3540,8 @@ struct gtls_batch {
     BatchCfg cfg;
     bool tuned = false;
     bool refines = false;              // some plan has a refinement stage
-    bool bounds_ok = true;             // every plan's templates admit the bounds kernel
+    bool bounds_ok = true;             // every plan's templates admit the window search by bounds
+    bool bounds_w_ok = true;           // ... with per-point weights, where these are tiled
     // graph of everything after the curve preparation, for one set of
     // per-curve kernel classes (uniform dy and tile fit)
     std::vector<uint8_t> graph_class;
@@ -3665,6 +3720,7 @@ Ctx batch_ctx(const gtls_batch* b, cudaStream_t st)
     }
     c.tc_maps = b->tc_maps;
     c.bounds_ok = b->bounds_ok;
+    c.bounds_w_ok = b->bounds_ok && b->bounds_w_ok;
     return c;
 }
 
@@ -3958,6 +4014,7 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
             any_tiled = true;
         }
         b->bounds_ok = b->bounds_ok && pl->bounds_ok;
+        b->bounds_w_ok = b->bounds_w_ok && (pl->bounds_w_ok || !pl->tile_w_ok);
     }
     b->fold_smem = fold_smem_bytes(bucket_log2);
     b->median_blocks = max_np_blocks;
@@ -4039,7 +4096,7 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     GTLS_TRY(batch_upload_tiles(b));
     if (b->bounds_ok) {
         int max_tiles = 1;
-        for (const DevTiles& t : b->tiles_host) max_tiles = std::max(max_tiles, t.count);
+        for (const DevTiles& t : b->tiles_host) max_tiles = std::max({max_tiles, t.count, t.count_w});
         GTLS_TRY(batch_alloc(b, &b->dk.dense, slots * (int64_t)max_tiles));
         GTLS_TRY(batch_alloc(b, &b->dk.pq, slots * pad_stride));
         b->dk.list_cap = std::max<int64_t>(4096, slots * kListPerSlot);

@@ -1,5 +1,5 @@
-// Window search by bounds (uniform weights): which windows can hold a
-// period's minimum at all.
+// Window search by bounds: which windows can hold a period's minimum at all.
+// First for uniform weights.
 //
 // Every window has delta-chi2 = w depth (depth sum s_k^2 - 2 C1), and for any
 // depth that is at least -w C1^2 / sum s_k^2.  C1 itself is bounded from
@@ -41,6 +41,16 @@
 // shifted right so far that any sum fits 31 bits; differences are then off by
 // at most one unit.
 //
+// Per-point weights (kW): delta-chi2 = depth (depth C2 - 2 C1) with
+// C1 = sum w r s_k and C2 = sum w s_k^2 is at least -C1^2 / C2 for any depth.
+// C1 is bounded as above with w r in the place of r; its 32-bit prefix sums are
+// those of w r rounded to a unit (weighted_prefix: half a unit per point).  C2
+// is at least sum_l c_l W_l over nested parts l of the window on which s_k^2
+// exceeds the sum of the c up to l; the first test takes for W_l the smallest
+// sum of w over any stretch of the length (weight_floors), the segment test the
+// window's own, with its exact depth.  (20,011 points with a dy of their own: the
+// window stage was 98 ms on the tiled kernel, 126 with the fold; now 71 in all.)
+//
 // What bounds it: shared-memory reads of the coarse prefix and about 50
 // instructions per window.  A lane that reads global memory at a cache line
 // of its own costs the L1 a cycle, which made the same tests on the prefix
@@ -65,7 +75,10 @@ constexpr int kRowBuf = 168;        // prefix sums at whole T0 steps a warp stag
 constexpr int kCutPoints = 60;      // windows of at least this many points are first tested by wide pieces
 constexpr int kCoarseSteps = 64;    // ... and from this many coarse steps on from the coarse prefix
 constexpr int kExactRoom = 24576;   // points of a window (and its template) staged by k_window_exact, at most
+constexpr int kFloorSpans = 48;     // stretches of blocks whose smallest weight is kept: 1 .. 15, then 16, 19, 22,
+                                    // 27 times powers of 2
 constexpr unsigned int kNone = 0xffffffffu;
+constexpr int kNoUnit = 1000;       // per-point weights whose sums do not fit the 32-bit prefix
 
 enum Mode : int { kModePairS = 0, kModeCols = 1, kModeRot = 2, kModeWin = 3 };
 enum Test : int { kTestSum = 0, kTestCuts = 1, kTestCutsDirect = 2, kTestCoarse = 3 };
@@ -76,10 +89,11 @@ struct Dur {
     int first;                  // first chunk (near durations: of a stretch)
     float emax;                 // upper bound of sum r^2 over any window of the duration
     float first_min, cmin;      // thresholds of the first test (32-bit prefix units) and of the segment bound
-    float smin;                 // lowest window sum that can have a depth (32-bit prefix units)
+    float smin;                 // lowest window sum that can have a depth (32-bit prefix units); kW: what the segment
+                                // bound can lose of C1
     float blur;                 // what FP32 sums of C1 can be off by
     float cmin_coarse;          // cmin for sums from the coarse prefix
-    int pad[1];
+    float c2_slack;             // relative error of FP32 sums of C2 (kW)
 };
 
 // Chunks of windows: durations of T0 steps above kNearStep (far ones) are cut
@@ -116,7 +130,11 @@ struct Smem {
     float wsum[kWarps], energy[kEnergySpans];
     float top[kWarps], c1[kWarps], s[kWarps], thr;
     int top_at[kWarps], cand[kCand];
+    int wmin[kFloorSpans], wlow;                     // smallest sums of w over whole blocks, smallest w (kW)
 };
+
+template <int T>
+constexpr int kWarpsOf = T / 32;
 
 __host__ inline size_t smem_bytes(int threads)
 {
@@ -140,6 +158,16 @@ __host__ inline int max_chunks(int threads) { return 2 * threads; }
 __device__ __forceinline__ float sum_slack(int n) { return 1.2e-7f * (float)(n + 8); }
 
 __device__ __forceinline__ float root(float x) { return x > 0.0f ? x * rsqrtf(x) : (x == 0.0f ? 0.0f : x); }
+
+// What delta-chi2 v of a window can differ between two orders of its sums: C1
+// off by at most off, the depth by dd (sums of its own: the (C1, S) pairs), C2
+// by c2_slack of itself (t2: C2, or sum s_k^2).
+__device__ __forceinline__ float sum_error(float w, float depth, float t2, float c1, float v, float off, float dd,
+                                           float c2_slack)
+{
+    return w * (2.0f * (depth + dd) * off + 2.0f * dd * fabsf(fmaf(depth, t2, -c1)) + dd * dd * t2) + 1e-6f * fabsf(v) +
+           2e-6f * w * depth * fabsf(c1) + w * depth * depth * t2 * c2_slack;
+}
 
 // Place of coarse entry e: one word further every 32, so that lanes whose
 // entries are a power of two apart read different banks.
@@ -450,8 +478,119 @@ __device__ __forceinline__ void scan_prefix(Smem<T>& S, const int* __restrict__ 
     }
 }
 
-// Steps 1 to 4 for one period, by a CTA of T threads.
+// Prefix sums of w r and of w over the folded, padded curve in 32 bits: every
+// value rounded to a unit (a = w r / unit, b = w / unit), positions 0 .. total;
+// S.wlow becomes the smallest b (set to INT_MAX before).
 template <int T>
+__device__ __forceinline__ void weighted_prefix(Smem<T>& S, const float* __restrict__ wrs, const float* __restrict__ ws,
+                                                int* __restrict__ pq, int* __restrict__ pw, int total, float per_a,
+                                                float per_b)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int carry_a = 0, carry_b = 0, low = INT_MAX;
+    bool odd = false;
+    for (int r0 = threadIdx.x * 8; r0 - (int)threadIdx.x * 8 <= total; r0 += T * 8, odd = !odd) {
+        int a[8], b[8], sa = 0, sb = 0;
+        float va[8], vb[8];
+#pragma unroll
+        for (int h = 0; h < 8; h += 4) {   // (zeros follow the padded curve)
+            const float4 x = r0 <= total ? *reinterpret_cast<const float4*>(wrs + r0 + h) : make_float4(0, 0, 0, 0);
+            const float4 y = r0 <= total ? *reinterpret_cast<const float4*>(ws + r0 + h) : make_float4(0, 0, 0, 0);
+            va[h] = x.x, va[h + 1] = x.y, va[h + 2] = x.z, va[h + 3] = x.w;
+            vb[h] = y.x, vb[h + 1] = y.y, vb[h + 2] = y.z, vb[h + 3] = y.w;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int qa = __float2int_rn(va[u] * per_a), qb = __float2int_rn(vb[u] * per_b);
+            if (r0 + u < total) low = min(low, qb);
+            a[u] = sa;
+            b[u] = sb;
+            sa += qa;
+            sb += qb;
+        }
+        int xa = sa, xb = sb;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int ya = __shfl_up_sync(0xffffffffu, xa, o), yb = __shfl_up_sync(0xffffffffu, xb, o);
+            if (lane >= o) {
+                xa += ya;
+                xb += yb;
+            }
+        }
+        // (two sets of warp sums in turn: one barrier per round)
+        int* const wa = reinterpret_cast<int*>(odd ? S.c1 : S.wsum);
+        int* const wb = reinterpret_cast<int*>(odd ? S.s : S.top);
+        if (lane == 31) {
+            wa[warp] = xa;
+            wb[warp] = xb;
+        }
+        __syncthreads();
+        const int ta = lane < kWarpsOf<T> ? wa[lane] : 0, tb = lane < kWarpsOf<T> ? wb[lane] : 0;
+        const int ea = carry_a + (int)__reduce_add_sync(0xffffffffu, lane < warp ? ta : 0) + xa - sa;
+        const int eb = carry_b + (int)__reduce_add_sync(0xffffffffu, lane < warp ? tb : 0) + xb - sb;
+        carry_a += (int)__reduce_add_sync(0xffffffffu, ta);
+        carry_b += (int)__reduce_add_sync(0xffffffffu, tb);
+        if (r0 <= total) {
+#pragma unroll
+            for (int h = 0; h < 8; h += 4) {
+                *reinterpret_cast<int4*>(pq + r0 + h) =
+                    make_int4(ea + a[h], ea + a[h + 1], ea + a[h + 2], ea + a[h + 3]);
+                *reinterpret_cast<int4*>(pw + r0 + h) =
+                    make_int4(eb + b[h], eb + b[h + 1], eb + b[h + 2], eb + b[h + 3]);
+            }
+        }
+    }
+    low = __reduce_min_sync(0xffffffffu, low);
+    if (lane == 0) atomicMin(&S.wlow, low);
+}
+
+// Blocks of floor span q.
+__device__ __forceinline__ int floor_span(int q)
+{
+    const int f = (q - 15) & 3;
+    return q < 15 ? q + 1 : (f == 0 ? 16 : f == 1 ? 19 : f == 2 ? 22 : 27) << ((q - 15) >> 2);
+}
+
+// Smallest sums of w over stretches of whole blocks of 2^lb points, by the
+// prefix of the blocks in S.pre (as integers).  Starts are taken 1/16 of the
+// stretch together: what all of them share.
+template <int T>
+__device__ __forceinline__ void weight_floors(Smem<T>& S, const int* __restrict__ pw, int total, int lb)
+{
+    int* const pre = reinterpret_cast<int*>(S.pre);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nb = total >> lb;
+    for (int b = threadIdx.x; b <= nb; b += T) pre[b] = pw[b << lb];
+    __syncthreads();
+    for (int q = warp; q < kFloorSpans; q += T / 32) {
+        const int m = floor_span(q), step = max(1, m >> 4);
+        int low = m <= nb ? INT_MAX : 0;
+#pragma unroll 4
+        for (int i = lane * step; i + m <= nb; i += 32 * step) low = min(low, pre[i + m] - pre[i + step - 1]);
+        low = __reduce_min_sync(0xffffffffu, low);
+        if (lane == 0) S.wmin[q] = low;
+    }
+    __syncthreads();   // (pre is written again)
+}
+
+// At most the sum of w over any len points, in units of its prefix.
+template <int T>
+__device__ __forceinline__ float weight_floor(const Smem<T>& S, int len, int lb)
+{
+    float sum = 0.0f;
+    for (int m = (len - (1 << lb) + 1) >> lb; m > 0;) {
+        int q = m - 1;
+        if (m > 15) {
+            const int o = 27 - __clz(m), x = m >> o;   // 16 .. 31
+            q = min(kFloorSpans - 1, 15 + 4 * o + (x >= 27 ? 3 : x >= 22 ? 2 : x >= 19 ? 1 : 0));
+        }
+        sum += (float)S.wmin[q] * (1.0f - 1e-6f);
+        m -= floor_span(q);
+    }
+    return fmaxf(sum, (float)len * (float)S.wlow * (1.0f - 1e-6f)) - 0.5f * (float)len;
+}
+
+// Steps 1 to 4 for one period, by a CTA of T threads (kW: per-point weights).
+template <int T, bool kW>
 __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet& ds, const DevChunk& dk, int slot, int lc,
                                               int p, int buf)
 {
@@ -461,20 +600,31 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
     Dur* const dur = S.dur;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const DevPlan& dp = ds.plans[lc];
-    const float w_uni = (float)ds.curves[lc].scal[2];
+    const float w_uni = kW ? 1.0f : (float)ds.curves[lc].scal[2];
     const int n = (int)dp.n;
     const int total = n + dp.dmax_p[p];
     float* const rb = S.row_buf + warp * kRowBuf;
-    const float* const rs = dk.rs + (int64_t)slot * dk.pad_stride;
+    const float* const rs = (kW ? dk.wrs : dk.rs) + (int64_t)slot * dk.pad_stride;   // what C1 sums
+    const float* const ws = kW ? dk.ws + (int64_t)slot * dk.pad_stride : nullptr;
     const int* const pq = dk.pq + (int64_t)slot * dk.pad_stride;
+    // (the fold is through with its keys)
+    int* const pw = reinterpret_cast<int*>(dk.keys + (int64_t)slot * dk.key_stride);
+    const long long* const pf = dk.pf + (int64_t)slot * dk.pad_stride;
     const int shift = (int)ds.curves[lc].scal[3];
-    const float unit = prefix_unit(shift);   // of the 32-bit prefix
+    const int shift_w = kW ? (int)ds.curves[lc].scal[4] : 0;
+    const bool in_range_32 = kW ? shift < kNoUnit && shift_w < kNoUnit : shift < 64;
+    // unit of the 32-bit prefix.  Per-point weights: C1 and energies are kept
+    // in units until the windows are summed
+    const float unit = kW ? 1.0f : prefix_unit(shift);
+    const float unit_a = kW ? ldexpf(1.0f, in_range_32 ? shift : 0) : 1.0f;
+    const float unit_w = kW ? ldexpf(1.0f, in_range_32 ? shift_w : 0) : 1.0f;
     const int lg = dp.bound_lg;
 
     if (warp == 0) {
         list_durations(dp, ds.curves[lc].check, p, n, dur, S.ck, lane);
         for (int k = lane; k < kEnergySpans; k += 32) S.energy[k] = 0.0f;
         if (lane == 0) S.next = S.sieved = S.n_fin = S.n_listed = S.dev = S.big = 0;
+        if (lane == 0) S.wlow = INT_MAX;
     }
     for (int i = threadIdx.x; i < M::kSieve; i += T) S.sieve[i] = kNone;
     __syncthreads();
@@ -495,6 +645,13 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
     while (((total + (1 << lb) - 1) >> lb) > M::kMaxBlocks) ++lb;
     while ((total >> clg) + 2 > M::kMaxCoarse) ++clg;
     const int bsize = 1 << lb, nb = (total + bsize - 1) >> lb;
+    int lbw = 2;   // blocks of the weights
+    if (kW) {
+        while ((total >> lbw) > M::kMaxBlocks) ++lbw;
+        weighted_prefix<T>(S, rs, ws, const_cast<int*>(pq), pw, total, 1.0f / unit_a, 1.0f / unit_w);
+        __syncthreads();
+        weight_floors<T>(S, pw, total, lbw);
+    }
     scan_prefix<T>(S, pq, total, lb, clg, unit);
     __syncthreads();
     {
@@ -659,12 +816,13 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         if (cand >= 0) {
             const BoundDur& t = dur[cand >> 24].b;
             const float* const r = rs + (cand & 0xffffff) * t.st;
+            const float* const w = ws + (cand & 0xffffff) * t.st;
             const float* const s = dp.tmpl + dp.tmpl_off[t.j];
 #pragma unroll 8
             for (int i = threadIdx.x % kTeamThreads; i < t.d; i += kTeamThreads) {
-                const float v = r[i];
-                c1 = fmaf(v, __ldg(s + i), c1);
-                sum += v;
+                const float v = r[i], sv = __ldg(s + i);
+                c1 = fmaf(v, sv, c1);
+                sum = kW ? fmaf(w[i], sv * sv, sum) : sum + v;   // C2, or the window sum
             }
         }
 #pragma unroll
@@ -678,18 +836,41 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         }
     }
     __syncthreads();
+    // rows a lane of the final sums adds to one window, what two orders of its
+    // sum can differ, and the same for C2
+    auto chain_of = [&](const Dur& t) {
+        const int lg = kW ? __ffs(dp.cfg_nc_w[t.b.j]) - 1 : t.b.lg_nc, nc = 1 << lg;
+        return ((t.b.st + nc - 1) >> lg) * ((t.b.d + t.b.st - 1) / t.b.st) + 6;
+    };
+    auto blur_of = [&](const Dur& t, int chain, float norm) {
+        return ((sum_slack(chain) + sum_slack(t.b.d / 32 + 8)) * norm + (kW ? 0.0f : (float)t.b.d * 1e-12f)) *
+               fmaxf(dp.bounds[t.b.j].t_max, 1.0f) * unit_a;
+    };
+    auto c2_slack_of = [&](const Dur& t, int chain) {
+        return kW ? sum_slack(chain) + sum_slack(t.b.d / 32 + 8) + 1e-6f : 1e-6f;
+    };
     if (threadIdx.x == 0) {
         float thr = INFINITY;
         for (int q = 0; q < kCand; ++q) {
             if (S.cand[q] < 0) continue;
-            const int j = dur[S.cand[q] >> 24].b.j;
+            const Dur& t = dur[S.cand[q] >> 24];
+            const int j = t.b.j;
             float c1 = 0.0f, sum = 0.0f;
             for (int w = q * kTeam; w < (q + 1) * kTeam; ++w) {
                 c1 += S.c1[w];
                 sum += S.s[w];
             }
-            const float depth = fmaxf(0.0f, sum * dp.inv_sum_t[j]);
-            const float v = w_uni * depth * fmaf(depth, dp.sum_t2[j], -2.0f * c1);
+            float depth = sum * dp.inv_sum_t[j];
+            if (kW) {
+                const int s = (S.cand[q] & 0xffffff) * t.b.st;
+                depth = tiles::fixed_to_float(pf[s + t.b.d] - pf[s]) * (dp.inv_sum_t[j] * (1.0f / 1099511627776.0f));
+            }
+            depth = fmaxf(0.0f, depth);
+            const float t2 = kW ? sum : dp.sum_t2[j];
+            const int chain = chain_of(t);
+            const float off = blur_of(t, chain, sqrtf((float)t.b.d * energy_of(t.b.d)));
+            float v = w_uni * depth * fmaf(depth, t2, -2.0f * c1);
+            v += sum_error(w_uni, depth, t2, c1, v, off, kW ? 0.0f : off * dp.inv_sum_t[j], c2_slack_of(t, chain));
             thr = v < thr || isnan(v) ? v : thr;
         }
         S.thr = thr;
@@ -698,27 +879,35 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
     __syncthreads();
     const float thr = S.thr;
     // no negative delta-chi2, or values out of range: the tiled kernel decides
-    const bool sane = thr < 0.0f && thr > -INFINITY && e_all < INFINITY && w_uni < INFINITY && shift < 64;
+    const bool sane = thr < 0.0f && thr > -INFINITY && e_all < INFINITY && w_uni < INFINITY && in_range_32;
     if (sane) {
         // thresholds of every duration.  A window whose C1 stays below cmin is
-        // above thr; 1e-4 of slack covers the rounding of thr and of
-        // delta-chi2 itself, and `lost` what FP32 summation, the 32-bit prefix
+        // above thr; 1e-4 of slack covers the rounding of delta-chi2, and `lost` what FP32 summation, the 32-bit prefix
         // and segment sums can lose of C1 (at most sum_slack(products in a
         // row) ||r|| ||s||, 2^-41 of fixed point per point, and the prefix
         // units of the sums)
-        const float reach = sqrtf(-thr / w_uni) * (1.0f - 1e-4f);
+        const float reach = sqrtf(-thr / w_uni) * (1.0f - 1e-4f);   // (kW: times the root of C2)
         for (int k = threadIdx.x; k < ndur; k += T) {
             Dur& t = dur[k];
             const BoundTab& bt = dp.bounds[t.b.j];
-            const int nc = 1 << t.b.lg_nc, d = t.b.d, st = t.b.st;
-            const int chain = ((st + nc - 1) >> t.b.lg_nc) * ((d + st - 1) / st) + 6;
+            if (kW) t.b.lg_nc = __ffs(dp.cfg_nc_w[t.b.j]) - 1;
+            const int d = t.b.d, st = t.b.st, chain = chain_of(t);
             t.emax = energy_of(d);
             const float norm = sqrtf((float)d * t.emax);
-            const float lost = (sum_slack(chain) + 8e-6f) * norm + (float)d * 1e-12f;
-            t.cmin = reach * bt.root_t2 - (lost + (float)(kBoundSegs + 1) * unit) * bt.t_max;
-            t.blur = ((sum_slack(chain) + sum_slack(d / 32 + 8)) * norm + (float)d * 1e-12f) * fmaxf(bt.t_max, 1.0f);
+            const float lost = (sum_slack(chain) + 8e-6f) * norm + (float)d * (kW ? 0.5f : 1e-12f);
+            t.c2_slack = c2_slack_of(t, chain);
+            float root_c2 = bt.root_t2;
+            if (kW) {
+                // the smallest C2 of any window, with what FP32 sums of it can lose
+                float c2 = 0.0f;
+                for (int l = 0; l < kBoundLevels; ++l)
+                    c2 = fmaf(bt.lev_up[l], fmaxf(0.0f, weight_floor(S, bt.lev_len[l], lbw)), c2);
+                root_c2 = sqrtf(c2 * unit_w * (1.0f - 1e-5f - t.c2_slack)) / unit_a;
+            }
+            t.cmin = reach * root_c2 - (lost + (float)(kBoundSegs + 1) * unit) * bt.t_max;
+            t.blur = blur_of(t, chain, norm);
             // depth is zero without a positive sum (exact, or FP32 for the pairs)
-            const float low = (t.b.mode == kModePairS ? -lost : 0.0f) - 2.0f * unit;
+            const float low = kW ? -INFINITY : (t.b.mode == kModePairS ? -lost : 0.0f) - 2.0f * unit;
             float c0;
             if (t.b.test == kTestSum) {
                 c0 = fmaxf((t.cmin - bt.nu_all * sqrtf(t.emax)) / bt.mean_all, low);
@@ -739,7 +928,7 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
                 c0 = t.cmin - lose;
             }
             t.first_min = (c0 - 1e-5f * fabsf(c0)) / unit;
-            t.smin = low / unit;
+            t.smin = kW ? (lost + (float)(kBoundSegs + 1) * unit) * bt.t_max : low / unit;
         }
     }
     __syncthreads();
@@ -823,8 +1012,39 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
                 if (c1 < t.cmin_coarse) continue;
             }
             int last = pq[s], e0 = s;
-            if ((float)(pq[s + t.b.d] - last) < t.smin) continue;
             float c1 = 0.0f;
+            if constexpr (kW) {
+                const long long sfx = pf[s + t.b.d] - pf[s];
+                if (sfx <= 0) continue;   // no depth
+                const float depth =
+                    tiles::fixed_to_float(sfx) * (dp.inv_sum_t[t.b.j] * (1.0f / 1099511627776.0f));
+                const float* const seg_low = dp.bounds[t.b.j].seg_low;
+                int lastw = pw[s];
+                float c2 = 0.0f;
+#pragma unroll 5
+                for (int g = 0; g < kBoundSegs; ++g) {
+                    const float4 q = __ldg(seg + g);   // end, mean, nu, 1 / length
+                    const int e1 = s + __float_as_int(q.x);
+                    const int nx = pq[e1], nw = pw[e1];
+                    const float sg = (float)(nx - last);
+                    const float en = fmaf(S.pre[(e1 + bsize - 1) >> lb] - S.pre[e0 >> lb], 1.0f + e_rel, e_abs);
+                    const float sm = fmaxf(fabsf(sg) - (1.0f + 0.5f * (float)(e1 - e0)), 0.0f);
+                    c1 += fmaf(q.y, sg, q.z * root(en - q.w * sm * sm));
+                    c2 = fmaf(__ldg(seg_low + g), fmaxf(0.0f, (float)(nw - lastw) - 0.5f * (float)(e1 - e0)), c2);
+                    last = nx;
+                    lastw = nw;
+                    e0 = e1;
+                }
+                c1 = (c1 + t.smin) * unit_a;
+                c2 *= unit_w * (1.0f - 1e-5f - t.c2_slack);
+                const float v = depth * fmaf(depth, c2, -2.0f * c1) -
+                                1e-6f * depth * (depth * c2 + 2.0f * fabsf(c1));
+                if (v > thr * (1.0f - 1e-4f)) continue;
+                const int to = atomicAdd(&S.n_fin, 1);
+                if (to < M::kFinal) S.fin[to] = e;
+                continue;
+            }
+            if ((float)(pq[s + t.b.d] - last) < t.smin) continue;
 #pragma unroll 5
             for (int g = 0; g < kBoundSegs; ++g) {
                 const float4 q = __ldg(seg + g);   // end, mean, nu, 1 / length
@@ -858,20 +1078,30 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
             const int s = (int)(e & 0xffffffu) * t.b.st, d = t.b.d;
             const float* const r = rs + s;
             const float* const tm = dp.tmpl + dp.tmpl_off[t.b.j];
-            const long long* const pf = dk.pf + (int64_t)slot * dk.pad_stride + s;
-            const long long sfx = pf[d] - pf[0];
-            float c1 = 0.0f;
+            const long long sfx = pf[s + d] - pf[s];
+            float c1 = 0.0f, c2 = 0.0f;
+            if (kW) {
+#pragma unroll 8
+                for (int q = lane; q < d; q += 32) {
+                    const float sv = __ldg(tm + q);
+                    c1 = fmaf(r[q], sv, c1);
+                    c2 = fmaf(ws[s + q], sv * sv, c2);
+                }
+            } else {
 #pragma unroll 16
-            for (int q = lane; q < d; q += 32) c1 = fmaf(r[q], __ldg(tm + q), c1);
+                for (int q = lane; q < d; q += 32) c1 = fmaf(r[q], __ldg(tm + q), c1);
+            }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) c1 += __shfl_xor_sync(0xffffffffu, c1, o);
-            const float inv = dp.inv_sum_t[t.b.j], t2 = dp.sum_t2[t.b.j];
+            for (int o = 16; o > 0; o >>= 1) {
+                c1 += __shfl_xor_sync(0xffffffffu, c1, o);
+                if (kW) c2 += __shfl_xor_sync(0xffffffffu, c2, o);
+            }
+            const float inv = dp.inv_sum_t[t.b.j], t2 = kW ? c2 : dp.sum_t2[t.b.j];
             const float depth = fmaxf(0.0f, tiles::fixed_to_float(sfx) * (inv * (1.0f / 1099511627776.0f)));
             const float v = w_uni * depth * fmaf(depth, t2, -2.0f * c1);
             // C1 is off by at most blur, the depth of the pairs by blur / sum s_k
-            const float off = t.blur, dd = t.b.mode == kModePairS ? off * inv : 0.0f;
-            const float err = w_uni * (2.0f * (depth + dd) * off + 2.0f * dd * fabsf(fmaf(depth, t2, -c1)) + dd * dd * t2) +
-                              1e-6f * fabsf(v) + 2e-6f * w_uni * depth * fabsf(c1);
+            const float off = t.blur, dd = !kW && t.b.mode == kModePairS ? off * inv : 0.0f;
+            const float err = sum_error(w_uni, depth, t2, c1, v, off, dd, t.c2_slack);
             if (lane == 0) S.fin_v[i] = v - err;
             odd = odd || !(v - err > -INFINITY && v + err < INFINITY);
             best = fminf(best, v + err);
@@ -896,7 +1126,7 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
                 else
                     S.n_listed = 2 * kListed;   // (more may be added: it stays above kListed)
             };
-            if (t.b.mode != kModeRot) {
+            if (kW || t.b.mode != kModeRot) {
                 push(0);
                 continue;
             }
@@ -922,7 +1152,7 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         fits = fits && S.n_listed <= kListed;
     }
     if (!fits && threadIdx.x == 0) {
-        const int tc = ds.tiles[lc].count;
+        const int tc = kW ? ds.tiles[lc].count_w : ds.tiles[lc].count;
         const unsigned int to = atomicAdd(dk.left_n + kListClasses, (unsigned int)tc);
         for (int tau = 0; tau < tc; ++tau) dk.dense[to + tau] = make_int2(slot, tau);
     }
@@ -975,6 +1205,72 @@ k_window_exact(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
             const float w_uni = (float)ds.curves[lc].scal[2];
             atomicMin(&ds.outs[lc].best[p],
                       tiles::window_key(w_uni * depth * fmaf(depth, dp.sum_t2[j], -2.0f * sum.x), j, m));
+        }
+        item -= cnt;
+    }
+}
+
+// The same for per-point weights: (w r, w) and (s_k, s_k^2) pairs, one
+// column per lane at a time.
+static __global__ void __launch_bounds__(32)
+k_window_exact_w(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk, int room)
+{
+    const SlotMap& sm = smq ? *smq : smv;
+    extern __shared__ float2 pair_smem[];
+    const int lane = threadIdx.x;
+    int item = blockIdx.x;
+    for (int q = 0; q < kListClasses; ++q) {
+        const int cnt = (int)min((int64_t)dk.left_n[q], dk.list_cap);
+        for (; item < cnt; item += gridDim.x) {
+            const unsigned long long en = dk.list[q * dk.list_cap + item];
+            const int slot = (int)(en >> 40), j = (int)(en >> 32) & 0xff, m = (int)(en & 0xffffffull);
+            int lc, p;
+            if (!resolve_slot(ds, sm, slot, lc, p)) continue;   // warp-uniform
+            const DevPlan& dp = ds.plans[lc];
+            const int d = dp.dpts[j], st = dp.stride[j], nc = 1 << q;
+            const int64_t base = (int64_t)slot * dk.pad_stride + (int64_t)m * st;
+            const float *const wr = dk.wrs + base, *const w = dk.ws + base;
+            const float2* const t = dp.tmplw + dp.tmplw_off[j];
+            const long long sfx = dk.pf[base + d] - dk.pf[base];
+            float x = 0.0f, y = 0.0f;
+            if (d <= room) {
+                __syncwarp();
+                for (int k = lane; k < d; k += 32) {
+                    const uint32_t to = (uint32_t)__cvta_generic_to_shared(pair_smem + k);
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to), "l"(wr + k) : "memory");
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to + 4), "l"(w + k) : "memory");
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(to + room * 8), "l"(t + k) : "memory");
+                }
+                asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+                __syncwarp();
+            }
+            if (lane < nc) {
+                for (int rho = lane; rho < st; rho += nc) {
+                    if (d <= room) {
+#pragma unroll 8
+                        for (int k = rho; k < d; k += st) {
+                            const float2 v = pair_smem[k], s = pair_smem[room + k];
+                            x = fmaf(v.x, s.x, x);
+                            y = fmaf(v.y, s.y, y);
+                        }
+                    } else {
+#pragma unroll 8
+                        for (int k = rho; k < d; k += st) {
+                            const float2 s = __ldg(t + k);
+                            x = fmaf(wr[k], s.x, x);
+                            y = fmaf(w[k], s.y, y);
+                        }
+                    }
+                }
+            }
+            for (int o = 1; o < nc; o <<= 1) {
+                x += __shfl_xor_sync(0xffffffffu, x, o);
+                y += __shfl_xor_sync(0xffffffffu, y, o);
+            }
+            if (lane != 0) continue;
+            const float depth =
+                fmaxf(0.0f, tiles::fixed_to_float(sfx) * (dp.inv_sum_t[j] * (1.0f / 1099511627776.0f)));
+            atomicMin(&ds.outs[lc].best[p], tiles::window_key(depth * fmaf(depth, y, -2.0f * x), j, m));
         }
         item -= cnt;
     }
