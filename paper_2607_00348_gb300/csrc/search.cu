@@ -219,6 +219,21 @@ __device__ long long block_exclusive_scan1(long long v, long long* warp_sums, lo
     return (warp > 0 ? base : 0) + x - v;
 }
 
+// The same for 32-bit values, without the total.
+__device__ __forceinline__ uint32_t block_exclusive_scan32(uint32_t v, uint32_t* warp_sums)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_sums[warp] = x;
+    __syncthreads();
+    return __reduce_add_sync(0xffffffffu, lane < warp ? warp_sums[lane] : 0u) + x - v;
+}
+
 // Light curve and period held by `slot` of a wave (segments ascend in
 // slot0); false past the wave's slots or when the period index is out of
 // range.
@@ -412,8 +427,12 @@ __global__ void k_curve_reduce(const double* __restrict__ dy, const int64_t* __r
 // whole buckets are ranked and scanned (in shared memory while a run fits,
 // else in global memory).
 
-constexpr int kFoldFineLog2 = 11;   // fine buckets per super-bucket (log2)
+// Fine buckets per super-bucket (log2): 1.75 points in each on average, whose
+// ranks need the comparison with all of them (3.5 at 11: 65 instead of 54
+// thousand cycles of a period of 62,363 points).
+constexpr int kFoldFineLog2 = 12;
 constexpr int kFoldMaxSbLog2 = 10;  // at most one super-bucket per fold thread
+constexpr float kFoldLookRun = 48.0f;   // points of a super-bucket and cycle from which warps look for sharing it
 constexpr int kFoldFillKeys = 7168; // mean points per super-bucket the plan aims at
 
 // Fine bucket of phase rho: floor((rho >> sh) mulf / 2^32) with
@@ -424,7 +443,7 @@ __device__ __forceinline__ uint32_t fold_fine(long long rho, int sh, uint32_t mu
     return (uint32_t)((((unsigned long long)rho >> sh) * (unsigned long long)mulf) >> 32);
 }
 
-// Shapes for CTAs of T threads: 8 T staged keys, two fine buckets per thread.
+// Shapes for CTAs of T threads: 8 T staged keys, four fine buckets per thread.
 // Curves of up to 8 T points take the smallest T (256, 512, 1024) and a single
 // super-bucket, whose keys never leave the CTA; several such CTAs share an SM
 // (1440 points: 0.27 ms at 1024 threads, 0.17 at 512).  At more than one
@@ -434,9 +453,9 @@ template <int T>
 struct FoldCfg {
     static constexpr bool kSingle = T < kFoldThreads;
     static constexpr int kSegKeys = 8 * T;
-    static constexpr int kFineLog2 = T == 1024 ? kFoldFineLog2 : T == 512 ? 10 : 9;
+    static constexpr int kFineLog2 = T == 1024 ? kFoldFineLog2 : T == 512 ? kFoldFineLog2 - 1 : kFoldFineLog2 - 2;
     static constexpr int kMaxSb = kSingle ? 2 : 1 << kFoldMaxSbLog2;
-    static constexpr int kStagedBytes = 33 * 8 + 2 * kSegKeys * 8 + (2 << kFineLog2) * 4 + 2 * kMaxSb * 4 +
+    static constexpr int kStagedBytes = 33 * 8 + 2 * kSegKeys * 8 + (1 << kFineLog2) * 4 + 2 * kMaxSb * 4 +
                                         2 * kSegKeys * 2 + 16;
 };
 
@@ -566,9 +585,10 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
     long long* total = warp_sums + 32;
     long long* srfx = reinterpret_cast<long long*>(total + 1);                  // rfx in final order (swizzled)
     unsigned long long* sorted = reinterpret_cast<unsigned long long*>(srfx + kFoldSegKeys);   // keys in fine-bucket order
-    uint32_t* fcnt = reinterpret_cast<uint32_t*>(sorted + kFoldSegKeys);
-    uint32_t* fcur = fcnt + (1 << kFoldFineLog2);
-    uint32_t* sb_cnt = fcur + (1 << kFoldFineLog2);
+    // fine buckets: keys in the upper half, place of the next one in the lower
+    uint32_t* fine = reinterpret_cast<uint32_t*>(sorted + kFoldSegKeys);
+    uint32_t* sb_cnt = fine + (1 << kFoldFineLog2);
+    static_assert(kFoldSegKeys <= 1 << 15, "counts and places are kept in 16 bits");
     uint32_t* sb_start = sb_cnt + L::kMaxSb;
     uint16_t* inv = reinterpret_cast<uint16_t*>(sb_start + L::kMaxSb);       // final position -> sorted position
     uint16_t* sorted_f = inv + kFoldSegKeys;                                              // fine bucket of sorted[q]
@@ -583,33 +603,56 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
         __syncthreads();
 
         // A. super-bucket of every point; its key goes to the next slot of the
-        // super-bucket's region (a shared-memory atomic per point: aggregating
-        // the lanes of a warp with equal super-buckets first measured slower)
-        const int64_t bs = blockDim.x;
-        for (int64_t g0 = 0; g0 < n; g0 += kFoldUnroll * bs) {
-            long long dl[kFoldUnroll];
-            float df[kFoldUnroll];
+        // super-bucket's region: one shared-memory atomic per point, or per
+        // warp where its points share the super-bucket.  Neighbours in time
+        // do at long periods, whose CTAs (several warps' points per cycle and
+        // super-bucket) look for it: 88 -> 63 thousand cycles of a 100-day
+        // period of 62,363 points; at 0.55 days, where no warp would, the
+        // look costs 51 -> 59.
+        auto scatter = [&](auto look) {
+            constexpr bool kLook = decltype(look)::value;
+            const int64_t bs = blockDim.x;
+            const int lane = threadIdx.x & 31;
+            for (int64_t g0 = 0; g0 < n; g0 += kFoldUnroll * bs) {
+                long long dl[kFoldUnroll];
+                float df[kFoldUnroll];
 #pragma unroll
-            for (int u = 0; u < kFoldUnroll; ++u) {
-                const int64_t i = g0 + u * bs + threadIdx.x;
-                dl[u] = i < n ? dc.d_lat[i] : 0;
-                df[u] = i < n ? dc.d_f[i] : 0.0f;
-            }
+                for (int u = 0; u < kFoldUnroll; ++u) {
+                    const int64_t i = g0 + u * bs + threadIdx.x;
+                    dl[u] = i < n ? dc.d_lat[i] : 0;
+                    df[u] = i < n ? dc.d_f[i] : 0.0f;
+                }
 #pragma unroll
-            for (int u = 0; u < kFoldUnroll; ++u) {
-                const int64_t i = g0 + u * bs + threadIdx.x;
-                const long long rho = lattice_rho(dl[u], df[u], P, inv_p);
-                const uint32_t sb = fold_fine(rho, sh, mulf) >> kFoldFineLog2;
-                const bool ok = i < n && in_range(dc.check, 2, rho, P) && in_range32(dc.check, 1, sb, nsb);
-                if (ok) {
-                    const uint32_t slot = atomicAdd(&sb_cnt[sb], 1u);
-                    if (slot < (uint32_t)kFoldSegKeys)
-                        keys[(int64_t)sb * kFoldSegKeys + slot] = ((unsigned long long)rho << ib) | (unsigned long long)i;
-                    else
-                        *overflow = 1;
+                for (int u = 0; u < kFoldUnroll; ++u) {
+                    const int64_t i = g0 + u * bs + threadIdx.x;
+                    const long long rho = lattice_rho(dl[u], df[u], P, inv_p);
+                    const uint32_t sb = fold_fine(rho, sh, mulf) >> kFoldFineLog2;
+                    const bool ok = i < n && in_range(dc.check, 2, rho, P) && in_range32(dc.check, 1, sb, nsb);
+                    uint32_t slot = 0;
+                    bool whole = false;
+                    if constexpr (kLook) {   // (every lane takes part in the exchanges)
+                        const uint32_t sb0 = __shfl_sync(0xffffffffu, sb, 0);
+                        whole = __all_sync(0xffffffffu, ok && sb == sb0);
+                        if (whole) {
+                            if (lane == 0) slot = atomicAdd(&sb_cnt[sb], 32u);
+                            slot = __shfl_sync(0xffffffffu, slot, 0) + (uint32_t)lane;
+                        }
+                    }
+                    if (ok) {
+                        if (!whole) slot = atomicAdd(&sb_cnt[sb], 1u);
+                        if (slot < (uint32_t)kFoldSegKeys)
+                            keys[(int64_t)sb * kFoldSegKeys + slot] =
+                                ((unsigned long long)rho << ib) | (unsigned long long)i;
+                        else
+                            *overflow = 1;
+                    }
                 }
             }
-        }
+        };
+        // points of a super-bucket in one cycle (for times in order)
+        const float cycles = fabsf(dc.d_f[n - 1] - dc.d_f[0]) * inv_p + 1.0f;
+        if ((float)n >= kFoldLookRun * cycles * (float)nsb) scatter(std::true_type{});
+        else scatter(std::false_type{});
         __syncthreads();
         if (*overflow) return false;
         {
@@ -639,7 +682,7 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
         const uint32_t k0 = single ? 0u : sb_start[sb], len = single ? (uint32_t)n : sb_cnt[sb];
         if (len == 0) continue;
         const unsigned long long* region = keys + (int64_t)sb * kFoldSegKeys;
-        for (int f = threadIdx.x; f < (1 << kFoldFineLog2); f += blockDim.x) fcnt[f] = 0;
+        for (int f = threadIdx.x; f < (1 << kFoldFineLog2); f += blockDim.x) fine[f] = 0;
         __syncthreads();
         // a thread's keys of the super-bucket and their fine buckets stay in
         // registers from the count to the scatter
@@ -677,7 +720,7 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
             const uint32_t f = fold_fine((long long)(kv[u] >> ib), sh, mulf) & kFineMask;
             if (u & 1) kf[u >> 1] |= f << 16;
             else kf[u >> 1] = f;
-            if (q < len) atomicAdd(&fcnt[f], 1u);
+            if (q < len) atomicAdd(&fine[f], 0x10000u);
         }
         __syncthreads();
         // every staged key of the super-bucket is in registers now: drop the
@@ -692,15 +735,17 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
         {
             constexpr int kPer = (1 << kFoldFineLog2) / kFoldThreads;
             const int f0 = threadIdx.x * kPer;
-            long long local = 0;
-#pragma unroll
-            for (int u = 0; u < kPer; ++u) local += fcnt[f0 + u];
-            long long sum;
-            long long run = block_exclusive_scan1(local, warp_sums, sum);
+            uint32_t c[kPer], local = 0;
 #pragma unroll
             for (int u = 0; u < kPer; ++u) {
-                fcur[f0 + u] = (uint32_t)run;
-                run += fcnt[f0 + u];
+                c[u] = fine[f0 + u];
+                local += c[u] >> 16;
+            }
+            uint32_t run = block_exclusive_scan32(local, reinterpret_cast<uint32_t*>(warp_sums));
+#pragma unroll
+            for (int u = 0; u < kPer; ++u) {
+                fine[f0 + u] = c[u] | run;
+                run += c[u] >> 16;
             }
         }
         __syncthreads();
@@ -709,18 +754,18 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
             const uint32_t q = threadIdx.x + u * kFoldThreads;
             if (q >= len) break;
             const uint32_t f = (kf[u >> 1] >> ((u & 1) * 16)) & 0xffffu;
-            const uint32_t d = atomicAdd(&fcur[f], 1u);   // fcur[f] ends as the end of bucket f
+            const uint32_t d = atomicAdd(&fine[f], 1u) & 0xffffu;   // the lower half ends as the end of bucket f
             if (in_range32(dc.check, 5, d, len)) {
                 sorted[d] = kv[u];
                 sorted_f[d] = (uint16_t)f;
             }
         }
         __syncthreads();
-        // rank inside the fine bucket: [fcur[f] - fcnt[f], fcur[f]) of sorted
+        // rank inside the fine bucket: [end - count, end) of sorted
         for (uint32_t q = threadIdx.x; q < len; q += blockDim.x) {
             const unsigned long long key = sorted[q];
             const uint32_t f = sorted_f[q];
-            const uint32_t cnt = fcnt[f], e = fcur[f];
+            const uint32_t cnt = fine[f] >> 16, e = fine[f] & 0xffffu;
             if (!in_range32(dc.check, 6, e, len + 1) || !in_range32(dc.check, 6, cnt, e + 1)) continue;
             const uint32_t lo = e - cnt;
             uint32_t rank = 0;
