@@ -24,6 +24,7 @@ struct alignas(16) BoundTab {
     float mean_all, nu_all;       // mean of s_k over the template, >= ||s_k - mean||
     float root_t2;                // sqrt(sum_k s_k^2)
     float t_max;                  // >= |s_k|
+    float change;                 // >= |s_0| + sum |s_k - s_{k-1}| + |s_{d-1}|
     int32_t cuts;                 // wide pieces (0: the window sum alone is tested)
     float cut_jumps, seg_jumps;   // sums of |mean - mean before| over the wide pieces, the segments
     float cut_nu[kBoundCuts];     // >= ||s_k - mean|| over the piece
@@ -73,6 +74,7 @@ struct DevPlan {
     const int32_t* stride;
     const int64_t* tmpl_off;
     const float* tmpl;
+    const float* tmpl_drop;   // s_{k-1} - s_k, k = 0 .. D (window search by bounds)
     const float* inv_sum_t;   // 1 / sum_k s_k
     const float* sum_t2;      // sum_k s_k^2
     const double* sum_t;      // FP64 sum_k s_k
@@ -106,6 +108,7 @@ struct DevCurve {
     int64_t* d_lat;           // rint((t - t_ref) 2^e)
     float* d_f;               // float(t - t_ref) (days): coarse cycle estimate
     PointVals* pv;            // rfx, r, w of every point
+    float* r;                 // r alone
     double* scal;             // [0] t_ref [1] chi2_0 [2] uniform weight w (0 if not uniform) [3] prefix shift (per-point
                               // weights: [3], [4] exponents of the units of the w r and w prefix sums)
     unsigned long long* tmin_key;  // ordered key of min(t)
@@ -128,9 +131,10 @@ struct DevChunk {
     float* ws;                // folded w (per-point weights only)
     float* wrs;               // folded w r (per-point weights only)
     long long* pf;            // prefix sums of rfx over the padded folded curve
-    // bounds kernel (uniform weights): the prefix sums in 32 bits, and what it
-    // leaves to sum in the wave
-    int32_t* pq;              // pf >> prefix_shift (modulo 2^32: window sums fit 31 bits)
+    // window search by bounds: prefix sums in 32 bits, and what it leaves to
+    // sum in the wave.  For uniform weights rs and pf are only written for
+    // periods that it leaves to the kernels that sum every window.
+    int32_t* pq;              // of r (per-point weights: w r) in units (modulo 2^32: window sums fit 31 bits)
     int64_t list_cap;         // windows per lane-group size
     unsigned long long* list; // windows to sum, kListClasses lists
     int2* dense;              // (slot, tile) items for the tiled kernel

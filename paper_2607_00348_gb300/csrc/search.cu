@@ -219,8 +219,8 @@ __device__ long long block_exclusive_scan1(long long v, long long* warp_sums, lo
     return (warp > 0 ? base : 0) + x - v;
 }
 
-// The same for 32-bit values, without the total.
-__device__ __forceinline__ uint32_t block_exclusive_scan32(uint32_t v, uint32_t* warp_sums)
+// The same for 32-bit values; the total only where it is asked for.
+__device__ __forceinline__ uint32_t block_exclusive_scan32(uint32_t v, uint32_t* warp_sums, uint32_t* total = nullptr)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t x = v;
@@ -231,7 +231,9 @@ __device__ __forceinline__ uint32_t block_exclusive_scan32(uint32_t v, uint32_t*
     }
     if (lane == 31) warp_sums[warp] = x;
     __syncthreads();
-    return __reduce_add_sync(0xffffffffu, lane < warp ? warp_sums[lane] : 0u) + x - v;
+    const uint32_t t = lane < (int)(blockDim.x >> 5) ? warp_sums[lane] : 0u;
+    if (total) *total = __reduce_add_sync(0xffffffffu, t);
+    return __reduce_add_sync(0xffffffffu, lane < warp ? t : 0u) + x - v;
 }
 
 // Light curve and period held by `slot` of a wave (segments ascend in
@@ -357,6 +359,7 @@ __global__ void k_curve_prep(const double* __restrict__ t, const double* __restr
         dc.d_lat[i] = __double2ll_rn(dt * scale);
         dc.d_f[i] = (float)dt;
         dc.pv[i] = PointVals{__double2ll_rn(r * kRScale), (float)r, (float)w};
+        dc.r[i] = (float)r;
         acc += w * r * r;
         wacc += w;
     }
@@ -475,8 +478,9 @@ struct FoldOut {
     float* ws;
     float* wrs;
     long long* pf;
-    int32_t* pq;              // 32-bit copy of pf, shifted right by `shift` (uniform weights)
+    int32_t* pq;              // kBounds: prefix sums of r in units of 2^(shift - 40), 32 bits
     int shift;
+    float per_unit;           // units of pq per unit of r
     bool uniform;
 };
 
@@ -594,6 +598,8 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
     uint16_t* sorted_f = inv + kFoldSegKeys;                                              // fine bucket of sorted[q]
     int* overflow = reinterpret_cast<int*>(sorted_f + kFoldSegKeys);
 
+    int* const sq = reinterpret_cast<int*>(srfx);   // kBounds: r in units, in fine-bucket order, then prefix sums
+
     // A single super-bucket (n <= kFoldSegKeys): its keys go straight to the
     // registers of step B.
     const bool single = nsb == 1;
@@ -668,7 +674,12 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
     // bucket, counting-sorted by fine bucket and ranked inside it, which
     // gives inv[final position] = sorted position; then, in final-position
     // order, the folded curve gathered (coalesced stores), rfx scanned and
-    // the prefix sums written.
+    // the prefix sums written.  When the bounds follow (kBounds) only the
+    // 32-bit prefix sums and the order are: r, rounded to their unit, is read
+    // where a key goes to its fine bucket, by lanes whose points are mostly
+    // neighbours in time, and moves with it.  A gather in folded order costs
+    // the L1 a cycle per point (130 of 660 thousand cycles of a period of
+    // 62,363 points); it is left to the few windows that are summed exactly.
     constexpr int kPerThread = kFoldSegKeys / kFoldThreads;
     static_assert(kFoldSegKeys % kFoldThreads == 0, "staged keys split evenly over the threads");
     static_assert(kPerThread == kScanPer, "one scan pass per super-bucket");
@@ -676,8 +687,9 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
     // srfx is read in blocks of kScanPer consecutive entries per thread; the
     // swizzle spreads the 16 lanes of a half-warp over 16 bank pairs
     auto swz = [](uint32_t i) { return i ^ ((i >> 4) & 7u); };
+    auto swz4 = [](uint32_t i) { return i ^ ((i >> 5) & 7u); };   // 32-bit values, 32 banks
     long long carry = 0;
-    if (threadIdx.x == 0) o.pf[0] = 0;
+    if (!kBounded && threadIdx.x == 0) o.pf[0] = 0;
     for (int sb = 0; sb < nsb; ++sb) {
         const uint32_t k0 = single ? 0u : sb_start[sb], len = single ? (uint32_t)n : sb_cnt[sb];
         if (len == 0) continue;
@@ -749,15 +761,29 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
             }
         }
         __syncthreads();
+        constexpr int kBatch = kBounded ? 4 : kPerThread;   // values in flight
 #pragma unroll
-        for (int u = 0; u < kPerThread; ++u) {
-            const uint32_t q = threadIdx.x + u * kFoldThreads;
-            if (q >= len) break;
-            const uint32_t f = (kf[u >> 1] >> ((u & 1) * 16)) & 0xffffu;
-            const uint32_t d = atomicAdd(&fine[f], 1u) & 0xffffu;   // the lower half ends as the end of bucket f
-            if (in_range32(dc.check, 5, d, len)) {
-                sorted[d] = kv[u];
-                sorted_f[d] = (uint16_t)f;
+        for (int h = 0; h < kPerThread; h += kBatch) {
+            float r[kBatch];
+            if (kBounded) {
+#pragma unroll
+                for (int u = 0; u < kBatch; ++u) {
+                    const uint32_t q = threadIdx.x + (h + u) * kFoldThreads;
+                    const uint32_t id = (uint32_t)(kv[h + u] & idx_mask);
+                    r[u] = q < len && id < (uint32_t)n ? __ldg(dc.r + id) : 0.0f;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kBatch; ++u) {
+                const uint32_t q = threadIdx.x + (h + u) * kFoldThreads;
+                if (q >= len) break;
+                const uint32_t f = (kf[(h + u) >> 1] >> (((h + u) & 1) * 16)) & 0xffffu;
+                const uint32_t d = atomicAdd(&fine[f], 1u) & 0xffffu;   // the lower half ends as the end of bucket f
+                if (in_range32(dc.check, 5, d, len)) {
+                    sorted[d] = kv[h + u];
+                    sorted_f[d] = (uint16_t)f;
+                    if (kBounded) sq[d] = __float2int_rn(r[u] * o.per_unit);
+                }
             }
         }
         __syncthreads();
@@ -773,73 +799,108 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
             if (in_range32(dc.check, 7, lo + rank, len)) inv[lo + rank] = (uint16_t)q;
         }
         __syncthreads();
-        // gather in final-position order (kRankBatch points' loads in flight;
-        // batches past the super-bucket's length skipped, block-uniform)
-#pragma unroll
-        for (int h = 0; h < kPerThread; h += kRankBatch) {
-            if ((uint32_t)h * kFoldThreads >= len) break;
-            int32_t id[kRankBatch];
-            bool ok[kRankBatch];
-#pragma unroll
-            for (int j = 0; j < kRankBatch; ++j) {
-                const uint32_t i = threadIdx.x + (h + j) * kFoldThreads;
-                ok[j] = false;
-                id[j] = 0;
-                if (i >= len) continue;
+        if constexpr (kBounded) {
+            for (uint32_t i = threadIdx.x; i < len; i += kFoldThreads) {
                 const uint32_t q = inv[i];
                 if (!in_range32(dc.check, 7, q, len)) continue;
-                id[j] = (int32_t)(sorted[q] & idx_mask);
-                ok[j] = in_range32(dc.check, 8, (uint32_t)id[j], (uint32_t)n);
+                const uint32_t id = (uint32_t)(sorted[q] & idx_mask);
+                if (in_range32(dc.check, 8, id, (uint32_t)n)) __stcs(o.sidx + (int64_t)k0 + i, (int32_t)id);
             }
-            PointVals pv[kRankBatch];
+        } else {
+            // gather in final-position order (kRankBatch points' loads in flight;
+            // batches past the super-bucket's length skipped, block-uniform)
 #pragma unroll
-            for (int j = 0; j < kRankBatch; ++j) pv[j] = ok[j] ? dc.pv[id[j]] : PointVals{0, 0.0f, 0.0f};
+            for (int h = 0; h < kPerThread; h += kRankBatch) {
+                if ((uint32_t)h * kFoldThreads >= len) break;
+                int32_t id[kRankBatch];
+                bool ok[kRankBatch];
 #pragma unroll
-            for (int j = 0; j < kRankBatch; ++j) {
-                const uint32_t i = threadIdx.x + (h + j) * kFoldThreads;
-                if (!ok[j]) continue;
-                const int64_t g = (int64_t)k0 + i;
-                // streaming stores: what the window kernels read after the
-                // whole chunk is folded comes from DRAM, so these lines go
-                // first when L2 needs room (the super-bucket regions stay, and
-                // what window_bounds reads right here)
-                __stcs(o.sidx + g, id[j]);
-                if (kBounded) o.rs[g] = pv[j].r;
-                else if (!kBoundedW) __stcs(o.rs + g, pv[j].r);
-                srfx[swz(i)] = pv[j].rfx;
-                if (kBoundedW) {
-                    o.ws[g] = pv[j].w;
-                    o.wrs[g] = pv[j].w * pv[j].r;
-                } else if (!kBounded && !o.uniform) {
-                    __stcs(o.ws + g, pv[j].w);
-                    __stcs(o.wrs + g, pv[j].w * pv[j].r);
+                for (int j = 0; j < kRankBatch; ++j) {
+                    const uint32_t i = threadIdx.x + (h + j) * kFoldThreads;
+                    ok[j] = false;
+                    id[j] = 0;
+                    if (i >= len) continue;
+                    const uint32_t q = inv[i];
+                    if (!in_range32(dc.check, 7, q, len)) continue;
+                    id[j] = (int32_t)(sorted[q] & idx_mask);
+                    ok[j] = in_range32(dc.check, 8, (uint32_t)id[j], (uint32_t)n);
+                }
+                PointVals pv[kRankBatch];
+#pragma unroll
+                for (int j = 0; j < kRankBatch; ++j) pv[j] = ok[j] ? dc.pv[id[j]] : PointVals{0, 0.0f, 0.0f};
+#pragma unroll
+                for (int j = 0; j < kRankBatch; ++j) {
+                    const uint32_t i = threadIdx.x + (h + j) * kFoldThreads;
+                    if (!ok[j]) continue;
+                    const int64_t g = (int64_t)k0 + i;
+                    // streaming stores: what the window kernels read after the
+                    // whole chunk is folded comes from DRAM, so these lines go
+                    // first when L2 needs room (the super-bucket regions stay, and
+                    // what window_bounds reads right here)
+                    __stcs(o.sidx + g, id[j]);
+                    if (!kBoundedW) __stcs(o.rs + g, pv[j].r);
+                    srfx[swz(i)] = pv[j].rfx;
+                    if (kBoundedW) {
+                        o.ws[g] = pv[j].w;
+                        o.wrs[g] = pv[j].w * pv[j].r;
+                    } else if (!o.uniform) {
+                        __stcs(o.ws + g, pv[j].w);
+                        __stcs(o.wrs + g, pv[j].w * pv[j].r);
+                    }
                 }
             }
+            __syncthreads();
         }
-        __syncthreads();
-        // inclusive prefix of rfx in final order, kScanPer consecutive
-        // entries per thread, written back in place
-        {
+        if constexpr (kBounded) {
+            // the same of the units: eight places of inv in two loads; every
+            // value is read before the scan's barrier, the sums written after it
             const uint32_t i0 = threadIdx.x * kScanPer;
-            long long v[kScanPer];
-            long long run = 0;
+            uint32_t at[kScanPer / 2];
+#pragma unroll
+            for (int u = 0; u < kScanPer / 4; ++u) {
+                const uint2 x = *reinterpret_cast<const uint2*>(inv + i0 + 4 * u);
+                at[2 * u] = x.x;
+                at[2 * u + 1] = x.y;
+            }
+            int v[kScanPer], run = 0;
 #pragma unroll
             for (int u = 0; u < kScanPer; ++u) {
-                run += i0 + u < len ? srfx[swz(i0 + u)] : 0;
+                const uint32_t q = (at[u >> 1] >> (16 * (u & 1))) & 0xffffu;
+                run += i0 + u < len ? sq[min(q, len - 1u)] : 0;
                 v[u] = run;
             }
-            long long sum;
-            const long long ex = block_exclusive_scan1(run, warp_sums, sum) + carry;
+            uint32_t sum;
+            const int ex = (int)block_exclusive_scan32((uint32_t)run, reinterpret_cast<uint32_t*>(warp_sums), &sum) +
+                           (int)carry;
 #pragma unroll
             for (int u = 0; u < kScanPer; ++u)
-                if (i0 + u < len) srfx[swz(i0 + u)] = ex + v[u];
-            carry += sum;
-        }
-        __syncthreads();
-        for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) {
-            const long long v = srfx[swz(i)];
-            __stcs(o.pf + (int64_t)k0 + 1 + i, v);
-            if (kBounded) o.pq[(int64_t)k0 + 1 + i] = (int32_t)(v >> o.shift);
+                if (i0 + u < len) sq[swz4(i0 + u)] = ex + v[u];
+            carry += (int)sum;
+            __syncthreads();
+            for (uint32_t i = threadIdx.x; i < len; i += kFoldThreads) o.pq[(int64_t)k0 + 1 + i] = sq[swz4(i)];
+        } else {
+            // inclusive prefix of rfx in final order, kScanPer consecutive
+            // entries per thread, written back in place
+            {
+                const uint32_t i0 = threadIdx.x * kScanPer;
+                long long v[kScanPer];
+                long long run = 0;
+#pragma unroll
+                for (int u = 0; u < kScanPer; ++u) {
+                    run += i0 + u < len ? srfx[swz(i0 + u)] : 0;
+                    v[u] = run;
+                }
+                long long sum;
+                const long long ex = block_exclusive_scan1(run, warp_sums, sum) + carry;
+#pragma unroll
+                for (int u = 0; u < kScanPer; ++u)
+                    if (i0 + u < len) srfx[swz(i0 + u)] = ex + v[u];
+                carry += sum;
+            }
+            __syncthreads();
+            for (uint32_t i = threadIdx.x; i < len; i += blockDim.x) {
+                __stcs(o.pf + (int64_t)k0 + 1 + i, srfx[swz(i)]);
+            }
         }
         __syncthreads();   // the next super-bucket overwrites the staged keys and rfx
     }
@@ -1012,7 +1073,7 @@ __device__ void fold_global(unsigned char* smem, const DevPlan& dp, const DevCur
 
 template <Fold kFold, int T>
 __global__ void __launch_bounds__(T, kFoldThreads * kFoldMinBlocks / T)
-k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk, int tile_buf)
+k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk, int tile_buf, int fill)
 {
     constexpr bool kBounded = kFold == Fold::kBounds, kBoundedW = kFold == Fold::kBoundsW;
     const SlotMap& sm = smq ? *smq : smv;
@@ -1032,6 +1093,7 @@ k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, 
     o.pq = dk.pq + (int64_t)slot_id * dk.pad_stride;
     o.uniform = dc.scal[2] > 0.0;
     o.shift = kBounded ? min((int)dc.scal[3], 63) : 0;
+    o.per_unit = kBounded ? 1.0f / prefix_unit(o.shift) : 0.0f;
     if (threadIdx.x == 0) {
         ds.outs[lc].best[p] = ~0ull;
         if (kFold != Fold::kPlain && slot_id == 0)
@@ -1043,31 +1105,34 @@ k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, 
         __syncthreads();   // the global path reuses the shared memory
         fold_global(smem, dp, dc, p, keys, o);
         __syncthreads();
-        if (kBounded)
+        if (kBounded) {
             for (int64_t k = threadIdx.x + 1; k <= dp.n; k += blockDim.x) o.pq[k] = (int32_t)(o.pf[k] >> o.shift);
+            __syncthreads();   // (the padding reads them)
+        }
     }
     if (kBounded && threadIdx.x == 0) o.pq[0] = 0;
 
     // padding: the first D_m folded points repeat after position N-1
     const int64_t n = dp.n;
     const int64_t dm = dp.dmax_p[p];
-    const long long tot = o.pf[n];
-    for (int64_t k = threadIdx.x; k < dm + kPadMargin; k += blockDim.x) {
-        const bool real = k < dm;
-        if (!kBoundedW) o.rs[n + k] = real ? o.rs[k] : 0.0f;
-        if (!o.uniform) {
-            o.ws[n + k] = real ? o.ws[k] : 0.0f;
-            o.wrs[n + k] = real ? o.wrs[k] : 0.0f;
-        }
-        if (real) {
-            const long long v = tot + o.pf[k + 1];
-            o.pf[n + k + 1] = v;
-            if (kBounded) o.pq[n + k + 1] = (int32_t)(v >> o.shift);
+    if constexpr (kBounded) {
+        const int tot = o.pq[n];
+        for (int64_t k = threadIdx.x; k < dm; k += blockDim.x) o.pq[n + k + 1] = tot + o.pq[k + 1];
+    } else {
+        const long long tot = o.pf[n];
+        for (int64_t k = threadIdx.x; k < dm + kPadMargin; k += blockDim.x) {
+            const bool real = k < dm;
+            if (!kBoundedW) o.rs[n + k] = real ? o.rs[k] : 0.0f;
+            if (!o.uniform) {
+                o.ws[n + k] = real ? o.ws[k] : 0.0f;
+                o.wrs[n + k] = real ? o.wrs[k] : 0.0f;
+            }
+            if (real) o.pf[n + k + 1] = tot + o.pf[k + 1];
         }
     }
     if (kFold != Fold::kPlain) {
         __syncthreads();
-        bounds::window_bounds<T, kBoundedW>(smem, ds, dk, slot_id, lc, p, tile_buf);
+        bounds::window_bounds<T, kBoundedW>(smem, ds, dk, slot_id, lc, p, tile_buf, fill != 0);
     }
 }
 
@@ -1792,37 +1857,75 @@ k_window_tc(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, 
 // per-period result: chi2(P), depth, T0 of the minimum
 // ---------------------------------------------------------------------------
 
+// Window of the minimum of period p: its duration and first point (false: a
+// failed check).
+__device__ __forceinline__ bool best_window(const DevPlan& dp, const DevCurve& dc, const DevPeriod& dq, int p,
+                                            int64_t pad_stride, int& j, int64_t& s)
+{
+    const unsigned long long b = dq.best[p];
+    j = (int)((b >> 24) & 0xffull);
+    if (!in_range(dc.check, 13, j, dp.nd)) return false;
+    s = (int64_t)(b & 0xffffffull) * dp.stride[j];
+    return in_range(dc.check, 14, s + dp.dpts[j], pad_stride);
+}
+
+// The period's outputs (sfx: exact sum of r over the window).
+__device__ __forceinline__ void finish_period(const DevPlan& dp, const DevCurve& dc, const DevPeriod& dq, int p,
+                                              const int32_t* sidx, int j, int64_t s, long long sfx)
+{
+    const int64_t n = dp.n;
+    const double depth = fmax(0.0, (double)sfx * (1.0 / kRScale) / dp.sum_t[j]);
+    const int32_t idx = sidx[(s + dp.dpts[j] / 2) % n];
+    if (!in_range(dc.check, 15, idx, n)) return;
+    const long long rho = lattice_rho(dc.d_lat[idx], dc.d_f[idx], dp.p_lat[p], dp.inv_p[p]);
+    dq.chi2[p] = dc.scal[1] + (double)float_from_order_key((unsigned int)(dq.best[p] >> 32));
+    dq.dur[p] = j;
+    dq.t0i[p] = (int32_t)s;
+    dq.depth[p] = depth;
+    dq.t0[p] = dc.scal[0] + ldexp((double)rho, -dp.time_exponent);
+}
+
 __global__ void k_period_finalize(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk)
 {
     const SlotMap& sm = smq ? *smq : smv;
     const int slot_id = blockIdx.x * blockDim.x + threadIdx.x;
     if (slot_id >= sm.slots) return;
-    int lc, p;
+    int lc, p, j;
+    int64_t s;
     if (!resolve_slot(ds, sm, slot_id, lc, p)) return;
     const DevPlan& dp = ds.plans[lc];
-    const DevCurve dc = ds.curves[lc];
-    const DevPeriod dq = ds.outs[lc];
-    const unsigned long long b = dq.best[p];
-    const float dchi = float_from_order_key((unsigned int)(b >> 32));
-    const int j = (int)((b >> 24) & 0xffull);
-    const int64_t m = (int64_t)(b & 0xffffffull);
-    if (!in_range(dc.check, 13, j, dp.nd)) return;
-    const int d = dp.dpts[j], st = dp.stride[j];
-    const int64_t s = m * st;
-    const int64_t n = dp.n;
-    if (!in_range(dc.check, 14, s + d, dk.pad_stride)) return;
+    if (!best_window(dp, ds.curves[lc], ds.outs[lc], p, dk.pad_stride, j, s)) return;
     const long long* pf = dk.pf + (int64_t)slot_id * dk.pad_stride;
-    const double sum_r = (double)(pf[s + d] - pf[s]) * (1.0 / kRScale);
-    const double depth = fmax(0.0, sum_r / dp.sum_t[j]);
-    const int64_t c = (s + d / 2) % n;
-    const int32_t idx = dk.sidx[(int64_t)slot_id * dk.fold_stride + c];
-    if (!in_range(dc.check, 15, idx, n)) return;
-    const long long rho = lattice_rho(dc.d_lat[idx], dc.d_f[idx], dp.p_lat[p], dp.inv_p[p]);
-    dq.chi2[p] = dc.scal[1] + (double)dchi;
-    dq.dur[p] = j;
-    dq.t0i[p] = (int32_t)s;
-    dq.depth[p] = depth;
-    dq.t0[p] = dc.scal[0] + ldexp((double)rho, -dp.time_exponent);
+    finish_period(dp, ds.curves[lc], ds.outs[lc], p, dk.sidx + (int64_t)slot_id * dk.fold_stride, j, s,
+                  pf[s + dp.dpts[j]] - pf[s]);
+}
+
+// After the window search by bounds (uniform weights), which leaves no exact
+// prefix sums: a warp per period adds the window's points, by their places in
+// the folded order.
+__global__ void __launch_bounds__(128)
+k_period_finalize_sum(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk)
+{
+    const SlotMap& sm = smq ? *smq : smv;
+    const int slot_id = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (slot_id >= sm.slots) return;   // (warp-uniform, as all that follows)
+    int lc, p, j;
+    int64_t s;
+    if (!resolve_slot(ds, sm, slot_id, lc, p)) return;
+    const DevPlan& dp = ds.plans[lc];
+    if (!best_window(dp, ds.curves[lc], ds.outs[lc], p, dk.pad_stride, j, s)) return;
+    const int32_t* const sidx = dk.sidx + (int64_t)slot_id * dk.fold_stride;
+    const PointVals* const pv = ds.curves[lc].pv;
+    const int n = (int)dp.n, d = dp.dpts[j];
+    long long sum = 0;
+#pragma unroll 8
+    for (int k = lane; k < d; k += 32) {
+        const int at = (int)s + k, id = sidx[at < n ? at : at - n];
+        sum += id >= 0 && id < n ? pv[id].rfx : 0;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) finish_period(dp, ds.curves[lc], ds.outs[lc], p, sidx, j, s, sum);
 }
 
 // ---------------------------------------------------------------------------
@@ -2579,6 +2682,9 @@ void bound_tables(const float* s, int j, int d, int st, int64_t n, int clg, int 
     for (int g = 0; g < kBoundSegs; ++g) b.seg_low[g] = (float)least(off[g], off[g + 1]);
     b.nu_all = piece(0, d, b.mean_all);
     b.root_t2 = (float)std::sqrt(t2);
+    double change = std::fabs((double)s[0]) + std::fabs((double)s[d - 1]);
+    for (int k = 1; k < d; ++k) change += std::fabs((double)s[k] - s[k - 1]);
+    b.change = (float)(change * (1.0 + 1e-6));
     b.t_max = (float)(top * (1.0 + 1e-6));
 
     bd.j = j;
@@ -2771,6 +2877,7 @@ gtls_status create_device(gtls_plan* pl)
     GTLS_TRY(dev_alloc(pl, &dc.d_lat, n));
     GTLS_TRY(dev_alloc(pl, &dc.d_f, n));
     GTLS_TRY(dev_alloc(pl, &dc.pv, n));
+    GTLS_TRY(dev_alloc(pl, &dc.r, n));
     GTLS_TRY(dev_alloc(pl, &dc.scal, 8));
     GTLS_TRY(dev_alloc(pl, &dc.tmin_key, 1));
     GTLS_TRY(dev_alloc(pl, &dc.flags, 1));
@@ -3099,6 +3206,17 @@ gtls_status create_device(gtls_plan* pl)
             GTLS_TRY(upload(pl, const_cast<BoundTab**>(&q.bounds), tab));
             GTLS_TRY(upload(pl, const_cast<BoundDur**>(&q.bound_durs), bd));
         }
+        if (pl->bounds_ok) {
+            // s_{k-1} - s_k of every template (0 before and after it), where dp.tmpl has s_k
+            std::vector<float> drop(pl->tmpl_pad.size(), 0.0f);
+            for (int j = 0; j < dp.nd; ++j) {
+                const float* const tj = pl->tmpl_pad.data() + pl->tmpl_pad_off[j];
+                for (int k = 0; k <= h.dpts[j]; ++k)
+                    drop[(size_t)(pl->tmpl_pad_off[j] + k)] = (float)((k > 0 ? (double)tj[k - 1] : 0.0) - tj[k]);
+            }
+            GTLS_TRY(upload(pl, const_cast<float**>(&dp.tmpl_drop), drop));
+            pl->dp_ref.tmpl_drop = dp.tmpl_drop;
+        }
         // (the 32-bit prefix sums of w take the fold's keys' place)
         pl->bounds_w_ok = pl->bounds_ok && pl->tile_w_ok && !pl->has_window_only &&
                           4 * (n + h.dmax + 16) <= 8 * pl->dk.key_stride;
@@ -3290,21 +3408,21 @@ gtls_status stage_mark(Ctx& c, int stage)
 }
 
 template <Fold kFold, int T>
-void launch_fold_as(Ctx& c, const DevSet& ds, const SlotMap& sm, const SlotMap* smq)
+void launch_fold_as(Ctx& c, const DevSet& ds, const SlotMap& sm, const SlotMap* smq, bool fill)
 {
     int smem = T == kFoldThreads ? c.fold_smem : FoldCfg<T>::kStagedBytes;
     if (kFold != Fold::kPlain) smem = std::max(smem, (int)bounds::smem_bytes(T));
-    k_fold_sort<kFold, T><<<sm.slots, T, smem, c.st>>>(ds, sm, smq, c.dk, c.tile_buf);
+    k_fold_sort<kFold, T><<<sm.slots, T, smem, c.st>>>(ds, sm, smq, c.dk, c.tile_buf, fill ? 1 : 0);
 }
 
 // The fold of one wave (with the first steps of the window search when
 // by bounds) in CTAs of `threads` threads.
 template <Fold kFold>
-void launch_fold(Ctx& c, const DevSet& ds, const SlotMap& sm, const SlotMap* smq, int threads)
+void launch_fold(Ctx& c, const DevSet& ds, const SlotMap& sm, const SlotMap* smq, int threads, bool fill = false)
 {
-    if (threads == 256) launch_fold_as<kFold, 256>(c, ds, sm, smq);
-    else if (threads == 512) launch_fold_as<kFold, 512>(c, ds, sm, smq);
-    else launch_fold_as<kFold, 1024>(c, ds, sm, smq);
+    if (threads == 256) launch_fold_as<kFold, 256>(c, ds, sm, smq, fill);
+    else if (threads == 512) launch_fold_as<kFold, 512>(c, ds, sm, smq, fill);
+    else launch_fold_as<kFold, 1024>(c, ds, sm, smq, fill);
 }
 
 // One wave: fold + sort, every window, per-period results.  `counter` must
@@ -3321,7 +3439,7 @@ gtls_status wave_pass(Ctx& c, bool ref, const SlotMap& sm, bool tiled, bool weig
     const int threads = fold_threads(max_n);
     if (!bounded) launch_fold<Fold::kPlain>(c, ds, sm, smq, threads);
     else if (weighted) launch_fold<Fold::kBoundsW>(c, ds, sm, smq, threads);
-    else launch_fold<Fold::kBounds>(c, ds, sm, smq, threads);
+    else launch_fold<Fold::kBounds>(c, ds, sm, smq, threads, window_only);   // (that kernel reads every folded curve)
     GTLS_CUDA(cudaGetLastError());
     GTLS_TRY(stage_mark(c, kStageFold));
     if (tiled) {
@@ -3332,9 +3450,12 @@ gtls_status wave_pass(Ctx& c, bool ref, const SlotMap& sm, bool tiled, bool weig
             // as many windows at a time as their points and templates leave room for
             const int per = 2 * (int)(weighted ? sizeof(float2) : sizeof(float));
             const int room = (int)std::min<int64_t>((c.max_d + 3) & ~3, bounds::kExactRoom * 8 / per);
-            const int ctas = std::max(1, std::min(16, 200000 / (room * per + 1024)));
+            // uniform weights: 16 points of the longest window per thread to fetch
+            int team = 32;
+            while (!weighted && team < bounds::kExactThreads && team * 16 < c.max_d) team *= 2;
+            const int ctas = std::max(1, std::min({16, 2048 / team, 200000 / (room * per + 1024)}));
             auto* const exact = weighted ? bounds::k_window_exact_w : bounds::k_window_exact;
-            exact<<<c.n_sm * ctas, 32, room * per, c.st>>>(ds, sm, smq, c.dk, room);
+            exact<<<c.n_sm * ctas, team, room * per, c.st>>>(ds, sm, smq, c.dk, room);
             GTLS_CUDA(cudaGetLastError());
             c.launches += 1;
         }
@@ -3362,7 +3483,8 @@ gtls_status wave_pass(Ctx& c, bool ref, const SlotMap& sm, bool tiled, bool weig
     }
     GTLS_CUDA(cudaGetLastError());
     GTLS_TRY(stage_mark(c, kStageWindow));
-    k_period_finalize<<<(sm.slots + 127) / 128, 128, 0, c.st>>>(ds, sm, smq, c.dk);
+    if (bounded && !weighted) k_period_finalize_sum<<<(sm.slots + 3) / 4, 128, 0, c.st>>>(ds, sm, smq, c.dk);
+    else k_period_finalize<<<(sm.slots + 127) / 128, 128, 0, c.st>>>(ds, sm, smq, c.dk);
     GTLS_CUDA(cudaGetLastError());
     GTLS_TRY(stage_mark(c, kStageFinalize));
     c.launches += 3;

@@ -74,6 +74,7 @@ constexpr int kCand = 2;            // windows summed for the threshold
 constexpr int kRowBuf = 168;        // prefix sums at whole T0 steps a warp stages for one group
 constexpr int kCutPoints = 60;      // windows of at least this many points are first tested by wide pieces
 constexpr int kCoarseSteps = 64;    // ... and from this many coarse steps on from the coarse prefix
+constexpr int kExactThreads = 256;
 constexpr int kExactRoom = 24576;   // points of a window (and its template) staged by k_window_exact, at most
 constexpr int kFloorSpans = 48;     // stretches of blocks whose smallest weight is kept: 1 .. 15, then 16, 19, 22,
                                     // 27 times powers of 2
@@ -177,8 +178,9 @@ __device__ __forceinline__ int at_coarse(int e) { return e + (e >> 5); }
 // kernel; every lane of the group returns the totals (y: window sum of the
 // (C1, S) pairs).  Lanes of groups that are not `on` only take part in the
 // exchanges.
-__device__ __forceinline__ float2 window_sum(const float* __restrict__ r, const float* __restrict__ t, int d, int st,
-                                             int lg_nc, int mode, int rot, bool on, int lane)
+template <typename Value>
+__device__ __forceinline__ float2 window_sum(Value r, const float* __restrict__ t, int d, int st, int lg_nc, int mode,
+                                             int rot, bool on, int lane)
 {
     const int nc = 1 << lg_nc, c = lane & (nc - 1);
     float x = 0.0f, y = 0.0f;
@@ -187,7 +189,7 @@ __device__ __forceinline__ float2 window_sum(const float* __restrict__ r, const 
             for (int rho = c; rho < st; rho += nc) {
 #pragma unroll 8
                 for (int k = rho; k < d; k += st) {
-                    const float v = r[k];
+                    const float v = r(k);
                     x = fmaf(v, t[k], x);
                     y = v + y;
                 }
@@ -195,7 +197,7 @@ __device__ __forceinline__ float2 window_sum(const float* __restrict__ r, const 
         } else if (mode == kModeWin) {
             for (int rho = c; rho < st; rho += nc) {
 #pragma unroll 8
-                for (int k = rho; k < d; k += st) x = fmaf(r[k], t[k], x);
+                for (int k = rho; k < d; k += st) x = fmaf(r(k), t[k], x);
             }
         } else {
             const int rounds = (st + 2 * nc - 1) >> (lg_nc + 1);
@@ -208,10 +210,10 @@ __device__ __forceinline__ float2 window_sum(const float* __restrict__ r, const 
                 int k = rho;
 #pragma unroll 8
                 for (; k < both; k += st) {
-                    x = fmaf(r[k], t[k], x);
-                    y = fmaf(r[k + nc], t[k + nc], y);
+                    x = fmaf(r(k), t[k], x);
+                    y = fmaf(r(k + nc), t[k + nc], y);
                 }
-                for (; k < end; k += st) x = fmaf(r[k], t[k], x);
+                for (; k < end; k += st) x = fmaf(r(k), t[k], x);
             }
         }
     }
@@ -592,7 +594,7 @@ __device__ __forceinline__ float weight_floor(const Smem<T>& S, int len, int lb)
 // Steps 1 to 4 for one period, by a CTA of T threads (kW: per-point weights).
 template <int T, bool kW>
 __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet& ds, const DevChunk& dk, int slot, int lc,
-                                              int p, int buf)
+                                              int p, int buf, bool fill)
 {
     using M = Smem<T>;
     constexpr int kWarps = T / 32;
@@ -604,7 +606,7 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
     const int n = (int)dp.n;
     const int total = n + dp.dmax_p[p];
     float* const rb = S.row_buf + warp * kRowBuf;
-    const float* const rs = (kW ? dk.wrs : dk.rs) + (int64_t)slot * dk.pad_stride;   // what C1 sums
+    const float* const rs = kW ? dk.wrs + (int64_t)slot * dk.pad_stride : nullptr;   // what C1 sums
     const float* const ws = kW ? dk.ws + (int64_t)slot * dk.pad_stride : nullptr;
     const int* const pq = dk.pq + (int64_t)slot * dk.pad_stride;
     // (the fold is through with its keys)
@@ -619,6 +621,17 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
     const float unit_a = kW ? ldexpf(1.0f, in_range_32 ? shift : 0) : 1.0f;
     const float unit_w = kW ? ldexpf(1.0f, in_range_32 ? shift_w : 0) : 1.0f;
     const int lg = dp.bound_lg;
+    // a sum of len points by the 32-bit prefix is off by at most this: half a
+    // unit per point, and for uniform weights the rounding of r to FP32 (units
+    // add up to at most 2^30 in size) and to the fixed point of exact sums
+    auto sum_blur = [&](int len) {
+        return (0.5f * (float)len + (kW ? 1.0f : 64.0f)) * unit + (kW ? 0.0f : 5e-13f * (float)len);
+    };
+    // depth of a window: exact (kW), or from the 32-bit prefix
+    auto depth_of = [&](int s, int d, float inv) {
+        if (kW) return fmaxf(0.0f, tiles::fixed_to_float(pf[s + d] - pf[s]) * (inv * (1.0f / 1099511627776.0f)));
+        return fmaxf(0.0f, (float)(pq[s + d] - pq[s]) * unit * inv);
+    };
 
     if (warp == 0) {
         list_durations(dp, ds.curves[lc].check, p, n, dur, S.ck, lane);
@@ -815,14 +828,22 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         float c1 = 0.0f, sum = 0.0f;
         if (cand >= 0) {
             const BoundDur& t = dur[cand >> 24].b;
-            const float* const r = rs + (cand & 0xffffff) * t.st;
-            const float* const w = ws + (cand & 0xffffff) * t.st;
-            const float* const s = dp.tmpl + dp.tmpl_off[t.j];
+            const int at = (cand & 0xffffff) * t.st;
+            if constexpr (kW) {
+                const float* const s = dp.tmpl + dp.tmpl_off[t.j];
 #pragma unroll 8
-            for (int i = threadIdx.x % kTeamThreads; i < t.d; i += kTeamThreads) {
-                const float v = r[i], sv = __ldg(s + i);
-                c1 = fmaf(v, sv, c1);
-                sum = kW ? fmaf(w[i], sv * sv, sum) : sum + v;   // C2, or the window sum
+                for (int i = threadIdx.x % kTeamThreads; i < t.d; i += kTeamThreads) {
+                    const float sv = __ldg(s + i);
+                    c1 = fmaf(rs[at + i], sv, c1);
+                    sum = fmaf(ws[at + i], sv * sv, sum);   // C2
+                }
+            } else {
+                // sum r s_k = sum (P_k - P_0) (s_{k-1} - s_k): r itself is not there
+                const float* const s = dp.tmpl_drop + dp.tmpl_off[t.j];
+                const int base = pq[at];
+#pragma unroll 8
+                for (int i = threadIdx.x % kTeamThreads; i <= t.d; i += kTeamThreads)
+                    c1 = fmaf((float)(pq[at + i] - base), __ldg(s + i), c1);
             }
         }
 #pragma unroll
@@ -842,12 +863,20 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         const int lg = kW ? __ffs(dp.cfg_nc_w[t.b.j]) - 1 : t.b.lg_nc, nc = 1 << lg;
         return ((t.b.st + nc - 1) >> lg) * ((t.b.d + t.b.st - 1) / t.b.st) + 6;
     };
+    // (uniform weights: the sums here are those of the rounded r)
     auto blur_of = [&](const Dur& t, int chain, float norm) {
-        return ((sum_slack(chain) + sum_slack(t.b.d / 32 + 8)) * norm + (kW ? 0.0f : (float)t.b.d * 1e-12f)) *
-               fmaxf(dp.bounds[t.b.j].t_max, 1.0f) * unit_a;
+        const float t_max = fmaxf(dp.bounds[t.b.j].t_max, 1.0f);
+        const float here = sum_slack(t.b.d / 32 + 8);
+        if (kW) return (sum_slack(chain) + here) * norm * t_max * unit_a;
+        return (sum_slack(chain) * norm + sum_blur(t.b.d)) * t_max +
+               (here + 3e-7f) * (norm + sum_blur(t.b.d)) * dp.bounds[t.b.j].change;
     };
     auto c2_slack_of = [&](const Dur& t, int chain) {
         return kW ? sum_slack(chain) + sum_slack(t.b.d / 32 + 8) + 1e-6f : 1e-6f;
+    };
+    // what the depth of depth_of can be off by (kW: nothing, it is exact)
+    auto depth_blur = [&](const Dur& t, float off, float inv) {
+        return kW ? 0.0f : (t.b.mode == kModePairS ? off : 0.0f) * inv + sum_blur(t.b.d) * inv;
     };
     if (threadIdx.x == 0) {
         float thr = INFINITY;
@@ -860,17 +889,14 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
                 c1 += S.c1[w];
                 sum += S.s[w];
             }
-            float depth = sum * dp.inv_sum_t[j];
-            if (kW) {
-                const int s = (S.cand[q] & 0xffffff) * t.b.st;
-                depth = tiles::fixed_to_float(pf[s + t.b.d] - pf[s]) * (dp.inv_sum_t[j] * (1.0f / 1099511627776.0f));
-            }
-            depth = fmaxf(0.0f, depth);
+            if (!kW) c1 *= unit;
+            const int s = (S.cand[q] & 0xffffff) * t.b.st;
+            const float depth = depth_of(s, t.b.d, dp.inv_sum_t[j]);
             const float t2 = kW ? sum : dp.sum_t2[j];
             const int chain = chain_of(t);
             const float off = blur_of(t, chain, sqrtf((float)t.b.d * energy_of(t.b.d)));
             float v = w_uni * depth * fmaf(depth, t2, -2.0f * c1);
-            v += sum_error(w_uni, depth, t2, c1, v, off, kW ? 0.0f : off * dp.inv_sum_t[j], c2_slack_of(t, chain));
+            v += sum_error(w_uni, depth, t2, c1, v, off, depth_blur(t, off, dp.inv_sum_t[j]), c2_slack_of(t, chain));
             thr = v < thr || isnan(v) ? v : thr;
         }
         S.thr = thr;
@@ -894,7 +920,7 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
             const int d = t.b.d, st = t.b.st, chain = chain_of(t);
             t.emax = energy_of(d);
             const float norm = sqrtf((float)d * t.emax);
-            const float lost = (sum_slack(chain) + 8e-6f) * norm + (float)d * (kW ? 0.5f : 1e-12f);
+            const float lost = (sum_slack(chain) + 8e-6f) * norm + sum_blur(d);
             t.c2_slack = c2_slack_of(t, chain);
             float root_c2 = bt.root_t2;
             if (kW) {
@@ -907,7 +933,7 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
             t.cmin = reach * root_c2 - (lost + (float)(kBoundSegs + 1) * unit) * bt.t_max;
             t.blur = blur_of(t, chain, norm);
             // depth is zero without a positive sum (exact, or FP32 for the pairs)
-            const float low = kW ? -INFINITY : (t.b.mode == kModePairS ? -lost : 0.0f) - 2.0f * unit;
+            const float low = kW ? -INFINITY : (t.b.mode == kModePairS ? -lost : 0.0f) - sum_blur(d);
             float c0;
             if (t.b.test == kTestSum) {
                 c0 = fmaxf((t.cmin - bt.nu_all * sqrtf(t.emax)) / bt.mean_all, low);
@@ -1052,7 +1078,7 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
                 const int nx = pq[e1];
                 const float sg = (float)(nx - last) * unit;
                 const float en = fmaf(S.pre[(e1 + bsize - 1) >> lb] - S.pre[e0 >> lb], 1.0f + e_rel, e_abs);
-                const float sm = fmaxf(fabsf(sg) - unit, 0.0f);
+                const float sm = fmaxf(fabsf(sg) - (1.0f + 0.5f * (float)(e1 - e0)) * unit, 0.0f);
                 c1 += fmaf(q.y, sg, q.z * root(en - q.w * sm * sm));
                 last = nx;
                 e0 = e1;
@@ -1076,20 +1102,21 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
             const unsigned int e = S.fin[i];
             const Dur& t = dur[e >> 24];
             const int s = (int)(e & 0xffffffu) * t.b.st, d = t.b.d;
-            const float* const r = rs + s;
-            const float* const tm = dp.tmpl + dp.tmpl_off[t.b.j];
-            const long long sfx = pf[s + d] - pf[s];
             float c1 = 0.0f, c2 = 0.0f;
             if (kW) {
+                const float* const tm = dp.tmpl + dp.tmpl_off[t.b.j];
 #pragma unroll 8
                 for (int q = lane; q < d; q += 32) {
                     const float sv = __ldg(tm + q);
-                    c1 = fmaf(r[q], sv, c1);
+                    c1 = fmaf(rs[s + q], sv, c1);
                     c2 = fmaf(ws[s + q], sv * sv, c2);
                 }
             } else {
+                const float* const tm = dp.tmpl_drop + dp.tmpl_off[t.b.j];
+                const int base = pq[s];
 #pragma unroll 16
-                for (int q = lane; q < d; q += 32) c1 = fmaf(r[q], __ldg(tm + q), c1);
+                for (int q = lane; q <= d; q += 32) c1 = fmaf((float)(pq[s + q] - base), __ldg(tm + q), c1);
+                c1 *= unit;
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
@@ -1097,10 +1124,9 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
                 if (kW) c2 += __shfl_xor_sync(0xffffffffu, c2, o);
             }
             const float inv = dp.inv_sum_t[t.b.j], t2 = kW ? c2 : dp.sum_t2[t.b.j];
-            const float depth = fmaxf(0.0f, tiles::fixed_to_float(sfx) * (inv * (1.0f / 1099511627776.0f)));
+            const float depth = depth_of(s, d, inv);
             const float v = w_uni * depth * fmaf(depth, t2, -2.0f * c1);
-            // C1 is off by at most blur, the depth of the pairs by blur / sum s_k
-            const float off = t.blur, dd = !kW && t.b.mode == kModePairS ? off * inv : 0.0f;
+            const float off = t.blur, dd = depth_blur(t, off, inv);
             const float err = sum_error(w_uni, depth, t2, c1, v, off, dd, t.c2_slack);
             if (lane == 0) S.fin_v[i] = v - err;
             odd = odd || !(v - err > -INFINITY && v + err < INFINITY);
@@ -1156,18 +1182,41 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         const unsigned int to = atomicAdd(dk.left_n + kListClasses, (unsigned int)tc);
         for (int tau = 0; tau < tc; ++tau) dk.dense[to + tau] = make_int2(slot, tau);
     }
+    if (!kW && (fill || !fits)) {
+        // the folded curve itself and its exact prefix sums, for the kernels
+        // that sum every window
+        float* const r = dk.rs + (int64_t)slot * dk.pad_stride;
+        long long* const sums = dk.pf + (int64_t)slot * dk.pad_stride;
+        const int* const sidx = dk.sidx + (int64_t)slot * dk.fold_stride;
+        const PointVals* const pv = ds.curves[lc].pv;
+        long long* const scratch = reinterpret_cast<long long*>(smem);   // (dur[] is not read any more)
+        __syncthreads();
+        long long carry = 0;
+        for (int k0 = 0; k0 < total + (int)kPadMargin; k0 += T) {
+            const int k = k0 + threadIdx.x;
+            const int id = k < total ? sidx[k < n ? k : k - n] : -1;
+            const PointVals v = id >= 0 && id < n ? pv[id] : PointVals{0, 0.0f, 0.0f};
+            const long long before = block_exclusive_scan(v.rfx, scratch, scratch + 32) + carry;
+            if (k <= total) sums[k] = before;
+            if (k < total + (int)kPadMargin) r[k] = v.r;
+            carry += scratch[32];
+            __syncthreads();
+        }
+    }
 }
 
-// 5. exact sums of the listed windows: one window per CTA of a warp at a time,
-// its points and its template staged in shared memory first (`room` floats
-// each; longer ones are read in place), because the chain of products would
-// wait for every row's loads (170 us per wave instead of 30).
-static __global__ void __launch_bounds__(32)
+// 5. exact sums of the listed windows: one window per CTA at a time, its
+// points (by their places in the folded order) and its template staged in
+// shared memory by all warps (`room` floats each; longer ones are read in
+// place), then summed by the first: the chain of products would wait for every
+// row's loads (170 us per wave instead of 30).
+static __global__ void __launch_bounds__(kExactThreads)
 k_window_exact(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk, int room)
 {
     const SlotMap& sm = smq ? *smq : smv;
     extern __shared__ float exact_smem[];
-    const int lane = threadIdx.x;
+    __shared__ long long part[kExactThreads / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int item = blockIdx.x;
     for (int q = 0; q < kListClasses; ++q) {
         const int cnt = (int)min((int64_t)dk.left_n[q], dk.list_cap);
@@ -1176,27 +1225,41 @@ k_window_exact(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
             const int slot = (int)(en >> 40), j = (int)(en >> 32) & 0xff, rot = (int)(en >> 24) & 0xff;
             const int m = (int)(en & 0xffffffull);
             int lc, p;
-            if (!resolve_slot(ds, sm, slot, lc, p)) continue;   // warp-uniform
+            if (!resolve_slot(ds, sm, slot, lc, p)) continue;   // block-uniform
             const DevPlan& dp = ds.plans[lc];
             const int d = dp.dpts[j], st = dp.stride[j], v = dp.cfg_variant[j];
             const int mode = v == tiles::kScalar15 ? kModePairS
                              : v == tiles::kCol16R || tiles::variant_colpair(v) ? kModeCols : kModeWin;
-            const int64_t base = (int64_t)slot * dk.pad_stride + (int64_t)m * st;
-            const float* r = dk.rs + base;
-            const float* t = dp.tmpl + dp.tmpl_off[j];
-            const long long sfx = dk.pf[base + d] - dk.pf[base];
-            if (d <= room) {
-                __syncwarp();
-                for (int k = lane; k < d; k += 32) {
-                    const uint32_t to = (uint32_t)__cvta_generic_to_shared(exact_smem + k);
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to), "l"(r + k) : "memory");
-                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(to + room * 4), "l"(t + k) : "memory");
+            const float* const t = dp.tmpl + dp.tmpl_off[j];
+            const int n = (int)dp.n, s = m * st;
+            const int* const sidx = dk.sidx + (int64_t)slot * dk.fold_stride;
+            const PointVals* const pv = ds.curves[lc].pv;
+            auto point = [&](int k) {
+                const int id = sidx[s + k < n ? s + k : s + k - n];
+                return id >= 0 && id < n ? pv[id] : PointVals{0, 0.0f, 0.0f};
+            };
+            long long sfx = 0;
+            __syncthreads();   // the window before is done with the staged points
+#pragma unroll 4
+            for (int k = threadIdx.x; k < d; k += blockDim.x) {
+                const PointVals v = point(k);
+                sfx += v.rfx;
+                if (d <= room) {
+                    exact_smem[k] = v.r;
+                    exact_smem[room + k] = __ldg(t + k);
                 }
-                asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
-                __syncwarp();
             }
-            const float2 sum = d <= room ? window_sum(exact_smem, exact_smem + room, d, st, q, mode, rot, lane < (1 << q), lane)
-                                         : window_sum(r, t, d, st, q, mode, rot, lane < (1 << q), lane);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) sfx += __shfl_xor_sync(0xffffffffu, sfx, o);
+            if (lane == 0) part[warp] = sfx;
+            __syncthreads();
+            if (warp != 0) continue;
+            sfx = 0;
+            for (int u = 0; u < (int)(blockDim.x >> 5); ++u) sfx += part[u];
+            const float2 sum = d <= room ? window_sum([&](int k) { return exact_smem[k]; }, exact_smem + room, d, st, q,
+                                                      mode, rot, lane < (1 << q), lane)
+                                         : window_sum([&](int k) { return point(k).r; }, t, d, st, q, mode, rot,
+                                                      lane < (1 << q), lane);
             if (lane != 0) continue;
             const float inv = dp.inv_sum_t[j];
             const float depth = fmaxf(0.0f, mode == kModePairS
