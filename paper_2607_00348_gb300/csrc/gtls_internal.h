@@ -47,7 +47,8 @@ struct alignas(16) BoundDur {
     float lam;                    // first-test value times lam estimates C1 / sqrt(sum s_k^2)
     float cut_last;               // mean of the last wide piece
     float coef0;                  // minus the mean of the first
-    int32_t pad[2];
+    float mean_all;               // mean of s_k over the template
+    int32_t pad;
     float coef[kBoundCutSlots];   // of the others: mean of the piece before minus its mean (Abel form; 0 past the last)
     int32_t row[kBoundCutSlots];  // their first T0 steps, or points
 };

@@ -2732,6 +2732,7 @@ void bound_tables(const float* s, int j, int d, int st, int64_t n, int clg, int 
         b.cut_jumps = (float)((jumps + std::fabs((double)before)) * (1.0 + 1e-6));
         bd.cuts4 = (b.cuts + 2) / 4 * 4;
     }
+    bd.mean_all = b.mean_all;
     bd.lam = (b.cuts == 0 ? b.mean_all : 1.0f) / b.root_t2;
 }
 

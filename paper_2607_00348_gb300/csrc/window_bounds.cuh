@@ -70,7 +70,6 @@ constexpr int kGroup = 128;         // windows a warp tests at a time (4 per lan
 constexpr int kChunkGroups = 4;     // groups per chunk (at most)
 constexpr int kNearStep = kTileStarts / kGroup;   // T0 steps up to this fill a group in one stretch
 constexpr int kListed = 256;        // windows listed of a period before the tiled kernel is cheaper
-constexpr int kCand = 2;            // windows summed for the threshold
 constexpr int kRowBuf = 168;        // prefix sums at whole T0 steps a warp stages for one group
 constexpr int kCutPoints = 60;      // windows of at least this many points are first tested by wide pieces
 constexpr int kCoarseSteps = 64;    // ... and from this many coarse steps on from the coarse prefix
@@ -88,7 +87,7 @@ enum Test : int { kTestSum = 0, kTestCuts = 1, kTestCutsDirect = 2, kTestCoarse 
 struct Dur {
     BoundDur b;
     int first;                  // first chunk (near durations: of a stretch)
-    float emax;                 // upper bound of sum r^2 over any window of the duration
+    float root_c2;              // root of the least C2 of its windows (uniform weights: of sum s_k^2)
     float first_min, cmin;      // thresholds of the first test (32-bit prefix units) and of the segment bound
     float smin;                 // lowest window sum that can have a depth (32-bit prefix units); kW: what the segment
                                 // bound can lose of C1
@@ -117,23 +116,26 @@ struct Smem {
     static constexpr int kMaxBlocks = T == 1024 ? 9 * T : 2 * T;
     static constexpr int kMaxCoarse = T == 1024 ? 18 * T : 3 * T;
     static constexpr int kMaxChunks = 2 * T;
-    static constexpr int kFinal = T;                 // windows past the segment bound
+    static constexpr int kFinal = 512;               // windows past the segment bound
     Dur dur[tiles::kMaxDur];
     unsigned int sieve[kSieve];                      // (duration, window) past the first test
     float pre[kMaxBlocks + 8];                       // energy prefix
-    float cmax[kMaxChunks];                          // largest first-test value per chunk
+    float cmax[kMaxChunks];                          // largest first-test value of a chunk
+    unsigned char cdur[kMaxChunks];                  // its duration
+    unsigned short pass[kMaxChunks];                 // chunks to walk again
     float row_buf[kWarps * kRowBuf];
     float coarse[kMaxCoarse + kMaxCoarse / 32 + 1];  // see at_coarse
     unsigned int fin[kFinal];
     float fin_v[kFinal];
     Chunks ck;
-    int next, sieved, n_fin, n_listed, dev, big;
+    int next, n_pass, sieved, n_fin, n_listed, dev, big;
     float wsum[kWarps], energy[kEnergySpans];
-    float top[kWarps], c1[kWarps], s[kWarps], thr;
-    int top_at[kWarps], cand[kCand];
+    float top[kWarps], c1[kWarps], s[kWarps];
+    int top_at[kWarps];
     int wmin[kFloorSpans], wlow;                     // smallest sums of w over whole blocks, smallest w (kW)
 };
 
+static_assert(sizeof(Smem<1024>) <= 195 * 1024, "see above");
 template <int T>
 constexpr int kWarpsOf = T / 32;
 
@@ -258,7 +260,6 @@ __device__ __forceinline__ void list_durations(const DevPlan& dp, unsigned int* 
         if (kept) {
             dur[k].b.j = j;
             dur[k].first = nearby ? run_near + a - a0 : run_far + b - b0;
-            dur[k].emax = 0.0f;
         }
         run_near += __shfl_sync(0xffffffffu, a, 31);
         run_far += __shfl_sync(0xffffffffu, b, 31);
@@ -636,7 +637,7 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
     if (warp == 0) {
         list_durations(dp, ds.curves[lc].check, p, n, dur, S.ck, lane);
         for (int k = lane; k < kEnergySpans; k += 32) S.energy[k] = 0.0f;
-        if (lane == 0) S.next = S.sieved = S.n_fin = S.n_listed = S.dev = S.big = 0;
+        if (lane == 0) S.next = S.n_pass = S.sieved = S.n_fin = S.n_listed = S.dev = S.big = 0;
         if (lane == 0) S.wlow = INT_MAX;
     }
     for (int i = threadIdx.x; i < M::kSieve; i += T) S.sieve[i] = kNone;
@@ -742,10 +743,69 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         return fmaf(S.energy[min(q, kEnergySpans - 1)], 1.0f + e_rel, e_abs);
     };
 
-    // 2. largest first-test value of every chunk; each warp's best group
-    float top = -INFINITY;   // this lane's best estimate of C1 / sqrt(sum s_k^2)
-    int top_at = 0;          // its duration and group of windows
-    int top_cnt = 0;
+    __syncthreads();
+
+    // what every duration's thresholds need besides the lowest known sum (eight
+    // lanes each, which share the pieces; kept in the fields of the thresholds).  A
+    // window whose C1 stays below cmin is above that sum: `lost` is what FP32
+    // summation, the 32-bit prefix and segment sums can lose of C1 (at most
+    // sum_slack(products in a row) ||r|| ||s||, and the units of the sums)
+    auto chain_of = [&](const Dur& t) {   // rows a lane of the final sums adds to one window
+        const int lg = kW ? __ffs(dp.cfg_nc_w[t.b.j]) - 1 : t.b.lg_nc, nc = 1 << lg;
+        return ((t.b.st + nc - 1) >> lg) * ((t.b.d + t.b.st - 1) / t.b.st) + 6;
+    };
+    for (int k0 = warp * 4; k0 < ndur; k0 += kWarps * 4) {
+        const int k = k0 + (lane >> 3);
+        Dur& t = dur[min(k, ndur - 1)];
+        const BoundTab& bt = dp.bounds[t.b.j];
+        const int d = t.b.d, st = t.b.st, chain = chain_of(t);
+        float lose = 0.0f, c2 = 0.0f;
+#pragma unroll
+        for (int u = 0; u < kBoundCuts; u += 8) {
+            const int at = u + (lane & 7);
+            if (at < bt.cuts) lose = fmaf(bt.cut_nu[at], sqrtf(energy_of(bt.cut_len[at])), lose);
+        }
+        static_assert(kBoundLevels <= 8, "a level per lane");
+        if (kW && (lane & 7) < kBoundLevels)
+            c2 = bt.lev_up[lane & 7] * fmaxf(0.0f, weight_floor(S, bt.lev_len[lane & 7], lbw));
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            lose += __shfl_xor_sync(0xffffffffu, lose, o);
+            if (kW) c2 += __shfl_xor_sync(0xffffffffu, c2, o);
+        }
+        if ((lane & 7) != 0 || k >= ndur) continue;
+        const float emax = energy_of(d), norm = sqrtf((float)d * emax), here = sum_slack(d / 32 + 8);
+        const float lost = (sum_slack(chain) + 8e-6f) * norm + sum_blur(d);
+        const float off = (lost + (float)(kBoundSegs + 1) * unit) * bt.t_max;
+        t.c2_slack = kW ? sum_slack(chain) + here + 1e-6f : 1e-6f;
+        // (kW: the smallest C2 of any window, less what FP32 sums of it can lose)
+        t.root_c2 = kW ? sqrtf(c2 * unit_w * (1.0f - 1e-5f - t.c2_slack)) / unit_a : bt.root_t2;
+        t.cmin = off;
+        // (uniform weights: the sums of steps 3 and 4 are those of the rounded r)
+        const float t_max = fmaxf(bt.t_max, 1.0f);
+        t.blur = kW ? (sum_slack(chain) + here) * norm * t_max * unit_a
+                    : (sum_slack(chain) * norm + sum_blur(d)) * t_max + (here + 3e-7f) * (norm + sum_blur(d)) * bt.change;
+        if (t.b.test == kTestSum) {
+            lose = bt.nu_all * sqrtf(emax);
+        } else if (t.b.test == kTestCoarse) {
+            // every position is off by at most S.dev in its prefix sum; the
+            // coarse entries are rounded to FP32
+            lose = fmaf(bt.cut_jumps * unit, (float)S.dev + 1.2e-7f * (float)(bt.cuts + 4) * (float)S.big, lose);
+            t.cmin_coarse = bt.seg_jumps * unit * ((float)S.dev + 1.2e-7f * (float)(2 * kBoundSegs + 4) * (float)S.big);
+        } else {
+            // rounding of the prefix sums, which reach over the whole group
+            const float over = (float)(kGroup * st) / (float)d + 2.0f;
+            lose += 1.2e-7f * (float)(bt.cuts + 4) * 2.0f * over * norm * bt.t_max;
+        }
+        t.first_min = lose;
+        // depth is zero without a positive sum (exact, or FP32 for the pairs)
+        t.smin = kW ? off : ((t.b.mode == kModePairS ? -lost : 0.0f) - sum_blur(d)) / unit;
+        if (kW) t.b.lg_nc = __ffs(dp.cfg_nc_w[t.b.j]) - 1;
+    }
+
+    // 2. largest first-test value of every chunk; each lane's best window
+    float top = -INFINITY;   // estimate of C1 / sqrt(sum s_k^2)
+    int top_at = 0;          // its duration and window
     for (;;) {
         int c = 0;
         if (lane == 0) c = atomicAdd(&S.next, 1);
@@ -759,14 +819,19 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
             // the largest sum of the chunk, in integers
             const int st = dur[k].b.st, d = dur[k].b.d;
             const int* a = pq + (lo + lane) * st;
-            int best = INT_MIN;
+            int best = INT_MIN, at = 0;
 #pragma unroll 4
-            for (int i = lo + lane; i < hi; i += 32, a += 32 * st) best = max(best, a[d] - a[0]);
+            for (int i = lo + lane; i < hi; i += 32, a += 32 * st) {
+                const int v = a[d] - a[0];
+                if (v > best) {
+                    best = v;
+                    at = i;
+                }
+            }
             if (best > INT_MIN) f = (float)best;
             if (f * lam > top) {
                 top = f * lam;
-                top_at = (k << 24) | lo;
-                top_cnt = hi - lo;
+                top_at = (k << 24) | at;
             }
         }
         for (int at = dur[k].b.test == kTestSum ? hi : lo; at < hi; at += kGroup) {
@@ -779,63 +844,56 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
             f = fmaxf(f, g);
             if (g * lam > top) {
                 top = g * lam;
-                top_at = (k << 24) | at;
-                top_cnt = cnt;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (q * 32 + lane < cnt && acc[q] == g) top_at = (k << 24) | (at + q * 32 + lane);
             }
         }
         f = float_from_order_key(__reduce_max_sync(0xffffffffu, float_order_key(f)));
-        if (lane == 0) S.cmax[c] = f;
+        if (lane == 0) {
+            S.cmax[c] = f;
+            S.cdur[c] = (unsigned char)k;
+        }
     }
 
-    // 3. threshold: the most promising windows of the warps, kWarps / kCand
+    // 3. threshold: the two most promising windows of the warps, half of the
     // warps to a window (any order: the result only has to be near)
     {
         const unsigned int key = __reduce_max_sync(0xffffffffu, float_order_key(top));
         const int who = __ffs(__ballot_sync(0xffffffffu, float_order_key(top) == key)) - 1;
-        const float most = __shfl_sync(0xffffffffu, top, who);
-        const int group = __shfl_sync(0xffffffffu, top_at, who), cnt = __shfl_sync(0xffffffffu, top_cnt, who);
-        if (most > -INFINITY) {   // the group again: which of the lane's windows it was
-            const BoundDur& t = dur[group >> 24].b;
-            const int g0 = group & 0xffffff;
-            int found = -1;
-            for (int at = g0; at < g0 + cnt; at += kGroup) {   // (one group, or the chunk of a sum test)
-                float acc[4];
-                first_test(t, pq, S.coarse, clg, at, min(kGroup, g0 + cnt - at), rb, lane, acc);
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (at + q * 32 + lane < g0 + cnt && acc[q] * t.lam == top) found = at + q * 32 + lane;
-            }
-            top_at = (group & ~0xffffff) | (found < 0 ? g0 : found);
-        }
         if (lane == who) {
             S.top[warp] = top;
             S.top_at[warp] = top_at;
         }
-        if (threadIdx.x < kCand) S.cand[threadIdx.x] = -1;
     }
     __syncthreads();
-    if (threadIdx.x < kWarps) {
-        const float v = S.top[threadIdx.x];
-        int rank = 0;
-        for (int w = 0; w < kWarps; ++w)
-            rank += S.top[w] > v || (S.top[w] == v && w < (int)threadIdx.x) ? 1 : 0;
-        if (rank < kCand && v > -INFINITY) S.cand[rank] = S.top_at[threadIdx.x];
-    }
-    __syncthreads();
-    constexpr int kTeam = kWarps / kCand, kTeamThreads = kTeam * 32;
+    constexpr int kTeam = kWarps / 2, kTeamThreads = kTeam * 32;
+    int cand[2];
     {
-        const int cand = S.cand[warp / kTeam];
-        float c1 = 0.0f, sum = 0.0f;
-        if (cand >= 0) {
-            const BoundDur& t = dur[cand >> 24].b;
-            const int at = (cand & 0xffffff) * t.st;
+        unsigned int key = lane < kWarps ? float_order_key(S.top[lane]) : 0u;
+        const int at = lane < kWarps ? S.top_at[lane] : 0;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const unsigned int most = __reduce_max_sync(0xffffffffu, key);
+            const int who = __ffs(__ballot_sync(0xffffffffu, key == most)) - 1;
+            const int from = __shfl_sync(0xffffffffu, at, who);
+            cand[q] = most > float_order_key(-INFINITY) ? from : -1;
+            if (lane == who) key = 0u;
+        }
+    }
+    {
+        const int mine = warp < kTeam ? cand[0] : cand[1];
+        float c1 = 0.0f, c2 = 0.0f;
+        if (mine >= 0) {
+            const BoundDur& t = dur[mine >> 24].b;
+            const int at = (mine & 0xffffff) * t.st;
             if constexpr (kW) {
                 const float* const s = dp.tmpl + dp.tmpl_off[t.j];
 #pragma unroll 8
                 for (int i = threadIdx.x % kTeamThreads; i < t.d; i += kTeamThreads) {
                     const float sv = __ldg(s + i);
                     c1 = fmaf(rs[at + i], sv, c1);
-                    sum = fmaf(ws[at + i], sv * sv, sum);   // C2
+                    c2 = fmaf(ws[at + i], sv * sv, c2);
                 }
             } else {
                 // sum r s_k = sum (P_k - P_0) (s_{k-1} - s_k): r itself is not there
@@ -849,134 +907,77 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             c1 += __shfl_xor_sync(0xffffffffu, c1, o);
-            sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (kW) c2 += __shfl_xor_sync(0xffffffffu, c2, o);
         }
         if (lane == 0) {
             S.c1[warp] = c1;
-            S.s[warp] = sum;
+            S.s[warp] = c2;
         }
+        if (threadIdx.x == 0) S.next = 0;
     }
     __syncthreads();
-    // rows a lane of the final sums adds to one window, what two orders of its
-    // sum can differ, and the same for C2
-    auto chain_of = [&](const Dur& t) {
-        const int lg = kW ? __ffs(dp.cfg_nc_w[t.b.j]) - 1 : t.b.lg_nc, nc = 1 << lg;
-        return ((t.b.st + nc - 1) >> lg) * ((t.b.d + t.b.st - 1) / t.b.st) + 6;
-    };
-    // (uniform weights: the sums here are those of the rounded r)
-    auto blur_of = [&](const Dur& t, int chain, float norm) {
-        const float t_max = fmaxf(dp.bounds[t.b.j].t_max, 1.0f);
-        const float here = sum_slack(t.b.d / 32 + 8);
-        if (kW) return (sum_slack(chain) + here) * norm * t_max * unit_a;
-        return (sum_slack(chain) * norm + sum_blur(t.b.d)) * t_max +
-               (here + 3e-7f) * (norm + sum_blur(t.b.d)) * dp.bounds[t.b.j].change;
-    };
-    auto c2_slack_of = [&](const Dur& t, int chain) {
-        return kW ? sum_slack(chain) + sum_slack(t.b.d / 32 + 8) + 1e-6f : 1e-6f;
-    };
     // what the depth of depth_of can be off by (kW: nothing, it is exact)
     auto depth_blur = [&](const Dur& t, float off, float inv) {
         return kW ? 0.0f : (t.b.mode == kModePairS ? off : 0.0f) * inv + sum_blur(t.b.d) * inv;
     };
-    if (threadIdx.x == 0) {
-        float thr = INFINITY;
-        for (int q = 0; q < kCand; ++q) {
-            if (S.cand[q] < 0) continue;
-            const Dur& t = dur[S.cand[q] >> 24];
-            const int j = t.b.j;
-            float c1 = 0.0f, sum = 0.0f;
-            for (int w = q * kTeam; w < (q + 1) * kTeam; ++w) {
-                c1 += S.c1[w];
-                sum += S.s[w];
-            }
-            if (!kW) c1 *= unit;
-            const int s = (S.cand[q] & 0xffffff) * t.b.st;
-            const float depth = depth_of(s, t.b.d, dp.inv_sum_t[j]);
-            const float t2 = kW ? sum : dp.sum_t2[j];
-            const int chain = chain_of(t);
-            const float off = blur_of(t, chain, sqrtf((float)t.b.d * energy_of(t.b.d)));
-            float v = w_uni * depth * fmaf(depth, t2, -2.0f * c1);
-            v += sum_error(w_uni, depth, t2, c1, v, off, depth_blur(t, off, dp.inv_sum_t[j]), c2_slack_of(t, chain));
-            thr = v < thr || isnan(v) ? v : thr;
+    float thr;   // (every warp for itself)
+    {
+        float c1 = lane < kWarps ? S.c1[lane] : 0.0f, c2 = lane < kWarps ? S.s[lane] : 0.0f, v = INFINITY;
+#pragma unroll
+        for (int o = kTeam / 2; o > 0; o >>= 1) {
+            c1 += __shfl_xor_sync(0xffffffffu, c1, o);
+            if (kW) c2 += __shfl_xor_sync(0xffffffffu, c2, o);
         }
-        S.thr = thr;
-        S.next = 0;
+        const int mine = lane < kTeam ? cand[0] : cand[1];
+        if (lane < kWarps && mine >= 0) {
+            const Dur& t = dur[mine >> 24];
+            const float inv = dp.inv_sum_t[t.b.j], t2 = kW ? c2 : dp.sum_t2[t.b.j];
+            if (!kW) c1 *= unit;
+            const float depth = depth_of((mine & 0xffffff) * t.b.st, t.b.d, inv);
+            v = w_uni * depth * fmaf(depth, t2, -2.0f * c1);
+            v += sum_error(w_uni, depth, t2, c1, v, t.blur, depth_blur(t, t.blur, inv), t.c2_slack);
+        }
+        const float v0 = __shfl_sync(0xffffffffu, v, 0), v1 = __shfl_sync(0xffffffffu, v, kTeam);
+        thr = isnan(v0) || isnan(v1) ? NAN : fminf(v0, v1);
     }
-    __syncthreads();
-    const float thr = S.thr;
     // no negative delta-chi2, or values out of range: the tiled kernel decides
     const bool sane = thr < 0.0f && thr > -INFINITY && e_all < INFINITY && w_uni < INFINITY && in_range_32;
     if (sane) {
-        // thresholds of every duration.  A window whose C1 stays below cmin is
-        // above thr; 1e-4 of slack covers the rounding of delta-chi2, and `lost` what FP32 summation, the 32-bit prefix
-        // and segment sums can lose of C1 (at most sum_slack(products in a
-        // row) ||r|| ||s||, 2^-41 of fixed point per point, and the prefix
-        // units of the sums)
-        const float reach = sqrtf(-thr / w_uni) * (1.0f - 1e-4f);   // (kW: times the root of C2)
+        // 1e-4 of slack covers the rounding of delta-chi2
+        const float reach = sqrtf(-thr / w_uni) * (1.0f - 1e-4f);   // (times the root of C2 or sum s_k^2)
         for (int k = threadIdx.x; k < ndur; k += T) {
             Dur& t = dur[k];
-            const BoundTab& bt = dp.bounds[t.b.j];
-            if (kW) t.b.lg_nc = __ffs(dp.cfg_nc_w[t.b.j]) - 1;
-            const int d = t.b.d, st = t.b.st, chain = chain_of(t);
-            t.emax = energy_of(d);
-            const float norm = sqrtf((float)d * t.emax);
-            const float lost = (sum_slack(chain) + 8e-6f) * norm + sum_blur(d);
-            t.c2_slack = c2_slack_of(t, chain);
-            float root_c2 = bt.root_t2;
-            if (kW) {
-                // the smallest C2 of any window, with what FP32 sums of it can lose
-                float c2 = 0.0f;
-                for (int l = 0; l < kBoundLevels; ++l)
-                    c2 = fmaf(bt.lev_up[l], fmaxf(0.0f, weight_floor(S, bt.lev_len[l], lbw)), c2);
-                root_c2 = sqrtf(c2 * unit_w * (1.0f - 1e-5f - t.c2_slack)) / unit_a;
-            }
-            t.cmin = reach * root_c2 - (lost + (float)(kBoundSegs + 1) * unit) * bt.t_max;
-            t.blur = blur_of(t, chain, norm);
-            // depth is zero without a positive sum (exact, or FP32 for the pairs)
-            const float low = kW ? -INFINITY : (t.b.mode == kModePairS ? -lost : 0.0f) - sum_blur(d);
-            float c0;
-            if (t.b.test == kTestSum) {
-                c0 = fmaxf((t.cmin - bt.nu_all * sqrtf(t.emax)) / bt.mean_all, low);
-            } else {
-                float lose = 0.0f;
-                for (int u = 0; u < bt.cuts; ++u) lose = fmaf(bt.cut_nu[u], sqrtf(energy_of(bt.cut_len[u])), lose);
-                if (t.b.test == kTestCoarse) {
-                    // every position is off by at most S.dev in its prefix
-                    // sum; the coarse entries are rounded to FP32
-                    lose = fmaf(bt.cut_jumps * unit, (float)S.dev + 1.2e-7f * (float)(bt.cuts + 4) * (float)S.big, lose);
-                    t.cmin_coarse = t.cmin - bt.seg_jumps * unit *
-                                                 ((float)S.dev + 1.2e-7f * (float)(2 * kBoundSegs + 4) * (float)S.big);
-                } else {
-                    // rounding of the prefix sums, which reach over the whole group
-                    const float over = (float)(kGroup * st) / (float)d + 2.0f;
-                    lose += 1.2e-7f * (float)(bt.cuts + 4) * 2.0f * over * norm * bt.t_max;
-                }
-                c0 = t.cmin - lose;
-            }
+            t.cmin = reach * t.root_c2 - t.cmin;
+            t.cmin_coarse = t.cmin - t.cmin_coarse;
+            const float c0 = t.b.test == kTestSum
+                                 ? fmaxf((t.cmin - t.first_min) / t.b.mean_all, kW ? -INFINITY : t.smin * unit)
+                                 : t.cmin - t.first_min;
             t.first_min = (c0 - 1e-5f * fabsf(c0)) / unit;
-            t.smin = kW ? (lost + (float)(kBoundSegs + 1) * unit) * bt.t_max : low / unit;
+        }
+    }
+    __syncthreads();
+    // the chunks to walk again
+    if (sane) {
+        for (int c = threadIdx.x; c < ck.total; c += T) {
+            if (!(S.cmax[c] < dur[S.cdur[c]].first_min)) S.pass[atomicAdd(&S.n_pass, 1)] = (unsigned short)c;
         }
     }
     __syncthreads();
 
-    // 4. windows that may hold the minimum: chunks whose largest value passes,
-    // their windows by the first test into the sieve, those by segments into
-    // the final list; a full sieve is emptied before the walk goes on
+    // 4. windows that may hold the minimum: those of the listed chunks by the
+    // first test into the sieve, those by segments into the final list; a full
+    // sieve is emptied before the walk goes on
     int c = -1, k = 0, at = 0, hi = 0;
     while (sane) {
         for (;;) {
             if (c < 0) {
                 if (lane == 0) c = atomicAdd(&S.next, 1);
                 c = __shfl_sync(0xffffffffu, c, 0);
-                if (c >= ck.total) {
+                if (c >= S.n_pass) {
                     c = -1;
                     break;
                 }
-                chunk_range(ck, dur, lg, c, lane, k, at, hi);
-                if (S.cmax[c] < dur[k].first_min) {
-                    c = -1;
-                    continue;
-                }
+                chunk_range(ck, dur, lg, S.pass[c], lane, k, at, hi);
             }
             const float first_min = dur[k].first_min;
             bool full = false;
