@@ -598,7 +598,8 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
     uint16_t* sorted_f = inv + kFoldSegKeys;                                              // fine bucket of sorted[q]
     int* overflow = reinterpret_cast<int*>(sorted_f + kFoldSegKeys);
 
-    int* const sq = reinterpret_cast<int*>(srfx);   // kBounds: r in units, in fine-bucket order, then prefix sums
+    int* const sq = reinterpret_cast<int*>(srfx);   // kBounds: r in units, in fine-bucket order
+    int* const sp = sq + kFoldSegKeys;              // ... in folded order (swizzled), then their prefix sums
 
     // A single super-bucket (n <= kFoldSegKeys): its keys go straight to the
     // registers of step B.
@@ -700,6 +701,7 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
         // registers from the count to the scatter
         unsigned long long kv[kPerThread];
         uint32_t kf[kPerThread / 2];   // two 16-bit fine buckets per register
+        float kr[kPerThread];          // (kBounds) r of the keys' points
         if (single) {
 #pragma unroll
             for (int h = 0; h < kPerThread; h += kFoldUnroll) {
@@ -730,6 +732,10 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
         for (int u = 0; u < kPerThread; ++u) {
             const uint32_t q = threadIdx.x + u * kFoldThreads;
             const uint32_t f = fold_fine((long long)(kv[u] >> ib), sh, mulf) & kFineMask;
+            if (kBounded) {   // (used after the next two barriers)
+                const uint32_t id = (uint32_t)(kv[u] & idx_mask);
+                kr[u] = q < len && id < (uint32_t)n ? __ldg(dc.r + id) : 0.0f;
+            }
             if (u & 1) kf[u >> 1] |= f << 16;
             else kf[u >> 1] = f;
             if (q < len) atomicAdd(&fine[f], 0x10000u);
@@ -761,29 +767,16 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
             }
         }
         __syncthreads();
-        constexpr int kBatch = kBounded ? 4 : kPerThread;   // values in flight
 #pragma unroll
-        for (int h = 0; h < kPerThread; h += kBatch) {
-            float r[kBatch];
-            if (kBounded) {
-#pragma unroll
-                for (int u = 0; u < kBatch; ++u) {
-                    const uint32_t q = threadIdx.x + (h + u) * kFoldThreads;
-                    const uint32_t id = (uint32_t)(kv[h + u] & idx_mask);
-                    r[u] = q < len && id < (uint32_t)n ? __ldg(dc.r + id) : 0.0f;
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kBatch; ++u) {
-                const uint32_t q = threadIdx.x + (h + u) * kFoldThreads;
-                if (q >= len) break;
-                const uint32_t f = (kf[(h + u) >> 1] >> (((h + u) & 1) * 16)) & 0xffffu;
-                const uint32_t d = atomicAdd(&fine[f], 1u) & 0xffffu;   // the lower half ends as the end of bucket f
-                if (in_range32(dc.check, 5, d, len)) {
-                    sorted[d] = kv[h + u];
-                    sorted_f[d] = (uint16_t)f;
-                    if (kBounded) sq[d] = __float2int_rn(r[u] * o.per_unit);
-                }
+        for (int u = 0; u < kPerThread; ++u) {
+            const uint32_t q = threadIdx.x + u * kFoldThreads;
+            if (q >= len) break;
+            const uint32_t f = (kf[u >> 1] >> ((u & 1) * 16)) & 0xffffu;
+            const uint32_t d = atomicAdd(&fine[f], 1u) & 0xffffu;   // the lower half ends as the end of bucket f
+            if (in_range32(dc.check, 5, d, len)) {
+                sorted[d] = kv[u];
+                sorted_f[d] = (uint16_t)f;
+                if (kBounded) sq[d] = __float2int_rn(kr[u] * o.per_unit);
             }
         }
         __syncthreads();
@@ -796,17 +789,18 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
             const uint32_t lo = e - cnt;
             uint32_t rank = 0;
             for (uint32_t u = 0; u < cnt; ++u) rank += sorted[lo + u] < key ? 1u : 0u;
-            if (in_range32(dc.check, 7, lo + rank, len)) inv[lo + rank] = (uint16_t)q;
+            if (!in_range32(dc.check, 7, lo + rank, len)) continue;
+            if constexpr (kBounded) {
+                // (neighbours in fine-bucket order are neighbours in the folded one)
+                const uint32_t id = (uint32_t)(key & idx_mask);
+                if (in_range32(dc.check, 8, id, (uint32_t)n)) __stcs(o.sidx + (int64_t)k0 + lo + rank, (int32_t)id);
+                sp[swz4(lo + rank)] = sq[q];
+            } else {
+                inv[lo + rank] = (uint16_t)q;
+            }
         }
         __syncthreads();
-        if constexpr (kBounded) {
-            for (uint32_t i = threadIdx.x; i < len; i += kFoldThreads) {
-                const uint32_t q = inv[i];
-                if (!in_range32(dc.check, 7, q, len)) continue;
-                const uint32_t id = (uint32_t)(sorted[q] & idx_mask);
-                if (in_range32(dc.check, 8, id, (uint32_t)n)) __stcs(o.sidx + (int64_t)k0 + i, (int32_t)id);
-            }
-        } else {
+        if constexpr (!kBounded) {
             // gather in final-position order (kRankBatch points' loads in flight;
             // batches past the super-bucket's length skipped, block-uniform)
 #pragma unroll
@@ -852,21 +846,12 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
             __syncthreads();
         }
         if constexpr (kBounded) {
-            // the same of the units: eight places of inv in two loads; every
-            // value is read before the scan's barrier, the sums written after it
+            // the same of the units, in place
             const uint32_t i0 = threadIdx.x * kScanPer;
-            uint32_t at[kScanPer / 2];
-#pragma unroll
-            for (int u = 0; u < kScanPer / 4; ++u) {
-                const uint2 x = *reinterpret_cast<const uint2*>(inv + i0 + 4 * u);
-                at[2 * u] = x.x;
-                at[2 * u + 1] = x.y;
-            }
             int v[kScanPer], run = 0;
 #pragma unroll
             for (int u = 0; u < kScanPer; ++u) {
-                const uint32_t q = (at[u >> 1] >> (16 * (u & 1))) & 0xffffu;
-                run += i0 + u < len ? sq[min(q, len - 1u)] : 0;
+                run += i0 + u < len ? sp[swz4(i0 + u)] : 0;
                 v[u] = run;
             }
             uint32_t sum;
@@ -874,10 +859,10 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
                            (int)carry;
 #pragma unroll
             for (int u = 0; u < kScanPer; ++u)
-                if (i0 + u < len) sq[swz4(i0 + u)] = ex + v[u];
+                if (i0 + u < len) sp[swz4(i0 + u)] = ex + v[u];
             carry += (int)sum;
             __syncthreads();
-            for (uint32_t i = threadIdx.x; i < len; i += kFoldThreads) o.pq[(int64_t)k0 + 1 + i] = sq[swz4(i)];
+            for (uint32_t i = threadIdx.x; i < len; i += kFoldThreads) o.pq[(int64_t)k0 + 1 + i] = sp[swz4(i)];
         } else {
             // inclusive prefix of rfx in final order, kScanPer consecutive
             // entries per thread, written back in place
