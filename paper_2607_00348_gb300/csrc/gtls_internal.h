@@ -36,6 +36,10 @@ struct alignas(16) BoundTab {
     float seg_low[kBoundSegs];
 };
 
+// Templates of at least kFineFrom points also in kFinePieces equal pieces: mean
+// of s_k and >= ||s_k - mean|| of every piece.
+constexpr int kFinePieces = 128, kFineFrom = 1024;
+
 // What the bounds need of one duration for every period (staged in shared
 // memory by the words).
 struct alignas(16) BoundDur {
@@ -93,6 +97,7 @@ struct DevPlan {
     const int64_t* tc_off;      // offset of duration j in tc_tab (floats; kTensor durations)
     const BoundTab* bounds;     // pieces of every duration's template
     const BoundDur* bound_durs;
+    const float2* bound_fine;   // kFinePieces per duration
     int32_t bound_lg;           // chunks of the window search are 2^bound_lg times the usual size
     const float* tc_tab;        // tensor-core template chunks: [chunk][hi, lo][32 x 32 core-matrix layout]
 };
@@ -138,7 +143,7 @@ struct DevChunk {
     int32_t* pq;              // of r (per-point weights: w r) in units (modulo 2^32: window sums fit 31 bits)
     int64_t list_cap;         // windows per lane-group size
     unsigned long long* list; // windows to sum, kListClasses lists
-    int2* dense;              // (slot, tile) items for the tiled kernel
+    int2* dense;              // items for the tiled kernel: slot, and tile | part << 20 | (parts - 1) << 24
     unsigned int* left_n;     // [0 .. kListClasses) windows listed, [kListClasses] items in `dense`
 };
 

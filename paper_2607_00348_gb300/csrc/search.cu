@@ -1211,7 +1211,7 @@ k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
     using namespace tiles;
     extern __shared__ float tile_smem[];
     __shared__ DurTask dur[kMaxDur];
-    __shared__ int s_item, s_ndur, s_total, s_task, s_lc, s_p, s_slot, s_x0, s_len, s_tau, s_tcount;
+    __shared__ int s_item, s_ndur, s_total, s_task, s_lc, s_p, s_slot, s_x0, s_len, s_tau, s_tcount, s_part, s_parts;
     __shared__ unsigned long long s_best[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the items the bounds kernel left, or every (period, tile) of the wave
@@ -1221,11 +1221,13 @@ k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
             const int item = (int)atomicAdd(counter, 1u);
             s_item = item < items ? 1 : 0;
             if (item < items) {
-                int lcg = 0, pp = -1, slot = 0, tau = 0;
+                int lcg = 0, pp = -1, slot = 0, tau = 0, part = 0, parts = 1;
                 if (listed) {
                     const int2 it = dk.dense[item];
                     slot = it.x;
-                    tau = it.y;
+                    tau = it.y & 0xfffff;
+                    part = (it.y >> 20) & 15;
+                    parts = (it.y >> 24) + 1;
                     if (!resolve_slot(ds, sm, slot, lcg, pp)) pp = -1;
                 } else {
                     int g = 0;
@@ -1247,6 +1249,8 @@ k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
                 s_x0 = tau * (weighted ? tl.len_w : tl.len);
                 s_len = weighted ? tl.len_w : tl.len;
                 s_tau = tau;
+                s_part = part;   // of the tile's tasks every parts-th, from the part-th on
+                s_parts = parts;
                 s_tcount = weighted ? tl.count_w : tl.count;
             }
         }
@@ -1350,7 +1354,7 @@ k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
         for (;;) {
             int task = 0;
             if (lane == 0) task = atomicAdd(&s_task, 1);
-            task = __shfl_sync(0xffffffffu, task, 0);
+            task = __shfl_sync(0xffffffffu, task, 0) * s_parts + s_part;
             if (task >= total) break;
             int lo_k = 0, hi_k = ndur - 1;   // last entry with first <= task
             while (lo_k < hi_k) {
@@ -3201,7 +3205,22 @@ gtls_status create_device(gtls_plan* pl)
                     drop[(size_t)(pl->tmpl_pad_off[j] + k)] = (float)((k > 0 ? (double)tj[k - 1] : 0.0) - tj[k]);
             }
             GTLS_TRY(upload(pl, const_cast<float**>(&dp.tmpl_drop), drop));
+            std::vector<float2> fine((size_t)dp.nd * kFinePieces, make_float2(0.0f, 0.0f));
+            for (int j = 0; j < dp.nd; ++j) {
+                const int64_t d = h.dpts[j];
+                const float* const tj = pl->tmpl_pad.data() + pl->tmpl_pad_off[j];
+                for (int64_t g = 0; g < kFinePieces && d >= kFineFrom; ++g) {
+                    const int64_t lo = g * d / kFinePieces, hi = (g + 1) * d / kFinePieces;
+                    double m = 0.0, v = 0.0;
+                    for (int64_t k = lo; k < hi; ++k) m += tj[k];
+                    const float mean = (float)(m / (double)(hi - lo));
+                    for (int64_t k = lo; k < hi; ++k) v += ((double)tj[k] - mean) * ((double)tj[k] - mean);
+                    fine[(size_t)(j * kFinePieces + g)] = make_float2(mean, (float)(std::sqrt(v) * (1.0 + 1e-6)));
+                }
+            }
+            GTLS_TRY(upload(pl, const_cast<float2**>(&dp.bound_fine), fine));
             pl->dp_ref.tmpl_drop = dp.tmpl_drop;
+            pl->dp_ref.bound_fine = dp.bound_fine;
         }
         // (the 32-bit prefix sums of w take the fold's keys' place)
         pl->bounds_w_ok = pl->bounds_ok && pl->tile_w_ok && !pl->has_window_only &&
@@ -3282,7 +3301,7 @@ gtls_status ensure_chunk(gtls_plan* pl)
         GTLS_TRY(dev_alloc(pl, &dk.pq, chunk * dk.pad_stride));
         dk.list_cap = std::max<int64_t>(4096, chunk * kListPerSlot);
         GTLS_TRY(dev_alloc(pl, &dk.list, kListClasses * dk.list_cap));
-        GTLS_TRY(dev_alloc(pl, &dk.dense, chunk * std::max({1, pl->tile_count, pl->tile_count_ref, pl->tile_count_w})));
+        GTLS_TRY(dev_alloc(pl, &dk.dense, chunk * bounds::kDenseParts * std::max({1, pl->tile_count, pl->tile_count_ref, pl->tile_count_w})));
         GTLS_TRY(dev_alloc(pl, &dk.left_n, kListClasses + 1));
     }
     if (pl->has_tensor) {
@@ -4250,7 +4269,7 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     if (b->bounds_ok) {
         int max_tiles = 1;
         for (const DevTiles& t : b->tiles_host) max_tiles = std::max({max_tiles, t.count, t.count_w});
-        GTLS_TRY(batch_alloc(b, &b->dk.dense, slots * (int64_t)max_tiles));
+        GTLS_TRY(batch_alloc(b, &b->dk.dense, slots * (int64_t)max_tiles * bounds::kDenseParts));
         GTLS_TRY(batch_alloc(b, &b->dk.pq, slots * pad_stride));
         b->dk.list_cap = std::max<int64_t>(4096, slots * kListPerSlot);
         GTLS_TRY(batch_alloc(b, &b->dk.list, kListClasses * b->dk.list_cap));

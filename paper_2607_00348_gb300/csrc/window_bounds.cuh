@@ -69,7 +69,9 @@ constexpr int kTileStarts = 8192;   // window starts walked before the next stre
 constexpr int kGroup = 128;         // windows a warp tests at a time (4 per lane)
 constexpr int kChunkGroups = 4;     // groups per chunk (at most)
 constexpr int kNearStep = kTileStarts / kGroup;   // T0 steps up to this fill a group in one stretch
-constexpr int kListed = 256;        // windows listed of a period before the tiled kernel is cheaper
+constexpr int kDenseParts = 16;     // items a tile is split into for the tiled kernel, at most
+constexpr int kListed = 256;        // windows listed of a period before the tiled kernel is cheaper, or a window in
+constexpr int kListedPart = 512;    // so many (a listed window costs about 3 us of an SM; all 1.2e6 at T0 step 1, 55 ms)
 constexpr int kRowBuf = 168;        // prefix sums at whole T0 steps a warp stages for one group
 constexpr int kCutPoints = 60;      // windows of at least this many points are first tested by wide pieces
 constexpr int kCoarseSteps = 64;    // ... and from this many coarse steps on from the coarse prefix
@@ -104,6 +106,8 @@ struct Chunks {
     int ndur, near_durs;        // durations (ascending); the first near_durs are near
     int far, per_tile;          // far chunks, near chunks per stretch
     int total;
+    int listed;                 // windows that may be listed
+    int parts;                  // items per tile for the tiled kernel
 };
 
 // Shared memory for CTAs of T threads (curves of up to 8 T points when
@@ -116,17 +120,21 @@ struct Smem {
     static constexpr int kMaxBlocks = T == 1024 ? 9 * T : 2 * T;
     static constexpr int kMaxCoarse = T == 1024 ? 18 * T : 3 * T;
     static constexpr int kMaxChunks = 2 * T;
-    static constexpr int kFinal = 512;               // windows past the segment bound
+    static constexpr int kFinal = kMaxChunks;        // windows past the segment bound
     Dur dur[tiles::kMaxDur];
-    unsigned int sieve[kSieve];                      // (duration, window) past the first test
+    union {
+        unsigned int sieve[kSieve];                  // (duration, window) past the first test
+        float fin_v[kFinal];                         // after the walk: lower ends of the sums of fin[]
+    };
     float pre[kMaxBlocks + 8];                       // energy prefix
-    float cmax[kMaxChunks];                          // largest first-test value of a chunk
+    union {
+        float cmax[kMaxChunks];                      // largest first-test value of a chunk
+        unsigned int fin[kFinal];                    // after the list of chunks is made: windows past the segment bound
+    };
     unsigned char cdur[kMaxChunks];                  // its duration
     unsigned short pass[kMaxChunks];                 // chunks to walk again
     float row_buf[kWarps * kRowBuf];
     float coarse[kMaxCoarse + kMaxCoarse / 32 + 1];  // see at_coarse
-    unsigned int fin[kFinal];
-    float fin_v[kFinal];
     Chunks ck;
     int next, n_pass, sieved, n_fin, n_listed, dev, big;
     float wsum[kWarps], energy[kEnergySpans];
@@ -237,10 +245,11 @@ __device__ __forceinline__ void list_durations(const DevPlan& dp, unsigned int* 
                                                int lane)
 {
     const int lo = dp.jlo[p], hi = dp.jhi[p];
-    int count = 0, run_near = 0, run_far = 0, near_durs = 0;
+    int count = 0, run_near = 0, run_far = 0, near_durs = 0, windows = 0;
     for (int base = 0; base <= hi - lo; base += 32) {
         const int j = lo + base + lane;
         const int subs = j <= hi ? dp.bound_durs[j].subs : 0;
+        const int wins = j <= hi ? dp.bound_durs[j].m_total : 0;
         const bool nearby = j <= hi && dp.bound_durs[j].st <= kNearStep;
         const int d = j <= hi ? dp.dpts[j] : 0, before = j <= hi && j > lo ? dp.dpts[j - 1] : -1;
         bool kept = j <= hi && d != before && subs > 0;
@@ -260,6 +269,7 @@ __device__ __forceinline__ void list_durations(const DevPlan& dp, unsigned int* 
         if (kept) {
             dur[k].b.j = j;
             dur[k].first = nearby ? run_near + a - a0 : run_far + b - b0;
+            windows += wins;
         }
         run_near += __shfl_sync(0xffffffffu, a, 31);
         run_far += __shfl_sync(0xffffffffu, b, 31);
@@ -267,9 +277,11 @@ __device__ __forceinline__ void list_durations(const DevPlan& dp, unsigned int* 
         count += __popc(mask);
     }
     const int tile = kTileStarts << dp.bound_lg;
+    windows = (int)__reduce_add_sync(0xffffffffu, (unsigned int)windows);
     if (lane == 0)
         ck = Chunks{min(count, tiles::kMaxDur), near_durs, run_far, run_near,
-                    run_far + (n + tile - 1) / tile * run_near};
+                    run_far + (n + tile - 1) / tile * run_near, max(kListed, windows / kListedPart),
+                    max(1, min(kDenseParts, windows >> 16))};
     __syncwarp();
 }
 
@@ -1104,6 +1116,38 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
             const Dur& t = dur[e >> 24];
             const int s = (int)(e & 0xffffffu) * t.b.st, d = t.b.d;
             float c1 = 0.0f, c2 = 0.0f;
+            if (!kW && T == 1024 && d >= kFineFrom) {   // (shorter curves have no such durations)
+                // the bound by kFinePieces pieces first, four per lane: it
+                // leaves a few of the windows, whose sums would read all
+                // their points (66 windows of up to 9,354 points at a
+                // period of 0.55 days: 43 thousand cycles of the CTA)
+                static_assert(kFinePieces == 128, "four pieces per lane");
+                const float4* const fine =
+                    reinterpret_cast<const float4*>(dp.bound_fine + t.b.j * kFinePieces + 4 * lane);
+                const float4 f01 = __ldg(fine), f23 = __ldg(fine + 1);
+                const float mean[4] = {f01.x, f01.z, f23.x, f23.z}, nu[4] = {f01.y, f01.w, f23.y, f23.w};
+                int at[5], p[5];
+#pragma unroll
+                for (int u = 0; u < 5; ++u) {
+                    at[u] = s + (((4 * lane + u) * d) >> 7);
+                    p[u] = pq[at[u]];
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int len = at[u + 1] - at[u];
+                    const float sg = (float)(p[u + 1] - p[u]) * unit;
+                    const float en = fmaf(S.pre[(at[u + 1] + bsize - 1) >> lb] - S.pre[at[u] >> lb], 1.0f + e_rel, e_abs);
+                    const float sm = fmaxf(fabsf(sg) - (1.0f + 0.5f * (float)len) * unit, 0.0f);
+                    c1 += fmaf(mean[u], sg, nu[u] * root(en - sm * sm * (1.0f - 1e-5f) / (float)len));
+                }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) c1 += __shfl_xor_sync(0xffffffffu, c1, o);
+                if (c1 < t.cmin) {   // (warp-uniform)
+                    if (lane == 0) S.fin_v[i] = INFINITY;
+                    continue;
+                }
+                c1 = 0.0f;
+            }
             if (kW) {
                 const float* const tm = dp.tmpl + dp.tmpl_off[t.b.j];
 #pragma unroll 8
@@ -1145,13 +1189,13 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
             const int m = (int)(e & 0xffffffu);
             auto push = [&](int rot) {
                 const unsigned int to =
-                    atomicAdd(&S.n_listed, 1) < kListed ? atomicAdd(dk.left_n + t.b.lg_nc, 1u) : 0xffffffffu;
+                    atomicAdd(&S.n_listed, 1) < S.ck.listed ? atomicAdd(dk.left_n + t.b.lg_nc, 1u) : 0xffffffffu;
                 if (to < dk.list_cap)
                     dk.list[t.b.lg_nc * dk.list_cap + to] = ((unsigned long long)slot << 40) |
                                                             ((unsigned long long)t.b.j << 32) |
                                                             ((unsigned long long)rot << 24) | (unsigned long long)m;
                 else
-                    S.n_listed = 2 * kListed;   // (more may be added: it stays above kListed)
+                    S.n_listed = 2 * S.ck.listed;   // (more may be added: it stays above)
             };
             if (kW || t.b.mode != kModeRot) {
                 push(0);
@@ -1176,12 +1220,15 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
             }
         }
         __syncthreads();
-        fits = fits && S.n_listed <= kListed;
+        fits = fits && S.n_listed <= S.ck.listed;
     }
     if (!fits && threadIdx.x == 0) {
-        const int tc = kW ? ds.tiles[lc].count_w : ds.tiles[lc].count;
-        const unsigned int to = atomicAdd(dk.left_n + kListClasses, (unsigned int)tc);
-        for (int tau = 0; tau < tc; ++tau) dk.dense[to + tau] = make_int2(slot, tau);
+        // (a tile's tasks shared by `parts` CTAs, about 65,536 windows each: the
+        // 1.2e6 windows of one period at T0 step 1 kept an SM for 15 ms)
+        const int tc = kW ? ds.tiles[lc].count_w : ds.tiles[lc].count, parts = S.ck.parts;
+        const unsigned int to = atomicAdd(dk.left_n + kListClasses, (unsigned int)(tc * parts));
+        for (int i = 0; i < tc * parts; ++i)
+            dk.dense[to + i] = make_int2(slot, (i / parts) | ((i % parts) << 20) | ((parts - 1) << 24));
     }
     if (!kW && (fill || !fits)) {
         // the folded curve itself and its exact prefix sums, for the kernels

@@ -92,3 +92,9 @@ def test_batch_of_both_kinds_equals_single_searches():
     batch.close()
     for p in plans:
         p.close()
+
+
+@pytest.mark.parametrize("flux", ["steps", "flat", "deep"])
+def test_periods_shared_by_several_ctas_of_the_tiled_kernel(flux):
+    # at T0 step 1 a period has more than 2 x 65,536 windows, most of them equal
+    _same(9001, 120.0, flux, "uniform", periods_days=np.geomspace(2.0, 50.0, 12), refine_periods=5)
