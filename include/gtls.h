@@ -83,9 +83,9 @@ typedef struct {
                                    phase that nothing completes, records the timeout and stops,
                                    so that the search returns GTLS_ERR_TIMEOUT: a test of the
                                    bounded-wait path that faults nothing.  Bit 1: every window
-                                   is summed (no window is ruled out by its bound), bit 2: the
-                                   bounds are used however small the search; for tests that
-                                   compare the two, results are the same */
+                                   is summed (no window is ruled out by its bound), for tests
+                                   that compare the two: results are the same.  Other bits are
+                                   ignored */
 } gtls_plan_params;
 
 /* Sizes of a plan (host struct filled by gtls_plan_get_info). */
@@ -139,8 +139,8 @@ typedef struct {
 /* Per-stage device time of the last search (host struct). */
 typedef struct {
     double ms_prepare;        /* per-curve arrays, t_ref, chi2_0, input checks */
-    double ms_fold_sort;      /* fold + sort + gather + prefix sums, all chunks */
-    double ms_window_search;  /* depth fit + chi2 of every window, all chunks */
+    double ms_fold_sort;      /* fold + sort + prefix sums, and the windows ruled out by bounds, all chunks */
+    double ms_window_search;  /* depth fit + chi2 of the windows left (of every window without bounds), all chunks */
     double ms_finalize;       /* per-period chi2(P), depth, T0 */
     double ms_sr_sde;         /* SR, SDE_raw, running median, argmax */
     int64_t kernel_launches;  /* kernels the last search launched */

@@ -7,20 +7,19 @@
 //   for every wave (chunk) of periods:
 //     k_fold_sort      fold on the exact phase lattice (Eq. phase), two-level
 //                      bucket sort by (phase, index) (super-buckets in global
-//                      memory, fine buckets in shared memory), gather the
-//                      folded curve, pad it with its first D_m points
-//                      (Sect. 2.3.2) and build the exact prefix sums that give
-//                      every moving average (Eq. cumsum)
-//     k_window_bounds, k_window_exact  (uniform weights) the windows that can
-//                      hold a period's minimum, and their sums
-//                      (window_bounds.cuh)
+//                      memory, fine buckets in shared memory), pad the folded
+//                      curve with its first D_m points (Sect. 2.3.2) and build
+//                      the prefix sums that give every moving average
+//                      (Eq. cumsum); then which windows can hold the
+//                      period's minimum (window_bounds.cuh)
+//     k_window_exact   the sums of those windows
 //     k_window_tiles   every duration and T0 start (Eq. N_skip): depth
 //                      (Eqs. k, depth), chi2 - chi2_0 (Eqs. out, in),
 //                      per-period minimum; staged tiles, window_tiles.cuh
-//                      (per-point weights, and periods the bounds leave;
+//                      (periods the bounds leave;
 //                      k_window_search: one thread per window, for plans
 //                      whose durations do not fit a tile)
-//     k_period_finalize chi2(P), depth, T0 of each period's minimum
+//     k_period_finalize(_sum) chi2(P), depth, T0 of each period's minimum
 //   k_sr_{min,sum,var}_set, k_median_sde_set   SR, SDE_raw, SDE (Sect. 2.4)
 //   k_topk + waves with T0 step 1           refinement of the best periods
 //                                           (Sect. 2.5), then SR/SDE again
@@ -81,7 +80,6 @@ constexpr int kScanPer = 8;           // consecutive prefix-sum positions per fo
 constexpr int kWeightedTilePairs = 24576;   // (w r, w) pairs staged per tile with per-point weights
 constexpr int kSearchThreads = 256;
 constexpr int kPrepBlocks = 1024;     // blocks per curve of its preparation, at most
-constexpr double kBoundsMinWpe = 5e8;  // window-point products of a search from which windows are ruled out by bounds
 constexpr int64_t kListPerSlot = 128;  // windows to sum per period and lane-group size a chunk has room for
 constexpr int kMedianThreads = 1024;
 constexpr int kMedianCap = 8192;       // values a median block sorts in shared memory
@@ -2865,9 +2863,9 @@ gtls_status create_device(gtls_plan* pl)
     const int64_t n = h.n;
     DevCurve& dc = pl->dc;
     GTLS_TRY(dev_alloc(pl, &dc.d_lat, n));
-    GTLS_TRY(dev_alloc(pl, &dc.d_f, n));
+    GTLS_TRY(dev_alloc(pl, &dc.d_f, 2 * n));
+    dc.r = dc.d_f + n;
     GTLS_TRY(dev_alloc(pl, &dc.pv, n));
-    GTLS_TRY(dev_alloc(pl, &dc.r, n));
     GTLS_TRY(dev_alloc(pl, &dc.scal, 8));
     GTLS_TRY(dev_alloc(pl, &dc.tmin_key, 1));
     GTLS_TRY(dev_alloc(pl, &dc.flags, 1));
@@ -3175,13 +3173,21 @@ gtls_status create_device(gtls_plan* pl)
 
     // tables of the window search by bounds
     {
-        // small searches are bound by launches: two kernels more cost what
-        // they save (0.29 ms and 6e7 window-point products: 18 us slower;
-        // 1.2 ms and 2.9e9: 140 us faster)
-        const bool worth = h.wpe >= kBoundsMinWpe || (h.prm.test_flags & 4);
-        pl->bounds_ok = !pl->has_tensor && worth && !(h.prm.test_flags & 2);
+        // at every size: 40 points and 2e5 window-point products 150 against
+        // 151 us by the tiled kernel, 257 and 6e7 196 against 207, 1000 and
+        // 1.3e9 371 against 556 (own dy: 157, 245, 656 against 163, 253, 827)
+        pl->bounds_ok = !pl->has_tensor && !(h.prm.test_flags & 2);
         std::vector<BoundTab> tab(dp.nd);
         std::vector<BoundDur> bd(dp.nd);
+        // (one allocation and copy for all tables)
+        std::vector<unsigned char> all;
+        auto place = [&](const auto& v) {
+            const size_t at = (all.size() + 255) & ~size_t(255), bytes = v.size() * sizeof(v[0]);
+            all.resize(at + bytes);
+            if (bytes) std::memcpy(all.data() + at, v.data(), bytes);
+            return at;
+        };
+        size_t at_tab[2] = {}, at_dur[2] = {}, at_drop = 0, at_fine = 0;
         const int threads = fold_threads(h.n), most = bounds::max_chunks(threads);
         const int clg = bounds::coarse_log2(threads, h.n, h.dmax);
         for (int pass = 0; pass < (pl->refine_k > 0 ? 2 : 1) && pl->bounds_ok; ++pass) {
@@ -3193,8 +3199,8 @@ gtls_status create_device(gtls_plan* pl)
             }
             DevPlan& q = pass ? pl->dp_ref : dp;
             q.bound_lg = bound_chunks(bd, var, h, most);
-            GTLS_TRY(upload(pl, const_cast<BoundTab**>(&q.bounds), tab));
-            GTLS_TRY(upload(pl, const_cast<BoundDur**>(&q.bound_durs), bd));
+            at_tab[pass] = place(tab);
+            at_dur[pass] = place(bd);
         }
         if (pl->bounds_ok) {
             // s_{k-1} - s_k of every template (0 before and after it), where dp.tmpl has s_k
@@ -3204,8 +3210,9 @@ gtls_status create_device(gtls_plan* pl)
                 for (int k = 0; k <= h.dpts[j]; ++k)
                     drop[(size_t)(pl->tmpl_pad_off[j] + k)] = (float)((k > 0 ? (double)tj[k - 1] : 0.0) - tj[k]);
             }
-            GTLS_TRY(upload(pl, const_cast<float**>(&dp.tmpl_drop), drop));
-            std::vector<float2> fine((size_t)dp.nd * kFinePieces, make_float2(0.0f, 0.0f));
+            at_drop = place(drop);
+            // (read for durations of at least kFineFrom points only)
+            std::vector<float2> fine(h.dmax >= kFineFrom ? (size_t)dp.nd * kFinePieces : 0, make_float2(0.0f, 0.0f));
             for (int j = 0; j < dp.nd; ++j) {
                 const int64_t d = h.dpts[j];
                 const float* const tj = pl->tmpl_pad.data() + pl->tmpl_pad_off[j];
@@ -3218,9 +3225,16 @@ gtls_status create_device(gtls_plan* pl)
                     fine[(size_t)(j * kFinePieces + g)] = make_float2(mean, (float)(std::sqrt(v) * (1.0 + 1e-6)));
                 }
             }
-            GTLS_TRY(upload(pl, const_cast<float2**>(&dp.bound_fine), fine));
-            pl->dp_ref.tmpl_drop = dp.tmpl_drop;
-            pl->dp_ref.bound_fine = dp.bound_fine;
+            at_fine = place(fine);
+            unsigned char* base = nullptr;
+            GTLS_TRY(upload(pl, &base, all));
+            for (int pass = 0; pass < (pl->refine_k > 0 ? 2 : 1); ++pass) {
+                DevPlan& q = pass ? pl->dp_ref : dp;
+                q.bounds = reinterpret_cast<const BoundTab*>(base + at_tab[pass]);
+                q.bound_durs = reinterpret_cast<const BoundDur*>(base + at_dur[pass]);
+                q.tmpl_drop = reinterpret_cast<const float*>(base + at_drop);
+                q.bound_fine = reinterpret_cast<const float2*>(base + at_fine);
+            }
         }
         // (the 32-bit prefix sums of w take the fold's keys' place)
         pl->bounds_w_ok = pl->bounds_ok && pl->tile_w_ok && !pl->has_window_only &&

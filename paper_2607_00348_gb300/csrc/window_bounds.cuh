@@ -22,7 +22,8 @@
 //      largest value of every chunk and the most promising windows are kept;
 //   3. those are summed: the lowest delta-chi2 T is the threshold;
 //   4. chunks whose largest value can beat T are walked again; windows that
-//      also pass the kBoundSegs-segment bound are summed, a warp each, and
+//      also pass the kBoundSegs-segment bound (long ones also the one by
+//      kFinePieces pieces) are summed, a warp each, and
 //      those within the rounding of the lowest sum are listed.
 // k_window_exact:
 //   5. the listed windows of all periods of the wave (one or two per period)
@@ -37,9 +38,9 @@
 // so that signed zeros decide; too many windows left; a value is not finite)
 // are listed for the tiled kernel, which then runs on that list.
 //
-// The window sums of steps 1 to 4 come from 32-bit prefix sums: the exact ones
-// shifted right so far that any sum fits 31 bits; differences are then off by
-// at most one unit.
+// The window sums of steps 1 to 4 come from 32-bit prefix sums of r rounded to
+// a unit with which any sum fits 31 bits: off by half a unit per point (the
+// unit is about 2e-4 of the noise of 62,363 points).
 //
 // Per-point weights (kW): delta-chi2 = depth (depth C2 - 2 C1) with
 // C1 = sum w r s_k and C2 = sum w s_k^2 is at least -C1^2 / C2 for any depth.
@@ -51,8 +52,12 @@
 // window's own, with its exact depth.  (20,011 points with a dy of their own: the
 // window stage was 98 ms on the tiled kernel, 126 with the fold; now 71 in all.)
 //
-// What bounds it: shared-memory reads of the coarse prefix and about 50
-// instructions per window.  A lane that reads global memory at a cache line
+// What bounds it (62,363 points, thousand cycles of a period's CTA at 0.55 / 5 /
+// 100 days): at short periods waiting between the steps (energies and
+// thresholds 34, first pass 24 / 68 / 271, threshold 6, second pass 18 / 41 / 42,
+// segments 28 / 33 / 21, sums 20 / 14 / 7; the tiled kernel took 1,100 on average
+// over the search), at long ones the instructions of the first pass, about 70
+// per 32 windows.  A lane that reads global memory at a cache line
 // of its own costs the L1 a cycle, which made the same tests on the prefix
 // sums themselves slower by half; only short windows (T0 steps of a few points, so
 // that neighbours share lines) read those,
