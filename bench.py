@@ -32,7 +32,6 @@ sys.path.insert(0, ROOT)
 
 METRIC = "Kepler-like light curves/hour on 1 GB300 (plain vs batched+learned, equal recall)"
 UNIT = "light curves/hour"
-FP32_LANES_PER_SM = 128          # FP32 FMA lanes per Blackwell SM (4 x 32)
 
 
 def _args():
@@ -174,9 +173,9 @@ class ClockSampler:
 
 
 def _kernel_sha():
-    """Hash of the window-search kernel's code (comments and blank space
-    removed): the k_window_tiles function, its warp tasks and the shared
-    device structures."""
+    """Hash of the code of the fold and the bounds that follow in its kernel
+    (comments and blank space removed): from FoldCfg to k_fold_sort, and the
+    shared device structures."""
     import re
 
     def code(src):
@@ -186,20 +185,28 @@ def _kernel_sha():
 
     csrc = os.path.join(ROOT, "paper_2607_00348_gb300", "csrc")
     search = open(os.path.join(csrc, "search.cu")).read()
-    start = search.index("k_window_tiles(DevSet")
-    body = search[start:search.index("\n}\n", start) + 3]
+    start = search.index("struct FoldCfg")
+    body = search[start:search.index("\n}\n", search.index("k_fold_sort(DevSet", start)) + 3]
     h = hashlib.sha256()
     for part in (open(os.path.join(csrc, "gtls_internal.h")).read(),
-                 open(os.path.join(csrc, "window_tiles.cuh")).read(), body):
+                 open(os.path.join(csrc, "window_bounds.cuh")).read(), body):
         h.update(code(part).encode())
     return h.hexdigest()[:16]
 
 
+def _hbm_peak_gbs():
+    """Measured copy bandwidth of this GPU type, or an earlier measurement."""
+    try:
+        return float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"]), "of measured"
+    except (OSError, KeyError, ValueError):
+        return 6800.0, "of fallback"
+
+
 def _ncu_traffic(workload):
-    """DRAM bytes per window-search launch from the committed ncu summary
-    (profiles/window_tiles_<workload>.md, lines 'kernel_sha: ...' and
+    """DRAM bytes per launch of the fold from the committed ncu summary
+    (profiles/fold_sort_<workload>.md, lines 'kernel_sha: ...' and
     'dram_bytes_per_launch: ...'), if it was taken on the current kernel."""
-    path = os.path.join(ROOT, "profiles", f"window_tiles_{workload}.md")
+    path = os.path.join(ROOT, "profiles", f"fold_sort_{workload}.md")
     vals = {}
     try:
         for line in open(path):
@@ -479,7 +486,7 @@ def run_gtls(args):
     clocks = ClockSampler(local)
     starts = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps)]
     ends = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps)]
-    win_ms, stage = [], []
+    stage = []
     launches = 0
     barrier()
     torch.cuda.synchronize()
@@ -490,7 +497,6 @@ def run_gtls(args):
         res = plan.search(t, y, dy, stream=stream)
         ends[k].record(stream)
         pr = plan.profile()
-        win_ms.append(pr.ms_window_search)
         stage.append(pr.as_dict())
         launches += int(pr.kernel_launches)
     torch.cuda.synchronize()
@@ -530,22 +536,21 @@ def run_gtls(args):
             torch.distributed.destroy_process_group()
         return 0
 
-    props = torch.cuda.get_device_properties(dev)
-    sm_max = (clk or {}).get("sm_max_mhz") or 2070.0
-    peak_tflops = 2.0 * props.multi_processor_count * FP32_LANES_PER_SM * sm_max * 1e6 / 1e12
-    win_s = statistics.mean(win_ms) / 1000.0
-    # 1 FMA per window-point evaluation with uniform dy; 2 (w r s and w s^2)
-    # with per-point dy
-    flop_per_wpe = 2.0 if res.uniform_dy else 4.0
-    achieved = flop_per_wpe * info["wpe"] / win_s / 1e12
-    traffic = _ncu_traffic(args.workload)
-    roofline = {"bound": "alu", "achieved": achieved, "peak": peak_tflops, "unit": "TFLOP/s",
-                "frac": achieved / peak_tflops, "traffic": traffic,
-                "kernel": "k_window_tiles",
-                "peak_basis": f"{props.multi_processor_count} SMs x {FP32_LANES_PER_SM} FP32 FMA "
-                              f"lanes x 2 flop x {sm_max:.0f} MHz (max SM clock)",
-                "achieved_basis": f"{flop_per_wpe:.0f} flop x window-point evaluations / mean "
-                                  "window-search stage time (CUDA events on the search stream)"}
+    # The fold, whose kernel also holds the bounds that leave one or two windows
+    # of a period to be summed, takes nearly all of the step.  It is bound by
+    # latency and instruction issue, not by bandwidth; the fraction says how far
+    # the bytes it has to move are from binding: per point and period a sort key
+    # written and read (16), the order (4) and the prefix sums (4; per-point
+    # weights: two of them, w, w r and exact sums of r, 24).
+    per_point = 24.0 if res.uniform_dy else 44.0
+    main_s = statistics.mean(s["ms_fold_sort"] + s["ms_window_search"] for s in stage) / 1000.0
+    achieved = per_point * info["n_periods"] * lc.n / main_s / 1e9
+    peak, basis = _hbm_peak_gbs()
+    roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+                "frac": achieved / peak, "traffic": _ncu_traffic(args.workload),
+                "kernel": "k_fold_sort", "peak_basis": f"copy bandwidth, {basis}",
+                "achieved_basis": f"{per_point:.0f} bytes per point and period / mean time of the fold and "
+                                  "window-search stages (CUDA events on the search stream)"}
     cpu = None
     if not args.no_cpu_baseline:
         v, threads, desc, dt, frac = oracle_sample(lc, args.cpu_seconds)
