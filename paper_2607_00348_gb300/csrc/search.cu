@@ -614,21 +614,25 @@ __device__ bool fold_staged(unsigned char* smem, const DevPlan& dp, const DevCur
         // super-bucket) look for it: 88 -> 63 thousand cycles of a 100-day
         // period of 62,363 points; at 0.55 days, where no warp would, the
         // look costs 51 -> 59.
+        // (loads of two points at a time: fold stage of the Kepler-like search
+        // 305.4 ms against 310.9 for four and 312.6 for eight; without the
+        // bounds four)
+        constexpr int kUnroll = kBounded ? 2 : kFoldUnroll;
         auto scatter = [&](auto look) {
             constexpr bool kLook = decltype(look)::value;
             const int64_t bs = blockDim.x;
             const int lane = threadIdx.x & 31;
-            for (int64_t g0 = 0; g0 < n; g0 += kFoldUnroll * bs) {
-                long long dl[kFoldUnroll];
-                float df[kFoldUnroll];
+            for (int64_t g0 = 0; g0 < n; g0 += kUnroll * bs) {
+                long long dl[kUnroll];
+                float df[kUnroll];
 #pragma unroll
-                for (int u = 0; u < kFoldUnroll; ++u) {
+                for (int u = 0; u < kUnroll; ++u) {
                     const int64_t i = g0 + u * bs + threadIdx.x;
                     dl[u] = i < n ? dc.d_lat[i] : 0;
                     df[u] = i < n ? dc.d_f[i] : 0.0f;
                 }
 #pragma unroll
-                for (int u = 0; u < kFoldUnroll; ++u) {
+                for (int u = 0; u < kUnroll; ++u) {
                     const int64_t i = g0 + u * bs + threadIdx.x;
                     const long long rho = lattice_rho(dl[u], df[u], P, inv_p);
                     const uint32_t sb = fold_fine(rho, sh, mulf) >> kFoldFineLog2;
