@@ -125,6 +125,14 @@ struct DevCurve {
 
 constexpr int kListClasses = 6;   // windows are summed by groups of 1, 2, 4, ..., 32 lanes
 
+// Words that the kernels of a wave count in (DevChunk::work): windows listed,
+// by class, items in `dense`, and the items that the tiled and the tensor-core
+// kernel have taken.  A wave starts with all of them at zero: they are cleared
+// in stream order before its first kernel (k_wave_next for waves cut on the
+// device), never by a kernel whose own CTAs add to them.
+constexpr int kWorkDense = kListClasses, kWorkTiles = kListClasses + 1, kWorkTensor = kListClasses + 2;
+constexpr int kWorkWords = kListClasses + 3;
+
 // Per-chunk scratch: `chunk` periods in flight.
 struct DevChunk {
     int32_t chunk;
@@ -144,7 +152,7 @@ struct DevChunk {
     int64_t list_cap;         // windows per lane-group size
     unsigned long long* list; // windows to sum, kListClasses lists
     int2* dense;              // items for the tiled kernel: slot, and tile | part << 20 | (parts - 1) << 24
-    unsigned int* left_n;     // [0 .. kListClasses) windows listed, [kListClasses] items in `dense`
+    unsigned int* work;       // kWorkWords counters of the wave in flight
 };
 
 // SR/SDE: blocks per curve of the reductions, and blocks of the running median
@@ -234,19 +242,17 @@ struct gtls_plan {
     // one-thread-per-window kernel in the same waves
     bool has_window_only = false, has_window_only_ref = false;
     // durations on the tensor-core window kernel (kTensor), the widest
-    // [jlo, jhi] span of a period (work items per period of that kernel),
-    // its counter, and the timeout test (a wait that nothing completes)
+    // [jlo, jhi] span of a period (work items per period of that kernel), and
+    // the timeout test (a wait that nothing completes)
     bool has_tensor = false;
     bool bounds_ok = false;              // the templates admit the bounds of window_bounds.cuh
     bool bounds_w_ok = false;            // ... with per-point weights
     int tc_jspan = 0;
-    unsigned int* tc_counter = nullptr;
     int tc_test_wait = 0;
     const void* tc_maps = nullptr;      // TMA maps of dk.rs (made with the chunk scratch)
     std::vector<int32_t> variant_host;   // window-kernel variant per duration (host copies)
     std::vector<int32_t> variant_ref_host, nc_host;
     int n_sm = 0;
-    unsigned int* tile_counter = nullptr;
     // refinement stage (T0 step 1 on the best periods): plan tables with
     // stride 1 and the (s_k, 1) pair tables, its tile configuration and the
     // device list of periods to re-search

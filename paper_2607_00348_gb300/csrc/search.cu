@@ -1081,11 +1081,7 @@ k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, 
     o.uniform = dc.scal[2] > 0.0;
     o.shift = kBounded ? min((int)dc.scal[3], 63) : 0;
     o.per_unit = kBounded ? 1.0f / prefix_unit(o.shift) : 0.0f;
-    if (threadIdx.x == 0) {
-        ds.outs[lc].best[p] = ~0ull;
-        if (kFold != Fold::kPlain && slot_id == 0)
-            for (int q = 0; q <= kListClasses; ++q) dk.left_n[q] = 0u;
-    }
+    if (threadIdx.x == 0) ds.outs[lc].best[p] = ~0ull;
 
     bool staged = fold_staged<kFold, T>(smem, dp, dc, p, keys, o);
     if constexpr (!FoldCfg<T>::kSingle) if (!staged) {
@@ -1207,7 +1203,7 @@ k_window_search(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* s
 
 __global__ void __launch_bounds__(tiles::kThreads, tiles::kCtasPerSm)
 k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, DevChunk dk, int buf, int weighted,
-               int listed, unsigned int* counter)
+               int listed)
 {
     const SlotMap& sm = smq ? *smq : smv;
     using namespace tiles;
@@ -1217,10 +1213,10 @@ k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
     __shared__ unsigned long long s_best[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the items the bounds kernel left, or every (period, tile) of the wave
-    const int items = listed ? (int)dk.left_n[kListClasses] : sm.items;
+    const int items = listed ? (int)dk.work[kWorkDense] : sm.items;
     for (;;) {
         if (threadIdx.x == 0) {
-            const int item = (int)atomicAdd(counter, 1u);
+            const int item = (int)atomicAdd(dk.work + kWorkTiles, 1u);
             s_item = item < items ? 1 : 0;
             if (item < items) {
                 int lcg = 0, pp = -1, slot = 0, tau = 0, part = 0, parts = 1;
@@ -1926,7 +1922,7 @@ k_period_finalize_sum(DevSet ds, const __grid_constant__ SlotMap smv, const Slot
 // The periods of a batch are a list of (curve, first, count) runs; a wave
 // takes the next at most `wave_slots` periods of the list in at most kMaxSeg
 // segments.  k_wave_next cuts the next wave from the queue's cursor into
-// device memory, clears the wave's window-kernel counters and, when the
+// device memory, clears the wave's counters and, when the
 // queue is empty after it, sets the condition of the enclosing graph loop to
 // zero, so that one loop node replays the wave kernels until the queue is
 // drained: the graph has the same nodes for any number of curves.
@@ -1942,7 +1938,7 @@ struct WaveQueue {
     int32_t from_list;
     int32_t* cursor;              // [0] run, [1] periods of that run taken, [2] waves cut
     SlotMap* wave;                // the wave being searched
-    unsigned int* counters;       // the window kernels' item counters (2)
+    unsigned int* work;           // the wave's counters (kWorkWords)
     cudaGraphConditionalHandle cond;
 };
 
@@ -1971,8 +1967,7 @@ __global__ void k_wave_next(WaveQueue q)
     q.cursor[0] = r;
     q.cursor[1] = off;
     q.cursor[2] += 1;
-    q.counters[0] = 0;
-    q.counters[1] = 0;
+    for (int k = 0; k < kWorkWords; ++k) q.work[k] = 0u;
     cudaGraphSetConditional(q.cond, r < q.nruns ? 1u : 0u);
 }
 
@@ -3171,8 +3166,6 @@ gtls_status create_device(gtls_plan* pl)
             GTLS_TRY(upload(pl, const_cast<int32_t**>(&pl->dp_ref.cfg_variant), var1));
             pl->variant_ref_host = var1;
         }
-        GTLS_TRY(dev_alloc(pl, &pl->tile_counter, 1));
-        GTLS_TRY(dev_alloc(pl, &pl->tc_counter, 1));
     }
 
     // tables of the window search by bounds
@@ -3315,12 +3308,12 @@ gtls_status ensure_chunk(gtls_plan* pl)
     GTLS_TRY(dev_alloc(pl, &dk.ws, chunk * dk.pad_stride));
     GTLS_TRY(dev_alloc(pl, &dk.wrs, chunk * dk.pad_stride));
     GTLS_TRY(dev_alloc(pl, &dk.pf, chunk * dk.pad_stride));
+    GTLS_TRY(dev_alloc(pl, &dk.work, kWorkWords));
     if (pl->bounds_ok) {
         GTLS_TRY(dev_alloc(pl, &dk.pq, chunk * dk.pad_stride));
         dk.list_cap = std::max<int64_t>(4096, chunk * kListPerSlot);
         GTLS_TRY(dev_alloc(pl, &dk.list, kListClasses * dk.list_cap));
         GTLS_TRY(dev_alloc(pl, &dk.dense, chunk * bounds::kDenseParts * std::max({1, pl->tile_count, pl->tile_count_ref, pl->tile_count_w})));
-        GTLS_TRY(dev_alloc(pl, &dk.left_n, kListClasses + 1));
     }
     if (pl->has_tensor) {
         unsigned char* maps = nullptr;
@@ -3339,7 +3332,7 @@ gtls_status trim_chunk(gtls_plan* pl)
     if (!pl->chunk_ready) return GTLS_OK;
     GTLS_CUDA(cudaDeviceSynchronize());
     const void* mine[] = {pl->dk.keys, pl->dk.sidx, pl->dk.rs, pl->dk.ws, pl->dk.wrs, pl->dk.pf,
-                          pl->dk.pq, pl->dk.list, pl->dk.dense, pl->dk.left_n, pl->tc_maps};
+                          pl->dk.pq, pl->dk.list, pl->dk.dense, pl->dk.work, pl->tc_maps};
     int kept = 0;
     for (int i = 0; i < pl->n_allocs; ++i) {
         bool chunk = false;
@@ -3359,7 +3352,7 @@ gtls_status trim_chunk(gtls_plan* pl)
     pl->dk.dense = nullptr;
     pl->dk.pq = nullptr;
     pl->dk.list = nullptr;
-    pl->dk.left_n = nullptr;
+    pl->dk.work = nullptr;
     pl->dk.chunk = chunk;
     pl->tc_maps = nullptr;
     pl->chunk_ready = false;
@@ -3448,25 +3441,23 @@ void launch_fold(Ctx& c, const DevSet& ds, const SlotMap& sm, const SlotMap* smq
     else launch_fold_as<kFold, 1024>(c, ds, sm, smq, fill);
 }
 
-// One wave: fold + sort, every window, per-period results.  `counter` must
-// be zero when the window kernel starts (reset here when reset_counter).
-// With smq (a wave cut on the device, see k_wave_next) the kernels read the
-// wave from device memory; sm.slots then only sizes the grids (the most
-// slots a wave of the queue can hold).
-gtls_status wave_pass(Ctx& c, bool ref, const SlotMap& sm, bool tiled, bool weighted, bool window_only,
-                      unsigned int* counter, bool reset_counter, int64_t max_n, int max_kept, bool tensor = false,
-                      unsigned int* tc_counter = nullptr, const SlotMap* smq = nullptr)
+// One wave: fold + sort, every window, per-period results.  With smq (a wave
+// cut on the device by k_wave_next, which has cleared the wave's counters) the
+// kernels read the wave from device memory; sm.slots then only sizes the grids
+// (the most slots a wave of the queue can hold).
+gtls_status wave_pass(Ctx& c, bool ref, const SlotMap& sm, bool tiled, bool weighted, bool window_only, int64_t max_n,
+                      int max_kept, bool tensor = false, const SlotMap* smq = nullptr)
 {
     const DevSet& ds = ref ? c.set_ref : c.set;
     const bool bounded = tiled && (weighted ? c.bounds_w_ok : c.bounds_ok);
     const int threads = fold_threads(max_n);
+    if (tiled && !smq) GTLS_CUDA(cudaMemsetAsync(c.dk.work, 0, kWorkWords * sizeof(unsigned int), c.st));
     if (!bounded) launch_fold<Fold::kPlain>(c, ds, sm, smq, threads);
     else if (weighted) launch_fold<Fold::kBoundsW>(c, ds, sm, smq, threads);
     else launch_fold<Fold::kBounds>(c, ds, sm, smq, threads, window_only);   // (that kernel reads every folded curve)
     GTLS_CUDA(cudaGetLastError());
     GTLS_TRY(stage_mark(c, kStageFold));
     if (tiled) {
-        if (reset_counter) GTLS_CUDA(cudaMemsetAsync(counter, 0, sizeof(unsigned int), c.st));
         const int buf = weighted ? c.tile_buf_w : c.tile_buf;
         const int bytes = buf * (int)(weighted ? sizeof(float2) : sizeof(float));
         if (bounded) {
@@ -3483,14 +3474,13 @@ gtls_status wave_pass(Ctx& c, bool ref, const SlotMap& sm, bool tiled, bool weig
             c.launches += 1;
         }
         k_window_tiles<<<c.n_sm * tiles::kCtasPerSm, tiles::kThreads, bytes, c.st>>>(
-            ds, sm, smq, c.dk, buf, weighted ? 1 : 0, bounded ? 1 : 0, counter);
-        if (tensor && !weighted && tc_counter) {
+            ds, sm, smq, c.dk, buf, weighted ? 1 : 0, bounded ? 1 : 0);
+        if (tensor && !weighted) {
             // the durations marked kTensor (the tiled kernel gave them no tasks)
             GTLS_CUDA(cudaGetLastError());
-            if (reset_counter) GTLS_CUDA(cudaMemsetAsync(tc_counter, 0, sizeof(unsigned int), c.st));
             if (!c.tc_maps) return fail(GTLS_ERR_INTERNAL, "tensor-core window kernel without tensor maps");
             k_window_tc<<<c.n_sm, tc::kThreads, tc::kSmemRequest, c.st>>>(ds, sm, smq, c.dk, c.tc_maps, c.tc_jspan,
-                                                                        tc_counter, c.tc_test);
+                                                                        c.dk.work + kWorkTensor, c.tc_test);
             c.launches += 1;
         }
     }
@@ -3642,8 +3632,8 @@ gtls_status run_search(gtls_plan* pl, const double* t, const double* y, const do
     for (int p0 = 0; p0 < dp.np; p0 += dk.chunk) {
         const int cnt = std::min<int>(dk.chunk, dp.np - p0);
         GTLS_TRY(wave_pass(c, false, single_wave(p0, cnt, wtiled ? pl->tile_count_w : pl->tile_count, false),
-                           tiled || wtiled, wtiled, tiled && pl->has_window_only, pl->tile_counter, true, n,
-                           h.max_kept, tiled && pl->has_tensor, pl->tc_counter));
+                           tiled || wtiled, wtiled, tiled && pl->has_window_only, n, h.max_kept,
+                           tiled && pl->has_tensor));
     }
     GTLS_TRY(sr_sde_pass(c));
     // two-stage T0 search (Sect. 2.5): the refine_k best periods by SDE(P)
@@ -3658,7 +3648,7 @@ gtls_status run_search(gtls_plan* pl, const double* t, const double* y, const do
         for (int r0 = 0; r0 < kref; r0 += dk.chunk) {
             const int cnt = std::min<int>(dk.chunk, kref - r0);
             GTLS_TRY(wave_pass(c, true, single_wave(r0, cnt, pl->tile_count_ref, true), tiled, false,
-                               tiled && pl->has_window_only_ref, pl->tile_counter, true, n, h.max_kept));
+                               tiled && pl->has_window_only_ref, n, h.max_kept));
         }
         GTLS_TRY(sr_sde_pass(c));
     }
@@ -3719,8 +3709,6 @@ struct gtls_batch {
     unsigned int* flags = nullptr;     // per curve validity flags
     unsigned int* checks = nullptr;    // 4 words per curve
     gtls_result* results = nullptr;
-    unsigned int* counters = nullptr;  // two per tiled wave (autotuner probes) or per graph loop
-    int n_counters = 0;
     // device work queues of the graph's loops: their (curve, first, count,
     // tiles per period) runs, the wave each loop is searching and the cursors
     int32_t* q_runs = nullptr;         // 4 words per run, at most 2 n_lc runs
@@ -3921,17 +3909,6 @@ gtls_status batch_upload_tiles(gtls_batch* b)
     return GTLS_OK;
 }
 
-// Makes sure there are two window-kernel counters (tiled, tensor-core) for
-// each of n waves or loops.
-gtls_status batch_counters(gtls_batch* b, int n)
-{
-    if (2 * n <= b->n_counters) return GTLS_OK;
-    const int m = std::max(2 * n, 2 * b->n_counters);
-    GTLS_TRY(batch_alloc(b, &b->counters, m));
-    b->n_counters = m;
-    return GTLS_OK;
-}
-
 // One loop of the batch graph: the runs of one kernel class, coarse or
 // refinement, and what its wave kernels need.
 constexpr int kMaxLoops = 6;   // classes 1, 2, 0 for the coarse and the refinement pass
@@ -4018,7 +3995,7 @@ gtls_status capture_loop(gtls_batch* b, Ctx& c, LoopSpec& L, int qi)
     q.from_list = L.ref ? 1 : 0;
     q.cursor = b->q_cursors + 3 * qi;
     q.wave = b->q_waves + qi;
-    q.counters = b->counters + 2 * qi;
+    q.work = b->dk.work;   // (the loops run one after the other)
     q.cond = h;
     GTLS_CUDA(cudaStreamBeginCaptureToGraph(b->body_stream, body, nullptr, nullptr, 0,
                                             cudaStreamCaptureModeThreadLocal));
@@ -4030,8 +4007,7 @@ gtls_status capture_loop(gtls_batch* b, Ctx& c, LoopSpec& L, int qi)
     SlotMap grid{};   // grid sizes: the most slots a wave can hold
     grid.slots = b->cfg.wave_slots;
     if (s == GTLS_OK)
-        s = wave_pass(cb, L.ref, grid, L.tiled, L.weighted, L.window_only, q.counters, false, L.max_n, L.max_kept,
-                      L.tensor, q.counters + 1, q.wave);
+        s = wave_pass(cb, L.ref, grid, L.tiled, L.weighted, L.window_only, L.max_n, L.max_kept, L.tensor, q.wave);
     cudaGraph_t out = nullptr;
     const cudaError_t e = cudaStreamEndCapture(b->body_stream, &out);
     if (s != GTLS_OK) return s;
@@ -4080,7 +4056,6 @@ gtls_status batch_capture(gtls_batch* b, cudaStream_t st, const std::vector<uint
     batch_loops(b, cls, runs, coarse, refine);
     if (coarse.size() + refine.size() > (size_t)kMaxLoops || runs.size() > 2 * (size_t)b->n_lc)
         return fail(GTLS_ERR_INTERNAL, "batch queue table overflow");
-    GTLS_TRY(batch_counters(b, kMaxLoops));
     if (!runs.empty())
         GTLS_CUDA(cudaMemcpy(b->q_runs, runs.data(), runs.size() * sizeof(QueueRun), cudaMemcpyHostToDevice));
     // captured on the batch's own stream (the caller's may be the legacy
@@ -4238,6 +4213,7 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     GTLS_TRY(batch_alloc(b, &dk.ws, slots * pad_stride));
     GTLS_TRY(batch_alloc(b, &dk.wrs, slots * pad_stride));
     GTLS_TRY(batch_alloc(b, &dk.pf, slots * pad_stride));
+    GTLS_TRY(batch_alloc(b, &dk.work, kWorkWords));
     {
         bool any_tensor = false;
         for (int i = 0; i < n_lc; ++i) any_tensor = any_tensor || plans[i]->has_tensor;
@@ -4291,7 +4267,6 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
         GTLS_TRY(batch_alloc(b, &b->dk.pq, slots * pad_stride));
         b->dk.list_cap = std::max<int64_t>(4096, slots * kListPerSlot);
         GTLS_TRY(batch_alloc(b, &b->dk.list, kListClasses * b->dk.list_cap));
-        GTLS_TRY(batch_alloc(b, &b->dk.left_n, kListClasses + 1));
     }
     return GTLS_OK;
 }
@@ -4360,17 +4335,13 @@ gtls_status batch_autotune(gtls_batch* b, const double* t, const double* y, cons
         for (int sc : slot_c) {
             std::vector<BatchWave> waves;
             build_waves(b, probe, true, false, false, sc, waves);
-            if ((s = batch_counters(b, (int)waves.size())) != GTLS_OK) break;
             Ctx c = batch_ctx(b, st);
             c.tile_buf = bc;
             float ms = 0.0f;
             for (int rep = 0; rep < 3 && s == GTLS_OK; ++rep) {
                 if (rep == 1 && cudaEventRecord(e0, st) != cudaSuccess) s = fail(GTLS_ERR_CUDA, "cudaEventRecord");
-                int ci = 0;
                 for (const BatchWave& w : waves) {
-                    unsigned int* cnt = b->counters + 2 * ci++;
-                    s = wave_pass(c, false, w.sm, true, false, false, cnt, true, w.max_n, w.max_kept, w.tensor,
-                                  cnt + 1);
+                    s = wave_pass(c, false, w.sm, true, false, false, w.max_n, w.max_kept, w.tensor);
                     if (s != GTLS_OK) break;
                 }
             }

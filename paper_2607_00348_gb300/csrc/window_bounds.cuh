@@ -1194,7 +1194,7 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
             const int m = (int)(e & 0xffffffu);
             auto push = [&](int rot) {
                 const unsigned int to =
-                    atomicAdd(&S.n_listed, 1) < S.ck.listed ? atomicAdd(dk.left_n + t.b.lg_nc, 1u) : 0xffffffffu;
+                    atomicAdd(&S.n_listed, 1) < S.ck.listed ? atomicAdd(dk.work + t.b.lg_nc, 1u) : 0xffffffffu;
                 if (to < dk.list_cap)
                     dk.list[t.b.lg_nc * dk.list_cap + to] = ((unsigned long long)slot << 40) |
                                                             ((unsigned long long)t.b.j << 32) |
@@ -1231,7 +1231,7 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         // (a tile's tasks shared by `parts` CTAs, about 65,536 windows each: the
         // 1.2e6 windows of one period at T0 step 1 kept an SM for 15 ms)
         const int tc = kW ? ds.tiles[lc].count_w : ds.tiles[lc].count, parts = S.ck.parts;
-        const unsigned int to = atomicAdd(dk.left_n + kListClasses, (unsigned int)(tc * parts));
+        const unsigned int to = atomicAdd(dk.work + kWorkDense, (unsigned int)(tc * parts));
         for (int i = 0; i < tc * parts; ++i)
             dk.dense[to + i] = make_int2(slot, (i / parts) | ((i % parts) << 20) | ((parts - 1) << 24));
     }
@@ -1272,7 +1272,7 @@ k_window_exact(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int item = blockIdx.x;
     for (int q = 0; q < kListClasses; ++q) {
-        const int cnt = (int)min((int64_t)dk.left_n[q], dk.list_cap);
+        const int cnt = (int)min((int64_t)dk.work[q], dk.list_cap);
         for (; item < cnt; item += gridDim.x) {
             const unsigned long long en = dk.list[q * dk.list_cap + item];
             const int slot = (int)(en >> 40), j = (int)(en >> 32) & 0xff, rot = (int)(en >> 24) & 0xff;
@@ -1336,7 +1336,7 @@ k_window_exact_w(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* 
     const int lane = threadIdx.x;
     int item = blockIdx.x;
     for (int q = 0; q < kListClasses; ++q) {
-        const int cnt = (int)min((int64_t)dk.left_n[q], dk.list_cap);
+        const int cnt = (int)min((int64_t)dk.work[q], dk.list_cap);
         for (; item < cnt; item += gridDim.x) {
             const unsigned long long en = dk.list[q * dk.list_cap + item];
             const int slot = (int)(en >> 40), j = (int)(en >> 32) & 0xff, m = (int)(en & 0xffffffull);
