@@ -151,6 +151,7 @@ struct DevChunk {
     int32_t* pq;              // of r (per-point weights: w r) in units (modulo 2^32: window sums fit 31 bits)
     int64_t list_cap;         // windows per lane-group size
     unsigned long long* list; // windows to sum, kListClasses lists
+    int64_t dense_cap;        // items
     int2* dense;              // items for the tiled kernel: slot, and tile | part << 20 | (parts - 1) << 24
     unsigned int* work;       // kWorkWords counters of the wave in flight
 };

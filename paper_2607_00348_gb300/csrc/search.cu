@@ -1213,7 +1213,7 @@ k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
     __shared__ unsigned long long s_best[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the items the bounds kernel left, or every (period, tile) of the wave
-    const int items = listed ? (int)dk.work[kWorkDense] : sm.items;
+    const int items = listed ? (int)min((int64_t)dk.work[kWorkDense], dk.dense_cap) : sm.items;
     for (;;) {
         if (threadIdx.x == 0) {
             const int item = (int)atomicAdd(dk.work + kWorkTiles, 1u);
@@ -3313,7 +3313,9 @@ gtls_status ensure_chunk(gtls_plan* pl)
         GTLS_TRY(dev_alloc(pl, &dk.pq, chunk * dk.pad_stride));
         dk.list_cap = std::max<int64_t>(4096, chunk * kListPerSlot);
         GTLS_TRY(dev_alloc(pl, &dk.list, kListClasses * dk.list_cap));
-        GTLS_TRY(dev_alloc(pl, &dk.dense, chunk * bounds::kDenseParts * std::max({1, pl->tile_count, pl->tile_count_ref, pl->tile_count_w})));
+        dk.dense_cap = chunk * bounds::kDenseParts *
+                       std::max({1, pl->tile_count, pl->tile_count_ref, pl->tile_count_w});
+        GTLS_TRY(dev_alloc(pl, &dk.dense, dk.dense_cap));
     }
     if (pl->has_tensor) {
         unsigned char* maps = nullptr;
@@ -4263,7 +4265,8 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     if (b->bounds_ok) {
         int max_tiles = 1;
         for (const DevTiles& t : b->tiles_host) max_tiles = std::max({max_tiles, t.count, t.count_w});
-        GTLS_TRY(batch_alloc(b, &b->dk.dense, slots * (int64_t)max_tiles * bounds::kDenseParts));
+        b->dk.dense_cap = slots * (int64_t)max_tiles * bounds::kDenseParts;
+        GTLS_TRY(batch_alloc(b, &b->dk.dense, b->dk.dense_cap));
         GTLS_TRY(batch_alloc(b, &b->dk.pq, slots * pad_stride));
         b->dk.list_cap = std::max<int64_t>(4096, slots * kListPerSlot);
         GTLS_TRY(batch_alloc(b, &b->dk.list, kListClasses * b->dk.list_cap));

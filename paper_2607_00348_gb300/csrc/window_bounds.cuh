@@ -1231,8 +1231,11 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         // (a tile's tasks shared by `parts` CTAs, about 65,536 windows each: the
         // 1.2e6 windows of one period at T0 step 1 kept an SM for 15 ms)
         const int tc = kW ? ds.tiles[lc].count_w : ds.tiles[lc].count, parts = S.ck.parts;
-        const unsigned int to = atomicAdd(dk.work + kWorkDense, (unsigned int)(tc * parts));
-        for (int i = 0; i < tc * parts; ++i)
+        const long long to = atomicAdd(dk.work + kWorkDense, (unsigned int)(tc * parts));
+        // (there is room for every period of a wave; as far as there is room,
+        // every item that the tiled kernel will read is written)
+        in_range(ds.curves[lc].check, 24, to + tc * parts - 1, dk.dense_cap);
+        for (int i = 0; i < tc * parts && to + i < dk.dense_cap; ++i)
             dk.dense[to + i] = make_int2(slot, (i / parts) | ((i % parts) << 20) | ((parts - 1) << 24));
     }
     if (!kW && (fill || !fits)) {

@@ -77,3 +77,17 @@ def test_batch_loops_in_small_waves():
     batch.close()
     for p in plans:
         p.close()
+
+
+@pytest.mark.parametrize("own_dy", [False, True])
+def test_list_for_the_tiled_kernel_filled_to_its_capacity(own_dy):
+    # 1.5 million windows a period at T0 step 1 (16 items a tile), every period
+    # of every wave left to the tiled kernel
+    n, kw = 70001, dict(periods_days=np.geomspace(1.0, 9.0, 8), refine_periods=8)
+    c = _curve(n, "flat", own_dy, 5)
+    got = []
+    for flags, chunk in ((0, 4), (2, 0)):
+        p = _plan(n, flags, periods_per_chunk=chunk, **kw)
+        got.append(gh.gpu_search(p, *c)[1])
+        p.close()
+    _equal(*got)
