@@ -825,12 +825,14 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
 // and then gives each bin to one thread, which needs two FP64 operations per
 // point (1 - y and its sum) and one reciprocal per bin while dy stays the
 // same.  kBinCtas CTAs share a curve, each a quarter of the bins.  Curves
-// whose points turn out not to be in order are flagged and left to
-// k_bin_any (shared-memory atomics).  256 curves of 20,000 to 72,000 points:
+// whose points turn out not to be in order, or that have too many of them for
+// its 32-bit counts, are flagged and left to k_bin_any (shared-memory atomics).  256 curves of 20,000 to 72,000 points:
 // 0.28 ms; 1.9 ms with two divisions and two atomics per point.
 constexpr int kBinThreads = 256;
 constexpr int kBinRun = 16;      // consecutive points of a thread (k_bin_any)
 constexpr int kBinCtas = 4;      // CTAs per curve
+constexpr int64_t kBinSortedMax = int64_t(1) << 30;   // points of a curve that k_bin_sorted takes (steps of a few
+                                                      // thousand past the last one still fit an int)
 constexpr long long kInfKey = 0x7ff0000000000000ll;
 
 // The bin formula.
@@ -873,8 +875,12 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_sorted(const double* __rest
     __shared__ int edge[2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int lc = blockIdx.x / kBinCtas, rank = blockIdx.x - lc * kBinCtas;
-    const int64_t o = off[lc];
-    const int n = (int)(off[lc + 1] - o);
+    const int64_t o = off[lc], points = off[lc + 1] - o;
+    if (points > kBinSortedMax) {   // (all CTAs of the curve)
+        if (threadIdx.x == 0) unsorted[lc] = 1u;
+        return;
+    }
+    const int n = (int)points;
     t += o;
     y += o;
     dy += o;
