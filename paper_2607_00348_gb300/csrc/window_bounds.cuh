@@ -35,8 +35,9 @@
 //      those of the tiled kernel.
 //
 // Periods for which nothing is gained (no window has a negative delta-chi2,
-// so that signed zeros decide; too many windows left; a value is not finite)
-// are listed for the tiled kernel, which then runs on that list.
+// so that signed zeros decide, or only subnormal ones, which are often equal;
+// too many windows left; a value is not finite) are listed for the tiled
+// kernel, which then runs on that list.
 //
 // The window sums of steps 1 to 4 come from 32-bit prefix sums of r rounded to
 // a unit with which any sum fits 31 bits: off by half a unit per point (the
@@ -85,6 +86,7 @@ constexpr int kExactRoom = 24576;   // points of a window (and its template) sta
 constexpr int kFloorSpans = 48;     // stretches of blocks whose smallest weight is kept: 1 .. 15, then 16, 19, 22,
                                     // 27 times powers of 2
 constexpr unsigned int kNone = 0xffffffffu;
+constexpr float kLeast = 1e-30f;    // smallest |delta-chi2| whose rounding is relative, w times the depth among its factors
 constexpr int kNoUnit = 1000;       // per-point weights whose sums do not fit the 32-bit prefix
 
 enum Mode : int { kModePairS = 0, kModeCols = 1, kModeRot = 2, kModeWin = 3 };
@@ -957,8 +959,10 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         const float v0 = __shfl_sync(0xffffffffu, v, 0), v1 = __shfl_sync(0xffffffffu, v, kTeam);
         thr = isnan(v0) || isnan(v1) ? NAN : fminf(v0, v1);
     }
-    // no negative delta-chi2, or values out of range: the tiled kernel decides
-    const bool sane = thr < 0.0f && thr > -INFINITY && e_all < INFINITY && w_uni < INFINITY && in_range_32;
+    // no negative delta-chi2, one so small that it or its factors are subnormal
+    // in FP32 (the slacks below are relative), or values out of range: the
+    // tiled kernel decides
+    const bool sane = thr < -kLeast && thr > -INFINITY && e_all < INFINITY && w_uni < INFINITY && in_range_32;
     if (sane) {
         // 1e-4 of slack covers the rounding of delta-chi2
         const float reach = sqrtf(-thr / w_uni) * (1.0f - 1e-4f);   // (times the root of C2 or sum s_k^2)
