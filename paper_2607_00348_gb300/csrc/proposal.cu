@@ -943,8 +943,9 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_sorted(const double* __rest
     for (int b = threadIdx.x; b < kShare; b += kBinThreads) {
         const int i1 = start[b + 1];
         int i = start[b];
-        double sw = 0.0, swr = 0.0, w = 0.0, sum = 0.0;
-        long long dy_bits = -1;   // (no dy has these bits)
+        double sw = 0.0, swr = 0.0, sum = 0.0;
+        long long dy_bits = -1;   // (the bits of a NaN, whose w is one too)
+        double w = __longlong_as_double(dy_bits);
         int cnt = 0;
 #pragma unroll 4
         for (; i < i1; ++i) {
@@ -1032,8 +1033,8 @@ k_bin_any(const double* __restrict__ t, const double* __restrict__ y, const doub
     }
     const double lo = key_time(klo), hi = key_time(khi);
     const double span = __dsub_rn(hi, lo);
-    double w = 0.0;
-    long long dy_bits = -1;   // (no dy has these bits)
+    long long dy_bits = -1;   // (the bits of a NaN, whose w is one too)
+    double w = __longlong_as_double(dy_bits);
     for (int64_t i0 = p0 + (int64_t)threadIdx.x * kBinRun; i0 < p1; i0 += (int64_t)kBinThreads * kBinRun) {
         const int len = (int)min((int64_t)kBinRun, p1 - i0);
         int bin = -1, cnt = 0;

@@ -36,3 +36,27 @@ def test_curve_of_more_points_than_32_bits_count():
     for got, want in zip((x, mean, wsum), alone):
         assert np.array_equal(got[1], want[0])
     net.close()
+
+
+@pytest.mark.parametrize("ordered", [True, False])
+@pytest.mark.parametrize("bits", [-1, 0x7ff8000000000000])
+def test_uncertainty_that_is_no_number(bits, ordered):
+    # sum w is NaN in the point's bin, whose values are then 0, whatever the
+    # NaN's bits; the other bins are those of the curve without the point
+    import torch
+    n, k = 640, 321
+    t = np.linspace(0.0, 10.0, n)
+    y = 1.0 + np.random.default_rng(1).normal(0.0, 1e-3, n)
+    dy = np.full(n, 1e-3)
+    dy[k] = np.array([bits], np.int64).view(np.float64)[0]
+    keep = np.arange(n) != k
+    order = np.arange(n) if ordered else np.roll(np.arange(n), 77)
+    dev = [torch.as_tensor(np.concatenate([a[order], a[keep]]), device="cuda:0") for a in (t, y, dy)]
+    net = pkg.Cnn(2)
+    x, mean, wsum = _bin(net, *dev, [0, n, 2 * n - 1])
+    net.close()
+    b = int(np.floor(t[k] / 10.0 * cnn.N_BINS))
+    assert np.isnan(wsum[0, b]) and x[0, b] == 0.0 and mean[0, b] == 0.0
+    others = np.arange(cnn.N_BINS) != b
+    for a in (x, mean, wsum):
+        np.testing.assert_allclose(a[0, others], a[1, others], rtol=1e-6, atol=0)
