@@ -4768,7 +4768,16 @@ extern "C" gtls_status gtls_sr_sde_noalloc(const double* chi2, int64_t n_periods
 
     DevPeriod dq{};
     dq.chi2 = const_cast<double*>(chi2);
-    dq.sr = sr_out ? sr_out : head + kNoAllocHead;
+    // the median's blocks read SR around their outputs while others write
+    // theirs: an SR array that shares memory with those is filled from the
+    // fixed one before they are written
+    auto shares = [&](const double* out) {
+        const uintptr_t a = reinterpret_cast<uintptr_t>(sr_out), b = reinterpret_cast<uintptr_t>(out);
+        const uintptr_t bytes = (uintptr_t)np * sizeof(double);
+        return sr_out && out && a < b + bytes && b < a + bytes;
+    };
+    const bool sr_shared = shares(sde_out) || shares(sde_raw_out);
+    dq.sr = sr_out && !sr_shared ? sr_out : head + kNoAllocHead;
     dq.sde_raw = sde_raw_out ? sde_raw_out : head + kNoAllocHead + kNoAllocMaxPeriods;
     dq.sde = sde_out;
     dq.stats = head;
@@ -4783,6 +4792,8 @@ extern "C" gtls_status gtls_sr_sde_noalloc(const double* chi2, int64_t n_periods
     GTLS_CUDA(cudaGetLastError());
     k_sr_var<<<sr_blocks(np), kSrThreads, 0, st>>>(np, dq);
     GTLS_CUDA(cudaGetLastError());
+    if (sr_shared)
+        GTLS_CUDA(cudaMemcpyAsync(sr_out, dq.sr, (size_t)np * sizeof(double), cudaMemcpyDeviceToDevice, st));
     k_median_sde<<<blocks, kMedianThreads, kMedianSmem, st>>>(np, hwin, outs, dq);
     GTLS_CUDA(cudaGetLastError());
     k_argmax_noalloc<<<1, 1024, 0, st>>>(np, blocks, dq, head);
