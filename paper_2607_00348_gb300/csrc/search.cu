@@ -1079,7 +1079,7 @@ k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, 
     o.pf = dk.pf + (int64_t)slot_id * dk.pad_stride;
     o.pq = dk.pq + (int64_t)slot_id * dk.pad_stride;
     o.uniform = dc.scal[2] > 0.0;
-    o.shift = kBounded ? min((int)dc.scal[3], 63) : 0;
+    o.shift = kBounded ? max(0, min((int)dc.scal[3], 63)) : 0;
     o.per_unit = kBounded ? 1.0f / prefix_unit(o.shift) : 0.0f;
     if (threadIdx.x == 0) ds.outs[lc].best[p] = ~0ull;
 
@@ -4287,8 +4287,8 @@ double period_wpe(const PlanHost& h, int p)
 
 // Picks the wave size and the staged tile size: every candidate runs the
 // coarse pass of a probe (runs of 256 periods spread over the grids of the
-// first tiled curves) once untimed and twice timed; the score is window-point
-// evaluations per second.
+// first tiled curves, each by the kernels of its class) once untimed and twice
+// timed; the score is window-point evaluations per second.
 gtls_status batch_autotune(gtls_batch* b, const double* t, const double* y, const double* dy,
                            const int64_t* offsets, cudaStream_t st)
 {
@@ -4298,7 +4298,7 @@ gtls_status batch_autotune(gtls_batch* b, const double* t, const double* y, cons
     int64_t launches = 0;
     GTLS_TRY(batch_prepare(b, t + o0, y + o0, dy + o0, st, flags, launches));
     std::vector<uint8_t> cls = batch_classes(b, flags);
-    std::vector<Run> probe;
+    std::vector<Run> probe[2];   // curves of class 1, of class 2 (per-point weights)
     double probe_wpe = 0.0;
     for (int i = 0, used = 0; i < b->n_lc && used < 4; ++i) {
         if (!cls[i]) continue;
@@ -4308,11 +4308,11 @@ gtls_status batch_autotune(gtls_batch* b, const double* t, const double* y, cons
         for (int k = 0; k < 4; ++k) {
             const int cnt = std::min(256, np);
             const int first = std::max(0, std::min(np - cnt, (int)((k + 0.5) * np / 4.0) - cnt / 2));
-            probe.push_back(Run{i, first, cnt});
+            probe[cls[i] == 2].push_back(Run{i, first, cnt});
             for (int p = first; p < first + cnt; ++p) probe_wpe += period_wpe(h, p);
         }
     }
-    if (probe.empty()) return GTLS_OK;   // no curve takes the tiled kernel: nothing to tune
+    if (probe[0].empty() && probe[1].empty()) return GTLS_OK;   // no curve takes the tiled kernel: nothing to tune
     std::vector<int> slot_c, buf_c;
     for (int sc : {b->max_slots, b->max_slots / 2, b->max_slots / 4})
         if (sc >= 128 && std::find(slot_c.begin(), slot_c.end(), sc) == slot_c.end()) slot_c.push_back(sc);
@@ -4332,19 +4332,20 @@ gtls_status batch_autotune(gtls_batch* b, const double* t, const double* y, cons
     for (int bc : buf_c) {
         batch_tiles(b, bc);
         bool ok = true;
-        for (const Run& r : probe) ok = ok && b->fits[r.lc];
+        for (const Run& r : probe[0]) ok = ok && b->fits[r.lc];
+        for (const Run& r : probe[1]) ok = ok && b->fits_w[r.lc];
         if (!ok) continue;
         if ((s = batch_upload_tiles(b)) != GTLS_OK) break;
         for (int sc : slot_c) {
             std::vector<BatchWave> waves;
-            build_waves(b, probe, true, false, false, sc, waves);
+            for (int w = 0; w < 2; ++w) build_waves(b, probe[w], true, w == 1, false, sc, waves);
             Ctx c = batch_ctx(b, st);
             c.tile_buf = bc;
             float ms = 0.0f;
             for (int rep = 0; rep < 3 && s == GTLS_OK; ++rep) {
                 if (rep == 1 && cudaEventRecord(e0, st) != cudaSuccess) s = fail(GTLS_ERR_CUDA, "cudaEventRecord");
                 for (const BatchWave& w : waves) {
-                    s = wave_pass(c, false, w.sm, true, false, false, w.max_n, w.max_kept, w.tensor);
+                    s = wave_pass(c, false, w.sm, true, w.weighted, false, w.max_n, w.max_kept, w.tensor);
                     if (s != GTLS_OK) break;
                 }
             }
