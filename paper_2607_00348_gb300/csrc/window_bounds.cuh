@@ -175,7 +175,8 @@ __host__ inline int max_chunks(int threads) { return 2 * threads; }
 // Relative error allowed for a sum of n products in FP32 (twice the bound).
 __device__ __forceinline__ float sum_slack(int n) { return 1.2e-7f * (float)(n + 8); }
 
-__device__ __forceinline__ float root(float x) { return x > 0.0f ? x * rsqrtf(x) : (x == 0.0f ? 0.0f : x); }
+// Root of an energy (NaN stays NaN; not negative but for rounding: then 0).
+__device__ __forceinline__ float root(float x) { return x > 0.0f ? x * rsqrtf(x) : (x <= 0.0f ? 0.0f : x); }
 
 // What delta-chi2 v of a window can differ between two orders of its sums: C1
 // off by at most off, the depth by dd (sums of its own: the (C1, S) pairs), C2
