@@ -2795,6 +2795,16 @@ gtls_status configure_kernels(int dev)
     return GTLS_OK;
 }
 
+// Bytes of chunk scratch per period in flight (strides set); `tiles`: most
+// tiles of a period, with the lists of the window search by bounds (0: without).
+int64_t slot_bytes(const DevChunk& dk, int64_t tiles)
+{
+    const int64_t folded = dk.key_stride * 8 + dk.fold_stride * 4 + dk.pad_stride * (4 + 4 + 4 + 8);
+    const int64_t lists = kListClasses * kListPerSlot * (int64_t)sizeof(*dk.list) +
+                          bounds::kDenseParts * tiles * (int64_t)sizeof(*dk.dense);
+    return folded + (tiles > 0 ? dk.pad_stride * 4 + lists : 0);
+}
+
 gtls_status create_device(gtls_plan* pl)
 {
     const PlanHost& h = pl->host;
@@ -2875,23 +2885,6 @@ gtls_status create_device(gtls_plan* pl)
     dk.fold_stride = (n + 31) & ~int64_t(31);
     dk.key_stride = std::max<int64_t>(dk.fold_stride, (int64_t)kFoldSegKeys * dp.fold_nsb);
     dk.pad_stride = (n + h.dmax + kPadMargin + 31) & ~int64_t(31);
-    const int64_t per_period = dk.key_stride * 8 + dk.fold_stride * 4 + dk.pad_stride * (4 + 4 + 4 + 8 + 4);
-    // 8 GiB of chunk scratch (measured on the Kepler-like search: 1024,
-    // 1520 and 3040 periods per chunk took 1013, 994 and 980 ms)
-    const int64_t budget = int64_t(8) << 30;
-    int64_t chunk = std::max<int64_t>(1, budget / per_period);
-    chunk = std::min<int64_t>(chunk, 4096);
-    {
-        // whole waves of the fold (one CTA per period and SM): a multiple of
-        // the SM count when at least one wave fits
-        int dev = 0, sms = 0;
-        GTLS_CUDA(cudaGetDevice(&dev));
-        GTLS_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        if (sms > 0 && chunk >= sms) chunk = chunk / sms * sms;
-    }
-    if (h.prm.periods_per_chunk > 0) chunk = h.prm.periods_per_chunk;
-    chunk = std::min<int64_t>(chunk, dp.np);
-    dk.chunk = (int32_t)chunk;   // allocated by the first single-curve search
 
     DevPeriod& dq = pl->dq;
     const int64_t np_ = dp.np;
@@ -3236,6 +3229,20 @@ gtls_status create_device(gtls_plan* pl)
         // (the 32-bit prefix sums of w take the fold's keys' place)
         pl->bounds_w_ok = pl->bounds_ok && pl->tile_w_ok && !pl->has_window_only &&
                           4 * (n + h.dmax + 16) <= 8 * pl->dk.key_stride;
+    }
+
+    // periods in flight: 8 GiB of chunk scratch (measured on the Kepler-like
+    // search when every window was summed: 1024, 1520 and 3040 periods per
+    // chunk took 1013, 994 and 980 ms), whole waves of the fold (one CTA per
+    // period and SM) when at least one fits
+    {
+        const int64_t budget = int64_t(8) << 30;
+        const int64_t tiles = std::max({1, pl->tile_count, pl->tile_count_ref, pl->tile_count_w});
+        int64_t chunk = std::max<int64_t>(1, budget / slot_bytes(dk, pl->bounds_ok ? tiles : 0));
+        chunk = std::min<int64_t>(chunk, 4096);
+        if (pl->n_sm > 0 && chunk >= pl->n_sm) chunk = chunk / pl->n_sm * pl->n_sm;
+        if (h.prm.periods_per_chunk > 0) chunk = h.prm.periods_per_chunk;
+        dk.chunk = (int32_t)std::min<int64_t>(chunk, dp.np);   // allocated by the first single-curve search
     }
 
     // one-entry descriptor sets of this plan's own searches
@@ -4201,9 +4208,12 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     dk.fold_stride = fold_stride;
     dk.key_stride = key_stride;
     dk.pad_stride = pad_stride;
-    const int64_t per_slot = key_stride * 8 + fold_stride * 4 + pad_stride * (4 + 4 + 4 + 8 + 4);
+    batch_tiles(b, b->cfg.tile_buf);
+    int64_t max_tiles = 1;
+    for (const DevTiles& t : b->tiles_host) max_tiles = std::max<int64_t>({max_tiles, t.count, t.count_w});
     const int64_t budget = int64_t(16) << 30;
-    int64_t slots = std::min<int64_t>(4096, std::max<int64_t>(1, budget / per_slot));
+    int64_t slots =
+        std::min<int64_t>(4096, std::max<int64_t>(1, budget / slot_bytes(dk, b->bounds_ok ? max_tiles : 0)));
     if (b->n_sm > 0 && slots >= 4 * b->n_sm) slots = slots / (4 * b->n_sm) * (4 * b->n_sm);   // whole fold waves at 1, 1/2, 1/4
     if (wave_slots > 0) slots = wave_slots;
     b->max_slots = (int)slots;
@@ -4260,12 +4270,9 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     GTLS_TRY(batch_alloc(b, &b->q_waves, (size_t)kMaxLoops));
     GTLS_TRY(batch_alloc(b, &b->q_cursors, 3 * (size_t)kMaxLoops));
     b->total_periods = total_periods;
-    batch_tiles(b, b->cfg.tile_buf);
     GTLS_TRY(batch_upload_tiles(b));
     if (b->bounds_ok) {
-        int max_tiles = 1;
-        for (const DevTiles& t : b->tiles_host) max_tiles = std::max({max_tiles, t.count, t.count_w});
-        b->dk.dense_cap = slots * (int64_t)max_tiles * bounds::kDenseParts;
+        b->dk.dense_cap = slots * max_tiles * bounds::kDenseParts;
         GTLS_TRY(batch_alloc(b, &b->dk.dense, b->dk.dense_cap));
         GTLS_TRY(batch_alloc(b, &b->dk.pq, slots * pad_stride));
         b->dk.list_cap = std::max<int64_t>(4096, slots * kListPerSlot);

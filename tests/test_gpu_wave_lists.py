@@ -91,3 +91,14 @@ def test_list_for_the_tiled_kernel_filled_to_its_capacity(own_dy):
         got.append(gh.gpu_search(p, *c)[1])
         p.close()
     _equal(*got)
+
+
+def test_chunk_scratch_holds_its_lists():
+    # sizes whose folded arrays alone fill 8 GiB but for a few MB
+    for n in (52702, 55691, 60409):
+        p = _plan(n, 0, periods_days=np.geomspace(1.0, 730.0, 4200))
+        before = p.device_bytes()
+        p.reserve()
+        assert p.device_bytes() - before <= 8 << 30, (n, p.info.periods_per_chunk)
+        assert p.info.periods_per_chunk % 152 == 0
+        p.close()
