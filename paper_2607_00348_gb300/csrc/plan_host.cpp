@@ -169,6 +169,14 @@ bool build_plan_host(const gtls_plan_params& p, PlanHost& h, std::string& err)
         h.dpts[j] = (int32_t)std::min<int64_t>(d, h.n);
         h.stride[j] = (int32_t)std::max<int64_t>(1, (int64_t)std::floor((double)h.dpts[j] * p.dt0));
     }
+    // windows and window-point products of every duration (divided out once,
+    // not at every period: 4.6 million divisions on the Kepler-like grid)
+    std::vector<int64_t> windows(nd);
+    std::vector<double> products(nd);
+    for (int32_t j = 0; j < nd; ++j) {
+        windows[j] = (h.n + h.stride[j] - 1) / h.stride[j];
+        products[j] = (double)windows[j] * (double)h.dpts[j];
+    }
     h.jlo.resize(np_);
     h.jhi.resize(np_);
     h.dmax_p.resize(np_);
@@ -188,9 +196,8 @@ bool build_plan_host(const gtls_plan_params& p, PlanHost& h, std::string& err)
             if (!kept_duration(h, j, a)) continue;
             ++kept;
             dm = std::max(dm, h.dpts[j]);
-            const int64_t m = (h.n + h.stride[j] - 1) / h.stride[j];
-            h.n_windows += m;
-            h.wpe += (double)m * (double)h.dpts[j];
+            h.n_windows += windows[j];
+            h.wpe += products[j];
         }
         h.dmax_p[i] = dm;
         h.max_kept = std::max(h.max_kept, kept);

@@ -2527,6 +2527,20 @@ gtls_status upload(gtls_plan* pl, T** ptr, const std::vector<T>& v)
     return GTLS_OK;
 }
 
+// Host arrays packed for one allocation and copy (each costs a plan about 8 us).
+struct Packed {
+    std::vector<unsigned char> bytes;
+
+    template <class T>
+    size_t place(const std::vector<T>& v)   // its offset
+    {
+        const size_t at = (bytes.size() + 255) & ~size_t(255), size = v.size() * sizeof(T);
+        bytes.resize(at + size);
+        if (size) std::memcpy(bytes.data() + at, v.data(), size);
+        return at;
+    }
+};
+
 #define GTLS_TRY(x)                     \
     do {                                \
         gtls_status s_ = (x);           \
@@ -3169,14 +3183,7 @@ gtls_status create_device(gtls_plan* pl)
         pl->bounds_ok = !pl->has_tensor && !(h.prm.test_flags & 2);
         std::vector<BoundTab> tab(dp.nd);
         std::vector<BoundDur> bd(dp.nd);
-        // (one allocation and copy for all tables)
-        std::vector<unsigned char> all;
-        auto place = [&](const auto& v) {
-            const size_t at = (all.size() + 255) & ~size_t(255), bytes = v.size() * sizeof(v[0]);
-            all.resize(at + bytes);
-            if (bytes) std::memcpy(all.data() + at, v.data(), bytes);
-            return at;
-        };
+        Packed all;
         size_t at_tab[2] = {}, at_dur[2] = {}, at_drop = 0, at_fine = 0;
         const int threads = fold_threads(h.n), most = bounds::max_chunks(threads);
         const int clg = bounds::coarse_log2(threads, h.n, h.dmax);
@@ -3189,8 +3196,8 @@ gtls_status create_device(gtls_plan* pl)
             }
             DevPlan& q = pass ? pl->dp_ref : dp;
             q.bound_lg = bound_chunks(bd, var, h, most);
-            at_tab[pass] = place(tab);
-            at_dur[pass] = place(bd);
+            at_tab[pass] = all.place(tab);
+            at_dur[pass] = all.place(bd);
         }
         if (pl->bounds_ok) {
             // s_{k-1} - s_k of every template (0 before and after it), where dp.tmpl has s_k
@@ -3200,7 +3207,7 @@ gtls_status create_device(gtls_plan* pl)
                 for (int k = 0; k <= h.dpts[j]; ++k)
                     drop[(size_t)(pl->tmpl_pad_off[j] + k)] = (float)((k > 0 ? (double)tj[k - 1] : 0.0) - tj[k]);
             }
-            at_drop = place(drop);
+            at_drop = all.place(drop);
             // (read for durations of at least kFineFrom points only)
             std::vector<float2> fine(h.dmax >= kFineFrom ? (size_t)dp.nd * kFinePieces : 0, make_float2(0.0f, 0.0f));
             for (int j = 0; j < dp.nd; ++j) {
@@ -3215,9 +3222,9 @@ gtls_status create_device(gtls_plan* pl)
                     fine[(size_t)(j * kFinePieces + g)] = make_float2(mean, (float)(std::sqrt(v) * (1.0 + 1e-6)));
                 }
             }
-            at_fine = place(fine);
+            at_fine = all.place(fine);
             unsigned char* base = nullptr;
-            GTLS_TRY(upload(pl, &base, all));
+            GTLS_TRY(upload(pl, &base, all.bytes));
             for (int pass = 0; pass < (pl->refine_k > 0 ? 2 : 1); ++pass) {
                 DevPlan& q = pass ? pl->dp_ref : dp;
                 q.bounds = reinterpret_cast<const BoundTab*>(base + at_tab[pass]);
@@ -3247,19 +3254,23 @@ gtls_status create_device(gtls_plan* pl)
 
     // one-entry descriptor sets of this plan's own searches
     {
-        DevPlan* d_plans = nullptr;
-        DevCurve* d_curves = nullptr;
-        DevPeriod* d_outs = nullptr;
-        DevTiles* d_tiles = nullptr;
-        GTLS_TRY(upload(pl, &d_plans, std::vector<DevPlan>{dp, pl->refine_k > 0 ? pl->dp_ref : dp}));
-        GTLS_TRY(upload(pl, &d_curves, std::vector<DevCurve>{dc}));
-        GTLS_TRY(upload(pl, &d_outs, std::vector<DevPeriod>{pl->dq}));
-        GTLS_TRY(upload(pl, &d_tiles,
-                        std::vector<DevTiles>{DevTiles{pl->tile_len, pl->tile_count, pl->tile_len_w, pl->tile_count_w},
-                                              DevTiles{pl->tile_len_ref, pl->tile_count_ref, 0, 0}}));
+        Packed all;
+        const size_t at_plans = all.place(std::vector<DevPlan>{dp, pl->refine_k > 0 ? pl->dp_ref : dp});
+        const size_t at_curves = all.place(std::vector<DevCurve>{dc});
+        const size_t at_outs = all.place(std::vector<DevPeriod>{pl->dq});
+        const size_t at_tiles = all.place(
+            std::vector<DevTiles>{DevTiles{pl->tile_len, pl->tile_count, pl->tile_len_w, pl->tile_count_w},
+                                  DevTiles{pl->tile_len_ref, pl->tile_count_ref, 0, 0}});
+        const size_t at_off = all.place(std::vector<int64_t>{0, n});
+        unsigned char* base = nullptr;
+        GTLS_TRY(upload(pl, &base, all.bytes));
+        DevPlan* const d_plans = reinterpret_cast<DevPlan*>(base + at_plans);
+        DevCurve* const d_curves = reinterpret_cast<DevCurve*>(base + at_curves);
+        DevPeriod* const d_outs = reinterpret_cast<DevPeriod*>(base + at_outs);
+        DevTiles* const d_tiles = reinterpret_cast<DevTiles*>(base + at_tiles);
         pl->set = DevSet{d_plans, d_curves, d_outs, d_tiles};
         pl->set_ref = DevSet{d_plans + 1, d_curves, d_outs, d_tiles + 1};
-        GTLS_TRY(upload(pl, &pl->prep_off, std::vector<int64_t>{0, n}));
+        pl->prep_off = reinterpret_cast<int64_t*>(base + at_off);
     }
     return GTLS_OK;
 }
