@@ -152,7 +152,7 @@ struct DevChunk {
     int64_t list_cap;         // windows per lane-group size
     unsigned long long* list; // windows to sum, kListClasses lists
     int64_t dense_cap;        // items
-    int2* dense;              // items for the tiled kernel: slot, and tile | part << 20 | (parts - 1) << 24
+    int2* dense;              // tiles for the tiled kernel: slot, and tile | CTAs that may share it << 24
     unsigned int* work;       // kWorkWords counters of the wave in flight
 };
 

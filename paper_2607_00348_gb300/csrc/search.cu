@@ -1212,8 +1212,14 @@ k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
     __shared__ int s_item, s_ndur, s_total, s_task, s_lc, s_p, s_slot, s_x0, s_len, s_tau, s_tcount, s_part, s_parts;
     __shared__ unsigned long long s_best[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // the items the bounds kernel left, or every (period, tile) of the wave
-    const int items = listed ? (int)min((int64_t)dk.work[kWorkDense], dk.dense_cap) : sm.items;
+    // the tiles the bounds left, or every (period, tile) of the wave.  A few
+    // tiles are shared by several CTAs, about 65,536 windows each at least (the
+    // 1.2e6 windows of one period at T0 step 1 kept an SM for 15 ms); many are
+    // not, as every CTA stages the tile again (1520 periods of 62,363 points,
+    // all left: 11.7 ms for the search in five parts, 10.1 undivided)
+    const int dense = listed ? (int)min((int64_t)dk.work[kWorkDense], dk.dense_cap) : 0;
+    const int split = max(1, min(bounds::kDenseParts, 4 * (int)gridDim.x / max(1, dense)));
+    const int items = listed ? dense * split : sm.items;
     for (;;) {
         if (threadIdx.x == 0) {
             const int item = (int)atomicAdd(dk.work + kWorkTiles, 1u);
@@ -1221,12 +1227,12 @@ k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
             if (item < items) {
                 int lcg = 0, pp = -1, slot = 0, tau = 0, part = 0, parts = 1;
                 if (listed) {
-                    const int2 it = dk.dense[item];
+                    const int2 it = dk.dense[item / split];
                     slot = it.x;
-                    tau = it.y & 0xfffff;
-                    part = (it.y >> 20) & 15;
-                    parts = (it.y >> 24) + 1;
-                    if (!resolve_slot(ds, sm, slot, lcg, pp)) pp = -1;
+                    tau = it.y & 0xffffff;
+                    part = item % split;
+                    parts = min(split, it.y >> 24);
+                    if (part >= parts || !resolve_slot(ds, sm, slot, lcg, pp)) pp = -1;
                 } else {
                     int g = 0;
                     while (g + 1 < sm.nseg && sm.seg[g + 1].item0 <= item) ++g;
@@ -2815,7 +2821,7 @@ int64_t slot_bytes(const DevChunk& dk, int64_t tiles)
 {
     const int64_t folded = dk.key_stride * 8 + dk.fold_stride * 4 + dk.pad_stride * (4 + 4 + 4 + 8);
     const int64_t lists = kListClasses * kListPerSlot * (int64_t)sizeof(*dk.list) +
-                          bounds::kDenseParts * tiles * (int64_t)sizeof(*dk.dense);
+                          tiles * (int64_t)sizeof(*dk.dense);
     return folded + (tiles > 0 ? dk.pad_stride * 4 + lists : 0);
 }
 
@@ -3331,8 +3337,7 @@ gtls_status ensure_chunk(gtls_plan* pl)
         GTLS_TRY(dev_alloc(pl, &dk.pq, chunk * dk.pad_stride));
         dk.list_cap = std::max<int64_t>(4096, chunk * kListPerSlot);
         GTLS_TRY(dev_alloc(pl, &dk.list, kListClasses * dk.list_cap));
-        dk.dense_cap = chunk * bounds::kDenseParts *
-                       std::max({1, pl->tile_count, pl->tile_count_ref, pl->tile_count_w});
+        dk.dense_cap = chunk * std::max({1, pl->tile_count, pl->tile_count_ref, pl->tile_count_w});
         GTLS_TRY(dev_alloc(pl, &dk.dense, dk.dense_cap));
     }
     if (pl->has_tensor) {
@@ -4283,7 +4288,7 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     b->total_periods = total_periods;
     GTLS_TRY(batch_upload_tiles(b));
     if (b->bounds_ok) {
-        b->dk.dense_cap = slots * max_tiles * bounds::kDenseParts;
+        b->dk.dense_cap = slots * max_tiles;
         GTLS_TRY(batch_alloc(b, &b->dk.dense, b->dk.dense_cap));
         GTLS_TRY(batch_alloc(b, &b->dk.pq, slots * pad_stride));
         b->dk.list_cap = std::max<int64_t>(4096, slots * kListPerSlot);

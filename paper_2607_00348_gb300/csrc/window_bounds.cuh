@@ -75,7 +75,7 @@ constexpr int kTileStarts = 8192;   // window starts walked before the next stre
 constexpr int kGroup = 128;         // windows a warp tests at a time (4 per lane)
 constexpr int kChunkGroups = 4;     // groups per chunk (at most)
 constexpr int kNearStep = kTileStarts / kGroup;   // T0 steps up to this fill a group in one stretch
-constexpr int kDenseParts = 16;     // items a tile is split into for the tiled kernel, at most
+constexpr int kDenseParts = 16;     // CTAs of the tiled kernel that share a tile, at most
 constexpr int kListed = 256;        // windows listed of a period before the tiled kernel is cheaper, or a window in
 constexpr int kListedPart = 512;    // so many (a listed window costs about 3 us of an SM; all 1.2e6 at T0 step 1, 55 ms)
 constexpr int kRowBuf = 168;        // prefix sums at whole T0 steps a warp stages for one group
@@ -114,7 +114,7 @@ struct Chunks {
     int far, per_tile;          // far chunks, near chunks per stretch
     int total;
     int listed;                 // windows that may be listed
-    int parts;                  // items per tile for the tiled kernel
+    int parts;                  // CTAs of the tiled kernel that may share a tile
 };
 
 // Shared memory for CTAs of T threads (curves of up to 8 T points when
@@ -1233,15 +1233,12 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         fits = fits && S.n_listed <= S.ck.listed;
     }
     if (!fits && threadIdx.x == 0) {
-        // (a tile's tasks shared by `parts` CTAs, about 65,536 windows each: the
-        // 1.2e6 windows of one period at T0 step 1 kept an SM for 15 ms)
-        const int tc = kW ? ds.tiles[lc].count_w : ds.tiles[lc].count, parts = S.ck.parts;
-        const long long to = atomicAdd(dk.work + kWorkDense, (unsigned int)(tc * parts));
+        const int tc = kW ? ds.tiles[lc].count_w : ds.tiles[lc].count;
+        const long long to = atomicAdd(dk.work + kWorkDense, (unsigned int)tc);
         // (there is room for every period of a wave; as far as there is room,
         // every item that the tiled kernel will read is written)
-        in_range(ds.curves[lc].check, 24, to + tc * parts - 1, dk.dense_cap);
-        for (int i = 0; i < tc * parts && to + i < dk.dense_cap; ++i)
-            dk.dense[to + i] = make_int2(slot, (i / parts) | ((i % parts) << 20) | ((parts - 1) << 24));
+        in_range(ds.curves[lc].check, 24, to + tc - 1, dk.dense_cap);
+        for (int i = 0; i < tc && to + i < dk.dense_cap; ++i) dk.dense[to + i] = make_int2(slot, i | (S.ck.parts << 24));
     }
     if (!kW && (fill || !fits)) {
         // the folded curve itself and its exact prefix sums, for the kernels

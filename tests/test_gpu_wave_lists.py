@@ -102,3 +102,24 @@ def test_chunk_scratch_holds_its_lists():
         assert p.device_bytes() - before <= 8 << 30, (n, p.info.periods_per_chunk)
         assert p.info.periods_per_chunk % 152 == 0
         p.close()
+
+
+def test_tiles_shared_by_unequal_numbers_of_ctas():
+    # a wave of periods left to the tiled kernel whose tiles one, two and
+    # sixteen CTAs may share
+    import torch
+    dev = torch.device("cuda:0")
+    sizes = (400, 9001, 70001)
+    curves = [_curve(n, "flat", False, n) for n in sizes]
+    kw = dict(periods_days=np.geomspace(1.0, 9.0, 5), refine_periods=5)
+    plans = [_plan(n, 0, **kw) for n in sizes]
+    batch = pkg.Batch(plans)
+    batch.search(*(torch.as_tensor(np.concatenate([c[k] for c in curves]), device=dev) for k in range(3)),
+                 np.cumsum((0,) + sizes).astype(np.int64))
+    for i, (n, c) in enumerate(zip(sizes, curves)):
+        every = _plan(n, 2, **kw)
+        _equal(gh.batch_outputs(batch, i, 5), gh.gpu_search(every, *c)[1])
+        every.close()
+    batch.close()
+    for p in plans:
+        p.close()
