@@ -76,8 +76,17 @@ constexpr int kGroup = 128;         // windows a warp tests at a time (4 per lan
 constexpr int kChunkGroups = 4;     // groups per chunk (at most)
 constexpr int kNearStep = kTileStarts / kGroup;   // T0 steps up to this fill a group in one stretch
 constexpr int kDenseParts = 16;     // CTAs of the tiled kernel that share a tile, at most
-constexpr int kListed = 256;        // windows listed of a period before the tiled kernel is cheaper, or a window in
-constexpr int kListedPart = 512;    // so many (a listed window costs about 3 us of an SM; all 1.2e6 at T0 step 1, 55 ms)
+// What is left of a period is cheaper on the tiled kernel when summing its
+// windows again would take longer than all of them there.  In ns of an SM, from
+// 1520 to 4000 periods of 1,440 to 62,363 points: the tiled kernel by points
+// and windows (own weights: 1.7 times that.  Per period 28 us by this, 35 as
+// measured, at 1,440 points, 65 and 65 at 3,900, 290 and 240 at 20,011, 810 and
+// 630 at 62,363), a listed window by its points, of which kListedRoom halve the
+// CTAs that an SM holds (0.6 us for 600 points, 2.5 us for 2,900, 13 to 16 us for
+// 9,000).  (A fixed limit of a window in 512: 27 ms for 1520 periods of 62,363
+// points 10 % below 1, which have hundreds of nearly equal long windows.)
+constexpr float kTiledPoint = 0.014f, kTiledWindow = 0.5f, kTiledOwn = 1.7f;   // ns of an SM
+constexpr float kListedPoint = 0.45f, kListedWindow = 300.0f, kListedRoom = 4096.0f;
 constexpr int kRowBuf = 168;        // prefix sums at whole T0 steps a warp stages for one group
 constexpr int kCutPoints = 60;      // windows of at least this many points are first tested by wide pieces
 constexpr int kCoarseSteps = 64;    // ... and from this many coarse steps on from the coarse prefix
@@ -113,7 +122,7 @@ struct Chunks {
     int ndur, near_durs;        // durations (ascending); the first near_durs are near
     int far, per_tile;          // far chunks, near chunks per stretch
     int total;
-    int listed;                 // windows that may be listed
+    float tiled;                // ns of an SM that the tiled kernel would take
     int parts;                  // CTAs of the tiled kernel that may share a tile
 };
 
@@ -143,7 +152,8 @@ struct Smem {
     float row_buf[kWarps * kRowBuf];
     float coarse[kMaxCoarse + kMaxCoarse / 32 + 1];  // see at_coarse
     Chunks ck;
-    int next, n_pass, sieved, n_fin, n_listed, dev, big;
+    int next, n_pass, sieved, n_fin, dev, big;
+    bool full;                                       // a list of the wave is
     float wsum[kWarps], energy[kEnergySpans];
     float top[kWarps], c1[kWarps], s[kWarps];
     int top_at[kWarps];
@@ -254,6 +264,7 @@ __device__ __forceinline__ void list_durations(const DevPlan& dp, unsigned int* 
 {
     const int lo = dp.jlo[p], hi = dp.jhi[p];
     int count = 0, run_near = 0, run_far = 0, near_durs = 0, windows = 0;
+    float points = 0.0f;
     for (int base = 0; base <= hi - lo; base += 32) {
         const int j = lo + base + lane;
         const int subs = j <= hi ? dp.bound_durs[j].subs : 0;
@@ -278,6 +289,7 @@ __device__ __forceinline__ void list_durations(const DevPlan& dp, unsigned int* 
             dur[k].b.j = j;
             dur[k].first = nearby ? run_near + a - a0 : run_far + b - b0;
             windows += wins;
+            points += (float)wins * (float)d;
         }
         run_near += __shfl_sync(0xffffffffu, a, 31);
         run_far += __shfl_sync(0xffffffffu, b, 31);
@@ -286,9 +298,11 @@ __device__ __forceinline__ void list_durations(const DevPlan& dp, unsigned int* 
     }
     const int tile = kTileStarts << dp.bound_lg;
     windows = (int)__reduce_add_sync(0xffffffffu, (unsigned int)windows);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) points += __shfl_xor_sync(0xffffffffu, points, o);
     if (lane == 0)
         ck = Chunks{min(count, tiles::kMaxDur), near_durs, run_far, run_near,
-                    run_far + (n + tile - 1) / tile * run_near, max(kListed, windows / kListedPart),
+                    run_far + (n + tile - 1) / tile * run_near, kTiledPoint * points + kTiledWindow * (float)windows,
                     max(1, min(kDenseParts, windows >> 16))};
     __syncwarp();
 }
@@ -657,7 +671,8 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
     if (warp == 0) {
         list_durations(dp, ds.curves[lc].check, p, n, dur, S.ck, lane);
         for (int k = lane; k < kEnergySpans; k += 32) S.energy[k] = 0.0f;
-        if (lane == 0) S.next = S.n_pass = S.sieved = S.n_fin = S.n_listed = S.dev = S.big = 0;
+        if (lane == 0) S.next = S.n_pass = S.sieved = S.n_fin = S.dev = S.big = 0;
+        if (lane == 0) S.full = false;
         if (lane == 0) S.wlow = INT_MAX;
     }
     for (int i = threadIdx.x; i < M::kSieve; i += T) S.sieve[i] = kNone;
@@ -1192,20 +1207,34 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         best = lane < kWarps ? S.top[lane] : INFINITY;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+        // what it takes to sum those near the lowest again
+        float again = 0.0f;
+        for (int i = threadIdx.x; i < nfin && fits; i += T)
+            if (!(S.fin_v[i] > best)) {
+                const float d = (float)dur[S.fin[i] >> 24].b.d;
+                again += kListedWindow + kListedPoint * d * (1.0f + d / kListedRoom);
+            }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) again += __shfl_xor_sync(0xffffffffu, again, o);
+        if (lane == 0) S.s[warp] = again;
+        __syncthreads();
+        again = lane < kWarps ? S.s[lane] : 0.0f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) again += __shfl_xor_sync(0xffffffffu, again, o);
+        fits = fits && again <= ck.tiled * (kW ? kTiledOwn : 1.0f);
         for (int i = threadIdx.x; i < nfin && fits; i += T) {
             if (S.fin_v[i] > best) continue;
             const unsigned int e = S.fin[i];
             const Dur& t = dur[e >> 24];
             const int m = (int)(e & 0xffffffu);
             auto push = [&](int rot) {
-                const unsigned int to =
-                    atomicAdd(&S.n_listed, 1) < S.ck.listed ? atomicAdd(dk.work + t.b.lg_nc, 1u) : 0xffffffffu;
+                const unsigned int to = atomicAdd(dk.work + t.b.lg_nc, 1u);
                 if (to < dk.list_cap)
                     dk.list[t.b.lg_nc * dk.list_cap + to] = ((unsigned long long)slot << 40) |
                                                             ((unsigned long long)t.b.j << 32) |
                                                             ((unsigned long long)rot << 24) | (unsigned long long)m;
                 else
-                    S.n_listed = 2 * S.ck.listed;   // (more may be added: it stays above)
+                    S.full = true;
             };
             if (kW || t.b.mode != kModeRot) {
                 push(0);
@@ -1230,7 +1259,7 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
             }
         }
         __syncthreads();
-        fits = fits && S.n_listed <= S.ck.listed;
+        fits = fits && !S.full;
     }
     if (!fits && threadIdx.x == 0) {
         const int tc = kW ? ds.tiles[lc].count_w : ds.tiles[lc].count;
