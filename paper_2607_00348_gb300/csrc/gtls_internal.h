@@ -121,6 +121,7 @@ struct DevCurve {
     unsigned int* flags;      // bit0 non-finite, bit1 dy <= 0, bit2 dy not uniform
     double* part;             // block partials of chi2_0
     unsigned int* check;      // [0] first failed device check (0 = none), [1..3] its values
+    int* given_up;            // periods that the bounds gave up lately: coarse pass, refinement
 };
 
 constexpr int kListClasses = 6;   // windows are summed by groups of 1, 2, 4, ..., 32 lanes

@@ -294,6 +294,7 @@ __global__ void k_curve_reset(DevSet ds, int lc0)
     if (threadIdx.x == 0) *dc.tmin_key = ~0ull;
     if (threadIdx.x == 1) *dc.flags = 0u;
     if (threadIdx.x >= 2 && threadIdx.x < 6) dc.check[threadIdx.x - 2] = 0u;
+    if (threadIdx.x >= 6 && threadIdx.x < 8) dc.given_up[threadIdx.x - 6] = 0;
 }
 
 // Curve lc = lc0 + blockIdx.y holds points off[lc] .. off[lc+1] of t, y, dy;
@@ -1115,7 +1116,8 @@ k_fold_sort(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* smq, 
     }
     if (kFold != Fold::kPlain) {
         __syncthreads();
-        bounds::window_bounds<T, kBoundedW>(smem, ds, dk, slot_id, lc, p, tile_buf, fill != 0);
+        bounds::window_bounds<T, kBoundedW>(smem, ds, dk, slot_id, lc, p, tile_buf, fill != 0,
+                                                  sm.from_list != 0);
     }
 }
 
@@ -1213,12 +1215,12 @@ k_window_tiles(DevSet ds, const __grid_constant__ SlotMap smv, const SlotMap* sm
     __shared__ unsigned long long s_best[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // the tiles the bounds left, or every (period, tile) of the wave.  A few
-    // tiles are shared by several CTAs, about 65,536 windows each at least (the
-    // 1.2e6 windows of one period at T0 step 1 kept an SM for 15 ms); many are
-    // not, as every CTA stages the tile again (1520 periods of 62,363 points,
-    // all left: 11.7 ms for the search in five parts, 10.1 undivided)
+    // tiles are shared by several CTAs, bounds::kPart each at least (the 1.2e6
+    // windows of one period at T0 step 1 kept an SM for 15 ms); many are not, as
+    // every CTA stages the tile again (1520 periods of 62,363 points, all left:
+    // 11.7 ms for the search in five parts, 10.1 undivided)
     const int dense = listed ? (int)min((int64_t)dk.work[kWorkDense], dk.dense_cap) : 0;
-    const int split = max(1, min(bounds::kDenseParts, 4 * (int)gridDim.x / max(1, dense)));
+    const int split = max(1, min(bounds::kDenseParts, 16 * (int)gridDim.x / max(1, dense)));
     const int items = listed ? dense * split : sm.items;
     for (;;) {
         if (threadIdx.x == 0) {
@@ -2899,7 +2901,8 @@ gtls_status create_device(gtls_plan* pl)
     GTLS_TRY(dev_alloc(pl, &dc.tmin_key, 1));
     GTLS_TRY(dev_alloc(pl, &dc.flags, 1));
     GTLS_TRY(dev_alloc(pl, &dc.part, 2 * kPrepBlocks));
-    GTLS_TRY(dev_alloc(pl, &dc.check, 4));
+    GTLS_TRY(dev_alloc(pl, &dc.check, 6));
+    dc.given_up = reinterpret_cast<int*>(dc.check + 4);
 
     DevChunk& dk = pl->dk;
     dk.fold_stride = (n + 31) & ~int64_t(31);

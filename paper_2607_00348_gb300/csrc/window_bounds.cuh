@@ -36,8 +36,9 @@
 //
 // Periods for which nothing is gained (no window has a negative delta-chi2,
 // so that signed zeros decide, or only subnormal ones, which are often equal;
-// too many windows left; a value is not finite) are listed for the tiled
-// kernel, which then runs on that list.
+// too many windows left, or through the sieve; a value is not finite) are
+// listed for the tiled kernel, which then runs on that list; curves most of
+// whose periods end there are not tried at every period (kGivenUp).
 //
 // The window sums of steps 1 to 4 come from 32-bit prefix sums of r rounded to
 // a unit with which any sum fits 31 bits: off by half a unit per point (the
@@ -83,9 +84,13 @@ constexpr int kDenseParts = 16;     // CTAs of the tiled kernel that share a til
 // measured, at 1,440 points, 65 and 65 at 3,900, 290 and 240 at 20,011, 810 and
 // 630 at 62,363), a listed window by its points, of which kListedRoom halve the
 // CTAs that an SM holds (0.6 us for 600 points, 2.5 us for 2,900, 13 to 16 us for
-// 9,000).  (A fixed limit of a window in 512: 27 ms for 1520 periods of 62,363
+// 9,000), and a window of the sieve its segment test (19 cycles of the CTA): a
+// period whose sieve takes longer than its tiles is given up there.  (A fixed limit of a window in 512: 27 ms for 1520 periods of 62,363
 // points 10 % below 1, which have hundreds of nearly equal long windows.)
 constexpr float kTiledPoint = 0.014f, kTiledWindow = 0.5f, kTiledOwn = 1.7f;   // ns of an SM
+constexpr float kPart = 2e5f;       // a tile's share that another CTA is worth staging the tile for
+constexpr int kFew = 16;            // windows always cheaper to sum again
+constexpr float kSieved = 10.0f;                                              // (two CTAs of an SM: half)
 constexpr float kListedPoint = 0.45f, kListedWindow = 300.0f, kListedRoom = 4096.0f;
 constexpr int kRowBuf = 168;        // prefix sums at whole T0 steps a warp stages for one group
 constexpr int kCutPoints = 60;      // windows of at least this many points are first tested by wide pieces
@@ -122,8 +127,6 @@ struct Chunks {
     int ndur, near_durs;        // durations (ascending); the first near_durs are near
     int far, per_tile;          // far chunks, near chunks per stretch
     int total;
-    float tiled;                // ns of an SM that the tiled kernel would take
-    int parts;                  // CTAs of the tiled kernel that may share a tile
 };
 
 // Shared memory for CTAs of T threads (curves of up to 8 T points when
@@ -154,6 +157,8 @@ struct Smem {
     Chunks ck;
     int next, n_pass, sieved, n_fin, dev, big;
     bool full;                                       // a list of the wave is
+    int given_up;                                    // DevCurve::given_up when the period began
+    int tested;                                      // windows that went through the sieve
     float wsum[kWarps], energy[kEnergySpans];
     float top[kWarps], c1[kWarps], s[kWarps];
     int top_at[kWarps];
@@ -263,12 +268,10 @@ __device__ __forceinline__ void list_durations(const DevPlan& dp, unsigned int* 
                                                int lane)
 {
     const int lo = dp.jlo[p], hi = dp.jhi[p];
-    int count = 0, run_near = 0, run_far = 0, near_durs = 0, windows = 0;
-    float points = 0.0f;
+    int count = 0, run_near = 0, run_far = 0, near_durs = 0;
     for (int base = 0; base <= hi - lo; base += 32) {
         const int j = lo + base + lane;
         const int subs = j <= hi ? dp.bound_durs[j].subs : 0;
-        const int wins = j <= hi ? dp.bound_durs[j].m_total : 0;
         const bool nearby = j <= hi && dp.bound_durs[j].st <= kNearStep;
         const int d = j <= hi ? dp.dpts[j] : 0, before = j <= hi && j > lo ? dp.dpts[j - 1] : -1;
         bool kept = j <= hi && d != before && subs > 0;
@@ -288,8 +291,6 @@ __device__ __forceinline__ void list_durations(const DevPlan& dp, unsigned int* 
         if (kept) {
             dur[k].b.j = j;
             dur[k].first = nearby ? run_near + a - a0 : run_far + b - b0;
-            windows += wins;
-            points += (float)wins * (float)d;
         }
         run_near += __shfl_sync(0xffffffffu, a, 31);
         run_far += __shfl_sync(0xffffffffu, b, 31);
@@ -297,14 +298,23 @@ __device__ __forceinline__ void list_durations(const DevPlan& dp, unsigned int* 
         count += __popc(mask);
     }
     const int tile = kTileStarts << dp.bound_lg;
-    windows = (int)__reduce_add_sync(0xffffffffu, (unsigned int)windows);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) points += __shfl_xor_sync(0xffffffffu, points, o);
     if (lane == 0)
         ck = Chunks{min(count, tiles::kMaxDur), near_durs, run_far, run_near,
-                    run_far + (n + tile - 1) / tile * run_near, kTiledPoint * points + kTiledWindow * (float)windows,
-                    max(1, min(kDenseParts, windows >> 16))};
+                    run_far + (n + tile - 1) / tile * run_near};
     __syncwarp();
+}
+
+// What the period would take on the tiled kernel (ns of an SM; by a whole warp).
+__device__ __forceinline__ float tiled_time(const DevPlan& dp, const Dur* dur, int ndur, bool own, int lane)
+{
+    float ns = 0.0f;
+    for (int k = lane; k < ndur; k += 32) {
+        const int j = dur[k].b.j;
+        ns += (float)dp.bound_durs[j].m_total * fmaf(kTiledPoint, (float)dp.dpts[j], kTiledWindow);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ns += __shfl_xor_sync(0xffffffffu, ns, o);
+    return own ? kTiledOwn * ns : ns;
 }
 
 // Duration k and windows [lo, hi) of chunk c (warp-uniform).
@@ -626,14 +636,14 @@ __device__ __forceinline__ float weight_floor(const Smem<T>& S, int len, int lb)
     return fmaxf(sum, (float)len * (float)S.wlow * (1.0f - 1e-6f)) - 0.5f * (float)len;
 }
 
-// Steps 1 to 4 for one period, by a CTA of T threads (kW: per-point weights).
+// Steps 1 to 4 for one period, by a CTA of T threads (kW: per-point weights):
+// true when its windows that may hold the minimum are listed, false when the
+// tiled kernel has to sum all of them.
 template <int T, bool kW>
-__device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet& ds, const DevChunk& dk, int slot, int lc,
-                                              int p, int buf, bool fill)
+__device__ __forceinline__ bool rule_out(Smem<T>& S, const DevSet& ds, const DevChunk& dk, int slot, int lc, int p, int buf)
 {
     using M = Smem<T>;
     constexpr int kWarps = T / 32;
-    M& S = *reinterpret_cast<M*>(smem);
     Dur* const dur = S.dur;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const DevPlan& dp = ds.plans[lc];
@@ -668,15 +678,6 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         return fmaxf(0.0f, (float)(pq[s + d] - pq[s]) * unit * inv);
     };
 
-    if (warp == 0) {
-        list_durations(dp, ds.curves[lc].check, p, n, dur, S.ck, lane);
-        for (int k = lane; k < kEnergySpans; k += 32) S.energy[k] = 0.0f;
-        if (lane == 0) S.next = S.n_pass = S.sieved = S.n_fin = S.dev = S.big = 0;
-        if (lane == 0) S.full = false;
-        if (lane == 0) S.wlow = INT_MAX;
-    }
-    for (int i = threadIdx.x; i < M::kSieve; i += T) S.sieve[i] = kNone;
-    __syncthreads();
     const Chunks ck = S.ck;
     const int ndur = ck.ndur;
     {
@@ -1126,8 +1127,19 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
             if (to < M::kFinal) S.fin[to] = e;
         }
         __syncthreads();
-        if (threadIdx.x == 0) S.sieved = 0;
+        if (threadIdx.x == 0) {
+            S.tested += sieved;
+            S.sieved = 0;
+        }
         if (!__syncthreads_or(c >= 0)) break;
+        // (a sieve that ran full)
+        if (S.n_fin > M::kFinal || (float)S.tested * (T == 1024 ? kSieved : 0.5f * kSieved) >
+                                       tiled_time(dp, dur, ndur, kW, lane)) {   // given up
+            __syncthreads();
+            if (threadIdx.x == 0) S.n_fin = M::kFinal + 1;
+            __syncthreads();
+            break;
+        }
     }
     // their sums (a warp each, any order): v - err <= delta-chi2 <= v + err,
     // whatever the order of the products
@@ -1207,21 +1219,23 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         best = lane < kWarps ? S.top[lane] : INFINITY;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
-        // what it takes to sum those near the lowest again
-        float again = 0.0f;
-        for (int i = threadIdx.x; i < nfin && fits; i += T)
-            if (!(S.fin_v[i] > best)) {
-                const float d = (float)dur[S.fin[i] >> 24].b.d;
-                again += kListedWindow + kListedPoint * d * (1.0f + d / kListedRoom);
-            }
+        if (nfin > kFew) {
+            // what it takes to sum those near the lowest again
+            float again = 0.0f;
+            for (int i = threadIdx.x; i < nfin; i += T)
+                if (!(S.fin_v[i] > best)) {
+                    const float d = (float)dur[S.fin[i] >> 24].b.d;
+                    again += kListedWindow + kListedPoint * d * (1.0f + d / kListedRoom);
+                }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) again += __shfl_xor_sync(0xffffffffu, again, o);
-        if (lane == 0) S.s[warp] = again;
-        __syncthreads();
-        again = lane < kWarps ? S.s[lane] : 0.0f;
+            for (int o = 16; o > 0; o >>= 1) again += __shfl_xor_sync(0xffffffffu, again, o);
+            if (lane == 0) S.s[warp] = again;
+            __syncthreads();
+            again = lane < kWarps ? S.s[lane] : 0.0f;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) again += __shfl_xor_sync(0xffffffffu, again, o);
-        fits = fits && again <= ck.tiled * (kW ? kTiledOwn : 1.0f);
+            for (int o = 16; o > 0; o >>= 1) again += __shfl_xor_sync(0xffffffffu, again, o);
+            fits = fits && again <= tiled_time(dp, dur, ndur, kW, lane);
+        }
         for (int i = threadIdx.x; i < nfin && fits; i += T) {
             if (S.fin_v[i] > best) continue;
             const unsigned int e = S.fin[i];
@@ -1261,34 +1275,110 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
         __syncthreads();
         fits = fits && !S.full;
     }
-    if (!fits && threadIdx.x == 0) {
+    return fits;
+}
+
+// The folded curve itself and its exact prefix sums, for the kernels that sum
+// every window (by the whole CTA; scratch: 33 words in shared memory).  Four
+// points per thread and scan: their gathers overlap.  Not inlined: the code
+// around it then stays as it is without it (Kepler-like search 327.1 against
+// 327.6 ms, 16 curves of 4,000 points 249.7 against 250.4).
+template <int T>
+__device__ __noinline__ void fill_folded(float* r, long long* sums, const int* sidx, const PointVals* pv, int n, int dm,
+                                         long long* scratch)
+{
+    constexpr int kPer = 4;
+    const int total = n + dm, padded = total + (int)kPadMargin;
+    long long carry = 0;
+    for (int k0 = 0; k0 < padded; k0 += kPer * T) {
+        const int k = k0 + kPer * threadIdx.x;
+        int id[kPer];
+        PointVals v[kPer];
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) id[u] = k + u < total ? sidx[k + u < n ? k + u : k + u - n] : -1;
+        long long sum = 0;
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            v[u] = id[u] >= 0 && id[u] < n ? pv[id[u]] : PointVals{0, 0.0f, 0.0f};
+            sum += v[u].rfx;
+        }
+        long long before = block_exclusive_scan(sum, scratch, scratch + 32) + carry;
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            if (k + u <= total) sums[k + u] = before;
+            if (k + u < padded) r[k + u] = v[u].r;
+            before += v[u].rfx;
+        }
+        carry += scratch[32];
+        __syncthreads();
+    }
+}
+
+// Whether the bounds are tried at a period (one thread decides for its CTA):
+// not while they gave up most periods of the curve lately, but at every 16th.
+// Curves whose windows they cannot tell apart (outliers above the flux, a flux
+// far from 1, no dip at all) so cost little more than the tiled kernel: 1520
+// periods of 62,363 points 33.6 to 9.8, 29.1 to 9.7 and 11.7 to 9.5 ms (8.5
+// with every window summed from the start), 4000 of 3,900 points 7.6 to 2.6, 3.3
+// to 2.4 and 2.6 to 2.3 ms (2.3); the code for it costs the Kepler-like search
+// 0.7 %, 16 curves of 4,000 points 0.9 %.  The count is of the search's pass over
+// the curve; which way a period takes changes none of its results.
+constexpr int kGivenUp = 32;
+
+__device__ __forceinline__ bool try_bounds(int given_up, int slot) { return given_up < kGivenUp || (slot & 15) == 0; }
+
+// (`then`: the count when the period began; others count too, so that it may
+// pass its ends by as many periods as are in flight)
+__device__ __forceinline__ void count_bounds(int* given_up, int then, bool fits)
+{
+    if (fits && then > 0) atomicSub(given_up, 1);
+    if (!fits && then < 2 * kGivenUp) atomicAdd(given_up, 1);
+}
+
+// The window search after the fold, for one period: by bounds, or left to the
+// tiled kernel.
+template <int T, bool kW>
+__device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet& ds, const DevChunk& dk, int slot, int lc,
+                                              int p, int buf, bool fill, bool ref)
+{
+    using M = Smem<T>;
+    M& S = *reinterpret_cast<M*>(smem);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const DevPlan& dp = ds.plans[lc];
+    if (warp == 0) {
+        list_durations(dp, ds.curves[lc].check, p, (int)dp.n, S.dur, S.ck, lane);
+        for (int k = lane; k < kEnergySpans; k += 32) S.energy[k] = 0.0f;
+        if (lane == 0) {
+            S.next = S.n_pass = S.sieved = S.tested = S.n_fin = S.dev = S.big = 0;
+            S.full = false;
+            S.wlow = INT_MAX;
+        }
+    }
+    if (threadIdx.x == 32) S.given_up = __ldcg(ds.curves[lc].given_up + (ref ? 1 : 0));
+    for (int i = threadIdx.x; i < M::kSieve; i += T) S.sieve[i] = kNone;
+    __syncthreads();
+    bool fits = false;
+    if (try_bounds(S.given_up, slot)) {   // (block-uniform)
+        fits = rule_out<T, kW>(S, ds, dk, slot, lc, p, buf);
+        if (threadIdx.x == 0 && (!fits || S.given_up > 0))
+            count_bounds(ds.curves[lc].given_up + (ref ? 1 : 0), S.given_up, fits);
+    }
+    if (!fits && warp == 0) {
         const int tc = kW ? ds.tiles[lc].count_w : ds.tiles[lc].count;
-        const long long to = atomicAdd(dk.work + kWorkDense, (unsigned int)tc);
-        // (there is room for every period of a wave; as far as there is room,
-        // every item that the tiled kernel will read is written)
-        in_range(ds.curves[lc].check, 24, to + tc - 1, dk.dense_cap);
-        for (int i = 0; i < tc && to + i < dk.dense_cap; ++i) dk.dense[to + i] = make_int2(slot, i | (S.ck.parts << 24));
+        const int parts = max(1, min(kDenseParts, (int)(tiled_time(dp, S.dur, S.ck.ndur, kW, lane) / (kPart * (float)tc))));
+        if (lane == 0) {
+            const long long to = atomicAdd(dk.work + kWorkDense, (unsigned int)tc);
+            // (there is room for every period of a wave; as far as there is room,
+            // every item that the tiled kernel will read is written)
+            in_range(ds.curves[lc].check, 24, to + tc - 1, dk.dense_cap);
+            for (int i = 0; i < tc && to + i < dk.dense_cap; ++i) dk.dense[to + i] = make_int2(slot, i | (parts << 24));
+        }
     }
     if (!kW && (fill || !fits)) {
-        // the folded curve itself and its exact prefix sums, for the kernels
-        // that sum every window
-        float* const r = dk.rs + (int64_t)slot * dk.pad_stride;
-        long long* const sums = dk.pf + (int64_t)slot * dk.pad_stride;
-        const int* const sidx = dk.sidx + (int64_t)slot * dk.fold_stride;
-        const PointVals* const pv = ds.curves[lc].pv;
-        long long* const scratch = reinterpret_cast<long long*>(smem);   // (dur[] is not read any more)
-        __syncthreads();
-        long long carry = 0;
-        for (int k0 = 0; k0 < total + (int)kPadMargin; k0 += T) {
-            const int k = k0 + threadIdx.x;
-            const int id = k < total ? sidx[k < n ? k : k - n] : -1;
-            const PointVals v = id >= 0 && id < n ? pv[id] : PointVals{0, 0.0f, 0.0f};
-            const long long before = block_exclusive_scan(v.rfx, scratch, scratch + 32) + carry;
-            if (k <= total) sums[k] = before;
-            if (k < total + (int)kPadMargin) r[k] = v.r;
-            carry += scratch[32];
-            __syncthreads();
-        }
+        __syncthreads();   // (dur[] is not read any more)
+        fill_folded<T>(dk.rs + (int64_t)slot * dk.pad_stride, dk.pf + (int64_t)slot * dk.pad_stride,
+                       dk.sidx + (int64_t)slot * dk.fold_stride, ds.curves[lc].pv, (int)dp.n, dp.dmax_p[p],
+                       reinterpret_cast<long long*>(smem));
     }
 }
 
