@@ -3189,7 +3189,9 @@ gtls_status create_device(gtls_plan* pl)
         // at every size: 40 points and 2e5 window-point products 150 against
         // 151 us by the tiled kernel, 257 and 6e7 196 against 207, 1000 and
         // 1.3e9 371 against 556 (own dy: 157, 245, 656 against 163, 253, 827)
-        pl->bounds_ok = !pl->has_tensor && !(h.prm.test_flags & 2);
+        // (more durations at a period than the tiled kernel lists: as there, an
+        // error at every curve, also when the bounds would leave it no period)
+        pl->bounds_ok = !pl->has_tensor && !(h.prm.test_flags & 2) && h.max_kept <= tiles::kMaxDur;
         std::vector<BoundTab> tab(dp.nd);
         std::vector<BoundDur> bd(dp.nd);
         Packed all;
