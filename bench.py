@@ -32,6 +32,7 @@ sys.path.insert(0, ROOT)
 
 METRIC = "Kepler-like light curves/hour on 1 GB300 (plain vs batched+learned, equal recall)"
 UNIT = "light curves/hour"
+SMS, MAX_SM_HZ = 152, 2.07e9   # GB300: SMs, maximum SM clock
 
 
 def _args():
@@ -194,30 +195,32 @@ def _kernel_sha():
     return h.hexdigest()[:16]
 
 
+def _ncu_profile(workload):
+    """Counters of the fold's kernel from the committed ncu summary
+    (profiles/fold_sort_<workload>.md, lines 'kernel_sha: ...' and
+    '<counter>_per_point: ...', per point and period), or None where it was
+    not taken on the current kernel."""
+    path = os.path.join(ROOT, "profiles", f"fold_sort_{workload}.md")
+    keys = ("warp_instructions_per_point", "dram_bytes_per_point")
+    vals = {}
+    try:
+        for line in open(path):
+            for key in ("kernel_sha",) + keys:
+                if line.strip().startswith(key + ":"):
+                    vals[key] = line.split(":", 1)[1].strip().strip("`")
+    except OSError:
+        return None
+    if vals.get("kernel_sha") != _kernel_sha() or not all(k in vals for k in keys):
+        return None
+    return {k: float(vals[k]) for k in keys}
+
+
 def _hbm_peak_gbs():
     """Measured copy bandwidth of this GPU type, or an earlier measurement."""
     try:
         return float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["hbm_gbs"]), "of measured"
     except (OSError, KeyError, ValueError):
         return 6800.0, "of fallback"
-
-
-def _ncu_traffic(workload):
-    """DRAM bytes per launch of the fold from the committed ncu summary
-    (profiles/fold_sort_<workload>.md, lines 'kernel_sha: ...' and
-    'dram_bytes_per_launch: ...'), if it was taken on the current kernel."""
-    path = os.path.join(ROOT, "profiles", f"fold_sort_{workload}.md")
-    vals = {}
-    try:
-        for line in open(path):
-            for key in ("kernel_sha", "dram_bytes_per_launch"):
-                if line.strip().startswith(key + ":"):
-                    vals[key] = line.split(":", 1)[1].strip().strip("`")
-    except OSError:
-        return None
-    if vals.get("kernel_sha") != _kernel_sha() or "dram_bytes_per_launch" not in vals:
-        return None
-    return float(vals["dram_bytes_per_launch"])
 
 
 def oracle_sample(lc, cpu_seconds):
@@ -537,20 +540,30 @@ def run_gtls(args):
         return 0
 
     # The fold, whose kernel also holds the bounds that leave one or two windows
-    # of a period to be summed, takes nearly all of the step.  It is bound by
-    # latency and instruction issue, not by bandwidth; the fraction says how far
-    # the bytes it has to move are from binding: per point and period a sort key
-    # written and read (16), the order (4) and the prefix sums (4; per-point
-    # weights: two of them, w, w r and exact sums of r, 24).
-    per_point = 24.0 if res.uniform_dy else 44.0
+    # of a period to be summed, takes nearly all of the step.  What binds it are
+    # issue slots and the shared-memory pipe (61 % and 55 % busy), not DRAM (6 %):
+    # the roofline is warp instructions, as ncu counts them per point and period,
+    # against one per cycle and scheduler.
     main_s = statistics.mean(s["ms_fold_sort"] + s["ms_window_search"] for s in stage) / 1000.0
-    achieved = per_point * info["n_periods"] * lc.n / main_s / 1e9
-    peak, basis = _hbm_peak_gbs()
-    roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                "frac": achieved / peak, "traffic": _ncu_traffic(args.workload),
-                "kernel": "k_fold_sort", "peak_basis": f"copy bandwidth, {basis}",
-                "achieved_basis": f"{per_point:.0f} bytes per point and period / mean time of the fold and "
-                                  "window-search stages (CUDA events on the search stream)"}
+    peak = SMS * 4 * MAX_SM_HZ / 1e9
+    prof = _ncu_profile(args.workload) if res.uniform_dy else None
+    points_s = info["n_periods"] * lc.n / main_s / 1e9
+    achieved = prof and prof["warp_instructions_per_point"] * points_s
+    hbm_peak, hbm_basis = _hbm_peak_gbs()
+    hbm = prof and prof["dram_bytes_per_point"] * points_s
+    per_launch = min(int(plan.info.periods_per_chunk), info["n_periods"])
+    roofline = {"bound": "issue", "achieved": achieved, "peak": peak, "unit": "G warp instructions/s",
+                "frac": achieved and achieved / peak,
+                "traffic": prof and prof["dram_bytes_per_point"] * lc.n * per_launch,
+                "kernel": "k_fold_sort",
+                "hbm": {"achieved": hbm, "peak": hbm_peak, "unit": "GB/s", "frac": hbm and hbm / hbm_peak,
+                        "peak_basis": f"copy bandwidth, {hbm_basis}"},
+                "peak_basis": f"{SMS} SMs x 4 schedulers x {MAX_SM_HZ / 1e6:.0f} MHz (max SM clock)",
+                "achieved_basis": "warp instructions per point and period (ncu, committed summary; null when the "
+                                  "kernel has changed since) x points x periods / mean time of the fold and "
+                                  "window-search stages (CUDA events on the search stream)",
+                "traffic_basis": f"DRAM bytes per point and period (the same summary) x points x the {per_launch} "
+                                 "periods of a launch"}
     cpu = None
     if not args.no_cpu_baseline:
         v, threads, desc, dt, frac = oracle_sample(lc, args.cpu_seconds)

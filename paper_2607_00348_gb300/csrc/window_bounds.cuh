@@ -52,7 +52,7 @@
 // exceeds the sum of the c up to l; the first test takes for W_l the smallest
 // sum of w over any stretch of the length (weight_floors), the segment test the
 // window's own, with its exact depth.  (20,011 points with a dy of their own: the
-// window stage was 98 ms on the tiled kernel, 126 with the fold; now 71 in all.)
+// window stage was 98 ms on the tiled kernel, 126 with the fold; now 66 in all.)
 //
 // What bounds it (62,363 points, thousand cycles of a period's CTA at 0.55 / 5 /
 // 100 days): at short periods waiting between the steps (energies and
@@ -89,7 +89,7 @@ constexpr int kDenseParts = 16;     // CTAs of the tiled kernel that share a til
 // points 10 % below 1, which have hundreds of nearly equal long windows.)
 constexpr float kTiledPoint = 0.014f, kTiledWindow = 0.5f, kTiledOwn = 1.7f;   // ns of an SM
 constexpr float kPart = 2e5f;       // a tile's share that another CTA is worth staging the tile for
-constexpr int kFew = 16;            // windows always cheaper to sum again
+constexpr int kFew = 64;            // windows that are not worth the estimate (at worst 1.6 times the tiled kernel)
 constexpr float kSieved = 10.0f;                                              // (two CTAs of an SM: half)
 constexpr float kListedPoint = 0.45f, kListedWindow = 300.0f, kListedRoom = 4096.0f;
 constexpr int kRowBuf = 168;        // prefix sums at whole T0 steps a warp stages for one group
