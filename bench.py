@@ -53,8 +53,7 @@ def _args():
     ap.add_argument("--refine", type=int, default=0,
                     help="periods re-searched with T0 step 1 after the coarse pass (Sect. 2.5)")
     ap.add_argument("--dy-jitter", type=float, default=0.0,
-                    help="multiply every dy by 1 + f * U(-1, 1) (seeded): per-point weights, which "
-                         "the one-thread-per-window kernel searches")
+                    help="multiply every dy by 1 + f * U(-1, 1) (seeded): per-point weights")
     ap.add_argument("--batch-curves", type=int, default=8,
                     help="curves of the uneven-length Kepler-like batch leg (0 = skip it)")
     ap.add_argument("--batch-steps", type=int, default=2)

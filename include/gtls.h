@@ -321,7 +321,8 @@ gtls_status gtls_plan_get_profile(const gtls_plan* plan, gtls_profile* out);
  * the process exits); larger inputs return GTLS_ERR_INVALID_ARG.
  *   chi2       device, n_periods doubles (input, read only)
  *   sr_out, sde_raw_out   device, n_periods doubles each, nullable (then
- *              kept in the fixed array)
+ *              kept in the fixed array); sr_out may share memory with the
+ *              other two, which are written after it
  *   sde_out    device, n_periods doubles (required)
  *   best_idx, best_sde    host, nullable: first index of the largest SDE
  *   median_window         0 => 2 floor(N_P/200) + 1, else odd
