@@ -3254,7 +3254,7 @@ gtls_status create_device(gtls_plan* pl)
     // chunk took 1013, 994 and 980 ms), whole waves of the fold (one CTA per
     // period and SM) when at least one fits
     {
-        const int64_t budget = int64_t(8) << 30;
+        const int64_t budget = (int64_t(8) << 30) - 8192;   // (less what aligning its arrays takes)
         const int64_t tiles = std::max({1, pl->tile_count, pl->tile_count_ref, pl->tile_count_w});
         int64_t chunk = std::max<int64_t>(1, budget / slot_bytes(dk, pl->bounds_ok ? tiles : 0));
         chunk = std::min<int64_t>(chunk, 4096);
@@ -3324,35 +3324,72 @@ gtls_status make_tc_maps(const DevChunk& dk, void* dev)
     return GTLS_OK;
 }
 
-// The chunk scratch of a plan's own searches (batches bring their own).
+// Takes the chunk scratch out of the plan's allocations and frees it.
+void free_chunk(gtls_plan* pl)
+{
+    void** const end = std::remove(pl->allocs, pl->allocs + pl->n_allocs, pl->chunk_mem);
+    pl->n_allocs = (int)(end - pl->allocs);
+    cudaFree(pl->chunk_mem);
+    pl->device_bytes -= pl->chunk_bytes;
+    pl->chunk_mem = nullptr;
+    pl->chunk_bytes = 0;
+    DevChunk none{};
+    none.chunk = pl->dk.chunk;
+    none.fold_stride = pl->dk.fold_stride;
+    none.key_stride = pl->dk.key_stride;
+    none.pad_stride = pl->dk.pad_stride;
+    pl->dk = none;
+    pl->tc_maps = nullptr;
+    pl->chunk_ready = false;
+}
+
+// The chunk scratch of a plan's own searches (batches bring their own): one
+// allocation (ten of them took a small plan's first search 100 us longer).
 gtls_status ensure_chunk(gtls_plan* pl)
 {
     if (pl->chunk_ready) return GTLS_OK;
-    DevChunk& dk = pl->dk;
+    DevChunk dk = pl->dk;
     const int64_t chunk = dk.chunk;
-    const int64_t bytes0 = pl->device_bytes;
-    GTLS_TRY(dev_alloc(pl, &dk.keys, chunk * dk.key_stride));
-    GTLS_TRY(dev_alloc(pl, &dk.sidx, chunk * dk.fold_stride));
-    GTLS_TRY(dev_alloc(pl, &dk.rs, chunk * dk.pad_stride));
-    GTLS_TRY(dev_alloc(pl, &dk.ws, chunk * dk.pad_stride));
-    GTLS_TRY(dev_alloc(pl, &dk.wrs, chunk * dk.pad_stride));
-    GTLS_TRY(dev_alloc(pl, &dk.pf, chunk * dk.pad_stride));
-    GTLS_TRY(dev_alloc(pl, &dk.work, kWorkWords));
+    unsigned char* maps = nullptr;
+    std::vector<std::pair<void*, int64_t>> parts;   // address of a pointer, its offset
+    int64_t bytes = 0;
+    auto part = [&](auto** ptr, int64_t count) {
+        parts.emplace_back(ptr, bytes);
+        bytes += (count * (int64_t)sizeof(**ptr) + 255) & ~int64_t(255);
+    };
+    part(&dk.keys, chunk * dk.key_stride);
+    part(&dk.sidx, chunk * dk.fold_stride);
+    part(&dk.rs, chunk * dk.pad_stride);
+    part(&dk.ws, chunk * dk.pad_stride);
+    part(&dk.wrs, chunk * dk.pad_stride);
+    part(&dk.pf, chunk * dk.pad_stride);
+    part(&dk.work, kWorkWords);
     if (pl->bounds_ok) {
-        GTLS_TRY(dev_alloc(pl, &dk.pq, chunk * dk.pad_stride));
+        part(&dk.pq, chunk * dk.pad_stride);
         dk.list_cap = std::max<int64_t>(4096, chunk * kListPerSlot);
-        GTLS_TRY(dev_alloc(pl, &dk.list, kListClasses * dk.list_cap));
+        part(&dk.list, kListClasses * dk.list_cap);
         dk.dense_cap = chunk * std::max({1, pl->tile_count, pl->tile_count_ref, pl->tile_count_w});
-        GTLS_TRY(dev_alloc(pl, &dk.dense, dk.dense_cap));
+        part(&dk.dense, dk.dense_cap);
     }
+    if (pl->has_tensor) part(&maps, (int64_t)(tc::kMaps * sizeof(CUtensorMap)));
+    unsigned char* base = nullptr;
+    GTLS_TRY(dev_alloc(pl, &base, (size_t)bytes));
+    for (const auto& [ptr, at] : parts) {
+        unsigned char* const p = base + at;
+        std::memcpy(ptr, &p, sizeof p);
+    }
+    pl->chunk_mem = base;
+    pl->chunk_bytes = bytes;
     if (pl->has_tensor) {
-        unsigned char* maps = nullptr;
-        GTLS_TRY(dev_alloc(pl, &maps, (size_t)tc::kMaps * sizeof(CUtensorMap)));
-        GTLS_TRY(make_tc_maps(dk, maps));
-        pl->tc_maps = maps;
+        const gtls_status s = make_tc_maps(dk, maps);
+        if (s != GTLS_OK) {
+            free_chunk(pl);
+            return s;
+        }
     }
+    pl->dk = dk;
+    pl->tc_maps = maps;
     pl->chunk_ready = true;
-    pl->chunk_bytes = pl->device_bytes - bytes0;
     return GTLS_OK;
 }
 
@@ -3361,31 +3398,7 @@ gtls_status trim_chunk(gtls_plan* pl)
 {
     if (!pl->chunk_ready) return GTLS_OK;
     GTLS_CUDA(cudaDeviceSynchronize());
-    const void* mine[] = {pl->dk.keys, pl->dk.sidx, pl->dk.rs, pl->dk.ws, pl->dk.wrs, pl->dk.pf,
-                          pl->dk.pq, pl->dk.list, pl->dk.dense, pl->dk.work, pl->tc_maps};
-    int kept = 0;
-    for (int i = 0; i < pl->n_allocs; ++i) {
-        bool chunk = false;
-        for (const void* m : mine) chunk = chunk || (m && m == pl->allocs[i]);
-        if (chunk) cudaFree(pl->allocs[i]);
-        else pl->allocs[kept++] = pl->allocs[i];
-    }
-    for (int i = kept; i < pl->n_allocs; ++i) pl->allocs[i] = nullptr;
-    pl->n_allocs = kept;
-    pl->device_bytes -= pl->chunk_bytes;
-    pl->chunk_bytes = 0;
-    const int32_t chunk = pl->dk.chunk;
-    pl->dk.keys = nullptr;
-    pl->dk.sidx = nullptr;
-    pl->dk.rs = pl->dk.ws = pl->dk.wrs = nullptr;
-    pl->dk.pf = nullptr;
-    pl->dk.dense = nullptr;
-    pl->dk.pq = nullptr;
-    pl->dk.list = nullptr;
-    pl->dk.work = nullptr;
-    pl->dk.chunk = chunk;
-    pl->tc_maps = nullptr;
-    pl->chunk_ready = false;
+    free_chunk(pl);
     return GTLS_OK;
 }
 
