@@ -3343,43 +3343,63 @@ void free_chunk(gtls_plan* pl)
     pl->chunk_ready = false;
 }
 
-// The chunk scratch of a plan's own searches (batches bring their own): one
-// allocation (ten of them took a small plan's first search 100 us longer).
+// The arrays of a chunk scratch, to be placed in one allocation (ten of them
+// took a small plan's first search 100 us longer).
+struct ChunkLayout {
+    std::vector<std::pair<void*, int64_t>> parts;   // address of a pointer, its offset
+    int64_t bytes = 0;
+
+    template <class T>
+    void part(T** ptr, int64_t count)
+    {
+        parts.emplace_back(ptr, bytes);
+        bytes += (count * (int64_t)sizeof(T) + 255) & ~int64_t(255);
+    }
+    void place(unsigned char* base) const
+    {
+        for (const auto& [ptr, at] : parts) {
+            unsigned char* const p = base + at;
+            std::memcpy(ptr, &p, sizeof p);
+        }
+    }
+};
+
+// Layout of dk's arrays (strides and slots set; sets the lists' capacities).
+// `tiles`: as for slot_bytes; maps: where the tensor-core kernel's TMA maps go, or null.
+ChunkLayout chunk_layout(DevChunk& dk, int64_t tiles, unsigned char** maps)
+{
+    ChunkLayout l;
+    const int64_t slots = dk.chunk;
+    l.part(&dk.keys, slots * dk.key_stride);
+    l.part(&dk.sidx, slots * dk.fold_stride);
+    l.part(&dk.rs, slots * dk.pad_stride);
+    l.part(&dk.ws, slots * dk.pad_stride);
+    l.part(&dk.wrs, slots * dk.pad_stride);
+    l.part(&dk.pf, slots * dk.pad_stride);
+    l.part(&dk.work, kWorkWords);
+    if (tiles > 0) {
+        l.part(&dk.pq, slots * dk.pad_stride);
+        dk.list_cap = std::max<int64_t>(4096, slots * kListPerSlot);
+        l.part(&dk.list, kListClasses * dk.list_cap);
+        dk.dense_cap = slots * tiles;
+        l.part(&dk.dense, dk.dense_cap);
+    }
+    if (maps) l.part(maps, (int64_t)(tc::kMaps * sizeof(CUtensorMap)));
+    return l;
+}
+
+// The chunk scratch of a plan's own searches (batches bring their own).
 gtls_status ensure_chunk(gtls_plan* pl)
 {
     if (pl->chunk_ready) return GTLS_OK;
     DevChunk dk = pl->dk;
-    const int64_t chunk = dk.chunk;
-    unsigned char* maps = nullptr;
-    std::vector<std::pair<void*, int64_t>> parts;   // address of a pointer, its offset
-    int64_t bytes = 0;
-    auto part = [&](auto** ptr, int64_t count) {
-        parts.emplace_back(ptr, bytes);
-        bytes += (count * (int64_t)sizeof(**ptr) + 255) & ~int64_t(255);
-    };
-    part(&dk.keys, chunk * dk.key_stride);
-    part(&dk.sidx, chunk * dk.fold_stride);
-    part(&dk.rs, chunk * dk.pad_stride);
-    part(&dk.ws, chunk * dk.pad_stride);
-    part(&dk.wrs, chunk * dk.pad_stride);
-    part(&dk.pf, chunk * dk.pad_stride);
-    part(&dk.work, kWorkWords);
-    if (pl->bounds_ok) {
-        part(&dk.pq, chunk * dk.pad_stride);
-        dk.list_cap = std::max<int64_t>(4096, chunk * kListPerSlot);
-        part(&dk.list, kListClasses * dk.list_cap);
-        dk.dense_cap = chunk * std::max({1, pl->tile_count, pl->tile_count_ref, pl->tile_count_w});
-        part(&dk.dense, dk.dense_cap);
-    }
-    if (pl->has_tensor) part(&maps, (int64_t)(tc::kMaps * sizeof(CUtensorMap)));
-    unsigned char* base = nullptr;
-    GTLS_TRY(dev_alloc(pl, &base, (size_t)bytes));
-    for (const auto& [ptr, at] : parts) {
-        unsigned char* const p = base + at;
-        std::memcpy(ptr, &p, sizeof p);
-    }
+    const int tiles = std::max({1, pl->tile_count, pl->tile_count_ref, pl->tile_count_w});
+    unsigned char *maps = nullptr, *base = nullptr;
+    const ChunkLayout l = chunk_layout(dk, pl->bounds_ok ? tiles : 0, pl->has_tensor ? &maps : nullptr);
+    GTLS_TRY(dev_alloc(pl, &base, (size_t)l.bytes));
+    l.place(base);
     pl->chunk_mem = base;
-    pl->chunk_bytes = bytes;
+    pl->chunk_bytes = l.bytes;
     if (pl->has_tensor) {
         const gtls_status s = make_tc_maps(dk, maps);
         if (s != GTLS_OK) {
@@ -4245,7 +4265,7 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     batch_tiles(b, b->cfg.tile_buf);
     int64_t max_tiles = 1;
     for (const DevTiles& t : b->tiles_host) max_tiles = std::max<int64_t>({max_tiles, t.count, t.count_w});
-    const int64_t budget = int64_t(16) << 30;
+    const int64_t budget = (int64_t(16) << 30) - 8192;   // (less what aligning its arrays takes)
     int64_t slots =
         std::min<int64_t>(4096, std::max<int64_t>(1, budget / slot_bytes(dk, b->bounds_ok ? max_tiles : 0)));
     if (b->n_sm > 0 && slots >= 4 * b->n_sm) slots = slots / (4 * b->n_sm) * (4 * b->n_sm);   // whole fold waves at 1, 1/2, 1/4
@@ -4253,22 +4273,15 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     b->max_slots = (int)slots;
     b->cfg.wave_slots = (int)slots;
     dk.chunk = (int32_t)slots;
-    GTLS_TRY(batch_alloc(b, &dk.keys, slots * key_stride));
-    GTLS_TRY(batch_alloc(b, &dk.sidx, slots * fold_stride));
-    GTLS_TRY(batch_alloc(b, &dk.rs, slots * pad_stride));
-    GTLS_TRY(batch_alloc(b, &dk.ws, slots * pad_stride));
-    GTLS_TRY(batch_alloc(b, &dk.wrs, slots * pad_stride));
-    GTLS_TRY(batch_alloc(b, &dk.pf, slots * pad_stride));
-    GTLS_TRY(batch_alloc(b, &dk.work, kWorkWords));
     {
         bool any_tensor = false;
         for (int i = 0; i < n_lc; ++i) any_tensor = any_tensor || plans[i]->has_tensor;
-        if (any_tensor) {
-            unsigned char* maps = nullptr;
-            GTLS_TRY(batch_alloc(b, &maps, (size_t)tc::kMaps * sizeof(CUtensorMap)));
-            GTLS_TRY(make_tc_maps(dk, maps));
-            b->tc_maps = maps;
-        }
+        unsigned char *maps = nullptr, *base = nullptr;
+        const ChunkLayout l = chunk_layout(dk, b->bounds_ok ? max_tiles : 0, any_tensor ? &maps : nullptr);
+        GTLS_TRY(batch_alloc(b, &base, (size_t)l.bytes));
+        l.place(base);
+        if (any_tensor) GTLS_TRY(make_tc_maps(dk, maps));
+        b->tc_maps = maps;
     }
 
     // per-curve descriptors
@@ -4305,13 +4318,6 @@ gtls_status batch_create(gtls_plan* const* plans, int64_t n_lc, int32_t wave_slo
     GTLS_TRY(batch_alloc(b, &b->q_cursors, 3 * (size_t)kMaxLoops));
     b->total_periods = total_periods;
     GTLS_TRY(batch_upload_tiles(b));
-    if (b->bounds_ok) {
-        b->dk.dense_cap = slots * max_tiles;
-        GTLS_TRY(batch_alloc(b, &b->dk.dense, b->dk.dense_cap));
-        GTLS_TRY(batch_alloc(b, &b->dk.pq, slots * pad_stride));
-        b->dk.list_cap = std::max<int64_t>(4096, slots * kListPerSlot);
-        GTLS_TRY(batch_alloc(b, &b->dk.list, kListClasses * b->dk.list_cap));
-    }
     return GTLS_OK;
 }
 
