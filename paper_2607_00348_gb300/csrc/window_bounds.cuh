@@ -157,7 +157,8 @@ struct Smem {
     Chunks ck;
     int next, n_pass, sieved, n_fin, dev, big;
     bool full;                                       // a list of the wave is
-    int given_up;                                    // DevCurve::given_up when the period began
+    int* given_at;                                   // the curve's DevCurve::given_up of this pass,
+    int given_up;                                    // and what it was when the period began
     int tested;                                      // windows that went through the sieve
     float wsum[kWarps], energy[kEnergySpans];
     float top[kWarps], c1[kWarps], s[kWarps];
@@ -678,7 +679,10 @@ __device__ __forceinline__ bool rule_out(Smem<T>& S, const DevSet& ds, const Dev
         return fmaxf(0.0f, (float)(pq[s + d] - pq[s]) * unit * inv);
     };
 
-    const Chunks ck = S.ck;
+    // (in registers only at 256 threads, whose CTAs wait for shared memory more
+    // than the spills cost: 1440 points 0.597 against 0.615 ms; 16 curves of 4,000
+    // points, at 512 threads, 250.8 against 247.3 ms)
+    std::conditional_t<T == 256, const Chunks, const Chunks&> ck = S.ck;
     const int ndur = ck.ndur;
     {
         // the plan's part of the durations
@@ -1321,7 +1325,7 @@ __device__ __noinline__ void fill_folded(float* r, long long* sums, const int* s
 // periods of 62,363 points 33.6 to 9.8, 29.1 to 9.7 and 11.7 to 9.5 ms (8.5
 // with every window summed from the start), 4000 of 3,900 points 7.6 to 2.6, 3.3
 // to 2.4 and 2.6 to 2.3 ms (2.3); the code for it costs the Kepler-like search
-// 0.7 %, 16 curves of 4,000 points 0.9 %.  The count is of the search's pass over
+// 0.3 %, curves of 1440 points 1 %.  The count is of the search's pass over
 // the curve; which way a period takes changes none of its results.
 constexpr int kGivenUp = 32;
 
@@ -1354,14 +1358,17 @@ __device__ __forceinline__ void window_bounds(unsigned char* smem, const DevSet&
             S.wlow = INT_MAX;
         }
     }
-    if (threadIdx.x == 32) S.given_up = __ldcg(ds.curves[lc].given_up + (ref ? 1 : 0));
+    if (threadIdx.x == 32) {
+        S.given_at = ds.curves[lc].given_up + (ref ? 1 : 0);
+        S.given_up = __ldcg(S.given_at);
+    }
     for (int i = threadIdx.x; i < M::kSieve; i += T) S.sieve[i] = kNone;
     __syncthreads();
     bool fits = false;
     if (try_bounds(S.given_up, slot)) {   // (block-uniform)
         fits = rule_out<T, kW>(S, ds, dk, slot, lc, p, buf);
         if (threadIdx.x == 0 && (!fits || S.given_up > 0))
-            count_bounds(ds.curves[lc].given_up + (ref ? 1 : 0), S.given_up, fits);
+            count_bounds(S.given_at, S.given_up, fits);
     }
     if (!fits && warp == 0) {
         const int tc = kW ? ds.tiles[lc].count_w : ds.tiles[lc].count;
