@@ -85,8 +85,9 @@ constexpr int kDenseParts = 16;     // CTAs of the tiled kernel that share a til
 // 630 at 62,363), a listed window by its points, of which kListedRoom halve the
 // CTAs that an SM holds (0.6 us for 600 points, 2.5 us for 2,900, 13 to 16 us for
 // 9,000), and a window of the sieve its segment test (19 cycles of the CTA): a
-// period whose sieve takes longer than its tiles is given up there.  (A fixed limit of a window in 512: 27 ms for 1520 periods of 62,363
-// points 10 % below 1, which have hundreds of nearly equal long windows.)
+// period whose sieve takes longer than its tiles is given up there.  (A fixed
+// limit of a window in 512: 27 ms for 1520 periods of 62,363 points 10 % below
+// 1, which have hundreds of nearly equal long windows.)
 constexpr float kTiledPoint = 0.014f, kTiledWindow = 0.5f, kTiledOwn = 1.7f;   // ns of an SM
 constexpr float kPart = 2e5f;       // a tile's share that another CTA is worth staging the tile for
 constexpr int kFew = 64;            // windows that are not worth the estimate (at worst 1.6 times the tiled kernel)
